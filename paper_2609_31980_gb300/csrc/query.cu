@@ -742,149 +742,6 @@ __global__ void __launch_bounds__(kQueryWarps * 32, QCfg<D, STAGE>::MINB) k_grid
     }
 }
 
-// ------------------------------------------------------------- overflow path
-// Exact selection for queries with more than kListCap neighbours (whether or
-// not that exceeds K): one warp per query scans the query's own +-m
-// neighbourhood with lanes over candidates, appends keys below the current
-// threshold to a shared buffer, and whenever the buffer is nearly full sorts
-// it and keeps the K smallest (the threshold becomes the K-th key).  Keys are
-// unique (indices differ), so the K smallest are unique.  The kernel always
-// follows the grid query on its stream; its last block to finish clears the
-// query's chunk counter (and, unless a compact fill pass still needs the
-// overflow list, the list) for the next query, so no host-side memset
-// interrupts the chain of programmatically dependent launches.
-
-constexpr int kOvfWarps = 4;
-
-__device__ void smem_bitonic(uint64_t* buf, int n) {
-    const int lane = threadIdx.x & 31;
-    for (int k = 2; k <= n; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            __syncwarp();
-            for (int i = lane; i < n / 2; i += 32) {
-                const int lo = ((i & ~(j - 1)) << 1) | (i & (j - 1));
-                const int hi = lo + j;
-                const bool up = (lo & k) == 0;
-                const uint64_t x = buf[lo], y = buf[hi];
-                if ((x > y) == up) {
-                    buf[lo] = y;
-                    buf[hi] = x;
-                }
-            }
-        }
-    }
-    __syncwarp();
-}
-
-__global__ void __launch_bounds__(kOvfWarps * 32) k_overflow(QueryArgs a, int cap) {
-    pdl_trigger();
-    pdl_wait();
-    extern __shared__ __align__(16) unsigned char smem_o[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint64_t* buf = reinterpret_cast<uint64_t*>(smem_o) + (size_t)warp * cap;
-    const int nov = min(*a.ovf_count, a.ovf_cap);
-    const int D = a.D, K = a.K;
-    const int DP = padded_dim(D);
-    for (int w = blockIdx.x * kOvfWarps + warp; w < nov; w += gridDim.x * kOvfWarps) {
-        const Overflow o = a.ovf[w];
-        const EventHdr& h = a.ev[o.ev];
-        int32_t* oidx = a.counts ? a.idx : h.idx;
-        float* od2 = a.counts ? a.dist2 : h.dist2;
-        const int qs = o.qslot;
-        const int qo = a.qperm[qs];
-        float qv[kMaxD];
-#pragma unroll
-        for (int k = 0; k < kMaxD; ++k) qv[k] = k < D ? a.qpts[pt_index(qs, k, DP)] : 0.f;
-        const int qc = a.qcell[qs];
-        const int dims0 = h.dims[0], m = h.m;
-        const int x = qc % dims0, qrow = qc / dims0;
-        const int self_slot = a.self ? qs : -1;
-        const bool count_only = a.ovf_mode == 1;
-        int fill = 0;
-        int64_t deg = 0;
-        uint64_t thr = ~0ull;
-        for (int i = lane; i < cap && !count_only; i += 32) buf[i] = ~0ull;
-        __syncwarp();
-        const int nrows = neighbour_rows(h);
-        for (int nr = 0; nr < nrows; ++nr) {
-            int64_t rowbase;
-            if (!neighbour_row(h, qrow, nr, rowbase)) continue;
-            {
-                const int rs = a.cstart[rowbase + max(x - m, 0)];
-                const int re = a.cstart[rowbase + min(x + m, dims0 - 1) + 1];
-                for (int c0 = rs; c0 < re; c0 += 32) {
-                    const int cs = c0 + lane;
-                    uint64_t key = ~0ull;
-                    if (cs < re && cs != self_slot) {
-                        float s = 0.f;
-#pragma unroll
-                        for (int k = 0; k < kMaxD; ++k) {
-                            if (k < D) {
-                                const float d = __fsub_rn(qv[k], a.rpts[pt_index(cs, k, DP)]);
-                                s = __fadd_rn(s, __fmul_rn(d, d));
-                            }
-                        }
-                        if (s <= a.r2) {
-                            ++deg;
-                            if (!count_only) {
-                                key = make_key(s, a.rperm[cs]);
-                                if (key >= thr) key = ~0ull;
-                            }
-                        }
-                    }
-                    if (count_only) continue;
-                    const unsigned bal = __ballot_sync(kFull, key != ~0ull);
-                    if (key != ~0ull) buf[fill + __popc(bal & ((1u << lane) - 1u))] = key;
-                    fill += __popc(bal);
-                    if (fill > cap - 32) {
-                        smem_bitonic(buf, cap);
-                        for (int i = K + lane; i < cap; i += 32) buf[i] = ~0ull;
-                        fill = K;
-                        thr = buf[K - 1];
-                        __syncwarp();
-                    }
-                }
-            }
-        }
-        for (int o2 = 16; o2 > 0; o2 >>= 1) deg += __shfl_xor_sync(kFull, deg, o2);
-        const int32_t c = (int32_t)(deg < K ? deg : K);
-        if (count_only) {
-            // compact output, first pass: the row's count (marked) and degree
-            if (lane == 0) {
-                (a.counts ? a.counts : h.counts)[qo] = c | kCsrSpill;
-                if (a.degree) a.degree[qo] = (int32_t)(deg < INT32_MAX ? deg : INT32_MAX);
-            }
-            continue;
-        }
-        const bool csr_rows = a.ovf_mode == 2;
-        // a compact output too small for the rows (its caller fails the
-        // call) is not written past its end
-        if (csr_rows && a.row_off[qo] + c > a.row_cap) continue;
-        smem_bitonic(buf, cap);
-        int32_t* irow = oidx + (csr_rows ? a.row_off[qo] : (int64_t)qo * K);
-        float* drow = od2 + (csr_rows ? a.row_off[qo] : (int64_t)qo * K);
-        for (int e = lane; e < (csr_rows ? c : K); e += 32) {
-            const uint64_t v = buf[e];
-            const bool real = v != ~0ull;
-            irow[e] = real ? (int32_t)(uint32_t)v : -1;
-            drow[e] = real ? __uint_as_float((uint32_t)(v >> 32)) : INFINITY;
-        }
-        if (lane == 0 && !csr_rows) (a.counts ? a.counts : h.counts)[qo] = c;
-        __syncwarp();
-    }
-    // the last block to finish clears the query's counters for the next launch
-    __syncthreads();
-    if (threadIdx.x == 0 && a.ovf_done) {
-        __threadfence();
-        if (atomicAdd(a.ovf_done, 1) == (int)gridDim.x - 1) {
-            *a.task_counter = 0;
-            if (a.reset_ovf) *a.ovf_count = 0;
-            __threadfence();
-            *a.ovf_done = 0;
-        }
-    }
-}
-
 // ------------------------------------------------------------- host launch
 
 template <int D, int STAGE>
@@ -998,24 +855,6 @@ frnn_status enqueue_overflow_only(const QueryLaunch& q, cudaStream_t st, std::st
     o.reset_ovf = 1;   // the fill pass consumes the list
     q.qset->ovf_stale = false;
     return enqueue_overflow(o, q.num_sms, st, err);
-}
-
-frnn_status enqueue_overflow(const QueryArgs& a, int num_sms, cudaStream_t st, std::string& err) {
-    // buffer of a power of two >= 2K keys per warp
-    int cap = 64;
-    while (cap < 2 * a.K) cap <<= 1;
-    const size_t osmem = (size_t)kOvfWarps * cap * sizeof(uint64_t);
-    cudaError_t ce =
-        cudaFuncSetAttribute(k_overflow, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)osmem);
-    if (ce == cudaSuccess) {
-        launch_pdl(k_overflow, dim3(num_sms), dim3(kOvfWarps * 32), osmem, st, a, cap);
-        ce = cudaGetLastError();
-    }
-    if (ce != cudaSuccess) {
-        err = std::string("selection kernel launch failed: ") + cudaGetErrorString(ce);
-        return FRNN_ERR_CUDA;
-    }
-    return FRNN_OK;
 }
 
 }  // namespace frnn
