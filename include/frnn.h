@@ -102,13 +102,15 @@ frnn_status frnn_destroy(frnn_ctx* ctx);
  *   grid  in/out.  If *grid is NULL a new grid is allocated.  If *grid is a
  *         grid from this context with D equal and capacity >= N, it is rebuilt
  *         in place without allocating (the previous contents are replaced).
- * The grid bins at most 5 coordinates (by default up to D = 8 the last
- * min(D, 5), or the last 4 when the cell budget would make five-axis cells
- * too coarse; from D = 9 the last 4; see FRNN_OPT_GRID_NAXES and
- * FRNN_OPT_GRID_AXES) with cells of edge (r/m)(1+2^-10), m = the
- * cell-multiple option, enlarged when needed so that the cell count stays
- * bounded; the choice never changes results (the cell assignment is proven
- * conservative).  A non-finite coordinate makes frnn_sync return
+ * The grid bins at most 5 coordinates (by default the last min(D, 5), or
+ * fewer when the cell budget would make the cells too coarse; from D = 9, up
+ * to 16,384 points or in a context with a memory budget, the last 4; see
+ * FRNN_OPT_GRID_NAXES and FRNN_OPT_GRID_AXES) with cells of edge
+ * (r/m)(1+2^-10), m = the cell-multiple option, enlarged when needed so that
+ * the cell count stays bounded.  The default grid of five or more dimensions
+ * stores cells two by two along every axis but the first and may divide them
+ * along one more coordinate.  The choice never changes results (the cell
+ * assignment is proven conservative).  A non-finite coordinate makes frnn_sync return
  * FRNN_ERR_NONFINITE and later queries on the grid return no neighbours.
  */
 frnn_status frnn_build_grid(frnn_ctx* ctx, const float* refs, int64_t N, int D, float r,
@@ -127,7 +129,9 @@ typedef struct frnn_grid_info {
     int64_t cells;      /* product of dims */
     int kernel;         /* grid scan used for this grid: 0 chunks of 16 queries
                            (candidates on lanes), 1 row tasks of 16 queries
-                           (grids requested with up to four axes) */
+                           (grids requested with up to four axes).  axes, dims
+                           and cells leave out the coordinate that a default
+                           grid may divide its cells along besides these */
     int valid;          /* 0 if a coordinate was non-finite */
 } frnn_grid_info;
 
@@ -283,9 +287,9 @@ const char* frnn_last_error(const frnn_ctx* ctx);
 /*
  * Autotuner.  Times the candidate configurations on the given point set (a
  * representative event, device memory, self-query): the automatic axis
- * choice with cell multiple m = 1 (five coordinates, or four when the cell
- * budget makes five-axis cells too coarse; scanned by chunks of 16 queries,
- * candidates on lanes, either candidate staging), four coordinates with
+ * choice with cell multiple m = 1 (scanned by chunks of 16 queries,
+ * candidates on lanes; up to D = 4 with either candidate staging), four
+ * coordinates with
  * m = 1 and three with m = 2 (scanned by 16-query row tasks, at the default
  * and a later warp vote); fewer axes when D is smaller; for D <= 4 the
  * automatic choice with m = 2 as well, and for D <= 3 with m = 3 (where
@@ -341,10 +345,12 @@ typedef enum frnn_option {
                                  with frnn_kernel_times; 0 (default): off.
                                  Setting it discards recorded pairs. */
     FRNN_OPT_GRID_NAXES = 10, /* gridded coordinates: 1..5 (at most D); 0
-                                 (default): autotuned, else up to D = 8 the
-                                 build's choice between min(D, 5) and one
-                                 fewer (the smaller expected neighbourhood
-                                 under the cell budget), from D = 9 four.
+                                 (default): autotuned, else the build's
+                                 choice (the smallest expected neighbourhood
+                                 under the cell budget among min(D, 5) axes,
+                                 one fewer and, from D = 6, one more), from
+                                 D = 9 four for up to 16,384 points or under
+                                 a memory budget.
                                  Grids requested with 1..4 axes are scanned by
                                  16-query row tasks, five-axis and automatic
                                  ones by 16-query chunks.  The cell multiple
@@ -355,7 +361,9 @@ typedef enum frnn_option {
                                  loads its candidate's row from global memory
                                  (L2), the next round in flight; 2 bulk copies
                                  (cp.async.bulk) of tiles into a shared-memory
-                                 ring; 0 (default): autotuned, else 1 */
+                                 ring; 0 (default): autotuned, else 1.  The
+                                 default grids of five or more dimensions and
+                                 row tasks have one staging each */
 } frnn_option;
 
 frnn_status frnn_set_option(frnn_ctx* ctx, frnn_option opt, int64_t value);

@@ -19,6 +19,7 @@ struct frnn_grid {
     int D = 0;
     float r = 0.f;
     int naxes = 0;   // gridded axes requested at the build
+    bool half = false;   // half cells (half_cells at the build)
 };
 
 struct frnn_ctx {
@@ -43,6 +44,7 @@ struct frnn_ctx {
     // workspaces
     GridBufs qset;            // cross-set query binning
     GridBufs batch;           // batched multi-event grid
+    int64_t batch_points = 0; // points of the batched call being served (0 outside of one)
     frnn_grid* host_grid = nullptr;   // grid of the host-buffer path
     void* hp_buf = nullptr;   // device buffers of the host-buffer path
     size_t hp_bytes = 0;
@@ -171,6 +173,7 @@ static size_t predict_grid_bytes(int E, const int64_t* n, int D, const int64_t* 
 }
 
 static int build_naxes(const frnn_ctx* ctx, int64_t N, int D);
+static int build_mult(const frnn_ctx* ctx, int64_t N, int D);
 // gridded axes a cell budget is sized for: the requested count, or for the
 // automatic choice (0) the most the build may take
 static int cap_axes(int naxes, int D) { return naxes > 0 ? naxes : std::min(D, kMaxAxes); }
@@ -179,7 +182,9 @@ static frnn_status alloc_accounted(frnn_ctx* c, GridBufs& g, int E, const int64_
                                    const int64_t* caps_in) {
     std::vector<int64_t> caps(E);
     for (int e = 0; e < E; ++e)
-        caps[e] = caps_in ? caps_in[e] : cell_cap_for(n[e], cap_axes(build_naxes(c, n[e], D), D));
+        caps[e] = caps_in ? caps_in[e]
+                          : cell_cap_for(n[e], cap_axes(build_naxes(c, n[e], D), D),
+                                         half_cells(D, build_naxes(c, n[e], D), build_mult(c, n[e], D)));
     const size_t old_bytes = g.bytes;
     const size_t need = predict_grid_bytes(E, n, D, caps.data());
     const bool reuse = g.base && need <= g.bytes;
@@ -288,18 +293,26 @@ static int build_mult(const frnn_ctx* ctx, int64_t N, int D) {
     const int na = build_naxes(ctx, N, D);
     return (na >= 1 && na <= 3 && D > 3) ? 2 : 1;
 }
-// gridded axes when neither the option nor the tuner fixes them.  Up to
-// D = 8: 0, the build's automatic choice (five axes, or four when the cell
-// budget makes five-axis cells too coarse; all of them for D < 5), scanned by
-// the chunk kernel.  From D = 9: four axes, scanned by the row-task kernel,
-// whose packed pre-screen costs less per candidate pair than the chunk
-// kernel's whole contract as D grows (measured build + query: 300k x 8 event
-// 0.306 ms five axes vs 0.318 ms four; 500k x 12 event 0.639 vs 0.546 ms).
-static int default_naxes(int D) { return D >= 9 ? 4 : 0; }
+// gridded axes when neither the option nor the tuner fixes them: 0, the
+// build's automatic choice (all of them for D < 5; from D = 5 half cells, six
+// to four axes).  From D = 9 three kinds of sets keep four axes and the
+// row-task scan: up to kRowsDefaultMax points, where that grid is the
+// documented default that frnn_grid_params reports (the half-cell scan is the
+// faster one there too: 13k x 12 points 41 against 61 us, build + query);
+// contexts with a memory budget, whose calls were sized for the four-axis
+// grid's smaller cell array; and batches whose cell arrays would not fit
+// their 2^30 entries.  Measured above that line (build + query, K = 64, row
+// tasks / half cells): 20k x 12 65 / 44 us, 100k x 12 128 / 77, 300k x 9
+// 313 / 167, 300k x 16 327 / 235.
+constexpr int64_t kRowsDefaultMax = 16384;
+constexpr int64_t kHalfBatchMax = (int64_t)1 << 26;   // points of a batch
+static int default_naxes(const frnn_ctx* ctx, int64_t N, int D) {
+    return D >= 9 && (N <= kRowsDefaultMax || ctx->budget != 0 || ctx->batch_points > kHalfBatchMax) ? 4 : 0;
+}
 static int build_naxes(const frnn_ctx* ctx, int64_t N, int D) {
     if (ctx->grid_naxes > 0) return std::min(ctx->grid_naxes, D);
     const frnn_ctx::Tuned* t = find_tuned(ctx, N, D, -1);
-    return std::min(t ? t->naxes : default_naxes(D), D);
+    return std::min(t ? t->naxes : default_naxes(ctx, N, D), D);
 }
 // default path when nothing is tuned: the tensor-core pre-filter beats the
 // grid scan over three gridded axes from about D = 10 on (0.90 vs 1.26 ms at
@@ -376,13 +389,13 @@ frnn_status frnn_grid_params(const frnn_grid* grid, frnn_grid_info* info) {
     EventHdr h{};
     if (e == cudaSuccess) e = cudaMemcpy(&h, grid->g.hdr, sizeof(h), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "reading the grid header");
-    info->naxes = h.naxes;
+    info->naxes = std::min(h.naxes, kMaxAxes);
     info->cell_mult = h.m;
     info->cells = 1;
     for (int a = 0; a < kMaxAxes; ++a) {
         info->axes[a] = a < h.naxes ? h.axes[a] : 0;
-        info->dims[a] = h.dims[a];
-        info->cells *= h.dims[a];
+        info->dims[a] = h.fdims[a];
+        info->cells *= h.fdims[a];
     }
     info->cell_edge = h.inv_h > 0.f ? 1.f / h.inv_h : INFINITY;
     info->valid = h.valid;
@@ -491,6 +504,8 @@ frnn_status frnn_build_grid(frnn_ctx* ctx, const float* refs, int64_t N, int D, 
     o.naxes = build_naxes(ctx, N, D);
     o.axes_mode = ctx->axes_mode;
     g->naxes = o.naxes;
+    g->half = half_cells(D, o.naxes, o.m);
+    g->g.h_hdr[0].half = g->half ? 1 : 0;
     std::string err;
     const float* ev_refs[1] = {refs};
     s = enqueue_build(g->g, ev_refs, o, nullptr, ctx->d_status, ctx->stream, false, err);
@@ -597,7 +612,7 @@ static frnn_status query_impl(frnn_ctx* ctx, const frnn_grid* grid, const float*
         q.tc_stats = ctx->d_tcstat;
         s = enqueue_tc_query(q, ctx->stream, err);
     } else {
-        q.kernel = grid_kernel(grid->naxes);
+        q.kernel = grid->half ? 2 : grid_kernel(grid->naxes);
         if (q.kernel == 1) {
             s = prepare_rows(ctx, rg, ctx->stream);
             if (s == FRNN_OK && !self) s = prepare_rows(ctx, ctx->qset, ctx->stream);
@@ -737,21 +752,25 @@ static bool same_events(const frnn_ctx* c, const frnn_event* ev, int n) {
     return true;
 }
 
-// Path of one event of a batch: 0 grid scan by chunks, 2 grid scan by row
-// tasks, 1 tensor core (autotuned per size class, else the defaults).
+// Path of one event of a batch: 0 grid scan by chunks, 3 half-cell scan, 2
+// grid scan by row tasks, 1 tensor core (autotuned per size class, else the
+// defaults).
 static int batch_path(const frnn_ctx* ctx, int64_t n, int D, int K, unsigned flags) {
     if (use_tc_path(ctx, D, flags, n, K)) return 1;
-    return grid_kernel(build_naxes(ctx, n, D)) == 1 ? 2 : 0;
+    const int naxes = build_naxes(ctx, n, D);
+    if (half_cells(D, naxes, build_mult(ctx, n, D))) return 3;
+    return grid_kernel(naxes) == 1 ? 2 : 0;
 }
 
-// ev: ordered by path (chunks, row tasks, tensor core), so that each path's
-// events occupy one range of chunks, cell-array entries and slots.
+// ev: ordered by path (chunks, half cells, row tasks, tensor core), so that
+// each path's events occupy one range of chunks, cell-array entries and slots.
 static frnn_status enqueue_batched(frnn_ctx* ctx, const frnn_event* ev, int n_events, int D,
                                    float r, int K, unsigned flags, bool capturing,
                                    cudaStream_t st) {
     std::vector<const float*> refs(n_events);
-    bool any_path[3] = {false, false, false};
-    int first_rows = n_events, first_tc = n_events;   // first event of each later path
+    bool any_path[4] = {false, false, false, false};
+    // first event of each later path
+    int first_half = n_events, first_rows = n_events, first_tc = n_events;
     for (int e = 0; e < n_events; ++e) {
         refs[e] = ev[e].pts;
         EventHdr& h = ctx->batch.h_hdr[e];
@@ -762,13 +781,16 @@ static frnn_status enqueue_batched(frnn_ctx* ctx, const frnn_event* ev, int n_ev
         h.m = build_mult(ctx, ev[e].n, D);
         h.naxes = build_naxes(ctx, ev[e].n, D);
         h.path = batch_path(ctx, ev[e].n, D, K, flags);
+        h.half = h.path == 3 ? 1 : 0;
         if (ev[e].n > 0) any_path[h.path] = true;
-        if (h.path != 0 && first_rows == n_events) first_rows = e;
+        if (h.path != 0 && first_half == n_events) first_half = e;
+        if (h.path != 0 && h.path != 3 && first_rows == n_events) first_rows = e;
         if (h.path == 1 && first_tc == n_events) first_tc = e;
     }
     const GridBufs& gb = ctx->batch;
     const auto slot_of = [&](int e) { return e < n_events ? gb.h_hdr[e].pt_off : gb.n_total; };
-    const bool any_grid = any_path[0], any_rows = any_path[2], any_tc = any_path[1];
+    const bool any_half = any_path[3], any_rows = any_path[2], any_tc = any_path[1];
+    const bool any_grid = any_path[0] || (!any_half && !any_rows && !any_tc);
     BuildOpts o;
     o.r = r;
     o.m = 1;
@@ -787,14 +809,22 @@ static frnn_status enqueue_batched(frnn_ctx* ctx, const frnn_event* ev, int n_ev
     q.stage = ctx->staging == 2 ? 1 : 0;
     q.d_status = ctx->d_status;
     q.num_sms = ctx->num_sms;
-    const bool mixed = (int)any_grid + (int)any_rows + (int)any_tc > 1;
-    if (any_grid || (!any_tc && !any_rows)) {
+    const bool mixed = (int)any_grid + (int)any_half + (int)any_rows + (int)any_tc > 1;
+    // the chunk scans: each ends at the chunks of the next path's events
+    if (any_grid) {
         q.kernel = 0;
         q.path_filter = mixed ? 0 : -1;
-        // the chunks of the chunk-scan events only
-        if (mixed && first_rows < n_events) q.chunk_end = gb.h_hdr[first_rows].qchunk0;
+        if (mixed && first_half < n_events) q.chunk_end = gb.h_hdr[first_half].qchunk0;
         s = enqueue_grid_query(q, st, err);
         if (s != FRNN_OK) return fail(ctx, s, err);
+    }
+    if (any_half) {
+        q.kernel = 2;
+        q.path_filter = mixed ? 3 : -1;
+        q.chunk_end = mixed && first_rows < n_events ? gb.h_hdr[first_rows].qchunk0 : -1;
+        s = enqueue_grid_query(q, st, err);
+        if (s != FRNN_OK) return fail(ctx, s, err);
+        q.kernel = 0;
     }
     if (any_rows) {
         // buffers were reserved before any capture; enqueue their build
@@ -855,6 +885,11 @@ frnn_status frnn_query_batched(frnn_ctx* ctx, const frnn_event* ev, int n_events
         if (x.n > 0 && (!x.pts || !x.counts || !x.idx || !x.dist2))
             return fail(ctx, FRNN_ERR_INVALID_ARG, "event pointer is NULL");
     }
+    struct BatchPoints {   // for the default axis choice while this call runs
+        frnn_ctx* c;
+        ~BatchPoints() { c->batch_points = 0; }
+    } batch_points{ctx};
+    for (int e = 0; e < n_events; ++e) ctx->batch_points += ev[e].n;
     const frnn_event* caller_ev = ev;
     const int opts[5] = {ctx->cell_mult, ctx->axes_mode, ctx->exit_dims, ctx->grid_naxes,
                          ctx->staging};
@@ -867,12 +902,12 @@ frnn_status frnn_query_batched(frnn_ctx* ctx, const frnn_event* ev, int n_events
         ctx->graph = nullptr;
         ctx->g_ev.clear();
     }
-    // the batch in path order (chunk scan, row-task scan, tensor core; stable
+    // the batch in path order (chunk scan, half-cell scan, row-task scan, tensor core; stable
     // within a path): each path's preparation and launch then covers only
     // its own events' chunks, cells and slots
     std::vector<frnn_event> ordered;
     ordered.reserve(n_events);
-    for (int want : {0, 2, 1})
+    for (int want : {0, 3, 2, 1})
         for (int e = 0; e < n_events; ++e)
             if (batch_path(ctx, ev[e].n, D, K, flags) == want) ordered.push_back(ev[e]);
     ev = ordered.data();
@@ -1305,7 +1340,7 @@ frnn_status frnn_autotune(frnn_ctx* ctx, const float* refs, int64_t N, int D, fl
         if (!(flags & FRNN_PATH_TC)) {
             if (grid_kernel(gcfg[gi].naxes) == 0) {
                 cands.push_back({FRNN_PATH_GRID, 1, 0});
-                cands.push_back({FRNN_PATH_GRID, 2, 0});
+                if (!half_cells(D, gcfg[gi].naxes, m)) cands.push_back({FRNN_PATH_GRID, 2, 0});
             } else {
                 cands.push_back({FRNN_PATH_GRID, 1, 0});
                 if (D >= 5) cands.push_back({FRNN_PATH_GRID, 1, 3});

@@ -130,17 +130,24 @@ __device__ __forceinline__ int cell_coord(float x, float lo, float hi, float inv
     return min(max(c, 0), dim - 1);
 }
 
+// A point's `cell` entry: its cell id (of a grid of half cells: the stored
+// cell id and the half bits).
 template <class Row>
 __device__ __forceinline__ int point_cell(const Row& p, const EventHdr& h) {
-    int c = 0, stride = 1;
+    int c = 0, stride = 1, bits = 0;
 #pragma unroll
-    for (int a = 0; a < kMaxAxes; ++a) {
+    for (int a = 0; a < kHdrAxes; ++a) {
         if (a < h.naxes) {
-            c += cell_coord(p[h.axes[a]], h.lo[a], h.hi[a], h.inv_h, h.dims[a]) * stride;
+            int x = cell_coord(p[h.axes[a]], h.lo[a], h.hi[a], h.inv_h, h.fdims[a]);
+            if (a > 0 && h.half) {
+                bits |= (x & 1) << (a - 1);
+                x >>= 1;
+            }
+            c += x * stride;
             stride *= h.dims[a];
         }
     }
-    return c;
+    return h.half ? (c << kHalfBits) | bits : c;
 }
 
 // ------------------------------------------------------------------ kernels
@@ -283,20 +290,21 @@ __global__ void __launch_bounds__(kBuildPtsPerBlock, 6) k_bbox(EventHdr* hdr,
 static_assert(kBBoxCopies == 32, "one copy per lane when the copies are combined");
 
 static_assert(kBuildPtsPerBlock == 256, "eight warps combine the box copies");
-static_assert(kMaxD <= 32 && kMaxAxes <= 32, "one lane per coordinate");
+static_assert(kMaxD <= 32 && kHdrAxes <= 32, "one lane per coordinate");
 
 // One candidate grid, held by warp 0: k gridded axes (the last k coordinates,
 // or the k widest), cell multiple m, the cell edge fitted to the proof's
 // condition, 1024 cells per axis and the event's cell budget, and the
 // expected fraction of the event a query's neighbourhood covers if the
 // points were spread evenly: the product over the gridded axes of
-// min(1, (2m+1) cells / extent).  The parameter step keeps the candidate
+// min(1, (2m+1) cells / extent) (4 cells on the axes of a grid of half cells,
+// whose budget counts stored cells).  The parameter step keeps the candidate
 // with the smallest fraction; the choice never changes results.  Lane a < k
 // holds gridded axis a (coordinate, cells, extremes); the other fields are
 // the same on every lane.
 struct GridFit {
     int naxes = 1, m = 1;
-    int axis = 0, dim = 1;
+    int axis = 0, dim = 1, sdim = 1;   // sdim: stored cells
     float lo = 0.f, hi = 0.f;
     float inv_h = 0.f;
     int32_t ncells = 1;
@@ -307,7 +315,7 @@ struct GridFit {
 // lo_j, hi_j: the extremes of coordinate j on lane j < D.  Called by all
 // lanes of warp 0.
 __device__ void grid_fit(GridFit& f, float lo_j, float hi_j, int D, int k, int m, int axes_mode,
-                         float r, int64_t cap, bool valid, int max_rows) {
+                         float r, int64_t cap, bool valid, int max_rows, bool half) {
     constexpr unsigned kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     f.naxes = k;
@@ -321,7 +329,10 @@ __device__ void grid_fit(GridFit& f, float lo_j, float hi_j, int D, int k, int m
         --mm;
     }
     f.m = mm;
-    int ax = lane < k ? D - k + lane : 0;
+    // the last k coordinates; a sixth axis (half cells) is the one before the
+    // last five
+    const int k5 = min(k, kMaxAxes);
+    int ax = lane < k5 ? D - k5 + lane : (lane < k ? D - 1 - lane : 0);
     if (valid && axes_mode == 1 && D > k) {
         // the k widest coordinates (ties by lower index), in index order
         const float wj = __fsub_rn(hi_j, lo_j);
@@ -331,11 +342,12 @@ __device__ void grid_fit(GridFit& f, float lo_j, float hi_j, int D, int k, int m
             if (wi > wj || (wi == wj && i < lane)) ++rank;
         }
         const unsigned sel = __ballot_sync(kAll, lane < D && rank < k);
+        const int want_pos = k > kMaxAxes ? (lane < kMaxAxes ? lane + 1 : 0) : lane;
         int cnt = 0;
         ax = 0;
         for (int j = 0; j < D; ++j) {
             if ((sel >> j) & 1u) {
-                if (cnt == lane) ax = j;
+                if (cnt == want_pos) ax = j;
                 ++cnt;
             }
         }
@@ -355,7 +367,7 @@ __device__ void grid_fit(GridFit& f, float lo_j, float hi_j, int D, int k, int m
     const float rho_up = __fmul_ru(r, 1.0f + 0x1p-20f);
     const float need = (float)mm - 0x1p-20f;
     float ih = __fdiv_rd((float)mm, __fmul_ru(r, 1.0f + 0x1p-10f));
-    int dim = 1;
+    int dim = 1, sdim = 1;
     int64_t cells = 1;
     bool fit = false;
     for (int it = 0; it < 4096; ++it) {
@@ -369,8 +381,9 @@ __device__ void grid_fit(GridFit& f, float lo_j, float hi_j, int D, int k, int m
                 __fadd_ru(__fmul_ru(ih, __fadd_ru(rho_up, __fmul_ru(0x1p-21f, ext_up))), 0x1p-148f);
             if (!(bound < need)) ok = false;
         }
+        sdim = half && lane > 0 ? (dim + 1) >> 1 : dim;
         cells = 1;
-        for (int a = 0; a < k; ++a) cells *= __shfl_sync(kAll, dim, a);
+        for (int a = 0; a < k; ++a) cells *= __shfl_sync(kAll, sdim, a);
         if (__all_sync(kAll, ok) && cells <= cap) {
             fit = true;
             f.at_start = it == 0;
@@ -382,14 +395,17 @@ __device__ void grid_fit(GridFit& f, float lo_j, float hi_j, int D, int k, int m
     if (!fit) {   // one cell is always safe
         ih = 0.f;
         dim = 1;
+        sdim = 1;
         cells = 1;
     }
     f.dim = lane < k ? dim : 1;
+    f.sdim = lane < k ? sdim : 1;
     f.inv_h = ih;
     f.ncells = (int32_t)cells;
     float fr = 1.f;
     if (lane < k && ext_up > 0.f) {
-        const float span = ih > 0.f ? (2.f * (float)mm + 1.f) / ih : INFINITY;
+        const float cover = half && lane > 0 ? 4.f : 2.f * (float)mm + 1.f;
+        const float span = ih > 0.f ? cover / ih : INFINITY;
         fr = fminf(1.f, span / ext_up);
     }
     float frac = 1.f;
@@ -439,9 +455,12 @@ __device__ void event_params(EventHdr* hdr, int e, int D, const int32_t* bbox, f
     const float hi_j = lane < D ? ordered_to_float(bb[16 + lane]) : 0.f;
     const bool fin = lane >= D || (isfinite(lo_j) && isfinite(hi_j));
     const bool valid = __all_sync(0xffffffffu, fin) && bb[32] == 0 && n > 0;
-    const int kmax = min(D, kMaxAxes);
+    // (half cells: six, five or four axes, always the automatic choice)
+    const bool half = H.half != 0;
+    const int kmax = min(D, half ? kHdrAxes : kMaxAxes);
     const int k_hi = want > 0 ? min(D, min(want, kMaxAxes)) : kmax;
-    const int k_lo = want > 0 ? k_hi : max(1, kmax - 1);
+    const int k_lo = want > 0 ? k_hi : max(1, kmax - (half ? 2 : 1));
+    const int64_t cap = half ? min((int64_t)cell_cap, kHalfMaxCells) : (int64_t)cell_cap;
     // grids requested with up to four axes are scanned by the row-task
     // kernel, whose lanes hold one neighbour row each
     const int max_rows = (want >= 1 && want <= 4) ? 32 : kMaxNbrRows;
@@ -449,17 +468,20 @@ __device__ void event_params(EventHdr* hdr, int e, int D, const int32_t* bbox, f
     best.frac = INFINITY;
     for (int k = k_hi; k >= k_lo; --k) {
         GridFit f;
-        grid_fit(f, lo_j, hi_j, D, k, m_req, axes_mode, r, cell_cap, valid, max_rows);
+        grid_fit(f, lo_j, hi_j, D, k, half ? 1 : m_req, axes_mode, r, cap, valid, max_rows, half);
         if (f.frac < best.frac) best = f;
         // at the starting cell edge a grid over more axes covers at most the
         // fraction of one over fewer (one factor <= 1 more): no need to try fewer
         if (f.at_start) break;
     }
     const int na = best.naxes;
-    if (lane < kMaxAxes) {
+    if (lane < kHdrAxes) {
         const bool gridded = lane < na;
+        const int sd = gridded && valid ? best.sdim : 1;
         H.axes[lane] = gridded ? best.axis : 0;
-        H.dims[lane] = gridded && valid ? best.dim : 1;
+        H.dims[lane] = sd;
+        H.fdims[lane] = gridded && valid ? best.dim : 1;
+        H.mag[lane] = ((1ull << 36) + (uint64_t)sd - 1) / (uint64_t)sd;
         H.lo[lane] = gridded && valid ? best.lo : 0.f;
         H.hi[lane] = gridded && valid ? best.hi : 0.f;
     }
@@ -494,9 +516,12 @@ __global__ void k_copy_params(EventHdr* dst, const EventHdr* src, int E, int32_t
     d.valid = s.valid;
     d.inv_h = s.inv_h;
     d.ncells = s.ncells;
-    for (int a = 0; a < kMaxAxes; ++a) {
+    d.half = s.half;
+    for (int a = 0; a < kHdrAxes; ++a) {
         d.axes[a] = s.axes[a];
         d.dims[a] = s.dims[a];
+        d.fdims[a] = s.fdims[a];
+        d.mag[a] = s.mag[a];
         d.lo[a] = s.lo[a];
         d.hi[a] = s.hi[a];
     }
@@ -534,7 +559,7 @@ __global__ void __launch_bounds__(kBuildPtsPerBlock) k_cellid(const EventHdr* hd
     if (h.valid) c = point_cell(p, h);
     const int64_t gi = h.pt_off + p0 + i;
     cid[gi] = c;
-    rnk[gi] = atomicAdd(counts + h.cell_off + c, 1);
+    rnk[gi] = atomicAdd(counts + h.cell_off + stored_cell(h, c), 1);
 }
 
 // Slot maps and cell-sorted coordinates: each point's slot (its cell's start
@@ -573,7 +598,7 @@ __global__ void __launch_bounds__(kBuildPtsPerBlock) k_scatter(const EventHdr* h
     if (i >= np) return;
     const int64_t gi = h.pt_off + p0 + i;
     const int c = cid[gi];
-    const int64_t slot = (int64_t)cstart[h.cell_off + c] + rnk[gi];
+    const int64_t slot = (int64_t)cstart[h.cell_off + stored_cell(h, c)] + rnk[gi];
     perm[slot] = (int32_t)(p0 + i);
     cell[slot] = c;
     const StagedRow src{sm, i * D, pad};
@@ -618,7 +643,7 @@ __global__ void k_rowtasks(const EventHdr* hdr, const int64_t* cell_off, int E, 
     const EventHdr& h = hdr[e];
     const int64_t row = i - cell_off[e];
     int64_t nrows = 1;   // rows: every gridded coordinate but the fastest
-    for (int a = 1; a < kMaxAxes && h.valid; ++a) nrows *= h.dims[a];
+    for (int a = 1; a < kHdrAxes && h.valid; ++a) nrows *= h.dims[a];
     int32_t nt = 0;
     // events another launch of a mixed batch queries get no tasks
     if (row < nrows && (path_filter < 0 || h.path == path_filter)) {
@@ -861,7 +886,8 @@ void enqueue_scan(int32_t* data, int64_t n, int32_t* parts, int32_t* total, cuda
 // build zeroes and scans the whole budget), and the parameter step falls
 // back to one axis fewer when the budget would make five-axis cells too
 // coarse.
-int64_t cell_cap_for(int64_t n, int naxes) {
+int64_t cell_cap_for(int64_t n, int naxes, bool half) {
+    if (half) return std::min<int64_t>(std::max<int64_t>(16384, 12 * n), kHalfMaxCells);
     const int64_t per = naxes >= 5 ? 18 : (naxes == 4 ? 2 : 0);
     int64_t c = per ? per * n : n / 2 + 1;
     c = std::max<int64_t>(16384, c);

@@ -97,7 +97,8 @@ constexpr int kTcRowPad = 512;      // rows readable past the last slot (chunk r
 
 // Cells allowed for an n-point event gridded over naxes coordinates (the
 // parameter step enlarges the cells when the grid would need more).
-int64_t cell_cap_for(int64_t n, int naxes);
+// half: a grid of half cells (stored cells).
+int64_t cell_cap_for(int64_t n, int naxes, bool half = false);
 
 // Compute the layout for E events of sizes n[e] and allocate (or reuse).
 // caps (optional): per-event cell capacities (a query set binned with a
@@ -106,6 +107,11 @@ int64_t cell_cap_for(int64_t n, int naxes);
 frnn_status grid_alloc(GridBufs& g, int E, const int64_t* n, int D, std::string& err,
                        const int64_t* caps = nullptr, int naxes = kMaxAxes);
 void grid_free(GridBufs& g);
+
+// Whether a grid requested with naxes gridded axes (0: the automatic choice)
+// and cell multiple m stores half cells (EventHdr::half) for the half-cell
+// scan (query_half.cu): the automatic grids of five or more dimensions.
+inline bool half_cells(int D, int naxes, int m) { return naxes == 0 && m == 1 && D > 4; }
 
 struct BuildOpts {
     float r = 0.f;          // grid radius
@@ -150,7 +156,8 @@ struct QueryLaunch {
     int self;
     int exit_dims;          // 0 = default
     int stage = 0;          // grid query candidate staging: 0 lanes load rows, 1 bulk copies
-    int kernel = 0;         // grid scan: 0 chunks (query.cu), 1 row tasks (query_rows.cu)
+    int kernel = 0;         // grid scan: 0 chunks (query.cu), 1 row tasks (query_rows.cu),
+                            // 2 half cells (query_half.cu)
     int32_t* counts;        // single event outputs, or NULL to use the event headers'
     int32_t* idx;
     float* dist2;
@@ -181,6 +188,7 @@ frnn_status rows_prepare(GridBufs& g, int32_t* d_status, cudaStream_t st, std::s
 void rows_free(GridBufs& g);
 frnn_status enqueue_row_query(const QueryLaunch& q, const QueryArgs& a, cudaStream_t st,
                               std::string& err);
+cudaError_t enqueue_half_query(const QueryArgs& a, int num_sms, cudaStream_t st);
 // The selection kernel alone over the rows the last query of q.qset listed
 // (compact output, second pass: q.ovf_mode 2, q.row_off).
 frnn_status enqueue_overflow_only(const QueryLaunch& q, cudaStream_t st, std::string& err);

@@ -12,7 +12,10 @@ namespace frnn {
 
 constexpr int kMaxD = 16;
 constexpr int kMaxK = 1024;
-constexpr int kMaxAxes = 5;
+constexpr int kMaxAxes = 5;             // gridded coordinates of a grid of plain cells
+constexpr int kHdrAxes = 6;             // of a grid of half cells (EventHdr::half)
+constexpr int kHalfBits = kHdrAxes - 1; // half-cell bits kept below a slot's cell id
+constexpr int64_t kHalfMaxCells = (int64_t)1 << 26;   // so that id and bits fit an int32
 constexpr int kMaxDimsPerAxis = 1024;   // the grid roundoff proof assumes <= 2^10 cells per axis
 constexpr int kTaskQueries = 16;        // task-list granularity of the build's task builder
 constexpr int kChunkQ = 16;             // query slots per chunk of the grid query kernel
@@ -58,15 +61,26 @@ struct EventHdr {
     int64_t cell_off;      // first entry of this event in the cell arrays (cap + 1 entries)
     int32_t cell_cap;      // cells allowed for this event
     int32_t ncells;        // product of dims (written by the parameter step)
-    int32_t naxes;         // gridded axes (1..5); preset by the host: requested count (0: default)
+    int32_t naxes;         // gridded axes (1..6); preset by the host: requested count (0: default)
     int32_t m;             // cell multiple: neighbours are within +-m cells per gridded axis
     int32_t valid;         // 0 if a coordinate was non-finite
-    int32_t axes[kMaxAxes];   // gridded coordinate indices; axes[0] varies fastest
-    int32_t dims[kMaxAxes];   // cells per gridded axis (1 for unused axes)
-    float lo[kMaxAxes];       // per-axis minimum coordinate
-    float hi[kMaxAxes];       // per-axis maximum coordinate
+    // 1: a grid of half cells (preset by the host).  Cell coordinates are those
+    // of a grid with m = 1, but along every axis except axes[0] two neighbouring
+    // cells share one stored cell: stored coordinate = cell coordinate >> 1,
+    // and the low bits say which half.  The cells within +-1 of cell c are then
+    // the stored cells c >> 1 and its one neighbour on the side of c's half, so
+    // a search visits 2 instead of 3 cells per axis.  A slot's `cell` entry is
+    // stored cell id << kHalfBits | half bits (axis a's at bit a - 1).
+    int32_t half;
+    int32_t axes[kHdrAxes];   // gridded coordinate indices; axes[0] varies fastest
+    int32_t dims[kHdrAxes];   // stored cells per gridded axis (1 for unused axes)
+    int32_t fdims[kHdrAxes];  // cells per gridded axis (= dims unless half)
+    uint64_t mag[kHdrAxes];   // ceil(2^36 / dims): v / dims = v * mag >> 36 for v < 2^26
+    float lo[kHdrAxes];       // per-axis minimum coordinate
+    float hi[kHdrAxes];       // per-axis maximum coordinate
     float inv_h;           // 1 / cell edge (float; the value the cell ids use)
-    int32_t path;          // batched queries: 0 = grid scan, 1 = tensor-core pre-filter
+    int32_t path;          // batched queries: 0 = chunk scan, 1 = tensor-core pre-filter,
+                           // 2 = row tasks, 3 = half-cell scan
     int32_t qchunk0;       // first query chunk (kChunkQ slots) of this event in its point set
     float ctr[16];         // per-dimension centre of the bounding box (tensor-core operands)
     // query outputs for batched self-queries (row = original point index)
@@ -83,6 +97,11 @@ struct Task {
     int32_t ev;      // event index
     int32_t row;     // row index within the event: c1 + dims[1] * (c2 + dims[2] * (c3 + ...))
 };
+
+// A slot's stored cell id (its `cell` entry without the half bits).
+__host__ __device__ inline int stored_cell(const EventHdr& h, int key) {
+    return h.half ? key >> kHalfBits : key;
+}
 
 // Neighbour rows of a row of cells.  A row fixes every gridded coordinate but
 // the fastest (c0); its neighbours are the rows whose coordinates c1..c4 each
@@ -101,16 +120,36 @@ __device__ __forceinline__ bool neighbour_row(const EventHdr& h, int row, int l,
     int64_t lin = 0, stride = 1;
     bool ok = true;
 #pragma unroll
-    for (int a = 1; a < kMaxAxes; ++a) {
+    for (int a = 1; a < kHdrAxes; ++a) {
+        if (a >= h.naxes) break;
         const int da = h.dims[a];
         const int c = row % da;
         row /= da;
-        int d = 0;
-        if (a < h.naxes) {
-            d = (l % side) - h.m;
-            l /= side;
-        }
+        const int d = (l % side) - h.m;
+        l /= side;
         const int cc = c + d;
+        ok = ok && cc >= 0 && cc < da;
+        lin += (int64_t)cc * stride;
+        stride *= da;
+    }
+    first_cell = h.cell_off + lin * h.dims[0];
+    return ok;
+}
+
+// The same for one query of a grid of half cells with half bits `bits`: row l
+// (0 <= l < 2^(naxes - 1)) moves along axis a (if bit a - 1 of l is set) to the
+// stored cell on the side of the query's half.
+__device__ __forceinline__ bool neighbour_row_half(const EventHdr& h, int row, int bits, int l,
+                                                   int64_t& first_cell) {
+    int64_t lin = 0, stride = 1;
+    bool ok = true;
+#pragma unroll
+    for (int a = 1; a < kHdrAxes; ++a) {
+        if (a >= h.naxes) break;
+        const int da = h.dims[a];
+        const int c = row % da;
+        row /= da;
+        const int cc = c + (((l >> (a - 1)) & 1) ? (((bits >> (a - 1)) & 1) ? 1 : -1) : 0);
         ok = ok && cc >= 0 && cc < da;
         lin += (int64_t)cc * stride;
         stride *= da;

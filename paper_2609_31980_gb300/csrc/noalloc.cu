@@ -58,7 +58,7 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 // the per-event tables the host would otherwise upload, and a clean status word
 __global__ void k_noalloc_tables(EventHdr* hdr, int32_t* blk_start, int64_t* cell_off,
                                  const float* pts, int64_t n, int32_t cap, int32_t nblk,
-                                 int32_t* status) {
+                                 int32_t half, int32_t* status) {
     if (threadIdx.x != 0) return;
     EventHdr h{};
     h.refs = pts;
@@ -67,6 +67,7 @@ __global__ void k_noalloc_tables(EventHdr* hdr, int32_t* blk_start, int64_t* cel
     h.cell_off = 0;
     h.cell_cap = cap;
     h.valid = 1;
+    h.half = half;
     *hdr = h;
     blk_start[0] = 0;
     blk_start[1] = nblk;
@@ -149,7 +150,7 @@ frnn_status frnn_self_query_noalloc(const float* pts, int64_t N, int D, float r,
     GridBufs g;
     int32_t* status = carve(g, base, N, D);
     k_noalloc_tables<<<1, 32, 0, st>>>(g.hdr, g.blk_start, g.cell_off, pts, N,
-                                      (int32_t)na_cap(N), (int32_t)g.nblk, status);
+                                      (int32_t)na_cap(N), (int32_t)g.nblk, half_cells(D, 0, 1), status);
     BuildOpts o;
     o.r = r;
     o.m = 1;
@@ -163,6 +164,7 @@ frnn_status frnn_self_query_noalloc(const float* pts, int64_t N, int D, float r,
     q.K = K;
     q.self = 1;
     q.exit_dims = 0;
+    q.kernel = half_cells(D, 0, 1) ? 2 : 0;
     q.counts = counts;
     q.idx = idx;
     q.dist2 = dist2;

@@ -829,6 +829,8 @@ frnn_status enqueue_grid_query(const QueryLaunch& q, cudaStream_t st, std::strin
         // grids of up to four axes: the row-task kernel (query_rows.cu)
         const frnn_status s = enqueue_row_query(q, a, st, err);
         if (s != FRNN_OK) return s;
+    } else if (q.kernel == 2) {
+        ce = enqueue_half_query(a, q.num_sms, st);
     } else if (a.nchunks > 0) {
         switch (rs.D) {
 #define FRNN_CASE(d) case d: ce = launch_grid_query_d<d>(a, q.stage, q.num_sms, st); break;

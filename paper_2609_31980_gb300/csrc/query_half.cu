@@ -1,0 +1,627 @@
+// query_half.cu — the grid scan for grids of half cells (EventHdr::half), the
+// automatic grids of five or more dimensions.
+//
+// Method (Eq. 1, Sec. 1): as in query.cu, every reference in the cells within
+// +-1 of the query's cell along each gridded axis is a candidate (complete by
+// the grid's roundoff-safe construction, build.cu), its squared distance is
+// computed under the fixed float32 contract and it is kept if <= fl(r*r).
+//
+// What half cells change.  Cells of about r need 3 look-ups per gridded axis
+// and query: 81 neighbour rows with five axes, three rounds of the warp's
+// lanes, most of them empty.  Storing two cells together along every axis but
+// the fastest leaves 2 per axis (a query in a stored cell's low half cannot
+// reach the stored cell above, and the other way round): with six axes 32
+// neighbour rows, exactly one per lane, whose row offsets and grid-edge tests
+// are a few operations on the lane's bits.  A sixth axis becomes affordable
+// (22 x 11^5 = 3.5 M stored cells instead of 22^5 = 5.2 M for the 300k x 8
+// event), so the candidates do not grow (a CPU model of that event: 10.7 M
+// evaluated pairs against 12.6 M, 144 k look-up rounds against 352 k).
+//
+// Organisation:
+//   * a persistent grid; a warp takes `per` (16, fewer for small sets)
+//     consecutive cell-sorted query slots at a time from an atomic counter,
+//     sorts them by (row of cells, half bits, cell along the fastest axis) and
+//     groups runs of equal row and half bits whose cells are equal or adjacent;
+//   * lane l looks up neighbour row l of a group (the next group's look-ups in
+//     flight), the non-empty slot ranges form one candidate stream over all
+//     the groups of the chunk;
+//   * each lane takes one candidate per round (its row and original index
+//     loaded from L2, the next round's in flight) and computes the contract's
+//     squared distance to every query of its group; which range a lane's
+//     stream position lies in follows from one load of the next range starts
+//     and one warp-wide OR of the positions where ranges start;
+//   * accepted (d2, original index) pairs are appended to the query's list in
+//     shared memory (at most kListCap; longer lists go to select.cu);
+//   * row sort: lanes q and q + 16 hold half of query q's list each, as 32-bit
+//     keys (the distance's bits with the low five cleared, then the entry's
+//     place in the list), sort them in registers (an odd-even merge network,
+//     every compare-exchange one min and one max) and merge the halves with
+//     one exchange between the two lanes: 16 rows at once in a few hundred
+//     instructions, where a network across the lanes takes about a hundred a
+//     row.  Rows in which two truncated distances agree are put in (d2, index)
+//     order by counting;
+//   * the sorted rows go back to shared memory and are written with 16-byte
+//     stores (row width a multiple of 4 and aligned outputs; else 4-byte).
+//
+// What bounds it: instruction issue (70 % of the slots, 84 M warp instructions
+// at 300k x 8 where the chunk scan over five axes took 143 M) and the
+// load/store pipe (65 %).  Kernel alone, 300k x 8, K = 64: 193 us (chunk scan)
+// -> 129 (8 CTAs per SM, 64 registers, 100 B of spills, one shared-memory
+// atomic per accepted pair) -> 111 (7 CTAs, 72 registers) -> 105 (places in the
+// lists by ballots instead of atomics, whose same-address conflicts were a
+// fifth of the load/store pipe, and 32-byte row loads).  Build + query: 300k x
+// 8 242 -> 151 us, 300k x 5 1334 -> 199, 500k x 12 (four-axis row tasks) 523
+// -> 350, 20k x 8 66 -> 45.
+#include <algorithm>
+#include <climits>
+
+#include "frnn_host.h"
+
+namespace frnn {
+namespace half {
+
+constexpr int kWarps = 4;
+constexpr uint32_t kFull = 0xffffffffu;
+constexpr int kListCap = 32;     // accepted entries a query keeps in the kernel
+constexpr int kListStr = 36;     // list row stride: 16-byte aligned rows
+constexpr int kRangeCap = 128;   // candidate ranges of one batch of groups
+constexpr int kQ = kChunkQ;      // queries a warp serves at once, at most
+static_assert(kQ == 16, "lanes q and q + 16 share query q's row");
+static_assert(kListCap <= kCsrStageW, "a staged compact row holds a whole kernel row");
+
+template <int D>
+struct Cfg {
+    static constexpr int DP = padded_dim(D);
+    static constexpr int MINB = DP <= 8 ? 7 : (DP <= 12 ? 5 : 4);
+};
+
+struct WarpSmem {
+    float* Q;         // [kQ][DP] query coordinates
+    float* Ld;        // [kQ][kListStr] squared distances
+    int32_t* Li;      // [kQ][kListStr] original indices
+    int32_t* rpre;    // [kRangeCap + 4] stream position of each range
+    int32_t* rdel;    // [kRangeCap] slot - stream position
+    uint16_t* rq;     // [kRangeCap] first and past-the-last query of the range's group
+    int32_t* cnt;     // [kQ] accepted entries
+    int32_t* qor;     // [kQ] original query index
+};
+
+template <int D>
+__host__ __device__ constexpr size_t warp_bytes() {
+    return ((size_t)kQ * Cfg<D>::DP * 4 + 2 * (size_t)kQ * kListStr * 4 + (size_t)(kRangeCap + 4) * 4 +
+            (size_t)kRangeCap * 4 + (size_t)kRangeCap * 2 + 2 * (size_t)kQ * 4 + 127) / 128 * 128;
+}
+
+template <int D>
+__device__ __forceinline__ WarpSmem carve(unsigned char* base) {
+    WarpSmem w;
+    w.Q = reinterpret_cast<float*>(base);
+    w.Ld = w.Q + kQ * Cfg<D>::DP;
+    w.Li = reinterpret_cast<int32_t*>(w.Ld + kQ * kListStr);
+    w.rpre = w.Li + kQ * kListStr;
+    w.rdel = w.rpre + kRangeCap + 4;
+    w.cnt = w.rdel + kRangeCap;
+    w.qor = w.cnt + kQ;
+    w.rq = reinterpret_cast<uint16_t*>(w.qor + kQ);
+    return w;
+}
+
+// v / d for v < 2^26 by the header's ceil(2^36 / d), d <= 1024: the error
+// v * (mag d - 2^36) is below 2^26 * 2^10 = 2^36, so the quotient is exact.
+__device__ __forceinline__ int div_mag(int v, uint64_t mag) {
+    return (int)(((uint64_t)(uint32_t)v * mag) >> 36);
+}
+
+// One point row of DP floats (32-byte rows with one 32-byte load).
+template <int DP>
+__device__ __forceinline__ void load_row(const float* p, float (&v)[DP]) {
+    static_assert(DP % 4 == 0, "rows are 16-byte multiples");
+    if constexpr (DP % 8 == 0) {
+#pragma unroll
+        for (int k = 0; k < DP; k += 8)
+            asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                : "=f"(v[k]), "=f"(v[k + 1]), "=f"(v[k + 2]), "=f"(v[k + 3]), "=f"(v[k + 4]), "=f"(v[k + 5]),
+                  "=f"(v[k + 6]), "=f"(v[k + 7])
+                : "l"(p + k));
+    } else {
+#pragma unroll
+        for (int k = 0; k < DP; k += 4) {
+            const float4 x = __ldg(reinterpret_cast<const float4*>(p + k));
+            v[k] = x.x;
+            v[k + 1] = x.y;
+            v[k + 2] = x.z;
+            v[k + 3] = x.w;
+        }
+    }
+}
+
+__device__ __forceinline__ int chunk_event(const EventHdr* qev, int E, int c) {
+    int lo = 0, hi = E - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (qev[mid].qchunk0 <= c) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
+__device__ __forceinline__ void cswap(uint32_t& a, uint32_t& b) {
+    const uint32_t lo = min(a, b), hi = max(a, b);
+    a = lo;
+    b = hi;
+}
+
+// Batcher's odd-even merge sort of P keys in registers.
+template <int P>
+__device__ __forceinline__ void sort_regs(uint32_t (&k)[P]) {
+#pragma unroll
+    for (int p = 1; p < P; p <<= 1) {
+#pragma unroll
+        for (int q = p; q >= 1; q >>= 1) {
+#pragma unroll
+            for (int i = 0; i < P; ++i) {
+                const int j = q % p;   // the step's first key
+                if (i >= j && (i - j) % (2 * q) < q && i + q < P && i / (2 * p) == (i + q) / (2 * p))
+                    cswap(k[i], k[i + q]);
+            }
+        }
+    }
+}
+
+// Sort every query's list (n entries of query lane % 16 on its two lanes, at
+// most 2 P; warp-wide call) in place by (d2, original index); the places from
+// n to 2 P get the padding.
+template <int P>
+__device__ __forceinline__ void sort_rows(const WarpSmem& w, int n) {
+    const int lane = threadIdx.x & 31;
+    const int q = lane & 15, hh = lane >> 4;
+    float* ld = w.Ld + q * kListStr;
+    int32_t* li = w.Li + q * kListStr;
+    uint32_t k[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+        const int e = hh * P + i;
+        // empty places: above every distance, 32 apart
+        const uint32_t v = __float_as_uint(ld[e]);
+        k[i] = e < n ? (v & ~31u) | (uint32_t)e : 0x80000000u | (uint32_t)(e * 33);
+    }
+    sort_regs<P>(k);
+    // the pair's halves: the lower lane keeps the P smallest, the upper the
+    // rest (each a bitonic sequence), then one merge in registers
+    {
+        uint32_t o[P];
+#pragma unroll
+        for (int i = 0; i < P; ++i) o[i] = __shfl_xor_sync(kFull, k[P - 1 - i], 16);
+#pragma unroll
+        for (int i = 0; i < P; ++i) k[i] = hh ? max(k[i], o[i]) : min(k[i], o[i]);
+    }
+#pragma unroll
+    for (int j = P / 2; j > 0; j >>= 1)
+#pragma unroll
+        for (int i = 0; i < P; ++i)
+            if ((i & j) == 0) cswap(k[i], k[i | j]);
+    // neighbouring keys equal but for the place: the order needs the whole key
+    uint32_t near = 32u;
+#pragma unroll
+    for (int i = 0; i + 1 < P; ++i) near = min(near, k[i] ^ k[i + 1]);
+    const uint32_t edge = hh ? k[0] : k[P - 1];
+    near = min(near, edge ^ __shfl_xor_sync(kFull, edge, 16));
+    const unsigned tied = __ballot_sync(kFull, near < 32u);
+    // entries to their places
+    {
+        float v[P];
+#pragma unroll
+        for (int i = 0; i < P; ++i) v[i] = ld[k[i] & 31];
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < P; i += 4) {
+            const int e = hh * P + i;
+            *reinterpret_cast<float4*>(ld + e) =
+                make_float4(e < n ? v[i] : INFINITY, e + 1 < n ? v[i + 1] : INFINITY,
+                            e + 2 < n ? v[i + 2] : INFINITY, e + 3 < n ? v[i + 3] : INFINITY);
+        }
+    }
+    {
+        int32_t v[P];
+#pragma unroll
+        for (int i = 0; i < P; ++i) v[i] = li[k[i] & 31];
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < P; i += 4) {
+            const int e = hh * P + i;
+            *reinterpret_cast<int4*>(li + e) = make_int4(e < n ? v[i] : -1, e + 1 < n ? v[i + 1] : -1,
+                                                         e + 2 < n ? v[i + 2] : -1, e + 3 < n ? v[i + 3] : -1);
+        }
+    }
+    __syncwarp();
+    // rows with ties among the truncated distances: each entry's place is the
+    // number of smaller (d2, index) keys
+    unsigned rows = (tied | (tied >> 16)) & 0xffffu;
+    while (rows) {
+        const int r = __ffs(rows) - 1;
+        rows &= rows - 1u;
+        const int nr = __shfl_sync(kFull, n, r);
+        const float d = lane < nr ? w.Ld[r * kListStr + lane] : 0.f;
+        const int32_t x = lane < nr ? w.Li[r * kListStr + lane] : 0;
+        int rank = 0;
+        for (int j = 0; j < nr; ++j) {
+            const float dj = __shfl_sync(kFull, d, j);
+            const int32_t xj = __shfl_sync(kFull, x, j);
+            rank += (dj < d || (dj == d && xj < x)) ? 1 : 0;
+        }
+        __syncwarp();
+        if (lane < nr) {
+            w.Ld[r * kListStr + rank] = d;
+            w.Li[r * kListStr + rank] = x;
+        }
+    }
+    __syncwarp();
+}
+
+template <int D>
+__global__ void __launch_bounds__(kWarps * 32, Cfg<D>::MINB) k_half_query(QueryArgs a, int sub_shift) {
+    pdl_trigger();
+    pdl_wait();
+    constexpr int DP = Cfg<D>::DP;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const WarpSmem w = carve<D>(smem + (size_t)warp * warp_bytes<D>());
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const unsigned le_mask = lt_mask | (1u << lane);
+    const float r2 = a.r2;
+    const int K = a.K;
+    const int per = kQ >> sub_shift;
+    const int ntasks = a.nchunks << sub_shift;
+    // row width of the output (compact staging rows have no padding) and, for
+    // the 16-byte stores, its quarter
+    const int width = a.csr ? kCsrStageW : K;
+    const int w4 = width >> 2;
+
+    for (;;) {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(a.task_counter, 1);
+        t = __shfl_sync(kFull, t, 0);
+        if (t >= ntasks) break;
+        const int c = t >> sub_shift;
+        const int e = a.nev > 1 ? chunk_event(a.qev, a.nev, c) : 0;
+        const EventHdr& hq = a.qev[e];
+        const EventHdr& h = a.ev[e];
+        if (a.path_filter >= 0 && h.path != a.path_filter) continue;   // another launch's event
+        int32_t* counts = a.counts ? a.counts : h.counts;
+        int32_t* oidx = a.counts ? a.idx : h.idx;
+        float* od2 = a.counts ? a.dist2 : h.dist2;
+        const int64_t q_end = hq.pt_off + hq.n;
+        const int s0 = (int)(hq.pt_off + (int64_t)(c - hq.qchunk0) * kQ) + (t & ((1 << sub_shift) - 1)) * per;
+        const int nqc = (int)min((int64_t)per, q_end - (int64_t)s0);
+        if (nqc <= 0) continue;   // past the event's last query
+        const bool act = lane < nqc;
+        const int qorig0 = act ? a.qperm[s0 + lane] : 0;
+        if (!h.valid) {
+            // grid built from non-finite input: empty rows (frnn_sync reports it)
+            for (int ql = 0; ql < nqc && !a.csr; ++ql) {
+                const int qo = __shfl_sync(kFull, qorig0, ql);
+                for (int e2 = lane; e2 < K; e2 += 32) {
+                    oidx[(int64_t)qo * K + e2] = -1;
+                    od2[(int64_t)qo * K + e2] = INFINITY;
+                }
+            }
+            if (act) counts[qorig0] = 0;
+            if (act && a.degree) a.degree[qorig0] = 0;
+            continue;
+        }
+        const int naxes = h.naxes, dims0 = h.dims[0];
+        const int32_t* cells = a.cstart + h.cell_off;
+
+        // the chunk's queries by (row of cells, half bits, cell on the row)
+        int x, row, src, pk;
+        {
+            const int key = act ? a.qcell[s0 + lane] : 0;
+            const int id = key >> kHalfBits;
+            row = div_mag(id, h.mag[0]);
+            x = id - row * dims0;
+            const int prev = __shfl_up_sync(kFull, row, 1);
+            const int rr = __popc(__ballot_sync(kFull, act && (lane == 0 || row != prev)) & le_mask);
+            uint32_t sk = act ? ((uint32_t)rr << 20) | ((uint32_t)(key & ((1 << kHalfBits) - 1)) << 15) |
+                                    ((uint32_t)x << 5) | (uint32_t)lane
+                              : 0xffffffffu;
+#pragma unroll
+            for (int k2 = 2; k2 <= kQ; k2 <<= 1) {
+#pragma unroll
+                for (int j = k2 >> 1; j > 0; j >>= 1) {
+                    const uint32_t o = __shfl_xor_sync(kFull, sk, j);
+                    const bool take_min = ((lane & j) == 0) == ((lane & k2) == 0 || k2 == kQ);
+                    sk = take_min ? min(sk, o) : max(sk, o);
+                }
+            }
+            src = (int)(sk & 31u);
+            pk = (int)(sk >> 5);
+            x = pk & 1023;
+            row = __shfl_sync(kFull, row, src);
+        }
+        const int bits = (pk >> 10) & 31;
+        const int qs = s0 + src;
+        const int qorig = __shfl_sync(kFull, qorig0, src);
+        if (act) {
+            const float4* q4 = reinterpret_cast<const float4*>(a.qpts + (int64_t)qs * DP);
+            float4* dst = reinterpret_cast<float4*>(w.Q + lane * DP);
+#pragma unroll
+            for (int k4 = 0; k4 < DP / 4; ++k4) dst[k4] = q4[k4];
+            w.qor[lane] = qorig;
+            w.cnt[lane] = 0;
+        }
+        // per query: the moves (bits of a neighbour row's number) that would
+        // leave the grid; per lane: the row offset its own bits move by
+        int bad = 0, mv[kHdrAxes - 1];
+        {
+            int v = row, rs = 1;
+#pragma unroll
+            for (int ax = 1; ax < kHdrAxes; ++ax) {
+                mv[ax - 1] = 0;
+                if (ax < naxes) {
+                    const int da = h.dims[ax];
+                    const int qv = div_mag(v, h.mag[ax]);
+                    const int ca = v - qv * da;
+                    v = qv;
+                    if (((bits >> (ax - 1)) & 1) ? ca == da - 1 : ca == 0) bad |= 1 << (ax - 1);
+                    if ((lane >> (ax - 1)) & 1) mv[ax - 1] = rs;
+                    rs *= da;
+                }
+            }
+        }
+        const int back = -(mv[0] + mv[1] + mv[2] + mv[3] + mv[4]);
+        const bool lane_row = lane < (1 << (naxes - 1));
+        const int gp = bits | (bad << 5) | (x << 10);
+        // groups
+        const int ppk = __shfl_up_sync(kFull, pk, 1);
+        const bool head = act && (lane == 0 || (pk >> 10) != (ppk >> 10) || x > (ppk & 1023) + 1);
+        const unsigned gmask = __ballot_sync(kFull, head);
+        const int ng = __popc(gmask);
+
+        // slot range of the neighbour row of group g (first query hl, past its
+        // last hn) on this lane
+        int nlo = 0, nhi = 0;
+        unsigned gleft = gmask;   // heads of the groups not fetched yet
+        int f_hl = 0, f_hn = 0;   // queries of the fetched group
+        auto fetch = [&]() {
+            f_hl = __ffs(gleft) - 1;
+            gleft &= gleft - 1u;
+            f_hn = gleft ? __ffs(gleft) - 1 : nqc;
+            const int g = __shfl_sync(kFull, gp, f_hl);
+            const int grow = __shfl_sync(kFull, row, f_hl);
+            const int xl = __shfl_sync(kFull, x, f_hn - 1);
+            const int x0 = max((g >> 10) - 1, 0), x1 = min(xl + 1, dims0 - 1) + 1;
+            nlo = 0;
+            nhi = 0;
+            if (lane_row && (lane & (g >> 5) & 31) == 0) {
+                int off = back;
+#pragma unroll
+                for (int ax = 0; ax < kHdrAxes - 1; ++ax)
+                    if ((g >> ax) & 1) off += 2 * mv[ax];
+                const int base = (grow + off) * dims0;
+                nlo = __ldg(cells + base + x0);
+                nhi = __ldg(cells + base + x1);
+            }
+        };
+        fetch();
+        __syncwarp();
+
+        int gdone = 0;   // groups taken into a batch
+        while (gdone < ng) {
+            int nr = 0;
+            for (;;) {
+                const int n = nhi - nlo;
+                const unsigned bal = __ballot_sync(kFull, n > 0);
+                if (nr + __popc(bal) > kRangeCap) break;   // this group opens the next batch
+                if (n > 0) {
+                    const int pos = nr + __popc(bal & lt_mask);
+                    w.rdel[pos] = nlo;
+                    w.rpre[pos] = n;   // a count until the batch's scan
+                    w.rq[pos] = (uint16_t)(f_hl | (f_hn << 8));
+                }
+                nr += __popc(bal);
+                if (++gdone == ng) break;
+                fetch();
+            }
+            // counts -> stream positions
+            __syncwarp();
+            int U = 0;
+            for (int b0 = 0; b0 < nr; b0 += 32) {
+                const int i = b0 + lane;
+                const int v = i < nr ? w.rpre[i] : 0;
+                int incl = v;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(kFull, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                if (i < nr) {
+                    const int start = U + incl - v;
+                    w.rpre[i] = start;
+                    w.rdel[i] -= start;
+                }
+                U += __shfl_sync(kFull, incl, 31);
+            }
+            __syncwarp();
+
+            int cur = -1;   // last range that starts before the next round
+            auto load_cand = [&](int k0, int& qq, int32_t& orig, float (&cv)[DP]) {
+                const int ri = cur + 1 + lane;
+                const int d = ri < nr ? w.rpre[ri] - k0 : 32;
+                const unsigned starts = __reduce_or_sync(kFull, d < 32 ? 1u << d : 0u);
+                const int i = cur + __popc(starts & le_mask);
+                cur += __popc(starts);
+                qq = 0;
+                orig = -1;
+#pragma unroll
+                for (int k = 0; k < DP; ++k) cv[k] = 0.f;
+                const int u = k0 + lane;
+                if (u < U) {
+                    const int slot = u + w.rdel[i];
+                    qq = w.rq[i];
+                    orig = __ldg(a.rperm + slot);
+                    load_row<DP>(a.rpts + (int64_t)slot * DP, cv);
+                }
+            };
+            int qq;
+            int32_t orig;
+            float cv[DP];
+            load_cand(0, qq, orig, cv);
+#pragma unroll 1
+            for (int k0 = 0; k0 < U; k0 += 32) {
+                int qq_n;
+                int32_t orig_n;
+                float cvn[DP];
+                load_cand(k0 + 32, qq_n, orig_n, cvn);   // next round in flight
+                const int qa = qq & 255;
+                const int nq = (qq >> 8) - qa;
+                const int mx = __reduce_max_sync(kFull, (unsigned)nq);
+                // the lanes of this lane's group before and after it (a group's
+                // lanes are consecutive)
+                const int qq_p = __shfl_up_sync(kFull, qq, 1);
+                const unsigned firsts = __ballot_sync(kFull, lane == 0 || qq != qq_p);
+                const unsigned g_lo = lt_mask & ~((1u << (31 - __clz(firsts & le_mask))) - 1u);
+                const unsigned later = firsts & ~le_mask;
+                const unsigned g_hi = ~le_mask & (later ? (later & (0u - later)) - 1u : kFull);
+                for (int j = 0; j < mx; ++j) {
+                    const bool on = j < nq;
+                    const int q = on ? qa + j : 0;
+                    const float4* qp = reinterpret_cast<const float4*>(w.Q + q * DP);
+                    const int held = w.cnt[q];
+                    float s = 0.f;
+#pragma unroll
+                    for (int k4 = 0; k4 < DP / 4; ++k4) {
+                        const float4 v = qp[k4];
+                        const float qv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            if (4 * k4 + k < D) {
+                                const float d = __fsub_rn(qv[k], cv[4 * k4 + k]);
+                                s = __fadd_rn(s, __fmul_rn(d, d));
+                            }
+                        }
+                    }
+                    bool acc = on && s <= r2;
+                    if (acc && a.self) acc = orig != w.qor[q];
+                    // places in the list by counting the group's accepting
+                    // lanes; the last of them writes the new count (a query
+                    // belongs to one group, so no other lane does)
+                    const unsigned am = __ballot_sync(kFull, acc);
+                    if (acc) {
+                        const int p = held + __popc(am & g_lo);
+                        if (p < kListCap) {
+                            w.Ld[q * kListStr + p] = s;
+                            w.Li[q * kListStr + p] = orig;
+                        }
+                        if ((am & g_hi) == 0) w.cnt[q] = p + 1;
+                    }
+                    __syncwarp();
+                }
+                qq = qq_n;
+                orig = orig_n;
+#pragma unroll
+                for (int k = 0; k < DP; ++k) cv[k] = cvn[k];
+            }
+            __syncwarp();   // the batch's ranges are rewritten by the next batch
+        }
+
+        // per query: counts, degree, rows for the selection kernel
+        const int kept = act ? w.cnt[lane] : 0;
+        const bool spill = kept > kListCap;
+        if (act && !spill) counts[qorig] = min(kept, K);
+        if (spill && a.csr) counts[qorig] = kCsrSpill;   // counted by the selection kernel
+        if (act && !spill && a.degree) a.degree[qorig] = kept;
+        if (spill) {
+            const int pos = atomicAdd(a.ovf_count, 1);
+            if (pos < a.ovf_cap) {
+                a.ovf[pos].qslot = qs;
+                a.ovf[pos].ev = e;
+            } else {
+                atomicOr(a.status, kStatusCapacity);
+            }
+        }
+        const unsigned rows = __ballot_sync(kFull, act && !spill);   // rows written here
+        const int n = __shfl_sync(kFull, spill ? 0 : kept, lane & 15);
+        const int most = __reduce_max_sync(kFull, (unsigned)n);
+        int sorted = 32;   // places of the lists that hold the row or its padding
+        if (most <= 8) {
+            sort_rows<4>(w, n);
+            sorted = 8;
+        } else if (most <= 16) {
+            sort_rows<8>(w, n);
+            sorted = 16;
+        } else {
+            sort_rows<16>(w, n);
+        }
+        const bool vec = (width & 3) == 0 &&
+                         ((reinterpret_cast<uintptr_t>(oidx) | reinterpret_cast<uintptr_t>(od2)) & 15) == 0;
+        if (vec) {
+            // quarter p of a row: its indices for p < w4, then its distances
+            for (int p0 = 0; p0 < 2 * w4; p0 += 32) {
+                const int p = p0 + lane;
+                const bool dist = p >= w4;
+                const int e0 = 4 * (dist ? p - w4 : p);
+                const bool lane_on = p < 2 * w4;
+                const bool listed = lane_on && e0 < sorted;   // else padding
+                const int pad = dist ? 0x7f800000 : -1;
+                const int32_t* src4 = (dist ? reinterpret_cast<const int32_t*>(w.Ld) : w.Li) + e0;
+                int32_t* dst = (dist ? reinterpret_cast<int32_t*>(od2) : oidx) + e0;
+                unsigned left = rows;
+                while (left) {
+                    const int q = __ffs(left) - 1;
+                    left &= left - 1u;
+                    int4 v = make_int4(pad, pad, pad, pad);
+                    if (listed) v = *reinterpret_cast<const int4*>(src4 + q * kListStr);
+                    if (lane_on && (!a.csr || e0 < w.cnt[q]))
+                        *reinterpret_cast<int4*>(dst + (int64_t)w.qor[q] * width) = v;
+                }
+            }
+        } else {
+            unsigned left = rows;
+            while (left) {
+                const int q = __ffs(left) - 1;
+                left &= left - 1u;
+                const int64_t at = (int64_t)w.qor[q] * width;
+                const int stop = a.csr ? min(w.cnt[q], width) : width;
+                for (int e2 = lane; e2 < stop; e2 += 32) {
+                    oidx[at + e2] = e2 < sorted ? w.Li[q * kListStr + e2] : -1;
+                    od2[at + e2] = e2 < sorted ? w.Ld[q * kListStr + e2] : INFINITY;
+                }
+            }
+        }
+        __syncwarp();
+    }
+}
+
+template <int D>
+cudaError_t launch(const QueryArgs& a, int num_sms, cudaStream_t st) {
+    auto kern = &k_half_query<D>;
+    const size_t smem = (size_t)kWarps * warp_bytes<D>();
+    cudaError_t ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (ce != cudaSuccess) return ce;
+    int per_sm = 0;
+    ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarps * 32, smem);
+    if (ce != cudaSuccess) return ce;
+    const int64_t blocks = (int64_t)num_sms * std::max(per_sm, 1);
+    // sets too small to give every resident warp a chunk of 16 queries are cut
+    // into chunks of 8 or 4 (a warp's chunk is a serial chain)
+    int sub = 0;
+    while (sub < 2 && ((int64_t)a.nchunks << sub) < blocks * kWarps) ++sub;
+    const int64_t need = ceil_div((int64_t)a.nchunks << sub, kWarps);
+    launch_pdl(kern, dim3((unsigned)std::min(blocks, std::max<int64_t>(need, 1))), dim3(kWarps * 32), smem, st,
+               a, sub);
+    return cudaGetLastError();
+}
+
+}  // namespace half
+
+cudaError_t enqueue_half_query(const QueryArgs& a, int num_sms, cudaStream_t st) {
+    if (a.nchunks <= 0) return cudaSuccess;
+    switch (a.D) {
+#define FRNN_CASE(d) case d: return half::launch<d>(a, num_sms, st);
+        FRNN_CASE(5) FRNN_CASE(6) FRNN_CASE(7) FRNN_CASE(8) FRNN_CASE(9) FRNN_CASE(10)
+        FRNN_CASE(11) FRNN_CASE(12) FRNN_CASE(13) FRNN_CASE(14) FRNN_CASE(15) FRNN_CASE(16)
+#undef FRNN_CASE
+    }
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace frnn

@@ -173,16 +173,20 @@ __global__ void __launch_bounds__(kWarps * 32, BIG ? 1 : (D <= 8 ? 8 : (D <= 12 
         // the neighbour rows' slot ranges, compact, as one candidate stream
         int nr = 0, U = 0;
         {
-            const int qc = a.qcell[qs];
+            const int key = a.qcell[qs];
+            const int qc = stored_cell(h, key);
             const int dims0 = h.dims[0], m = h.m;
+            const bool half = h.half != 0;
+            const int bits = key & ((1 << kHalfBits) - 1);
             const int x = qc % dims0, qrow = qc / dims0;
             const int x0 = max(x - m, 0), x1 = min(x + m, dims0 - 1);
-            const int nrows = neighbour_rows(h);
+            const int nrows = half ? 1 << (h.naxes - 1) : neighbour_rows(h);
             for (int l0 = 0; l0 < nrows; l0 += 32) {
                 const int l = l0 + lane;
                 int lo = 0, n = 0;
                 int64_t rowbase;
-                if (l < nrows && neighbour_row(h, qrow, l, rowbase)) {
+                if (l < nrows && (half ? neighbour_row_half(h, qrow, bits, l, rowbase)
+                                       : neighbour_row(h, qrow, l, rowbase))) {
                     lo = __ldg(a.cstart + rowbase + x0);
                     n = __ldg(a.cstart + rowbase + x1 + 1) - lo;
                 }

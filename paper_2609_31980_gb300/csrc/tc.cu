@@ -64,7 +64,7 @@ constexpr int kTcEpi = 256;      // epilogue threads: warp w < 8 owns TMEM lanes
 constexpr int kTcThreads = kTcEpi + 32;   // + one producer warp (bulk copies, MMA issue)
 constexpr int kTcLStr = kTcM + 1;         // list table: one column per query row
 constexpr int kTcMaxChunks = 128;         // chunk table entries kept in shared memory
-constexpr int kTcMaxRows = kMaxNbrRows;   // neighbour rows per task
+constexpr int kTcMaxRows = 256;           // neighbour rows per task (3^5 on a six-axis grid of half cells)
 constexpr int kTcCols = 256;     // TMEM columns per CTA: two accumulators (2 CTAs / SM)
 // (the producer warp is warp 4; epilogue warps 0..3 own the TMEM lane quarters)
 constexpr int kTcList = 30;      // per-query survivor list capacity (2 CTAs / SM up to D = 12)
@@ -314,7 +314,7 @@ struct TcArgs {
 // operand rows start at b8 = rs rounded down to 8 and end at e8 = re rounded
 // up to 8; chunks of up to 256 rows (the MMA N, rounded up to 16).
 struct ChunkTab {
-    int rs[kTcMaxRows], re[kTcMaxRows], b8[kTcMaxRows], pref[kTcMaxRows + 1];
+    int rs[kTcMaxRows], re[kTcMaxRows], pref[kTcMaxRows + 1];
     int nrows, nch;
     int4 chunk[kTcMaxChunks];   // (start, n, lo, hi) of the first chunks
 };
@@ -323,7 +323,7 @@ __device__ __forceinline__ void chunk_info_slow(const ChunkTab& t, int c, int& s
                                                 int& lo, int& hi) {
     int L = 0;
     while (L + 1 < t.nrows && t.pref[L + 1] <= c) ++L;
-    start = t.b8[L] + (c - t.pref[L]) * kTcN;
+    start = (t.rs[L] & ~7) + (c - t.pref[L]) * kTcN;
     const int e8 = (t.re[L] + 7) & ~7;
     n = min(kTcN, e8 - start);
     n = (n + 31) & ~31;   // whole 32-column TMEM loads; extra rows are masked by [lo, hi)
@@ -449,8 +449,8 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_query(TcArgs a) {
         if (producer) {
             // neighbour rows and chunk table
             const int dims0 = h.dims[0], m = h.m;
-            const int xa = a.qcell[tk.qslot] % dims0;
-            const int xb = a.qcell[tk.qslot + tk.nq - 1] % dims0;
+            const int xa = stored_cell(h, a.qcell[tk.qslot]) % dims0;
+            const int xb = stored_cell(h, a.qcell[tk.qslot + tk.nq - 1]) % dims0;
             // (2m+1)^(naxes-1) <= kTcMaxRows rows (the grid parameters ensure
             // it), 32 per round with a running chunk count
             const int nrows = neighbour_rows(h);
@@ -475,7 +475,6 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_query(TcArgs a) {
                 if (l < kTcMaxRows) {
                     s_ct.rs[l] = rs;
                     s_ct.re[l] = re;
-                    s_ct.b8[l] = b8;
                     s_ct.pref[l] = carry + pre - nch;
                 }
                 // this lane's row: its chunks' (start, n, lo, hi)
