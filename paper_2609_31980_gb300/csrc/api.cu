@@ -1340,7 +1340,9 @@ frnn_status frnn_autotune(frnn_ctx* ctx, const float* refs, int64_t N, int D, fl
         if (!(flags & FRNN_PATH_TC)) {
             if (grid_kernel(gcfg[gi].naxes) == 0) {
                 cands.push_back({FRNN_PATH_GRID, 1, 0});
-                if (!half_cells(D, gcfg[gi].naxes, m)) cands.push_back({FRNN_PATH_GRID, 2, 0});
+                // the chunk scan's other staging (half cells and grids of up to
+                // four dimensions have scans of their own)
+                if (D > 4 && !half_cells(D, gcfg[gi].naxes, m)) cands.push_back({FRNN_PATH_GRID, 2, 0});
             } else {
                 cands.push_back({FRNN_PATH_GRID, 1, 0});
                 if (D >= 5) cands.push_back({FRNN_PATH_GRID, 1, 3});

@@ -879,16 +879,18 @@ void enqueue_scan(int32_t* data, int64_t n, int32_t* parts, int32_t* total, cuda
 
 // ------------------------------------------------------------------ host
 
-// Five gridded axes at a cell edge of about r need about (extent / r)^5
-// cells (5.15 M = 17.2 n for the 300k x 8 tracking-like event, whose
-// coordinates span [-1.06, 1.06] at r = 0.1), four about (extent / r)^4; the
-// budget grows with n so that the cells stay near r on such events (every
-// build zeroes and scans the whole budget), and the parameter step falls
-// back to one axis fewer when the budget would make five-axis cells too
-// coarse.
+// The budget grows with n so that the cells stay near r on the sets the
+// library is for, and not faster, since every build zeroes and scans it all;
+// the parameter step falls back to fewer axes when it would make the cells too
+// coarse.  Half cells: 12 n, just what six axes need for the 300k x 8
+// tracking-like event (22 x 11^5 = 3.5 M; 6 n 171 us, 12 n 151, 18 n 156, 30 n
+// 166, build + query), flat within 3 us for smaller sets.  Five axes of plain
+// cells: 18 n (22^5 = 5.2 M there).  Up to four: 4 n (1 M x 3, two neighbours
+// each: n / 2 269 us, n 236, 2 n 217, 4 n 219; 300k x 4: n 133, 2 n 119, 4 n
+// 108).
 int64_t cell_cap_for(int64_t n, int naxes, bool half) {
     if (half) return std::min<int64_t>(std::max<int64_t>(16384, 12 * n), kHalfMaxCells);
-    const int64_t per = naxes >= 5 ? 18 : (naxes == 4 ? 2 : 0);
+    const int64_t per = naxes >= 5 ? 18 : 4;
     int64_t c = per ? per * n : n / 2 + 1;
     c = std::max<int64_t>(16384, c);
     return std::min<int64_t>(c, naxes >= 5 ? ((int64_t)1 << 27) : ((int64_t)1 << 24));

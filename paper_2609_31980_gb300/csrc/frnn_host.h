@@ -189,6 +189,8 @@ void rows_free(GridBufs& g);
 frnn_status enqueue_row_query(const QueryLaunch& q, const QueryArgs& a, cudaStream_t st,
                               std::string& err);
 cudaError_t enqueue_half_query(const QueryArgs& a, int num_sms, cudaStream_t st);
+// The scan of the automatic grids of up to four dimensions (query_low.cu).
+cudaError_t enqueue_low_query(const QueryArgs& a, int num_sms, cudaStream_t st);
 // The selection kernel alone over the rows the last query of q.qset listed
 // (compact output, second pass: q.ovf_mode 2, q.row_off).
 frnn_status enqueue_overflow_only(const QueryLaunch& q, cudaStream_t st, std::string& err);

@@ -831,11 +831,12 @@ frnn_status enqueue_grid_query(const QueryLaunch& q, cudaStream_t st, std::strin
         if (s != FRNN_OK) return s;
     } else if (q.kernel == 2) {
         ce = enqueue_half_query(a, q.num_sms, st);
+    } else if (rs.D <= 4) {
+        ce = enqueue_low_query(a, q.num_sms, st);
     } else if (a.nchunks > 0) {
         switch (rs.D) {
 #define FRNN_CASE(d) case d: ce = launch_grid_query_d<d>(a, q.stage, q.num_sms, st); break;
-            FRNN_CASE(1) FRNN_CASE(2) FRNN_CASE(3) FRNN_CASE(4) FRNN_CASE(5) FRNN_CASE(6)
-            FRNN_CASE(7) FRNN_CASE(8) FRNN_CASE(9) FRNN_CASE(10) FRNN_CASE(11) FRNN_CASE(12)
+            FRNN_CASE(5) FRNN_CASE(6) FRNN_CASE(7) FRNN_CASE(8) FRNN_CASE(9) FRNN_CASE(10) FRNN_CASE(11) FRNN_CASE(12)
             FRNN_CASE(13) FRNN_CASE(14) FRNN_CASE(15) FRNN_CASE(16)
 #undef FRNN_CASE
             default:
