@@ -45,6 +45,7 @@ struct frnn_ctx {
     GridBufs qset;            // cross-set query binning
     GridBufs batch;           // batched multi-event grid
     int64_t batch_points = 0; // points of the batched call being served (0 outside of one)
+    bool small_cells = false; // serving slot under a memory budget (see cell_kind)
     frnn_grid* host_grid = nullptr;   // grid of the host-buffer path
     void* hp_buf = nullptr;   // device buffers of the host-buffer path
     size_t hp_bytes = 0;
@@ -112,6 +113,7 @@ void ctx_copy_tuning(frnn_ctx* dst, const frnn_ctx* src) {
     dst->auto_tc = src->auto_tc;
     dst->tuned = src->tuned;
 }
+void ctx_small_cells(frnn_ctx* ctx) { ctx->small_cells = true; }
 void ctx_set_error(frnn_ctx* ctx, const char* msg) {
     if (ctx) ctx->err = msg;
 }
@@ -178,13 +180,21 @@ static int build_mult(const frnn_ctx* ctx, int64_t N, int D);
 // automatic choice (0) the most the build may take
 static int cap_axes(int naxes, int D) { return naxes > 0 ? naxes : std::min(D, kMaxAxes); }
 
+// The cell budget a set's grid gets.  Contexts (and serving slots) under a
+// memory budget keep the smaller plain budget at D <= 4: requests were sized
+// by it.
+static CellKind cell_kind(const frnn_ctx* ctx, int64_t N, int D) {
+    const int naxes = build_naxes(ctx, N, D);
+    if (half_cells(D, naxes, build_mult(ctx, N, D))) return CellKind::kHalf;
+    return D <= 4 && naxes == 0 && ctx->budget == 0 && !ctx->small_cells ? CellKind::kLow : CellKind::kPlain;
+}
+
 static frnn_status alloc_accounted(frnn_ctx* c, GridBufs& g, int E, const int64_t* n, int D,
                                    const int64_t* caps_in) {
     std::vector<int64_t> caps(E);
     for (int e = 0; e < E; ++e)
         caps[e] = caps_in ? caps_in[e]
-                          : cell_cap_for(n[e], cap_axes(build_naxes(c, n[e], D), D),
-                                         half_cells(D, build_naxes(c, n[e], D), build_mult(c, n[e], D)));
+                          : cell_cap_for(n[e], cap_axes(build_naxes(c, n[e], D), D), cell_kind(c, n[e], D));
     const size_t old_bytes = g.bytes;
     const size_t need = predict_grid_bytes(E, n, D, caps.data());
     const bool reuse = g.base && need <= g.bytes;

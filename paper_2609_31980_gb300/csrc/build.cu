@@ -887,10 +887,12 @@ void enqueue_scan(int32_t* data, int64_t n, int32_t* parts, int32_t* total, cuda
 // 166, build + query), flat within 3 us for smaller sets.  Five axes of plain
 // cells: 18 n (22^5 = 5.2 M there).  Up to four: 4 n (1 M x 3, two neighbours
 // each: n / 2 269 us, n 236, 2 n 217, 4 n 219; 300k x 4: n 133, 2 n 119, 4 n
-// 108).
-int64_t cell_cap_for(int64_t n, int naxes, bool half) {
-    if (half) return std::min<int64_t>(std::max<int64_t>(16384, 12 * n), kHalfMaxCells);
-    const int64_t per = naxes >= 5 ? 18 : 4;
+// 108) on automatic grids of up to four dimensions; requested axes as before
+// (2 n for four, n / 2 for fewer: row tasks and tensor-core tiles want long
+// rows of cells).
+int64_t cell_cap_for(int64_t n, int naxes, CellKind kind) {
+    if (kind == CellKind::kHalf) return std::min<int64_t>(std::max<int64_t>(16384, 12 * n), kHalfMaxCells);
+    const int64_t per = naxes >= 5 ? 18 : (kind == CellKind::kLow ? 4 : (naxes == 4 ? 2 : 0));
     int64_t c = per ? per * n : n / 2 + 1;
     c = std::max<int64_t>(16384, c);
     return std::min<int64_t>(c, naxes >= 5 ? ((int64_t)1 << 27) : ((int64_t)1 << 24));

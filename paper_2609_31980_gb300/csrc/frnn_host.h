@@ -97,8 +97,8 @@ constexpr int kTcRowPad = 512;      // rows readable past the last slot (chunk r
 
 // Cells allowed for an n-point event gridded over naxes coordinates (the
 // parameter step enlarges the cells when the grid would need more).
-// half: a grid of half cells (stored cells).
-int64_t cell_cap_for(int64_t n, int naxes, bool half = false);
+enum class CellKind { kPlain, kHalf, kLow };   // kHalf: stored half cells; kLow: automatic, D <= 4
+int64_t cell_cap_for(int64_t n, int naxes, CellKind kind = CellKind::kPlain);
 
 // Compute the layout for E events of sizes n[e] and allocate (or reuse).
 // caps (optional): per-event cell capacities (a query set binned with a
@@ -218,6 +218,7 @@ frnn_status enqueue_overflow(const QueryArgs& a, int num_sms, cudaStream_t st, s
 
 // Context helpers for the serving loop (defined with the context, api.cu).
 void ctx_copy_tuning(frnn_ctx* dst, const frnn_ctx* src);
+void ctx_small_cells(frnn_ctx* ctx);   // keep the plain cell budget at D <= 4
 // Launch a kernel with programmatic stream serialization (see pdl_wait).
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,

@@ -88,6 +88,7 @@ frnn_status frnn_serve_run(frnn_ctx* ctx, const frnn_request* reqs, int n_reqs, 
         if (status != FRNN_OK) break;
         // children inherit the parent's options; every batch is new, so no graph
         ctx_copy_tuning(s.ctx, ctx);
+        if (mem_budget_bytes) ctx_small_cells(s.ctx);   // admission estimates by the plain cell budget
         frnn_set_option(s.ctx, FRNN_OPT_USE_GRAPH, 0);
     }
 
