@@ -19,7 +19,10 @@
 //   k_scatter   slot -> original index, slot -> cell, and the point's row of
 //               DP floats at its slot (cell-sorted coordinates)
 // (the tensor-core path adds its 128-query tiles: k_rowtasks, a scan, k_emit)
+#include <cooperative_groups.h>
+
 #include <algorithm>
+#include <climits>
 #include <cmath>
 
 #include "frnn_host.h"
@@ -90,6 +93,22 @@ struct StagedRow {
     __device__ __forceinline__ float operator[](int k) const { return sm[stage_slot(j0 + k, pad)]; }
 };
 
+// One cell-sorted row of DP floats (zero padding), written in 32-byte or
+// 16-byte pieces.
+__device__ __forceinline__ void write_row(float* dst, const StagedRow& src, int D, int DP) {
+    auto at = [&](int k) { return k < D ? src[k] : 0.f; };
+    if ((DP & 7) == 0) {
+        for (int k = 0; k < DP; k += 8)
+            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + k), "f"(at(k)),
+                         "f"(at(k + 1)), "f"(at(k + 2)), "f"(at(k + 3)), "f"(at(k + 4)), "f"(at(k + 5)),
+                         "f"(at(k + 6)), "f"(at(k + 7))
+                         : "memory");
+    } else {
+        for (int k = 0; k < DP; k += 4)
+            *reinterpret_cast<float4*>(dst + k) = make_float4(at(k), at(k + 1), at(k + 2), at(k + 3));
+    }
+}
+
 // Stage nf consecutive floats of a row-major point array into shared memory
 // (at stage_slot), using 16-byte vector loads for the aligned body.
 __device__ __forceinline__ void stage_floats(float* sm, const float* src, int nf, bool pad) {
@@ -100,13 +119,25 @@ __device__ __forceinline__ void stage_floats(float* sm, const float* src, int nf
     for (int i = threadIdx.x; i < head; i += blockDim.x) sm[stage_slot(i, pad)] = __ldg(src + i);
     const int n4 = (nf - head) >> 2;
     const float4* s4 = reinterpret_cast<const float4*>(src + head);
-    for (int i = threadIdx.x; i < n4; i += blockDim.x) {
-        float4 v = __ldg(s4 + i);
-        const int j = head + 4 * i;
-        sm[stage_slot(j, pad)] = v.x;
-        sm[stage_slot(j + 1, pad)] = v.y;
-        sm[stage_slot(j + 2, pad)] = v.z;
-        sm[stage_slot(j + 3, pad)] = v.w;
+    constexpr int kAhead = 3;   // loads in flight per thread
+    for (int i0 = threadIdx.x; i0 < n4; i0 += kAhead * blockDim.x) {
+        float4 v[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int i = i0 + u * blockDim.x;
+            v[u] = i < n4 ? __ldg(s4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int i = i0 + u * blockDim.x;
+            const int j = head + 4 * i;
+            if (i < n4) {
+                sm[stage_slot(j, pad)] = v[u].x;
+                sm[stage_slot(j + 1, pad)] = v[u].y;
+                sm[stage_slot(j + 2, pad)] = v[u].z;
+                sm[stage_slot(j + 3, pad)] = v[u].w;
+            }
+        }
     }
     for (int i = head + 4 * n4 + threadIdx.x; i < nf; i += blockDim.x)
         sm[stage_slot(i, pad)] = __ldg(src + i);
@@ -318,6 +349,13 @@ __device__ void grid_fit(GridFit& f, float lo_j, float hi_j, int D, int k, int m
                          float r, int64_t cap, bool valid, int max_rows, bool half) {
     constexpr unsigned kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
+    const int la = lane & 7;   // the lane's axis (every eighth lane alike, for the products below)
+    // product of an axis value over the axes, on every lane
+    auto over_axes = [&](auto x) {
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) x *= __shfl_xor_sync(kAll, x, o);
+        return x;
+    };
     f.naxes = k;
     // neighbour rows, (2m+1)^(k-1): at most max_rows (the chunk kernel
     // enumerates kMaxNbrRows, 32 per round; the row-task kernel one per lane)
@@ -332,7 +370,7 @@ __device__ void grid_fit(GridFit& f, float lo_j, float hi_j, int D, int k, int m
     // the last k coordinates; a sixth axis (half cells) is the one before the
     // last five
     const int k5 = min(k, kMaxAxes);
-    int ax = lane < k5 ? D - k5 + lane : (lane < k ? D - 1 - lane : 0);
+    int ax = la < k5 ? D - k5 + la : (la < k ? D - 1 - la : 0);
     if (valid && axes_mode == 1 && D > k) {
         // the k widest coordinates (ties by lower index), in index order
         const float wj = __fsub_rn(hi_j, lo_j);
@@ -342,7 +380,7 @@ __device__ void grid_fit(GridFit& f, float lo_j, float hi_j, int D, int k, int m
             if (wi > wj || (wi == wj && i < lane)) ++rank;
         }
         const unsigned sel = __ballot_sync(kAll, lane < D && rank < k);
-        const int want_pos = k > kMaxAxes ? (lane < kMaxAxes ? lane + 1 : 0) : lane;
+        const int want_pos = k > kMaxAxes ? (la < kMaxAxes ? la + 1 : 0) : la;
         int cnt = 0;
         ax = 0;
         for (int j = 0; j < D; ++j) {
@@ -354,7 +392,7 @@ __device__ void grid_fit(GridFit& f, float lo_j, float hi_j, int D, int k, int m
     }
     const float lo = __shfl_sync(kAll, lo_j, ax);
     const float hi = __shfl_sync(kAll, hi_j, ax);
-    f.axis = lane < k ? ax : 0;
+    f.axis = la < k ? ax : 0;
     f.lo = lo;
     f.hi = hi;
     if (!valid) {
@@ -373,7 +411,7 @@ __device__ void grid_fit(GridFit& f, float lo_j, float hi_j, int D, int k, int m
     for (int it = 0; it < 4096; ++it) {
         bool ok = true;
         dim = 1;
-        if (lane < k) {
+        if (la < k) {
             const float c = floorf(__fmul_rn(ext, ih)) + 1.0f;
             if (!(c <= (float)kMaxDimsPerAxis)) ok = false;
             else dim = (int)c;
@@ -381,15 +419,21 @@ __device__ void grid_fit(GridFit& f, float lo_j, float hi_j, int D, int k, int m
                 __fadd_ru(__fmul_ru(ih, __fadd_ru(rho_up, __fmul_ru(0x1p-21f, ext_up))), 0x1p-148f);
             if (!(bound < need)) ok = false;
         }
-        sdim = half && lane > 0 ? (dim + 1) >> 1 : dim;
-        cells = 1;
-        for (int a = 0; a < k; ++a) cells *= __shfl_sync(kAll, sdim, a);
+        sdim = half && la > 0 ? (dim + 1) >> 1 : dim;
+        cells = over_axes((int64_t)sdim);   // (1 beyond the k axes; at most 1024^6)
         if (__all_sync(kAll, ok) && cells <= cap) {
             fit = true;
             f.at_start = it == 0;
             break;
         }
-        ih = __fmul_rd(ih, 0.9f);
+        // too many cells: by the ratio the budget asks for (the dims' rounding
+        // may need another step); a failed bound or axis limit: by a tenth
+        float shrink = 0.9f;
+        if (__all_sync(kAll, ok)) {
+            shrink = exp2f(log2f((float)cap / (float)cells) / (float)k);
+            shrink = fminf(fmaxf(shrink, 0.5f), 0.97f);
+        }
+        ih = __fmul_rd(ih, shrink);
         if (!(ih > 0.f)) break;
     }
     if (!fit) {   // one cell is always safe
@@ -398,19 +442,98 @@ __device__ void grid_fit(GridFit& f, float lo_j, float hi_j, int D, int k, int m
         sdim = 1;
         cells = 1;
     }
-    f.dim = lane < k ? dim : 1;
-    f.sdim = lane < k ? sdim : 1;
+    f.dim = la < k ? dim : 1;
+    f.sdim = la < k ? sdim : 1;
     f.inv_h = ih;
     f.ncells = (int32_t)cells;
     float fr = 1.f;
-    if (lane < k && ext_up > 0.f) {
-        const float cover = half && lane > 0 ? 4.f : 2.f * (float)mm + 1.f;
+    if (la < k && ext_up > 0.f) {
+        const float cover = half && la > 0 ? 4.f : 2.f * (float)mm + 1.f;
         const float span = ih > 0.f ? cover / ih : INFINITY;
         fr = fminf(1.f, span / ext_up);
     }
-    float frac = 1.f;
-    for (int a = 0; a < k; ++a) frac *= __shfl_sync(kAll, fr, a);
-    f.frac = frac;
+    f.frac = over_axes(fr);
+}
+
+// ceil(2^36 / d) for 1 <= d <= 1024 (EventHdr::mag) in 32-bit divisions: with
+// 2^32 = q d + rem, 0 < rem <= d, it is 16 q + ceil(16 rem / d).
+__device__ __forceinline__ uint64_t division_multiplier(uint32_t d) {
+    const uint32_t q = 0xffffffffu / d;
+    const uint32_t rem = 0xffffffffu - q * d + 1u;
+    return 16ull * q + (16u * rem + d - 1u) / d;
+}
+
+// The grid parameters of one event from its bounding box, by a whole block (at
+// least kFitWarps warps): box[j], box[kMaxD + j] are the ordered-int extremes of
+// coordinate j in shared memory, bad a non-finite input.  Warp w fits the
+// candidate of k_hi - w axes; the best one's warp writes the parameters.
+// H: the event's header (global or shared memory), everything else of it set.
+constexpr int kFitWarps = 3;
+__device__ void derive_params(EventHdr& H, const int32_t* box, bool bad, int D, float r, int m, int axes_mode,
+                              int naxes_req) {
+    __shared__ float s_frac[kFitWarps];
+    __shared__ int s_start[kFitWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t n = H.n;
+    // per-event presets (batched autotuning) win over the call's options; 0 =
+    // automatic: the candidate with the smallest expected neighbourhood under
+    // the cell budget among the widest count and one axis fewer (half cells:
+    // six, five and four axes)
+    const int want = H.naxes > 0 ? H.naxes : naxes_req;
+    const int m_req = H.m > 0 ? H.m : m;
+    const bool half = H.half != 0;
+    const float lo_j = lane < D ? ordered_to_float(box[lane]) : 0.f;
+    const float hi_j = lane < D ? ordered_to_float(box[kMaxD + lane]) : 0.f;
+    const bool fin = lane >= D || (isfinite(lo_j) && isfinite(hi_j));
+    const bool valid = __all_sync(0xffffffffu, fin) && !bad && n > 0;
+    const int kmax = min(D, half ? kHdrAxes : kMaxAxes);
+    const int k_hi = want > 0 ? min(D, min(want, kMaxAxes)) : kmax;
+    const int k_lo = want > 0 ? k_hi : max(1, kmax - (half ? 2 : 1));
+    const int64_t cap = half ? min((int64_t)H.cell_cap, kHalfMaxCells) : (int64_t)H.cell_cap;
+    // grids requested with up to four axes are scanned by the row-task
+    // kernel, whose lanes hold one neighbour row each
+    const int max_rows = (want >= 1 && want <= 4) ? 32 : kMaxNbrRows;
+    GridFit f;
+    f.frac = INFINITY;
+    if (warp < kFitWarps && k_hi - warp >= k_lo)
+        grid_fit(f, lo_j, hi_j, D, k_hi - warp, half ? 1 : m_req, axes_mode, r, cap, valid, max_rows, half);
+    if (warp < kFitWarps && lane == 0) {
+        s_frac[warp] = f.frac;
+        s_start[warp] = f.at_start ? 1 : 0;
+    }
+    __syncthreads();   // (also: every warp has read the header before it is written)
+    // at the starting cell edge a grid over more axes covers at most the
+    // fraction of one over fewer (one factor <= 1 more): those are not taken
+    int best = 0;
+    for (int w = 1; w < kFitWarps && k_hi - w >= k_lo && !s_start[w - 1]; ++w)
+        if (s_frac[w] < s_frac[best]) best = w;
+    if (warp != best) return;
+    const int na = f.naxes;
+    if (lane < kHdrAxes) {
+        const bool gridded = lane < na;
+        const int sd = gridded && valid ? f.sdim : 1;
+        H.axes[lane] = gridded ? f.axis : 0;
+        H.dims[lane] = sd;
+        H.fdims[lane] = gridded && valid ? f.dim : 1;
+        H.mag[lane] = division_multiplier((uint32_t)sd);
+        H.lo[lane] = gridded && valid ? f.lo : 0.f;
+        H.hi[lane] = gridded && valid ? f.hi : 0.f;
+    }
+    if (lane < kMaxD) {
+        float c = 0.f;
+        if (valid && lane < D) {
+            c = __fadd_rn(lo_j, __fmul_rn(0.5f, __fsub_rn(hi_j, lo_j)));
+            if (!isfinite(c)) c = 0.f;
+        }
+        H.ctr[lane] = c;
+    }
+    if (lane == 0) {
+        H.naxes = na;
+        H.m = f.m;
+        H.valid = valid ? 1 : 0;
+        H.inv_h = valid ? f.inv_h : 0.f;
+        H.ncells = valid ? f.ncells : 1;
+    }
 }
 
 __device__ void event_params(EventHdr* hdr, int e, int D, const int32_t* bbox, float r, int m,
@@ -430,76 +553,17 @@ __device__ void event_params(EventHdr* hdr, int e, int D, const int32_t* bbox, f
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
         const int k = warp + 8 * i;
-        for (int o = 16; o > 0; o >>= 1) {
-            const int32_t x = __shfl_xor_sync(0xffffffffu, v[i], o);
-            v[i] = k < 16 ? min(v[i], x) : (k < 32 ? max(v[i], x) : (v[i] | x));
-        }
-        if (lane == 0 && k < kBBoxStride) bb[k] = v[i];
+        const int32_t x = k < 16 ? __reduce_min_sync(0xffffffffu, v[i])
+                                 : (k < 32 ? __reduce_max_sync(0xffffffffu, v[i])
+                                           : (int32_t)__reduce_or_sync(0xffffffffu, (unsigned)v[i]));
+        if (lane == 0 && k < kBBoxStride) bb[k] = x;
     }
     __syncthreads();
-    if (warp != 0) return;
     EventHdr& H = hdr[e];
-    const int64_t n = H.n;
-    const int64_t cell_off = H.cell_off;
-    const int32_t cell_cap = H.cell_cap;
-    // per-event presets (batched autotuning) win over the call's options;
-    // 0 = automatic: the widest count up to kMaxAxes, or one fewer axis when
-    // the cell budget makes that grid's neighbourhoods smaller
-    const int want = H.naxes > 0 ? H.naxes : naxes_req;
-    const int m_req = H.m > 0 ? H.m : m;
-    __syncwarp();   // every lane has read the header before it is written
     // the last cell-array entry of the event counts its pair padding slot, so
     // the next event's slots start on a pair boundary
-    if (lane == 0) counts[cell_off + cell_cap] = (int32_t)(n & 1);
-    const float lo_j = lane < D ? ordered_to_float(bb[lane]) : 0.f;
-    const float hi_j = lane < D ? ordered_to_float(bb[16 + lane]) : 0.f;
-    const bool fin = lane >= D || (isfinite(lo_j) && isfinite(hi_j));
-    const bool valid = __all_sync(0xffffffffu, fin) && bb[32] == 0 && n > 0;
-    // (half cells: six, five or four axes, always the automatic choice)
-    const bool half = H.half != 0;
-    const int kmax = min(D, half ? kHdrAxes : kMaxAxes);
-    const int k_hi = want > 0 ? min(D, min(want, kMaxAxes)) : kmax;
-    const int k_lo = want > 0 ? k_hi : max(1, kmax - (half ? 2 : 1));
-    const int64_t cap = half ? min((int64_t)cell_cap, kHalfMaxCells) : (int64_t)cell_cap;
-    // grids requested with up to four axes are scanned by the row-task
-    // kernel, whose lanes hold one neighbour row each
-    const int max_rows = (want >= 1 && want <= 4) ? 32 : kMaxNbrRows;
-    GridFit best;
-    best.frac = INFINITY;
-    for (int k = k_hi; k >= k_lo; --k) {
-        GridFit f;
-        grid_fit(f, lo_j, hi_j, D, k, half ? 1 : m_req, axes_mode, r, cap, valid, max_rows, half);
-        if (f.frac < best.frac) best = f;
-        // at the starting cell edge a grid over more axes covers at most the
-        // fraction of one over fewer (one factor <= 1 more): no need to try fewer
-        if (f.at_start) break;
-    }
-    const int na = best.naxes;
-    if (lane < kHdrAxes) {
-        const bool gridded = lane < na;
-        const int sd = gridded && valid ? best.sdim : 1;
-        H.axes[lane] = gridded ? best.axis : 0;
-        H.dims[lane] = sd;
-        H.fdims[lane] = gridded && valid ? best.dim : 1;
-        H.mag[lane] = ((1ull << 36) + (uint64_t)sd - 1) / (uint64_t)sd;
-        H.lo[lane] = gridded && valid ? best.lo : 0.f;
-        H.hi[lane] = gridded && valid ? best.hi : 0.f;
-    }
-    if (lane < kMaxD) {
-        float c = 0.f;
-        if (valid && lane < D) {
-            c = __fadd_rn(lo_j, __fmul_rn(0.5f, __fsub_rn(hi_j, lo_j)));
-            if (!isfinite(c)) c = 0.f;
-        }
-        H.ctr[lane] = c;
-    }
-    if (lane == 0) {
-        H.naxes = na;
-        H.m = best.m;
-        H.valid = valid ? 1 : 0;
-        H.inv_h = valid ? best.inv_h : 0.f;
-        H.ncells = valid ? best.ncells : 1;
-    }
+    if (threadIdx.x == 0) counts[H.cell_off + H.cell_cap] = (int32_t)(H.n & 1);
+    derive_params(H, bb, bb[32] != 0, D, r, m, axes_mode, naxes_req);
 }
 
 // Cross-set binning: take the reference grid's parameters for each event.
@@ -601,16 +665,7 @@ __global__ void __launch_bounds__(kBuildPtsPerBlock) k_scatter(const EventHdr* h
     const int64_t slot = (int64_t)cstart[h.cell_off + stored_cell(h, c)] + rnk[gi];
     perm[slot] = (int32_t)(p0 + i);
     cell[slot] = c;
-    const StagedRow src{sm, i * D, pad};
-    float4* dst = reinterpret_cast<float4*>(pts + slot * DP);
-    for (int j = 0; j < DP / 4; ++j) {
-        float4 v;
-        v.x = 4 * j + 0 < D ? src[4 * j + 0] : 0.f;
-        v.y = 4 * j + 1 < D ? src[4 * j + 1] : 0.f;
-        v.z = 4 * j + 2 < D ? src[4 * j + 2] : 0.f;
-        v.w = 4 * j + 3 < D ? src[4 * j + 3] : 0.f;
-        dst[j] = v;
-    }
+    write_row(pts + slot * DP, StagedRow{sm, i * D, pad}, D, DP);
 }
 
 // Per row of cells (all gridded coordinates but the fastest fixed): number of
@@ -877,6 +932,266 @@ void enqueue_scan(int32_t* data, int64_t n, int32_t* parts, int32_t* total, cuda
     }
 }
 
+// ------------------------------------------------------------------ small sets
+// The whole build of one small event in one launch: a cluster of kSmallCtas
+// CTAs, cluster barriers where the chain above has kernel boundaries.  A set of
+// a few thousand points leaves the six kernels of the chain nothing to do but
+// launch, read the previous one's results from L2 and drain (about 3 us each);
+// a cluster's SMs hold the points' cell ids and ranks in registers, and
+// the barriers cost 0.5 us each.  All of the memory it shares across CTAs is
+// read past L1 (ld.cg) after a cluster barrier.  Bound by the latency of its
+// phases (4096 x 3: 10.4 us, 2.7 of them the grid parameters, 5.5 the cell
+// counts' four round trips); sixteen SMs are enough up to 32,768 points, where
+// the chain catches up.  Build + query, chain / cluster: 4096 x 3 30.8 / 21.1
+// us, 5,000 x 8 40.5 / 24.4, 20,000 x 8 45.8 / 38.4, 32,000 x 8 52.2 / 49.9
+// (eight CTAs without staged rows lost from 13,000 points on).
+//   1 bounding box of the CTA's points (input only, so before the wait for the
+//     previous kernel), zeroing of the cell counts; boxes to every CTA
+//   2 grid parameters (one warp of every CTA, redundantly); cell ids, ranks
+//   3 per-warp sums of the counts; CTA sums to every CTA
+//   4 exclusive scan of the counts in place
+//   5 slot maps and cell-sorted coordinates
+// With `src` (cross-set queries) the parameters are those of src's grid.
+
+constexpr int kSmallCtas = 16;
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallPer = 2;    // points of a thread, at most
+constexpr int kSmallQuads = 2;  // 128-entry steps of a warp's scan segment kept in registers
+constexpr int64_t kSmallMax = (int64_t)kSmallCtas * kSmallThreads * kSmallPer;
+constexpr int64_t kSmallCells = 16 * kSmallMax;   // cell-array entries
+
+__host__ __device__ constexpr size_t small_stage_floats(int64_t per, int D) {
+    return (size_t)per * D + (size_t)per * D / 32 + 1;
+}
+
+__global__ void __launch_bounds__(kSmallThreads, 1)
+    k_build_small(OneEventTables t1, const EventHdr* src, int per, int D, int DP, float r, int m, int axes_mode,
+                  int naxes_req, EventHdr* hdr, int32_t* blk_start, int64_t* cell_off, int32_t* counts,
+                  int32_t* scalars, float* pts, int32_t* perm, int32_t* cell, int32_t* status) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    constexpr int kWarps = kSmallThreads / 32;
+    constexpr unsigned kAll = 0xffffffffu;
+    extern __shared__ float sm[];   // this CTA's input rows (staged_slot layout)
+    __shared__ EventHdr sh;
+    __shared__ int32_t s_mn[kMaxD], s_mx[kMaxD], s_bad;
+    __shared__ int32_t s_box[kSmallCtas][2 * kMaxD + 1], s_all[2 * kMaxD];
+    __shared__ int32_t s_wt[kWarps], s_tot[kSmallCtas];
+    pdl_trigger();
+    cluster.barrier_arrive();   // (every CTA must run before its shared memory is written)
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = (int)cluster.block_rank(), ctas = (int)cluster.num_blocks();
+    const int n = (int)t1.hdr.n;
+    const float* refs = t1.hdr.refs;
+    const bool pad = (D & 3) == 0;
+    // this CTA's points [p0, p0 + np); thread t has the t-th, t + 1024-th, ...
+    const int p0 = min(rank * per, n), np = min(per, n - p0);
+    const int first = rank * kSmallThreads + tid, step = ctas * kSmallThreads;
+    if (tid < kMaxD) {
+        s_mn[tid] = INT_MAX;
+        s_mx[tid] = INT_MIN;
+    }
+    if (tid == 0) s_bad = 0;
+    for (int i = tid; i < (int)(sizeof(EventHdr) / 4); i += kSmallThreads)
+        reinterpret_cast<int32_t*>(&sh)[i] = reinterpret_cast<const int32_t*>(&t1.hdr)[i];
+    stage_floats(sm, refs + (int64_t)p0 * D, np * D, pad);
+    __syncthreads();
+    {
+        // warp w takes coordinate w % D of every (32 / D)-th run of 32 points
+        const int runs = kWarps / D, k = warp % D, g = warp / D;
+        if (g < runs) {
+            bool bad = false;
+            float mn = INFINITY, mx = -INFINITY;
+#pragma unroll 4
+            for (int i = g * 32 + lane; i < np; i += runs * 32) {
+                const float v = sm[stage_slot(i * D + k, pad)];
+                bad |= !isfinite(v);
+                mn = fminf(mn, v);
+                mx = fmaxf(mx, v);
+            }
+            const int32_t a = __reduce_min_sync(kAll, float_to_ordered(mn));
+            const int32_t b = __reduce_max_sync(kAll, float_to_ordered(mx));
+            const bool any_bad = __any_sync(kAll, bad);
+            if (lane == 0) {
+                atomicMin(s_mn + k, a);
+                atomicMax(s_mx + k, b);
+                if (any_bad) atomicOr(&s_bad, 1);
+            }
+        }
+    }
+    pdl_wait();   // the previous work on the stream may still read what is written from here on
+    {
+        const int L = t1.hdr.cell_cap + 1;
+        int4* c4 = reinterpret_cast<int4*>(counts);
+        for (int j = first; j < L / 4; j += step) c4[j] = make_int4(0, 0, 0, 0);
+        for (int j = L / 4 * 4 + first; j < L; j += step) counts[j] = 0;
+    }
+    if (rank == 0 && tid < kScalars) scalars[tid] = 0;
+    __syncthreads();
+    cluster.barrier_wait();
+    // this CTA's box to every CTA
+    if (tid < ctas * 64) {
+        const int to = tid >> 6, k = tid & 63;
+        if (k <= 2 * kMaxD)
+            *cluster.map_shared_rank(&s_box[rank][k], to) =
+                k < kMaxD ? s_mn[k] : (k < 2 * kMaxD ? s_mx[k - kMaxD] : s_bad);
+    }
+    cluster.sync();
+    int bad = 0;
+    for (int c = 0; c < ctas; ++c) bad |= s_box[c][2 * kMaxD];
+    if (rank == 0 && tid == 0 && bad) atomicOr(status, kStatusNonFinite);
+    if (tid < 2 * kMaxD) {
+        int32_t v = s_box[0][tid];
+        for (int c = 1; c < ctas; ++c) v = tid < kMaxD ? min(v, s_box[c][tid]) : max(v, s_box[c][tid]);
+        s_all[tid] = v;
+    }
+    __syncthreads();
+    if (src) {
+        // the parameters of the foreign header
+        if (tid == 0) {
+            sh.naxes = src->naxes;
+            sh.m = src->m;
+            sh.valid = src->valid;
+            sh.inv_h = src->inv_h;
+            sh.ncells = src->ncells;
+            sh.half = src->half;
+        }
+        if (tid < kHdrAxes) {
+            sh.axes[tid] = src->axes[tid];
+            sh.dims[tid] = src->dims[tid];
+            sh.fdims[tid] = src->fdims[tid];
+            sh.mag[tid] = src->mag[tid];
+            sh.lo[tid] = src->lo[tid];
+            sh.hi[tid] = src->hi[tid];
+        }
+        if (tid < kMaxD) sh.ctr[tid] = src->ctr[tid];
+    } else {
+        derive_params(sh, s_all, bad != 0, D, r, m, axes_mode, naxes_req);
+    }
+    __syncthreads();
+    if (rank == 0) {
+        const int words = (int)(sizeof(EventHdr) / 4);
+        for (int i = tid; i < words; i += kSmallThreads)
+            reinterpret_cast<int32_t*>(hdr)[i] = reinterpret_cast<const int32_t*>(&sh)[i];
+        if (tid == 0) {
+            blk_start[0] = 0;
+            blk_start[1] = t1.nblk;
+            cell_off[0] = 0;
+            cell_off[1] = t1.cell_end;
+        }
+    }
+    // cell ids and ranks, kept in registers
+    int32_t key[kSmallPer], rnk[kSmallPer];
+#pragma unroll
+    for (int j = 0; j < kSmallPer; ++j) {
+        const int i = tid + j * kSmallThreads;
+        key[j] = 0;
+        rnk[j] = 0;
+        if (i < np) {
+            if (sh.valid) key[j] = point_cell(StagedRow{sm, i * D, pad}, sh);
+            rnk[j] = atomicAdd(counts + stored_cell(sh, key[j]), 1);
+        }
+    }
+    cluster.sync();
+    // exclusive scan of the used entries, the one past the last cell among
+    // them: warp g of the cluster takes the g-th segment of `seg` entries
+    const int used = sh.ncells + 1;
+    const int seg = ((used + ctas * kWarps - 1) / (ctas * kWarps) + 127) / 128 * 128;
+    const int s0 = (rank * kWarps + warp) * seg, s1 = min(s0 + seg, used);
+    // four entries from i on (zero past the segment's end)
+    auto quad = [&](int i) -> int4 {
+        if (i + 4 <= s1) return __ldcg(reinterpret_cast<const int4*>(counts + i));
+        int4 v = make_int4(0, 0, 0, 0);
+        if (i < s1) v.x = __ldcg(counts + i);
+        if (i + 1 < s1) v.y = __ldcg(counts + i + 1);
+        if (i + 2 < s1) v.z = __ldcg(counts + i + 2);
+        return v;
+    };
+    int4 held[kSmallQuads];   // the segment's first steps, for both passes
+    int sum = 0;
+#pragma unroll
+    for (int j = 0; j < kSmallQuads; ++j) {
+        const int o = s0 + 128 * j + 4 * lane;
+        held[j] = o < s1 ? quad(o) : make_int4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int j = 0; j < kSmallQuads; ++j) sum += held[j].x + held[j].y + held[j].z + held[j].w;
+#pragma unroll 4
+    for (int o = s0 + 128 * kSmallQuads + 4 * lane; o < s1; o += 128) {
+        const int4 v = quad(o);
+        sum += v.x + v.y + v.z + v.w;
+    }
+    sum = __reduce_add_sync(kAll, sum);
+    if (lane == 0) s_wt[warp] = sum;
+    __syncthreads();
+    if (warp == 0) {
+        const int v = s_wt[lane];
+        int incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(kAll, incl, o);
+            if (lane >= o) incl += y;
+        }
+        s_wt[lane] = incl - v;
+        const int total = __shfl_sync(kAll, incl, 31);
+        if (lane < ctas) *cluster.map_shared_rank(&s_tot[rank], lane) = total;
+    }
+    cluster.sync();
+    int carry = s_wt[warp];
+    for (int c = 0; c < rank; ++c) carry += s_tot[c];
+    auto scan_step = [&](int b, const int4 v) {
+        const int i = b + 4 * lane;
+        const int t = v.x + v.y + v.z + v.w;
+        int incl = t;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(kAll, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const int x = carry + incl - t;
+        const int4 w = make_int4(x, x + v.x, x + v.x + v.y, x + v.x + v.y + v.z);
+        if (i + 4 <= s1) {
+            *reinterpret_cast<int4*>(counts + i) = w;
+        } else {
+            if (i < s1) counts[i] = w.x;
+            if (i + 1 < s1) counts[i + 1] = w.y;
+            if (i + 2 < s1) counts[i + 2] = w.z;
+        }
+        carry += __shfl_sync(kAll, incl, 31);
+    };
+#pragma unroll
+    for (int j = 0; j < kSmallQuads; ++j)
+        if (s0 + 128 * j < s1) scan_step(s0 + 128 * j, held[j]);
+    if (s0 + 128 * kSmallQuads < s1) {
+        // (the next step's entries in flight)
+        int4 next = quad(s0 + 128 * kSmallQuads + 4 * lane);
+#pragma unroll 1
+        for (int b = s0 + 128 * kSmallQuads; b < s1; b += 128) {
+            const int4 v = next;
+            next = quad(b + 128 + 4 * lane);
+            scan_step(b, v);
+        }
+    }
+    cluster.sync();
+#pragma unroll
+    for (int j = 0; j < kSmallPer; ++j) {
+        const int i = tid + j * kSmallThreads;
+        if (i < np) {
+            const int slot = __ldcg(counts + stored_cell(sh, key[j])) + rnk[j];
+            perm[slot] = p0 + i;
+            cell[slot] = key[j];
+            write_row(pts + (int64_t)slot * DP, StagedRow{sm, i * D, pad}, D, DP);
+        }
+    }
+    if (rank == 0 && tid == 0 && (n & 1)) {   // an odd event's padding slot
+        perm[n] = -1;
+        cell[n] = 0;
+        const float nan = __int_as_float(0x7fc00000);
+        float4* dst = reinterpret_cast<float4*>(pts + (int64_t)n * DP);
+        for (int q = 0; q < DP / 4; ++q) dst[q] = make_float4(nan, nan, nan, nan);
+    }
+}
+
 // ------------------------------------------------------------------ host
 
 // The budget grows with n so that the cells stay near r on the sets the
@@ -1090,6 +1405,26 @@ frnn_status enqueue_build(GridBufs& g, const float* const* refs, const BuildOpts
     if (!capturing) cudaEventRecord(g.h_pinned_free, st);
     }
 
+    // (a cross-set query's cells are its reference grid's: not a small set's)
+    if (t1.set && t1.hdr.n > 0 && t1.hdr.n <= kSmallMax && g.L <= kSmallCells) {
+        const int per = (int)ceil_div(t1.hdr.n, kSmallCtas);   // at most kSmallPer * kSmallThreads
+        const size_t smem = sizeof(float) * small_stage_floats(per, D);
+        cudaError_t ce = cudaFuncSetAttribute(k_build_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (ce == cudaSuccess)
+            ce = cudaFuncSetAttribute(k_build_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (ce == cudaSuccess)
+            ce = launch_pdl_cluster(k_build_small, dim3(kSmallCtas), dim3(kSmallThreads), smem, st, kSmallCtas, t1,
+                                    params_from ? (const EventHdr*)params_from->hdr : nullptr, per, D, g.DP, o.r, o.m,
+                                    o.axes_mode, o.naxes, g.hdr, g.blk_start, g.cell_off, g.cstart, g.scalars, g.pts,
+                                    g.perm, g.cell, d_status);
+        g.tc_ready = false;
+        g.rows_ready = false;
+        if (ce != cudaSuccess) {
+            err = std::string("grid build launch failed: ") + cudaGetErrorString(ce);
+            return FRNN_ERR_CUDA;
+        }
+        return FRNN_OK;
+    }
     const int32_t bbmin = host_float_to_ordered(INFINITY);
     const int32_t bbmax = host_float_to_ordered(-INFINITY);
     const int64_t init_n = std::max<int64_t>(g.L, (int64_t)E * kBBoxCopies * kBBoxStride);
