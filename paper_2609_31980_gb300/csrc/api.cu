@@ -45,6 +45,8 @@ struct frnn_ctx {
     GridBufs qset;            // cross-set query binning
     GridBufs batch;           // batched multi-event grid
     int64_t batch_points = 0; // points of the batched call being served (0 outside of one)
+    uint64_t* scratch = nullptr;   // half-cell scan's long lists (half_scratch_keys)
+    bool scratch_tried = false;
     bool small_cells = false; // serving slot under a memory budget (see cell_kind)
     frnn_grid* host_grid = nullptr;   // grid of the host-buffer path
     void* hp_buf = nullptr;   // device buffers of the host-buffer path
@@ -88,6 +90,8 @@ struct frnn_ctx {
     int32_t* csr_idx = nullptr;     // [M * kCsrStageW] staged rows
     float* csr_d2 = nullptr;
     int64_t* csr_parts = nullptr;
+    unsigned long long* csr_pool_count = nullptr;   // entries taken of the long rows' pool
+    int64_t csr_pool0 = 0, csr_pool_cap = 0;        // its first entry and size
     bool csr_pending = false;
     QueryLaunch csr_q{};
     int64_t csr_M = 0, csr_E = 0;
@@ -187,6 +191,20 @@ static CellKind cell_kind(const frnn_ctx* ctx, int64_t N, int D) {
     const int naxes = build_naxes(ctx, N, D);
     if (half_cells(D, naxes, build_mult(ctx, N, D))) return CellKind::kHalf;
     return D <= 4 && naxes == 0 && ctx->budget == 0 && !ctx->small_cells ? CellKind::kLow : CellKind::kPlain;
+}
+
+// The half-cell scan's scratch array, made with the first call that keeps long
+// rows (about 52 MB; none under a memory budget, whose contexts send them to
+// the selection kernel, as when the allocation fails).
+static void ensure_scratch(frnn_ctx* c, int K) {
+    if (K <= kLongK || c->scratch_tried || c->budget != 0 || c->small_cells) return;
+    c->scratch_tried = true;
+    void* p = nullptr;
+    if (cudaMalloc(&p, half_scratch_keys(c->num_sms) * sizeof(uint64_t)) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    c->scratch = static_cast<uint64_t*>(p);
 }
 
 static frnn_status alloc_accounted(frnn_ctx* c, GridBufs& g, int E, const int64_t* n, int D,
@@ -471,6 +489,7 @@ frnn_status frnn_destroy(frnn_ctx* ctx) {
     if (ctx->hp_buf) cudaFree(ctx->hp_buf);
     if (ctx->hr_buf) cudaFree(ctx->hr_buf);
     if (ctx->csr_buf) cudaFree(ctx->csr_buf);
+    if (ctx->scratch) cudaFree(ctx->scratch);
     cudaFree(ctx->d_status);
     cudaFreeHost(ctx->h_status);
     delete ctx;
@@ -584,6 +603,9 @@ static frnn_status query_impl(frnn_ctx* ctx, const frnn_grid* grid, const float*
         q.csr = 1;
         q.ovf_mode = 1;
         q.degree = csr->degree;
+        q.pool0 = ctx->csr_pool0;
+        q.pool_cap = ctx->csr_pool_cap;
+        q.pool_count = ctx->csr_pool_count;
     }
     if (ctx->ktime && ctx->kev_used < kMaxTimedCalls) {
         const size_t need = 2 * (size_t)(ctx->kev_used + 1);
@@ -623,6 +645,10 @@ static frnn_status query_impl(frnn_ctx* ctx, const frnn_grid* grid, const float*
         s = enqueue_tc_query(q, ctx->stream, err);
     } else {
         q.kernel = grid->half ? 2 : grid_kernel(grid->naxes);
+        if (q.kernel == 2) {
+            ensure_scratch(ctx, K);
+            q.scratch = ctx->scratch;
+        }
         if (q.kernel == 1) {
             s = prepare_rows(ctx, rg, ctx->stream);
             if (s == FRNN_OK && !self) s = prepare_rows(ctx, ctx->qset, ctx->stream);
@@ -647,12 +673,34 @@ frnn_status frnn_query(frnn_ctx* ctx, const frnn_grid* grid, const float* querie
     return query_impl(ctx, grid, queries, M, r, K, flags, counts, idx, dist2, nullptr, nullptr);
 }
 
-static frnn_status csr_reserve(frnn_ctx* ctx, int64_t M) {
+static frnn_status csr_reserve(frnn_ctx* ctx, int64_t M, int K) {
     auto al = [](size_t x) { return (x + 255) / 256 * 256; };
     const size_t rows = (size_t)std::max<int64_t>(M, 1);
-    const size_t b_cnt = al(rows * 4), b_stage = al(rows * kCsrStageW * 4);
+    const size_t b_cnt = al(rows * 4);
     const size_t b_parts = al((size_t)csr_parts_needed(M) * 8);
-    const size_t need = b_cnt + 2 * b_stage + b_parts;
+    // behind the staging rows, without a memory budget: a pool of as many
+    // entries for rows longer than a staging row (none if it cannot be had)
+    const auto stage_bytes = [&](bool pool) { return al(rows * kCsrStageW * 4 * (pool ? 2 : 1)); };
+    const auto total = [&](bool pool) { return b_cnt + 2 * stage_bytes(pool) + b_parts + 256; };
+    ensure_scratch(ctx, K);
+    bool pool = K > kLongK && ctx->scratch != nullptr;
+    if (pool && total(true) > ctx->csr_bytes) {
+        cudaStreamSynchronize(ctx->stream);
+        void* p = nullptr;
+        if (ctx->csr_buf) cudaFree(ctx->csr_buf);
+        ctx->held -= ctx->csr_bytes;
+        ctx->csr_buf = nullptr;
+        ctx->csr_bytes = 0;
+        if (cudaMalloc(&p, total(true)) == cudaSuccess) {
+            ctx->csr_buf = p;
+            ctx->csr_bytes = total(true);
+            ctx->held += ctx->csr_bytes;
+        } else {
+            cudaGetLastError();
+            pool = false;
+        }
+    }
+    const size_t b_stage = stage_bytes(pool), need = total(pool);
     if (need > ctx->csr_bytes) {
         if (!budget_allows(ctx, ctx->csr_bytes, need))
             return fail(ctx, FRNN_ERR_BUDGET, "request exceeds the context's memory budget");
@@ -673,6 +721,10 @@ static frnn_status csr_reserve(frnn_ctx* ctx, int64_t M) {
     ctx->csr_idx = reinterpret_cast<int32_t*>(b + b_cnt);
     ctx->csr_d2 = reinterpret_cast<float*>(b + b_cnt + b_stage);
     ctx->csr_parts = reinterpret_cast<int64_t*>(b + b_cnt + 2 * b_stage);
+    ctx->csr_pool_count = reinterpret_cast<unsigned long long*>(b + b_cnt + 2 * b_stage + b_parts);
+    ctx->csr_pool0 = (int64_t)rows * kCsrStageW;
+    ctx->csr_pool_cap = pool ? ctx->csr_pool0 : 0;
+    cudaMemsetAsync(ctx->csr_pool_count, 0, sizeof(unsigned long long), ctx->stream);
     return FRNN_OK;
 }
 
@@ -686,7 +738,7 @@ static frnn_status csr_count_enqueue(frnn_ctx* ctx, const frnn_grid* grid, const
     int32_t dummy = 0;   // check_query_args wants row outputs: the staging is ours
     frnn_status s = check_query_args(ctx, M, r, K, flags, &dummy, &dummy, reinterpret_cast<float*>(&dummy));
     if (s != FRNN_OK) return s;
-    s = csr_reserve(ctx, M);
+    s = csr_reserve(ctx, M, K);
     if (s != FRNN_OK) return s;
     *q = QueryLaunch{};
     if (M > 0) {
@@ -830,6 +882,7 @@ static frnn_status enqueue_batched(frnn_ctx* ctx, const frnn_event* ev, int n_ev
     }
     if (any_half) {
         q.kernel = 2;
+        q.scratch = ctx->scratch;
         q.path_filter = mixed ? 3 : -1;
         q.chunk_end = mixed && first_rows < n_events ? gb.h_hdr[first_rows].qchunk0 : -1;
         s = enqueue_grid_query(q, st, err);
@@ -928,6 +981,7 @@ frnn_status frnn_query_batched(frnn_ctx* ctx, const frnn_event* ev, int n_events
     bool batch_tc = false, batch_rows = false;
     for (int e = 0; e < n_events; ++e) {
         if (ev[e].n <= 0) continue;
+        if (batch_path(ctx, ev[e].n, D, K, flags) == 3) ensure_scratch(ctx, K);   // outside any capture
         if (use_tc_path(ctx, D, flags, ev[e].n, K)) batch_tc = true;
         else if (grid_kernel(build_naxes(ctx, ev[e].n, D)) == 1) batch_rows = true;
     }

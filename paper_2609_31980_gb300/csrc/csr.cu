@@ -122,12 +122,12 @@ __global__ void __launch_bounds__(kCsrThreads) k_csr_down(const int32_t* cnt, in
         offsets[M] = tot + (parts ? parts[blockIdx.x] : 0);
 }
 
-// One warp per 32 consecutive rows.  Their entries are contiguous in the
-// output ([offsets[r0], offsets[r0 + 32]) minus the rows the selection
-// kernel writes), so the warp walks them as one flat range: entry t of the
-// range belongs to the row whose exclusive prefix (within the 32) is the last
-// one <= t (a binary search over the lanes' prefixes with shuffles); every
-// lane copies one entry per step and the stores of a step are contiguous.
+// One warp per 32 consecutive rows, one row a step, its entries on the lanes:
+// a row's entries lie side by side in the staging area (or the pool) and in
+// the output.  Steps are independent and four are in flight, which is what
+// bounds this kernel; finding each lane's row in the 32 rows' flat range of
+// entries first (a five-step search before every load) measured 33 us a
+// quarter of the 300k x 8 event's rows, this 8.
 __global__ void __launch_bounds__(256) k_csr_gather(const int32_t* cnt, const int64_t* offsets,
                                                     const int32_t* sidx, const float* sd2,
                                                     int64_t M, int32_t* idx, float* dist2,
@@ -139,36 +139,31 @@ __global__ void __launch_bounds__(256) k_csr_gather(const int32_t* cnt, const in
     // rows [row0, row1) (row0 a multiple of 32)
     for (int64_t w = (row0 >> 5) + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
          w * 32 < row1; w += nw) {
-        const int64_t r0 = w * 32;
-        const int64_t i = r0 + lane;
+        const int64_t i = w * 32 + lane;
         const int32_t c = i < row1 ? cnt[i] : 0;
-        const int own = (c & kCsrSpill) ? 0 : c;   // spilled rows: written by the selection kernel
-        int incl = own;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        const int excl = incl - own;
-        const int T = __shfl_sync(0xffffffffu, incl, 31);
-        const int64_t o_lane = i < row1 ? offsets[i] : 0;
-        for (int base = 0; base < T; base += 32) {
-            const int t = base + lane;
-            int R = 0;
-#pragma unroll
-            for (int st = 16; st > 0; st >>= 1) {
-                const int v = __shfl_sync(0xffffffffu, excl, R + st);
-                if (v <= t) R += st;
-            }
-            const int e = t - __shfl_sync(0xffffffffu, excl, R);
-            const int64_t dst = __shfl_sync(0xffffffffu, o_lane, R) + e;
+        // spilled rows: written by the selection kernel
+        const int own = (c & kCsrSpill) ? 0 : (c & kCsrCountMask);
+        const int64_t src = (c & kCsrPool) ? *reinterpret_cast<const int64_t*>(sidx + i * kCsrStageW)
+                                           : i * kCsrStageW;
+        const int64_t dst = i < row1 ? offsets[i] : 0;
+        const int rows = (int)min((int64_t)32, row1 - w * 32);
+#pragma unroll 4
+        for (int r = 0; r < rows; ++r) {
+            const int n = __shfl_sync(0xffffffffu, own, r);
+            const int64_t s = __shfl_sync(0xffffffffu, src, r);
+            const int64_t d = __shfl_sync(0xffffffffu, dst, r);
             // cap: entries the output holds (a caller that gathers before
             // it knows the edge count passes its capacity; the call then
             // fails when the count exceeds it, and nothing past it is written)
-            if (t < T && dst < cap) {
-                const int64_t src = (r0 + R) * kCsrStageW + e;
-                idx[dst] = sidx[src];
-                dist2[dst] = sd2[src];
+            if (lane < n && d + lane < cap) {
+                idx[d + lane] = __ldg(sidx + s + lane);
+                dist2[d + lane] = __ldg(sd2 + s + lane);
+            }
+            for (int e = 32 + lane; e < n; e += 32) {
+                if (d + e < cap) {
+                    idx[d + e] = __ldg(sidx + s + e);
+                    dist2[d + e] = __ldg(sd2 + s + e);
+                }
             }
         }
     }

@@ -174,7 +174,12 @@ struct QueryLaunch {
     int32_t* degree = nullptr;
     const int64_t* row_off = nullptr;
     int64_t row_cap = INT64_MAX;   // compact rows: entries the output holds
+    uint64_t* scratch = nullptr;   // half-cell scan: see QueryArgs
+    int64_t pool0 = 0, pool_cap = 0;
+    unsigned long long* pool_count = nullptr;
 };
+// Keys of the scratch array of a device with num_sms SMs.
+inline size_t half_scratch_keys(int num_sms) { return (size_t)num_sms * 28 * kScratchKeys; }
 frnn_status enqueue_grid_query(const QueryLaunch& q, cudaStream_t st, std::string& err);
 // Row-task kernel: allocate (outside any capture) and build (enqueued) the
 // pair-interleaved copy and 16-query tasks of a point set; the launch itself

@@ -32,7 +32,16 @@ constexpr int kStatusCapacity = 4;
 // with kCsrSpill set belongs to a row the selection kernel writes itself
 constexpr int kCsrStageW = 32;
 constexpr int32_t kCsrSpill = 0x40000000;
-constexpr int32_t kCsrCountMask = 0x3fffffff;
+// or with kCsrPool set: to a row longer than that in the pool behind the staging
+// rows, its first pool entry in the row's first two staged indices
+constexpr int32_t kCsrPool = 0x20000000;
+constexpr int32_t kCsrCountMask = 0x1fffffff;
+
+// The half-cell scan keeps up to kMoreCap entries of each query beyond the
+// shared-memory lists in its warp's part of a context-owned scratch array.
+constexpr int kMoreCap = 96;
+constexpr int kLongK = 128;   // in calls that keep more than this many neighbours (query_half.cu says why)
+constexpr int kScratchKeys = kChunkQ * kMoreCap;   // 8-byte keys per resident warp
 
 // Bounded waits: an mbarrier wait gives up after about two seconds of wall
 // time (%globaltimer), far above any legitimate wait, with an iteration cap as
@@ -204,6 +213,13 @@ struct QueryArgs {
     int32_t* degree;             // optional full degree per query (csr)
     const int64_t* row_off;      // CSR row offsets (ovf_mode 2)
     int64_t row_cap;             // entries idx / dist2 hold (ovf_mode 2): rows past it are skipped
+    uint64_t* scratch;           // half-cell scan: kScratchKeys keys per warp (NULL: none)
+    uint64_t f2_one, f2_neg_one, f2_neg_zero;   // 1, -1 and -0 twice (query_half.cu, fma2)
+    int32_t list_cap;            // entries it keeps per query: the list's, and kMoreCap with the scratch
+    // compact output of the half-cell scan: pool entries behind the staging
+    // rows (idx / dist2 from entry pool0 on), and the counter of those taken
+    int64_t pool0, pool_cap;
+    unsigned long long* pool_count;
 };
 
 // ---------------------------------------------------------------- PTX helpers

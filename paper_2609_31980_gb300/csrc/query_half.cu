@@ -31,7 +31,13 @@
 //     stream position lies in follows from one load of the next range starts
 //     and one warp-wide OR of the positions where ranges start;
 //   * accepted (d2, original index) pairs are appended to the query's list in
-//     shared memory (at most kListCap; longer lists go to select.cu);
+//     shared memory (kListCap entries), with K > kLongK then to the warp's part
+//     of a scratch array in global memory (kMoreCap more); longer lists go to
+//     select.cu, which searches again;
+//   * rows past the shared-memory list: one at a time by a network across the
+//     lanes, two or four keys a lane; compact rows among them go to a pool
+//     behind the 32-wide staging rows, so no row is searched twice (calls with
+//     K > kLongK);
 //   * row sort: lanes q and q + 16 hold half of query q's list each, as 32-bit
 //     keys (the distance's bits with the low five cleared, then the entry's
 //     place in the list), sort them in registers (an odd-even merge network,
@@ -56,18 +62,19 @@
 #include <climits>
 
 #include "frnn_host.h"
+#include "warp_sort.cuh"
 
 namespace frnn {
 namespace half {
 
 constexpr int kWarps = 4;
-constexpr uint32_t kFull = 0xffffffffu;
 constexpr int kListCap = 32;     // accepted entries a query keeps in the kernel
 constexpr int kListStr = 36;     // list row stride: 16-byte aligned rows
 constexpr int kRangeCap = 128;   // candidate ranges of one batch of groups
 constexpr int kQ = kChunkQ;      // queries a warp serves at once, at most
 static_assert(kQ == 16, "lanes q and q + 16 share query q's row");
 static_assert(kListCap <= kCsrStageW, "a staged compact row holds a whole kernel row");
+static_assert(kListCap + kMoreCap <= 128, "four keys a lane sort a long row");
 
 template <int D>
 struct Cfg {
@@ -257,7 +264,58 @@ __device__ __forceinline__ void sort_rows(const WarpSmem& w, int n) {
     __syncwarp();
 }
 
-template <int D>
+// Sort and write one row of more than kListCap entries (n of them: the list,
+// then the query's part of the scratch) with the whole warp, 32 P >= n keys.
+// width: entries written, those from n on padding.  Not inlined: the scan's
+// registers and instruction cache are for the rows that fit the lists.
+template <int P>
+__device__ __noinline__ void write_long_row(const float* ld, const int32_t* li, const uint64_t* scr, int n,
+                                            int width, int32_t* irow, float* drow) {
+    const int lane = threadIdx.x & 31;
+    uint64_t k[P];
+    k[0] = make_key(ld[lane], li[lane]);
+#pragma unroll
+    for (int p = 1; p < P; ++p)
+        k[p] = 32 * p + lane < n ? __ldcg(scr + 32 * (p - 1) + lane) : ~0ull;
+    warp_sort<P>(k);
+    const bool vec = (width & 3) == 0 &&
+                     ((reinterpret_cast<uintptr_t>(irow) | reinterpret_cast<uintptr_t>(drow)) & 15) == 0;
+    const int e0 = lane * P;
+    int32_t vi[P];
+    float vd[P];
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        vi[p] = e0 + p < n ? (int32_t)(uint32_t)k[p] : -1;
+        vd[p] = e0 + p < n ? __uint_as_float((uint32_t)(k[p] >> 32)) : INFINITY;
+    }
+    if (vec && P == 4) {
+        if (e0 < width) {
+            *reinterpret_cast<int4*>(irow + e0) = make_int4(vi[0], vi[1], vi[P - 2], vi[P - 1]);
+            *reinterpret_cast<float4*>(drow + e0) = make_float4(vd[0], vd[1], vd[P - 2], vd[P - 1]);
+        }
+    } else if (vec) {
+        if (e0 < width) {
+            *reinterpret_cast<int2*>(irow + e0) = make_int2(vi[0], vi[1]);
+            *reinterpret_cast<float2*>(drow + e0) = make_float2(vd[0], vd[1]);
+        }
+    } else {
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            if (e0 + p < width) {
+                irow[e0 + p] = vi[p];
+                drow[e0 + p] = vd[p];
+            }
+        }
+    }
+    for (int e = 32 * P + lane; e < width; e += 32) {
+        irow[e] = -1;
+        drow[e] = INFINITY;
+    }
+}
+
+// LONG: rows past the shared-memory lists are kept (scratch, pool) and written
+// here; else they go to select.cu.
+template <int D, bool LONG>
 __global__ void __launch_bounds__(kWarps * 32, Cfg<D>::MINB) k_half_query(QueryArgs a, int sub_shift) {
     pdl_trigger();
     pdl_wait();
@@ -275,6 +333,10 @@ __global__ void __launch_bounds__(kWarps * 32, Cfg<D>::MINB) k_half_query(QueryA
     // the 16-byte stores, its quarter
     const int width = a.csr ? kCsrStageW : K;
     const int w4 = width >> 2;
+    // this warp's part of the scratch (formed where it is used: long rows only)
+    auto scratch = [&](int q) {
+        return a.scratch + (size_t)(blockIdx.x * kWarps + (threadIdx.x >> 5)) * kScratchKeys + q * kMoreCap;
+    };
 
     for (;;) {
         int t = 0;
@@ -505,13 +567,17 @@ __global__ void __launch_bounds__(kWarps * 32, Cfg<D>::MINB) k_half_query(QueryA
                     // lanes; the last of them writes the new count (a query
                     // belongs to one group, so no other lane does)
                     const unsigned am = __ballot_sync(kFull, acc);
-                    if (acc) {
-                        const int p = held + __popc(am & g_lo);
-                        if (p < kListCap) {
-                            w.Ld[q * kListStr + p] = s;
-                            w.Li[q * kListStr + p] = orig;
+                    const int p = held + __popc(am & g_lo);
+                    if (acc && p < kListCap) {
+                        w.Ld[q * kListStr + p] = s;
+                        w.Li[q * kListStr + p] = orig;
+                    }
+                    if (acc && (am & g_hi) == 0) w.cnt[q] = p + 1;
+                    if constexpr (LONG) {
+                        const bool over = acc && p >= kListCap;
+                        if (__any_sync(kFull, over)) {
+                            if (over && p < a.list_cap) scratch(q)[p - kListCap] = make_key(s, orig);
                         }
-                        if ((am & g_hi) == 0) w.cnt[q] = p + 1;
                     }
                     __syncwarp();
                 }
@@ -525,8 +591,15 @@ __global__ void __launch_bounds__(kWarps * 32, Cfg<D>::MINB) k_half_query(QueryA
 
         // per query: counts, degree, rows for the selection kernel
         const int kept = act ? w.cnt[lane] : 0;
-        const bool spill = kept > kListCap;
-        if (act && !spill) counts[qorig] = min(kept, K);
+        bool spill = kept > (LONG ? a.list_cap : kListCap);
+        const bool is_long = LONG && kept > kListCap && !spill;
+        int64_t pool_at = 0;   // compact output: a long row's place in the pool
+        if (LONG && is_long && a.csr) {
+            const int need = (min(kept, K) + 3) & ~3;
+            pool_at = (int64_t)atomicAdd(a.pool_count, (unsigned long long)need);
+            spill = pool_at + need > a.pool_cap;
+        }
+        if (act && !spill) counts[qorig] = min(kept, K) | (is_long && a.csr ? kCsrPool : 0);
         if (spill && a.csr) counts[qorig] = kCsrSpill;   // counted by the selection kernel
         if (act && !spill && a.degree) a.degree[qorig] = kept;
         if (spill) {
@@ -538,8 +611,24 @@ __global__ void __launch_bounds__(kWarps * 32, Cfg<D>::MINB) k_half_query(QueryA
                 atomicOr(a.status, kStatusCapacity);
             }
         }
-        const unsigned rows = __ballot_sync(kFull, act && !spill);   // rows written here
-        const int n = __shfl_sync(kFull, spill ? 0 : kept, lane & 15);
+        // rows longer than the lists, one by one (before the lists are sorted)
+        unsigned long_rows = LONG ? __ballot_sync(kFull, is_long && !spill) : 0u;
+        while (long_rows) {
+            const int q = __ffs(long_rows) - 1;
+            long_rows &= long_rows - 1u;
+            const int nl = __shfl_sync(kFull, kept, q);
+            const int64_t row = __shfl_sync(kFull, qorig, q);
+            const int64_t pool = a.pool0 + __shfl_sync(kFull, pool_at, q);
+            const int64_t at = a.csr ? pool : row * K;
+            const int wide = a.csr ? (min(nl, K) + 3) & ~3 : K;
+            const float* ld = w.Ld + q * kListStr;
+            const int32_t* li = w.Li + q * kListStr;
+            if (nl <= 64) write_long_row<2>(ld, li, scratch(q), nl, wide, oidx + at, od2 + at);
+            else write_long_row<4>(ld, li, scratch(q), nl, wide, oidx + at, od2 + at);
+            if (a.csr && lane == 0) *reinterpret_cast<int64_t*>(oidx + row * kCsrStageW) = pool;
+        }
+        const unsigned rows = __ballot_sync(kFull, act && kept <= kListCap);   // the other rows written here
+        const int n = __shfl_sync(kFull, kept > kListCap ? 0 : kept, lane & 15);
         const int most = __reduce_max_sync(kFull, (unsigned)n);
         int sorted = 32;   // places of the lists that hold the row or its padding
         if (most <= 8) {
@@ -591,16 +680,16 @@ __global__ void __launch_bounds__(kWarps * 32, Cfg<D>::MINB) k_half_query(QueryA
     }
 }
 
-template <int D>
-cudaError_t launch(const QueryArgs& a, int num_sms, cudaStream_t st) {
-    auto kern = &k_half_query<D>;
+template <int D, bool LONG>
+cudaError_t launch_l(const QueryArgs& a, int num_sms, cudaStream_t st) {
+    auto kern = &k_half_query<D, LONG>;
     const size_t smem = (size_t)kWarps * warp_bytes<D>();
     cudaError_t ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (ce != cudaSuccess) return ce;
     int per_sm = 0;
     ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarps * 32, smem);
     if (ce != cudaSuccess) return ce;
-    const int64_t blocks = (int64_t)num_sms * std::max(per_sm, 1);
+    const int64_t blocks = (int64_t)num_sms * std::min(std::max(per_sm, 1), 28 / kWarps);   // the scratch's warps
     // sets too small to give every resident warp a chunk of 16 queries are cut
     // into chunks of 8 or 4 (a warp's chunk is a serial chain)
     int sub = 0;
@@ -609,6 +698,17 @@ cudaError_t launch(const QueryArgs& a, int num_sms, cudaStream_t st) {
     launch_pdl(kern, dim3((unsigned)std::min(blocks, std::max<int64_t>(need, 1))), dim3(kWarps * 32), smem, st,
                a, sub);
     return cudaGetLastError();
+}
+
+// Keeping long rows costs the scan's inner loop a vote per step (300k x 8 147
+// -> 151 us, 500k x 12 346 -> 361, build + query, none of whose rows are long)
+// and saves searching them again (271,663 x 12, compact, K = 1000, two rows in
+// three long: 758 -> 430).  Calls that keep more than 128 neighbours expect
+// such rows; the others leave the few they meet to the selection kernel.
+template <int D>
+cudaError_t launch(const QueryArgs& a, int num_sms, cudaStream_t st) {
+    return a.K > kLongK && a.list_cap > kListCap ? launch_l<D, true>(a, num_sms, st)
+                                                 : launch_l<D, false>(a, num_sms, st);
 }
 
 }  // namespace half

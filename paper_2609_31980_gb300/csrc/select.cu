@@ -20,60 +20,22 @@
 // list with 2K keys a warp in shared memory.  A launch with an empty list ends
 // at once.  The kernel this replaces walked the neighbour rows one after
 // another (27 to 81 dependent look-ups a row) and always sorted 2K keys in
-// shared memory at 12 warps an SM.  Measured (build + compact query, 271,663 x
-// 12 clustered points, r = 0.12, K = 1000, mean degree 34, two rows in three
-// selected): 56.1 -> 1.24 ms; with no row to select, 4096 x 3, K = 32: 41.9 ->
-// 38.7 us.
+// shared memory at 12 warps an SM.  Measured (build + query, 271,663 x 12
+// clustered points, r = 0.12, mean degree 34, two rows in three selected): compact,
+// K = 1000, 56.1 -> 1.24 ms (0.43 since the half-cell scan keeps these rows
+// itself at K > 128); dense, K = 100, 0.51 ms; with no row to select, 4096 x 3:
+// 41.9 -> 38.7 us.
 #include <algorithm>
 
 #include "frnn_host.h"
+#include "warp_sort.cuh"
 
 namespace frnn {
 namespace sel {
 
-constexpr uint32_t kFull = 0xffffffffu;
 constexpr int kWarps = 4;
 constexpr int kSelKeys = 256;                 // buffer of the first pass (keys a warp)
 constexpr int kSelMaxCut = kSelKeys - 64;     // largest K whose cut leaves two rounds of room
-
-__device__ __forceinline__ uint64_t make_key(float d2, int32_t j) {
-    return ((uint64_t)__float_as_uint(d2) << 32) | (uint32_t)j;
-}
-
-// Ascending sort of 32 P keys held P a lane (key i = lane * P + p): a bitonic
-// network, steps within a lane on registers, across lanes by shuffles.
-template <int P>
-__device__ __forceinline__ void warp_sort(uint64_t (&k)[P]) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int len = 2; len <= 32 * P; len <<= 1) {
-#pragma unroll
-        for (int j = len >> 1; j > 0; j >>= 1) {
-            if (j >= P) {
-                const int jl = j / P;   // lanes apart
-                // direction from the key's index: the bits at and above P are the lane's
-                const bool up = len >= 32 * P || ((lane * P) & len) == 0;
-                const bool take_min = ((lane & jl) == 0) == up;
-#pragma unroll
-                for (int p = 0; p < P; ++p) {
-                    const uint64_t o = __shfl_xor_sync(kFull, k[p], jl);
-                    k[p] = (take_min == (o < k[p])) ? o : k[p];
-                }
-            } else {
-#pragma unroll
-                for (int p = 0; p < P; ++p) {
-                    if ((p & j) == 0) {
-                        const bool up = len >= P ? ((lane * P) & len) == 0 || len >= 32 * P : (p & len) == 0;
-                        const uint64_t x = k[p], y = k[p | j];
-                        const bool sw = (x > y) == up;
-                        k[p] = sw ? y : x;
-                        k[p | j] = sw ? x : y;
-                    }
-                }
-            }
-        }
-    }
-}
 
 // Sort the first 32 P keys of buf (entries past n hold any value).
 template <int P>
@@ -151,9 +113,30 @@ __global__ void __launch_bounds__(kWarps * 32, BIG ? 1 : (D <= 8 ? 8 : (D <= 12 
     const bool csr_rows = a.ovf_mode == 2;
     const unsigned lt_mask = (1u << lane) - 1u;
     const int stride = gridDim.x * kWarps;
-    for (int w = blockIdx.x * kWarps + warp; w < nov; w += stride) {
-        const Overflow o = a.ovf[w];
-        if (BIG && o.ev >= 0) continue;   // finished by the first pass
+    // the first pass takes the list's rows one by one; the second looks for the
+    // marked ones 32 entries at a time
+    int w = (blockIdx.x * kWarps + warp) * (BIG ? 32 : 1) - (BIG ? 0 : stride);
+    unsigned marked = 0;
+    int w_base = 0;
+    for (;;) {
+        if constexpr (BIG) {
+            while (!marked && w < nov) {
+                const int i = w + lane;
+                marked = __ballot_sync(kFull, i < nov && a.ovf[i].ev < 0);
+                w_base = w;
+                w += stride * 32;
+            }
+            if (!marked) break;
+        } else {
+            w += stride;
+            if (w >= nov) break;
+        }
+        int at_entry = w;
+        if constexpr (BIG) {
+            at_entry = w_base + __ffs(marked) - 1;
+            marked &= marked - 1u;
+        }
+        const Overflow o = a.ovf[at_entry];
         const int ev = BIG ? ~o.ev : o.ev;
         const EventHdr& h = a.ev[ev];
         const int qs = o.qslot;
@@ -288,7 +271,7 @@ __global__ void __launch_bounds__(kWarps * 32, BIG ? 1 : (D <= 8 ? 8 : (D <= 12 
             for (int k = 0; k < DP; ++k) cv[k] = cvn[k];
         }
         if (left) {   // mark the entry for the second pass
-            if (lane == 0) a.ovf[w].ev = ~ev;
+            if (lane == 0) a.ovf[at_entry].ev = ~ev;
             __syncwarp();
             continue;
         }

@@ -107,3 +107,28 @@ def test_batches_mix_half_cells_and_row_tasks(ctx):
         rows = np.arange(0, len(p), max(1, len(p) // 1500))
         if len(p):
             _same(tuple(x[torch.from_numpy(rows).cuda()] for x in o), oracle.self_query(p, 0.1, 24, rows=rows))
+
+
+@pytest.mark.parametrize("size", [40, 100, 129, 140])
+@pytest.mark.parametrize("budget", [0, 1 << 28])
+def test_long_rows_beyond_the_pool(size, budget):
+    # every row is longer than the lists; from 100 points a cluster on the
+    # compact rows' pool (32 entries a query) runs out, from 130 the scratch
+    import torch
+    from paper_2609_31980_gb300 import frnn
+    p = synth.clustered(30, size, 40, 8, 0.01, seed=850 + size)
+    t = torch.from_numpy(p).cuda()
+    for K in (129, 400):
+        want = oracle.self_query(p, 0.1, K)
+        with frnn.Context(budget_bytes=budget) as ctx:
+            g = ctx.build_grid(t, 0.1)
+            got = ctx.query(g, t, 0.1, K, path="grid")
+            ctx.sync()
+            _same(got, want)
+            off, ci, cd, deg = ctx.query_csr(g, t, 0.1, K, degree=True)
+            ctx.sync()
+        keep = np.arange(K)[None, :] < want[0][:, None]
+        np.testing.assert_array_equal(np.diff(off.cpu().numpy()), want[0])
+        np.testing.assert_array_equal(ci.cpu().numpy(), want[1][keep])
+        np.testing.assert_array_equal(cd.cpu().numpy().view(np.uint32), want[2][keep].view(np.uint32))
+        np.testing.assert_array_equal(deg.cpu().numpy(), want[3])
