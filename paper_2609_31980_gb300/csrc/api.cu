@@ -166,7 +166,7 @@ static size_t predict_grid_bytes(int E, const int64_t* n, int D, const int64_t* 
     int64_t nt = 0, L = 0;
     for (int e = 0; e < E; ++e) {
         nt += n[e] + 1;
-        L += caps[e] + 1;
+        L += cell_entries(caps[e]);
     }
     nt = std::max<int64_t>(nt, 1);
     size_t b = 0;
@@ -631,6 +631,9 @@ static frnn_status query_impl(frnn_ctx* ctx, const frnn_grid* grid, const float*
         const int64_t cap = grid->g.h_hdr[0].cell_cap;
         s = alloc_accounted(ctx, ctx->qset, 1, &M, grid->D, &cap);
         if (s != FRNN_OK) return s;
+        // the half-cell scan needs its queries by rows of cells only
+        ctx->qset.h_hdr[0].rowsort =
+            grid->half && !use_tc_path(ctx, grid->D, flags, grid->N, K, grid->naxes) ? 1 : 0;
         BuildOpts o;
         const float* ev_q[1] = {queries};
         s = enqueue_build(ctx->qset, ev_q, o, &grid->g, ctx->d_status, ctx->stream, false, err);
@@ -1010,6 +1013,7 @@ frnn_status frnn_query_batched(frnn_ctx* ctx, const frnn_event* ev, int n_events
     // the pinned table mirror must be free before its upload is captured, and
     // the previous replay must be done before the tables change
     cudaStreamSynchronize(ctx->gstream);
+    grid_clean(ctx->batch, ctx->gstream);
     if (ctx->batch.h_pinned_free) cudaEventSynchronize(ctx->batch.h_pinned_free);
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamBeginCapture(ctx->gstream, cudaStreamCaptureModeThreadLocal);

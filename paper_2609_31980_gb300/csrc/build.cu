@@ -9,16 +9,18 @@
 // event_params below).
 //
 // Steps, all on the device, no host synchronisation:
-//   k_init      zero the cell counts, reset bounding boxes (and, for one event,
-//               write the per-event tables passed by value)
-//   k_bbox      per-event per-axis min / max (+ non-finite flag), float4 staged;
-//               the event's last block to finish derives the grid parameters:
-//               gridded axes, cell edge, cells per axis
+//   k_bbox      zero the cell counts; per-event per-axis min / max (+ non-finite
+//               flag), float4 staged; the event's last block to finish writes the
+//               tables of a one-event build (passed by value) and derives the
+//               grid parameters: gridded axes, cell edge, cells per axis
+//               (k_begin_foreign instead when the parameters are another grid's)
 //   k_cellid    cell id of every point and its rank inside the cell (atomics)
-//   scan        exclusive warp-shuffle prefix scan of the counts -> cell starts
+//   k_cells_*   exclusive prefix scan of the used counts -> cell starts
 //   k_scatter   slot -> original index, slot -> cell, and the point's row of
 //               DP floats at its slot (cell-sorted coordinates)
-// (the tensor-core path adds its 128-query tiles: k_rowtasks, a scan, k_emit)
+// Sets of up to 32,768 points are built by one launch instead (k_build_small).
+// (row tasks and tensor-core tiles are listed at query time: k_rowtasks, a
+// scan, k_emit)
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -31,12 +33,39 @@ namespace frnn {
 
 // ------------------------------------------------------------------ helpers
 
+// An entry of a box copy before any point.
+__device__ __forceinline__ int32_t empty_box_entry(int k) {
+    return k < 16 ? INT_MAX : (k < 32 ? INT_MIN : 0);   // minima, maxima; flag, block counter
+}
+
+// The grid parameters of src, by a whole block (or more than kMaxD threads).
+__device__ __forceinline__ void copy_params(EventHdr& dst, const EventHdr& src) {
+    const int t = threadIdx.x;
+    if (t == 0) {
+        dst.naxes = src.naxes;
+        dst.m = src.m;
+        dst.valid = src.valid;
+        dst.inv_h = src.inv_h;
+        dst.ncells = src.ncells;
+        dst.half = src.half;
+    }
+    if (t < kHdrAxes) {
+        dst.axes[t] = src.axes[t];
+        dst.dims[t] = src.dims[t];
+        dst.fdims[t] = src.fdims[t];
+        dst.mag[t] = src.mag[t];
+        dst.lo[t] = src.lo[t];
+        dst.hi[t] = src.hi[t];
+    }
+    if (t < kMaxD) dst.ctr[t] = src.ctr[t];
+}
+
 // Entry of each event's box copy 0 that counts its finished k_bbox blocks.
 constexpr int kBBoxDone = 33;
 static_assert(kBBoxDone >= 33 && kBBoxDone < kBBoxStride, "after the minima, maxima and flag");
 
 // The tables of a one-event build (header, block starts, cell offsets), passed
-// to k_init by value instead of being copied from the host.
+// to the first kernel by value instead of being copied from the host.
 struct OneEventTables {
     EventHdr hdr;
     int64_t cell_end;   // cell_off[1]
@@ -47,7 +76,7 @@ struct OneEventTables {
 // A one-event build's input, passed by value to the kernels that stage it:
 // they stage their block's points before waiting for the previous kernel of
 // the chain (no kernel of the chain writes the caller's points, and the
-// header that would locate them is written by k_init in this case).
+// header that would locate them is written by k_bbox in this case).
 struct EarlyPts {
     const float* refs;
     int64_t n;
@@ -183,121 +212,185 @@ __device__ __forceinline__ int point_cell(const Row& p, const EventHdr& h) {
 
 // ------------------------------------------------------------------ kernels
 
-__global__ void k_init(int32_t* counts, int64_t L, int32_t* bbox, int E, int32_t* scalars,
-                       int32_t bb_min_init, int32_t bb_max_init, OneEventTables t1,
-                       EventHdr* hdr, int32_t* blk_start, int64_t* cell_off) {
-    pdl_trigger();
-    pdl_wait();   // the previous work on the stream may still read the tables
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t1.set && i == 0) {
-        hdr[0] = t1.hdr;
-        blk_start[0] = 0;
-        blk_start[1] = t1.nblk;
-        cell_off[0] = 0;
-        cell_off[1] = t1.cell_end;
-    }
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // counts: 16-byte stores (the array starts 256-byte aligned)
+// Zero the counters and this block's share of the cell array (n4 quads).
+__device__ __forceinline__ void zero_share(int32_t* counts, int64_t n4, int32_t* scalars) {
     int4* c4 = reinterpret_cast<int4*>(counts);
-    const int64_t L4 = L / 4;
-    for (int64_t j = i; j < L4; j += stride) c4[j] = make_int4(0, 0, 0, 0);
-    for (int64_t j = 4 * L4 + i; j < L; j += stride) counts[j] = 0;
-    for (int64_t j = i; j < (int64_t)E * kBBoxCopies * kBBoxStride; j += stride) {
-        int k = (int)(j % kBBoxStride);
-        bbox[j] = k < 16 ? bb_min_init : (k < 32 ? bb_max_init : 0);   // flag, block counter: 0
-    }
-    if (i < kScalars) scalars[i] = 0;
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n4; j += (int64_t)gridDim.x * blockDim.x)
+        c4[j] = make_int4(0, 0, 0, 0);
+    if (blockIdx.x == 0 && threadIdx.x < kScalars) scalars[threadIdx.x] = 0;
 }
 
-__device__ void event_params(EventHdr* hdr, int e, int D, const int32_t* bbox, float r, int m,
-                             int axes_mode, int naxes_req, int32_t* counts);
+// One header by a whole block, word by word.
+__device__ __forceinline__ void copy_header(EventHdr* dst, const EventHdr& src) {
+    for (int i = threadIdx.x; i < (int)(sizeof(EventHdr) / 4); i += blockDim.x)
+        reinterpret_cast<int32_t*>(dst)[i] = reinterpret_cast<const int32_t*>(&src)[i];
+}
 
-// Per-event bounding boxes.  One CTA per build block (256 points staged
-// through shared memory with 16-byte loads) reduces its points and merges the
-// result into one of kBBoxCopies copies of the event's box (copy = block mod
-// kBBoxCopies), so that no address takes more than a few dozen atomics.  The
-// event's last block to finish (a counter beside copy 0, taken after a memory
-// fence) combines the copies and derives the grid parameters.
-// (at most 40 registers, as without the parameter step: six CTAs per SM; the
-// one-thread parameter code may spill)
-__global__ void __launch_bounds__(kBuildPtsPerBlock, 6) k_bbox(EventHdr* hdr,
-                                                            const int32_t* blk_start, int E,
-                                                            int D, int32_t* bbox,
-                                                            int32_t* status, float r, int m,
-                                                            int axes_mode, int naxes_req,
-                                                            int32_t* counts, EarlyPts ep) {
+// The boxes of E events before any point (new buffers; afterwards the
+// parameter step leaves them like this).
+__global__ void k_box_reset(int32_t* bbox, int E) {
+    pdl_trigger();
+    pdl_wait();
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < E * kBBoxCopies * kBBoxStride) bbox[j] = empty_box_entry(j % kBBoxStride);
+}
+
+__device__ void event_params(EventHdr* hdr, int e, int D, int32_t* bbox, float r, int m,
+                             int axes_mode, int naxes_req);
+
+// Per-event bounding boxes, and the zeroing of the cell counts.  One CTA takes
+// `sub` build blocks (256 points each, staged through shared memory with
+// 16-byte loads), keeps its points' extremes in registers and merges them once
+// per event into one of kBBoxCopies copies of the event's box (copy = block mod
+// kBBoxCopies), so that no address takes more than a few atomics.  The event's
+// last block to finish (a counter beside copy 0, taken after a memory fence)
+// combines the copies and derives the grid parameters; the zeroing of the other
+// blocks runs beside that chain.  `sub` build blocks a CTA: as many as make one
+// wave of kBoxWave CTAs, at most eight (each costs a round trip: 300k x 8 build
+// + query with 2, 4 and 8: 141, 148, 155 us; 1 M x 3 216, 214, 213).  One build
+// block a CTA, reduced by shuffles, and the zeroing in a launch of its own
+// measured 14 + 5 us at 300k x 8.
+constexpr int kBoxWave = 608;
+constexpr int kBoxMost = 8;
+__global__ void __launch_bounds__(kBuildPtsPerBlock, 4) k_bbox(EventHdr* hdr, int32_t* blk_start, int64_t* cell_off,
+                                                            int E, int nblk, int sub, int D, int32_t* bbox,
+                                                            int32_t* status, float r, int m, int axes_mode, int naxes_req,
+                                                            int32_t* counts, int64_t L, int32_t* scalars,
+                                                            OneEventTables t1) {
     pdl_trigger();
     extern __shared__ float sm[];
+    __shared__ int32_t red_mn[kMaxD][kBuildPtsPerBlock / 32];
+    __shared__ int32_t red_mx[kMaxD][kBuildPtsPerBlock / 32];
+    __shared__ int red_bad, s_last;
     const bool pad = (D & 3) == 0;
-    const bool staged = stage_early(sm, ep, D, pad);
-    pdl_wait();
-    __shared__ float red_mn[kMaxD][kBuildPtsPerBlock / 32];
-    __shared__ float red_mx[kMaxD][kBuildPtsPerBlock / 32];
-    __shared__ int red_bad;
-    const int e = find_event(blk_start, E, blockIdx.x);
-    const EventHdr& h = hdr[e];
-    const int64_t p0 = (int64_t)(blockIdx.x - blk_start[e]) * kBuildPtsPerBlock;
-    const int np = (int)min((int64_t)kBuildPtsPerBlock, h.n - p0);
-    if (threadIdx.x == 0) red_bad = 0;
-    if (!staged && np > 0) stage_floats(sm, h.refs + p0 * D, np * D, pad);
-    __syncthreads();
-    float mn[kMaxD], mx[kMaxD];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // a one-event build reads its input (which no kernel of the chain writes)
+    // before it waits for the previous work; else the tables come first
+    if (!t1.set) pdl_wait();
+    int32_t mn[kMaxD], mx[kMaxD];   // ordered ints
     bool bad = false;
+    auto clear = [&]() {
 #pragma unroll
-    for (int k = 0; k < kMaxD; ++k) { mn[k] = INFINITY; mx[k] = -INFINITY; }
-    if ((int)threadIdx.x < np) {
-        const StagedRow p{sm, (int)threadIdx.x * D, pad};
+        for (int k = 0; k < kMaxD; ++k) {
+            mn[k] = INT_MAX;
+            mx[k] = INT_MIN;
+        }
+        bad = false;
+    };
+    // merge what the registers hold of event e (nb of its build blocks)
+    auto flush = [&](int e, int nb) {
+        if (threadIdx.x == 0) red_bad = 0;
+        __syncthreads();
 #pragma unroll
         for (int k = 0; k < kMaxD; ++k) {
             if (k < D) {
-                float v = p[k];
-                bad |= !isfinite(v);
-                mn[k] = fminf(mn[k], v);
-                mx[k] = fmaxf(mx[k], v);
+                const int32_t a = __reduce_min_sync(0xffffffffu, mn[k]);
+                const int32_t b = __reduce_max_sync(0xffffffffu, mx[k]);
+                if (lane == 0) {
+                    red_mn[k][warp] = a;
+                    red_mx[k][warp] = b;
+                }
             }
         }
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&red_bad, 1);
+        __syncthreads();
+        int32_t* bb = bbox + ((int64_t)e * kBBoxCopies + (blockIdx.x % kBBoxCopies)) * kBBoxStride;
+        if (threadIdx.x < (unsigned)D) {
+            const int k = threadIdx.x;
+            int32_t a = INT_MAX, b = INT_MIN;
+            for (int w = 0; w < kBuildPtsPerBlock / 32; ++w) {
+                a = min(a, red_mn[k][w]);
+                b = max(b, red_mx[k][w]);
+            }
+            atomicMin(bb + k, a);
+            atomicMax(bb + 16 + k, b);
+        }
+        if (threadIdx.x == 0 && red_bad) {
+            atomicOr(bb + 32, 1);
+            atomicOr(status, kStatusNonFinite);
+        }
+        __threadfence();   // this block's box updates before its count
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const int total = t1.set ? t1.nblk : blk_start[e + 1] - blk_start[e];
+            int32_t* done = bbox + (int64_t)e * kBBoxCopies * kBBoxStride + kBBoxDone;
+            s_last = atomicAdd(done, nb) == total - nb;
+        }
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();   // every other block's updates before the reads
+        if (t1.set) {
+            copy_header(hdr, t1.hdr);
+            if (threadIdx.x == 0) {
+                blk_start[0] = 0;
+                blk_start[1] = t1.nblk;
+                cell_off[0] = 0;
+                cell_off[1] = t1.cell_end;
+            }
+            __syncthreads();
+        }
+        event_params(hdr, e, D, bbox, r, m, axes_mode, naxes_req);
+        __syncthreads();
+    };
+    clear();
+    int e_cur = -1, e_blocks = 0;
+    const int b1 = min((int)(blockIdx.x + 1) * sub, nblk);
+    bool waited = !t1.set;
+    for (int b = blockIdx.x * sub; b < b1; ++b) {
+        const int e = t1.set ? 0 : find_event(blk_start, E, b);
+        if (e != e_cur && e_cur >= 0) {   // (several events only: the wait is done)
+            flush(e_cur, e_blocks);
+            clear();
+            e_blocks = 0;
+        }
+        e_cur = e;
+        ++e_blocks;
+        const float* refs = t1.set ? t1.hdr.refs : hdr[e].refs;
+        const int64_t n = t1.set ? t1.hdr.n : hdr[e].n;
+        const int64_t p0 = (int64_t)(t1.set ? b : b - blk_start[e]) * kBuildPtsPerBlock;
+        const int np = (int)max((int64_t)0, min((int64_t)kBuildPtsPerBlock, n - p0));
+        __syncthreads();   // the previous block's rows have been read
+        if (np > 0) stage_floats(sm, refs + p0 * D, np * D, pad);
+        __syncthreads();
+        if ((int)threadIdx.x < np) {
+            const StagedRow p{sm, (int)threadIdx.x * D, pad};
 #pragma unroll
-    for (int k = 0; k < kMaxD; ++k) {
-        if (k < D) {
-            float a = mn[k], b = mx[k];
-            for (int o = 16; o > 0; o >>= 1) {
-                a = fminf(a, __shfl_xor_sync(0xffffffffu, a, o));
-                b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, o));
+            for (int k = 0; k < kMaxD; ++k) {
+                if (k < D) {
+                    const float v = p[k];
+                    bad |= !isfinite(v);
+                    const int32_t x = float_to_ordered(v);
+                    mn[k] = min(mn[k], x);
+                    mx[k] = max(mx[k], x);
+                }
             }
-            if (lane == 0) { red_mn[k][warp] = a; red_mx[k][warp] = b; }
         }
     }
-    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&red_bad, 1);
-    __syncthreads();
-    int32_t* bb = bbox + ((int64_t)e * kBBoxCopies + (blockIdx.x % kBBoxCopies)) * kBBoxStride;
-    if (threadIdx.x < (unsigned)D) {
-        const int k = threadIdx.x;
-        float a = INFINITY, b = -INFINITY;
-        for (int w = 0; w < kBuildPtsPerBlock / 32; ++w) {
-            a = fminf(a, red_mn[k][w]);
-            b = fmaxf(b, red_mx[k][w]);
+    if (!waited) pdl_wait();
+    zero_share(counts, L / 4, scalars);
+    if (e_cur >= 0) flush(e_cur, e_blocks);
+}
+
+// The start of a build with foreign parameters (a cross-set query's points,
+// binned by the reference grid's header src): tables, parameters, zeroed counts.
+__global__ void k_begin_foreign(OneEventTables t1, const EventHdr* src, EventHdr* hdr, int32_t* blk_start,
+                                int64_t* cell_off, int32_t* counts, int32_t* scalars) {
+    pdl_trigger();
+    pdl_wait();
+    if (blockIdx.x == 0) {
+        copy_header(hdr, t1.hdr);
+        __syncthreads();
+        copy_params(*hdr, *src);
+        if (threadIdx.x == 0) {
+            blk_start[0] = 0;
+            blk_start[1] = t1.nblk;
+            cell_off[0] = 0;
+            cell_off[1] = t1.cell_end;
         }
-        atomicMin(bb + k, float_to_ordered(a));
-        atomicMax(bb + 16 + k, float_to_ordered(b));
     }
-    if (threadIdx.x == 0 && red_bad) {
-        atomicOr(bb + 32, 1);
-        atomicOr(status, kStatusNonFinite);
-    }
-    __shared__ int s_last;
-    __threadfence();   // this block's box updates before its count
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const int nb = blk_start[e + 1] - blk_start[e];
-        int32_t* done = bbox + (int64_t)e * kBBoxCopies * kBBoxStride + kBBoxDone;
-        s_last = atomicAdd(done, 1) == nb - 1;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();   // every other block's updates before the reads
-    event_params(hdr, e, D, bbox, r, m, axes_mode, naxes_req, counts);
+    // (t1.hdr.rowsort: used_entries of the finished header)
+    const int used = (t1.hdr.rowsort ? src->ncells / src->dims[0] : src->ncells) + 1;
+    zero_share(counts, (used + kCellChunk - 1) / kCellChunk * (kCellChunk / 4), scalars);
 }
 
 // Grid parameters of one event (one CTA: its warps combine the box copies,
@@ -536,8 +629,8 @@ __device__ void derive_params(EventHdr& H, const int32_t* box, bool bad, int D, 
     }
 }
 
-__device__ void event_params(EventHdr* hdr, int e, int D, const int32_t* bbox, float r, int m,
-                             int axes_mode, int naxes_req, int32_t* counts) {
+__device__ void event_params(EventHdr* hdr, int e, int D, int32_t* bbox, float r, int m,
+                             int axes_mode, int naxes_req) {
     __shared__ int32_t bb[kBBoxStride];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // lane c holds copy c of entry k; a warp reduction combines them (all of a
@@ -547,8 +640,11 @@ __device__ void event_params(EventHdr* hdr, int e, int D, const int32_t* bbox, f
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
         const int k = warp + 8 * i;
-        // L2 reads: the copies were updated by other blocks' atomics
-        v[i] = k < kBBoxStride ? __ldcg(bbox + ((int64_t)e * kBBoxCopies + lane) * kBBoxStride + k) : 0;
+        // L2 reads: the copies were updated by other blocks' atomics; they are
+        // left empty for the next build
+        int32_t* at = bbox + ((int64_t)e * kBBoxCopies + lane) * kBBoxStride + k;
+        v[i] = k < kBBoxStride ? __ldcg(at) : 0;
+        if (k < kBBoxStride) *at = empty_box_entry(k);
     }
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
@@ -559,37 +655,7 @@ __device__ void event_params(EventHdr* hdr, int e, int D, const int32_t* bbox, f
         if (lane == 0 && k < kBBoxStride) bb[k] = x;
     }
     __syncthreads();
-    EventHdr& H = hdr[e];
-    // the last cell-array entry of the event counts its pair padding slot, so
-    // the next event's slots start on a pair boundary
-    if (threadIdx.x == 0) counts[H.cell_off + H.cell_cap] = (int32_t)(H.n & 1);
-    derive_params(H, bb, bb[32] != 0, D, r, m, axes_mode, naxes_req);
-}
-
-// Cross-set binning: take the reference grid's parameters for each event.
-__global__ void k_copy_params(EventHdr* dst, const EventHdr* src, int E, int32_t* counts) {
-    pdl_trigger();
-    pdl_wait();
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= E) return;
-    EventHdr& d = dst[e];
-    counts[d.cell_off + d.cell_cap] = (int32_t)(d.n & 1);
-    const EventHdr& s = src[e];
-    d.naxes = s.naxes;
-    d.m = s.m;
-    d.valid = s.valid;
-    d.inv_h = s.inv_h;
-    d.ncells = s.ncells;
-    d.half = s.half;
-    for (int a = 0; a < kHdrAxes; ++a) {
-        d.axes[a] = s.axes[a];
-        d.dims[a] = s.dims[a];
-        d.fdims[a] = s.fdims[a];
-        d.mag[a] = s.mag[a];
-        d.lo[a] = s.lo[a];
-        d.hi[a] = s.hi[a];
-    }
-    for (int k = 0; k < kMaxD; ++k) d.ctr[k] = s.ctr[k];
+    derive_params(hdr[e], bb, bb[32] != 0, D, r, m, axes_mode, naxes_req);
 }
 
 // Non-finite check of a query set binned with foreign parameters (the bbox
@@ -623,7 +689,7 @@ __global__ void __launch_bounds__(kBuildPtsPerBlock) k_cellid(const EventHdr* hd
     if (h.valid) c = point_cell(p, h);
     const int64_t gi = h.pt_off + p0 + i;
     cid[gi] = c;
-    rnk[gi] = atomicAdd(counts + h.cell_off + stored_cell(h, c), 1);
+    rnk[gi] = atomicAdd(counts + h.cell_off + count_entry(h, c), 1);
 }
 
 // Slot maps and cell-sorted coordinates: each point's slot (its cell's start
@@ -662,7 +728,7 @@ __global__ void __launch_bounds__(kBuildPtsPerBlock) k_scatter(const EventHdr* h
     if (i >= np) return;
     const int64_t gi = h.pt_off + p0 + i;
     const int c = cid[gi];
-    const int64_t slot = (int64_t)cstart[h.cell_off + stored_cell(h, c)] + rnk[gi];
+    const int64_t slot = (int64_t)cstart[h.cell_off + count_entry(h, c)] + rnk[gi];
     perm[slot] = (int32_t)(p0 + i);
     cell[slot] = c;
     write_row(pts + slot * DP, StagedRow{sm, i * D, pad}, D, DP);
@@ -932,6 +998,147 @@ void enqueue_scan(int32_t* data, int64_t n, int32_t* parts, int32_t* total, cuda
     }
 }
 
+// ------------------------------------------------------------------ cell scan
+// Exclusive scan of the cell counts, every event's on its own: an event's first
+// slot is known, so events share nothing, and only the entries a grid uses are
+// scanned.  Blocks of kCellChunk entries (an event's region starts on one), 16
+// entries a thread in four 16-byte loads; the down pass sums the totals of its
+// event's blocks before it (beyond kCellSumParts of them a pass of one block per
+// event scans the totals first).  300k x 8 (3.5 M cells), reduce + down: 5.0 +
+// 9.6 us with 2,048-entry blocks and 4-byte accesses through shared memory.
+
+constexpr int kCellThreads = 256;
+constexpr int kCellSumParts = 4096;
+static_assert(kCellChunk == 16 * kCellThreads, "four quads a thread");
+
+// Event of a block, its first block, whether the block holds used entries.
+struct CellBlock {
+    int e, first;
+    bool used;
+    __device__ CellBlock(const EventHdr* hdr, int E) {
+        int lo = 0, hi = E - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (hdr[mid].cell_off <= (int64_t)blockIdx.x * kCellChunk) lo = mid; else hi = mid - 1;
+        }
+        e = lo;
+        first = (int)(hdr[lo].cell_off / kCellChunk);
+        used = ((int)blockIdx.x - first) * kCellChunk < used_entries(hdr[lo]);
+    }
+};
+
+__global__ void __launch_bounds__(kCellThreads) k_cells_reduce(const EventHdr* hdr, int E, const int32_t* counts,
+                                                               int32_t* parts) {
+    pdl_trigger();
+    pdl_wait();
+    __shared__ int32_t red[kCellThreads / 32];
+    const CellBlock cb(hdr, E);
+    if (!cb.used) return;
+    const int4* c4 = reinterpret_cast<const int4*>(counts + (int64_t)blockIdx.x * kCellChunk) + threadIdx.x;
+    int4 v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = c4[j * kCellThreads];
+    int s = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) s += v[j].x + v[j].y + v[j].z + v[j].w;
+    s = __reduce_add_sync(0xffffffffu, s);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+        for (int w = 0; w < kCellThreads / 32; ++w) t += red[w];
+        parts[blockIdx.x] = t;
+    }
+}
+
+// Exclusive scan of one event's block totals in place.
+__global__ void __launch_bounds__(1024) k_cells_parts(const EventHdr* hdr, int32_t* parts) {
+    pdl_trigger();
+    pdl_wait();
+    __shared__ int32_t wt[32];
+    const EventHdr& h = hdr[blockIdx.x];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nb = (used_entries(h) + kCellChunk - 1) / kCellChunk;
+    int32_t* p = parts + h.cell_off / kCellChunk;
+    int carry = 0;
+    for (int b0 = 0; b0 < nb; b0 += 1024) {
+        const int i = b0 + threadIdx.x;
+        const int v = i < nb ? p[i] : 0;
+        int incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) wt[warp] = incl;
+        __syncthreads();
+        int below = 0, all = 0;
+        for (int w = 0; w < 32; ++w) {
+            below += w < warp ? wt[w] : 0;
+            all += wt[w];
+        }
+        if (i < nb) p[i] = carry + below + incl - v;
+        carry += all;
+        __syncthreads();
+    }
+}
+
+// scanned: the totals were scanned (k_cells_parts).
+__global__ void __launch_bounds__(kCellThreads) k_cells_down(const EventHdr* hdr, int E, int32_t* counts,
+                                                             const int32_t* parts, int scanned) {
+    pdl_trigger();
+    pdl_wait();
+    constexpr int kW = kCellThreads / 32;
+    __shared__ int32_t tot[4 * kW], red[kW];
+    const CellBlock cb(hdr, E);
+    if (!cb.used) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int4* c4 = reinterpret_cast<int4*>(counts + (int64_t)blockIdx.x * kCellChunk) + threadIdx.x;
+    int4 v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = c4[j * kCellThreads];
+    int before = 0;   // the event's entries before this block
+    if (scanned) {
+        if (threadIdx.x == 0) before = parts[blockIdx.x];
+    } else {
+        for (int j = cb.first + threadIdx.x; j < (int)blockIdx.x; j += kCellThreads) before += parts[j];
+    }
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 0) red[warp] = before;
+    int excl[4];   // of each quad within its warp's 128 entries
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int t = v[j].x + v[j].y + v[j].z + v[j].w;
+        int incl = t;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        excl[j] = incl - t;
+        if (lane == 31) tot[j * kW + warp] = incl;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        static_assert(4 * kW == 32, "one total per lane");
+        const int t = tot[lane];
+        int incl = t;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const int base = (int)hdr[cb.e].pt_off + __reduce_add_sync(0xffffffffu, lane < kW ? red[lane] : 0);
+        tot[lane] = base + incl - t;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int x = tot[j * kW + warp] + excl[j];
+        c4[j * kCellThreads] = make_int4(x, x + v[j].x, x + v[j].x + v[j].y, x + v[j].x + v[j].y + v[j].z);
+    }
+}
+
 // ------------------------------------------------------------------ small sets
 // The whole build of one small event in one launch: a cluster of kSmallCtas
 // CTAs, cluster barriers where the chain above has kernel boundaries.  A set of
@@ -1021,7 +1228,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     }
     pdl_wait();   // the previous work on the stream may still read what is written from here on
     {
-        const int L = t1.hdr.cell_cap + 1;
+        // all of the cell array, or what the foreign parameters use of it
+        const int L = src ? (t1.hdr.rowsort ? src->ncells / src->dims[0] : src->ncells) + 1 : t1.hdr.cell_cap + 1;
         int4* c4 = reinterpret_cast<int4*>(counts);
         for (int j = first; j < L / 4; j += step) c4[j] = make_int4(0, 0, 0, 0);
         for (int j = L / 4 * 4 + first; j < L; j += step) counts[j] = 0;
@@ -1047,24 +1255,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     }
     __syncthreads();
     if (src) {
-        // the parameters of the foreign header
-        if (tid == 0) {
-            sh.naxes = src->naxes;
-            sh.m = src->m;
-            sh.valid = src->valid;
-            sh.inv_h = src->inv_h;
-            sh.ncells = src->ncells;
-            sh.half = src->half;
-        }
-        if (tid < kHdrAxes) {
-            sh.axes[tid] = src->axes[tid];
-            sh.dims[tid] = src->dims[tid];
-            sh.fdims[tid] = src->fdims[tid];
-            sh.mag[tid] = src->mag[tid];
-            sh.lo[tid] = src->lo[tid];
-            sh.hi[tid] = src->hi[tid];
-        }
-        if (tid < kMaxD) sh.ctr[tid] = src->ctr[tid];
+        copy_params(sh, *src);
     } else {
         derive_params(sh, s_all, bad != 0, D, r, m, axes_mode, naxes_req);
     }
@@ -1089,13 +1280,13 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
         rnk[j] = 0;
         if (i < np) {
             if (sh.valid) key[j] = point_cell(StagedRow{sm, i * D, pad}, sh);
-            rnk[j] = atomicAdd(counts + stored_cell(sh, key[j]), 1);
+            rnk[j] = atomicAdd(counts + count_entry(sh, key[j]), 1);
         }
     }
     cluster.sync();
     // exclusive scan of the used entries, the one past the last cell among
     // them: warp g of the cluster takes the g-th segment of `seg` entries
-    const int used = sh.ncells + 1;
+    const int used = used_entries(sh);
     const int seg = ((used + ctas * kWarps - 1) / (ctas * kWarps) + 127) / 128 * 128;
     const int s0 = (rank * kWarps + warp) * seg, s1 = min(s0 + seg, used);
     // four entries from i on (zero past the segment's end)
@@ -1177,7 +1368,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     for (int j = 0; j < kSmallPer; ++j) {
         const int i = tid + j * kSmallThreads;
         if (i < np) {
-            const int slot = __ldcg(counts + stored_cell(sh, key[j])) + rnk[j];
+            const int slot = __ldcg(counts + count_entry(sh, key[j])) + rnk[j];
             perm[slot] = p0 + i;
             cell[slot] = key[j];
             write_row(pts + (int64_t)slot * DP, StagedRow{sm, i * D, pad}, D, DP);
@@ -1243,7 +1434,7 @@ frnn_status grid_alloc(GridBufs& g, int E, const int64_t* n, int D, std::string&
         g.h_blk_start[e] = (int32_t)nblk;
         g.h_cell_off[e] = L;
         n_total += (n[e] + 1) & ~(int64_t)1;   // pair-aligned event regions
-        L += cap + 1;
+        L += cell_entries(cap);
         nblk += std::max<int64_t>(1, ceil_div(n[e], kBuildPtsPerBlock));
     }
     g.h_blk_start[E] = (int32_t)nblk;
@@ -1259,7 +1450,7 @@ frnn_status grid_alloc(GridBufs& g, int E, const int64_t* n, int D, std::string&
     g.n_total = n_total;
     g.L = L;
     g.nblk = nblk;
-    g.nparts = scan_parts_needed(L);
+    g.nparts = std::max(scan_parts_needed(L), L / kCellChunk);
     g.nchunks = nchunks;
     // the buffers are reused only if every region is large enough, the
     // point rows included (a set of a higher dimension needs wider rows)
@@ -1295,7 +1486,7 @@ frnn_status grid_alloc(GridBufs& g, int E, const int64_t* n, int D, std::string&
         if (ce != cudaSuccess) {
             cudaGetLastError();
             err = std::string("cudaMalloc of grid buffers failed: ") + cudaGetErrorString(ce);
-            g.cap_n = g.cap_L = g.cap_E = g.cap_blk = 0;
+            g.cap_n = g.cap_L = g.cap_E = g.cap_blk = g.clean_E = 0;
             g.cap_DP = 0;
             return FRNN_ERR_OUT_OF_MEMORY;
         }
@@ -1320,6 +1511,7 @@ frnn_status grid_alloc(GridBufs& g, int E, const int64_t* n, int D, std::string&
         g.cap_DP = DP;
         g.cap_L = L;
         g.cap_E = E;
+        g.clean_E = 0;
         g.cap_blk = nblk;
     }
     // page-locked mirror for the per-event tables
@@ -1346,11 +1538,7 @@ frnn_status grid_alloc(GridBufs& g, int E, const int64_t* n, int D, std::string&
     return FRNN_OK;
 }
 
-// k_init's blocks: four per SM of the GB300's 152, all resident at once, so
-// that every block triggers the next kernel at once and the bounding-box
-// blocks can stage their points while k_init finishes (2, 4 and 8 per SM
-// measured the same build time at 300k x 8, 0.051 ms; the gain over 0.057
-// is the early staging)
+// k_begin_foreign's blocks: four per SM of the GB300's 152, all resident at once
 constexpr unsigned kInitBlocks = 608;
 
 static inline unsigned blocks_for(int64_t n, int t) {
@@ -1361,12 +1549,34 @@ static inline unsigned blocks_for(int64_t n, int t) {
 static void enqueue_sort(GridBufs& g, size_t smem_pts, int check_finite, int32_t* d_status,
                          cudaStream_t st, EarlyPts ep) {
     const int E = g.E, D = g.D;
+    // (without host headers, the one event's entries are all of them)
+    auto cap_of = [&](int e) -> int64_t { return g.h_hdr.empty() ? g.L - 1 : g.h_hdr[e].cell_cap; };
     launch_pdl(k_cellid, dim3((unsigned)g.nblk), dim3(kBuildPtsPerBlock), smem_pts, st,
                g.hdr, g.blk_start, E, D, g.cstart, g.cid, g.rnk, check_finite, d_status, ep);
-    enqueue_scan(g.cstart, g.L, g.parts, g.scalars + kScCellTotal, st);
+    const int64_t nb = g.L / kCellChunk;
+    int64_t most = 0;   // blocks of the largest event
+    for (int e = 0; e < E; ++e) most = std::max(most, cell_entries(cap_of(e)) / kCellChunk);
+    launch_pdl(k_cells_reduce, dim3((unsigned)nb), dim3(kCellThreads), 0, st, g.hdr, E, g.cstart, g.parts);
+    if (most > kCellSumParts)
+        launch_pdl(k_cells_parts, dim3((unsigned)E), dim3(1024), 0, st, g.hdr, g.parts);
+    launch_pdl(k_cells_down, dim3((unsigned)nb), dim3(kCellThreads), 0, st, g.hdr, E, g.cstart, g.parts,
+               most > kCellSumParts ? 1 : 0);
     launch_pdl(k_scatter, dim3((unsigned)g.nblk), dim3(kBuildPtsPerBlock), smem_pts, st,
                g.hdr, g.blk_start, E, D, g.DP, g.cstart, g.cid, g.rnk, g.pts, g.perm, g.cell, ep);
     // no task list: the grid query takes chunks of kChunkQ slots in slot order
+}
+
+static int box_sub(int64_t nblk) {
+    return (int)std::min<int64_t>(std::max<int64_t>(ceil_div(nblk, kBoxWave), 1), kBoxMost);
+}
+
+// Empty the boxes of buffers that no build has used yet (not inside a capture:
+// a replay would find them empty already).
+void grid_clean(GridBufs& g, cudaStream_t st) {
+    if (g.clean_E >= g.E) return;
+    launch_pdl(k_box_reset, dim3(blocks_for((int64_t)g.cap_E * kBBoxCopies * kBBoxStride, 256)), dim3(256), 0, st,
+               g.bbox, (int)g.cap_E);
+    g.clean_E = g.cap_E;
 }
 
 frnn_status enqueue_build(GridBufs& g, const float* const* refs, const BuildOpts& o,
@@ -1377,7 +1587,7 @@ frnn_status enqueue_build(GridBufs& g, const float* const* refs, const BuildOpts
         g.h_hdr[e].refs = refs[e];
         g.h_hdr[e].valid = 1;
     }
-    // one event outside a capture: k_init writes the tables from its
+    // one event outside a capture: the first kernel writes the tables from its
     // arguments (no copy on the stream, so the chain stays one run of
     // programmatically dependent kernels)
     OneEventTables t1{};
@@ -1406,7 +1616,8 @@ frnn_status enqueue_build(GridBufs& g, const float* const* refs, const BuildOpts
     }
 
     // (a cross-set query's cells are its reference grid's: not a small set's)
-    if (t1.set && t1.hdr.n > 0 && t1.hdr.n <= kSmallMax && g.L <= kSmallCells) {
+    if (t1.set && t1.hdr.n > 0 && t1.hdr.n <= kSmallMax &&
+        g.L <= (params_from && t1.hdr.rowsort ? 16 * kSmallCells : kSmallCells)) {
         const int per = (int)ceil_div(t1.hdr.n, kSmallCtas);   // at most kSmallPer * kSmallThreads
         const size_t smem = sizeof(float) * small_stage_floats(per, D);
         cudaError_t ce = cudaFuncSetAttribute(k_build_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -1425,19 +1636,21 @@ frnn_status enqueue_build(GridBufs& g, const float* const* refs, const BuildOpts
         }
         return FRNN_OK;
     }
-    const int32_t bbmin = host_float_to_ordered(INFINITY);
-    const int32_t bbmax = host_float_to_ordered(-INFINITY);
-    const int64_t init_n = std::max<int64_t>(g.L, (int64_t)E * kBBoxCopies * kBBoxStride);
-    launch_pdl(k_init, dim3(std::min<unsigned>(blocks_for(init_n, 256), kInitBlocks)), dim3(256), 0, st,
-        g.cstart, g.L, g.bbox, E, g.scalars, bbmin, bbmax, t1, g.hdr, g.blk_start, g.cell_off);
     const size_t smem_pts = sizeof(float) * staged_floats(D);
     const EarlyPts ep{t1.hdr.refs, t1.hdr.n, t1.set};
     if (params_from) {
-        launch_pdl(k_copy_params, dim3(blocks_for(E, 128)), dim3(128), 0, st, g.hdr, params_from->hdr, E,
-                   g.cstart);
+        if (!t1.set) {
+            err = "foreign grid parameters need a one-event build";
+            return FRNN_ERR_INVALID_ARG;
+        }
+        launch_pdl(k_begin_foreign, dim3(std::min<unsigned>(blocks_for(g.L / 4, 256), kInitBlocks)), dim3(256), 0, st,
+                   t1, (const EventHdr*)params_from->hdr, g.hdr, g.blk_start, g.cell_off, g.cstart, g.scalars);
     } else {
-        launch_pdl(k_bbox, dim3((unsigned)g.nblk), dim3(kBuildPtsPerBlock), smem_pts, st, g.hdr, g.blk_start, E, D,
-                   g.bbox, d_status, o.r, o.m, o.axes_mode, o.naxes, g.cstart, ep);
+        if (!capturing) grid_clean(g, st);
+        const int sub = box_sub(g.nblk);
+        launch_pdl(k_bbox, dim3((unsigned)ceil_div(g.nblk, sub)), dim3(kBuildPtsPerBlock), smem_pts, st, g.hdr,
+                   g.blk_start, g.cell_off, E, (int)g.nblk, sub, D, g.bbox, d_status, o.r, o.m, o.axes_mode, o.naxes,
+                   g.cstart, g.L, g.scalars, t1);
     }
     enqueue_sort(g, smem_pts, params_from ? 1 : 0, d_status, st, ep);
     g.tc_ready = false;     // tensor-core operands describe the previous contents
@@ -1456,15 +1669,13 @@ frnn_status enqueue_build(GridBufs& g, const float* const* refs, const BuildOpts
 frnn_status enqueue_build_resident(GridBufs& g, const BuildOpts& o, int32_t* d_status,
                                    cudaStream_t st, std::string& err) {
     const int E = g.E, D = g.D;
-    const int32_t bbmin = host_float_to_ordered(INFINITY);
-    const int32_t bbmax = host_float_to_ordered(-INFINITY);
-    const int64_t init_n = std::max<int64_t>(g.L, (int64_t)E * kBBoxCopies * kBBoxStride);
-    launch_pdl(k_init, dim3(std::min<unsigned>(blocks_for(init_n, 256), kInitBlocks)), dim3(256), 0, st,
-        g.cstart, g.L, g.bbox, E, g.scalars, bbmin, bbmax, OneEventTables{}, g.hdr, g.blk_start,
-        g.cell_off);
     const size_t smem_pts = sizeof(float) * staged_floats(D);
-    launch_pdl(k_bbox, dim3((unsigned)g.nblk), dim3(kBuildPtsPerBlock), smem_pts, st, g.hdr, g.blk_start, E, D,
-               g.bbox, d_status, o.r, o.m, o.axes_mode, o.naxes, g.cstart, EarlyPts{});
+    // (the array's contents are anybody's: its boxes are emptied first)
+    launch_pdl(k_box_reset, dim3(blocks_for((int64_t)E * kBBoxCopies * kBBoxStride, 256)), dim3(256), 0, st, g.bbox, E);
+    const int sub = box_sub(g.nblk);
+    launch_pdl(k_bbox, dim3((unsigned)ceil_div(g.nblk, sub)), dim3(kBuildPtsPerBlock), smem_pts, st, g.hdr,
+               g.blk_start, g.cell_off, E, (int)g.nblk, sub, D, g.bbox, d_status, o.r, o.m, o.axes_mode, o.naxes, g.cstart,
+               g.L, g.scalars, OneEventTables{});
     enqueue_sort(g, smem_pts, 0, d_status, st, EarlyPts{});
     g.tc_ready = false;
     g.rows_ready = false;

@@ -29,6 +29,7 @@ struct GridBufs {
     void* base = nullptr;
     size_t bytes = 0;
     int64_t cap_n = 0, cap_L = 0, cap_E = 0, cap_blk = 0;
+    int64_t clean_E = 0;    // events whose bounding boxes hold no points (grid_clean)
     int cap_DP = 0;         // row width the point rows were carved for
     void* h_pinned = nullptr;      // page-locked host mirror of the small tables
     size_t h_pinned_bytes = 0;
@@ -86,7 +87,6 @@ constexpr int kScanChunk = 2048;     // entries per block of the exclusive scan
 constexpr int kBuildPtsPerBlock = 256;
 // indices into GridBufs::scalars
 constexpr int kScNTasks = 0;        // number of warp tasks
-constexpr int kScCellTotal = 1;     // total of the cell-count scan (= n_total)
 constexpr int kScTaskCounter = 2;   // chunk counter of the grid query kernel
 constexpr int kScOvfCount = 3;      // overflowed queries
 constexpr int kScTcCounter = 4;     // task counter of the tensor-core kernel
@@ -107,6 +107,7 @@ int64_t cell_cap_for(int64_t n, int naxes, CellKind kind = CellKind::kPlain);
 frnn_status grid_alloc(GridBufs& g, int E, const int64_t* n, int D, std::string& err,
                        const int64_t* caps = nullptr, int naxes = kMaxAxes);
 void grid_free(GridBufs& g);
+void grid_clean(GridBufs& g, cudaStream_t st);
 
 // Whether a grid requested with naxes gridded axes (0: the automatic choice)
 // and cell multiple m stores half cells (EventHdr::half) for the half-cell

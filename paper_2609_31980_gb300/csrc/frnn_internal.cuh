@@ -81,6 +81,10 @@ struct EventHdr {
     // a search visits 2 instead of 3 cells per axis.  A slot's `cell` entry is
     // stored cell id << kHalfBits | half bits (axis a's at bit a - 1).
     int32_t half;
+    // 1: a query set of a half-cell scan (preset by the host), sorted by rows of
+    // stored cells only (the scan sorts its chunks itself and looks nothing up
+    // in a query set's cell array, which then has one entry per row)
+    int32_t rowsort;
     int32_t axes[kHdrAxes];   // gridded coordinate indices; axes[0] varies fastest
     int32_t dims[kHdrAxes];   // stored cells per gridded axis (1 for unused axes)
     int32_t fdims[kHdrAxes];  // cells per gridded axis (= dims unless half)
@@ -107,9 +111,32 @@ struct Task {
     int32_t row;     // row index within the event: c1 + dims[1] * (c2 + dims[2] * (c3 + ...))
 };
 
+// Cell-array entries of an event allowed `cap` cells: one more than the cells
+// (the end of the last one), in whole blocks of the prefix scan.
+constexpr int kCellChunk = 4096;
+__host__ __device__ constexpr int64_t cell_entries(int64_t cap) {
+    return (cap + kCellChunk) / kCellChunk * kCellChunk;
+}
+
 // A slot's stored cell id (its `cell` entry without the half bits).
 __host__ __device__ inline int stored_cell(const EventHdr& h, int key) {
     return h.half ? key >> kHalfBits : key;
+}
+
+// v / d for v < 2^26 by EventHdr::mag = ceil(2^36 / d), d <= 1024: the error
+// v * (mag d - 2^36) is below 2^26 * 2^10 = 2^36, so the quotient is exact.
+__device__ __forceinline__ int div_mag(int v, uint64_t mag) {
+    return (int)(((uint64_t)(uint32_t)v * mag) >> 36);
+}
+
+// Entry of the cell array that counts a slot with this `cell` entry, and the
+// entries a set uses (the one past its last cell among them).
+__device__ __forceinline__ int count_entry(const EventHdr& h, int key) {
+    const int c = stored_cell(h, key);
+    return h.rowsort ? div_mag(c, h.mag[0]) : c;
+}
+__device__ __forceinline__ int used_entries(const EventHdr& h) {
+    return (h.rowsort ? h.ncells / h.dims[0] : h.ncells) + 1;
 }
 
 // Neighbour rows of a row of cells.  A row fixes every gridded coordinate but

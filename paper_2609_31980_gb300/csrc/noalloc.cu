@@ -43,7 +43,7 @@ constexpr size_t na_al(size_t x) { return (x + 255) / 256 * 256; }
 // bytes of the grid of one n-point event in D dimensions, carved as below
 constexpr size_t na_bytes(int64_t n, int D) {
     const int64_t cn = ((n + 1) & ~(int64_t)1) > 0 ? ((n + 1) & ~(int64_t)1) : 1;
-    const int64_t L = na_cap(n) + 1;
+    const int64_t L = cell_entries(na_cap(n));
     const int64_t parts = (L + kScanChunk - 1) / kScanChunk > 0 ? (L + kScanChunk - 1) / kScanChunk : 1;
     return na_al(sizeof(EventHdr)) + na_al(sizeof(int32_t) * 2) + na_al(sizeof(int64_t) * 2) +
            na_al(sizeof(int32_t) * kBBoxStride * kBBoxCopies) +
@@ -72,7 +72,7 @@ __global__ void k_noalloc_tables(EventHdr* hdr, int32_t* blk_start, int64_t* cel
     blk_start[0] = 0;
     blk_start[1] = nblk;
     cell_off[0] = 0;
-    cell_off[1] = cap + 1;
+    cell_off[1] = cell_entries(cap);
     *status = 0;
 }
 
@@ -85,7 +85,7 @@ static int32_t* carve(GridBufs& g, char* b, int64_t n, int D) {
     g.D = D;
     g.DP = padded_dim(D);
     g.n_total = (n + 1) & ~(int64_t)1;
-    g.L = cap + 1;
+    g.L = cell_entries(cap);
     g.nblk = std::max<int64_t>(1, ceil_div(n, kBuildPtsPerBlock));
     g.nparts = scan_parts_needed(g.L);
     g.nchunks = ceil_div(n, kChunkQ);   // the header's first chunk is 0

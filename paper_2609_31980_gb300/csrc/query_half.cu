@@ -113,12 +113,6 @@ __device__ __forceinline__ WarpSmem carve(unsigned char* base) {
     return w;
 }
 
-// v / d for v < 2^26 by the header's ceil(2^36 / d), d <= 1024: the error
-// v * (mag d - 2^36) is below 2^26 * 2^10 = 2^36, so the quotient is exact.
-__device__ __forceinline__ int div_mag(int v, uint64_t mag) {
-    return (int)(((uint64_t)(uint32_t)v * mag) >> 36);
-}
-
 // One point row of DP floats (32-byte rows with one 32-byte load).
 template <int DP>
 __device__ __forceinline__ void load_row(const float* p, float (&v)[DP]) {

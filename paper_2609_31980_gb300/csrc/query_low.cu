@@ -69,10 +69,6 @@ constexpr size_t kWarpBytes = 2 * 32 * kListStr * 4 + 32 * 4;
 static_assert(kRows * 32 * 8 <= 32 * kListStr * 4, "the ranges fit the distances' rows");
 static_assert(kWarpBytes % 16 == 0, "aligned warp areas");
 
-__device__ __forceinline__ int div_mag(int v, uint64_t mag) {   // v < 2^26 (EventHdr::mag)
-    return (int)(((uint64_t)(uint32_t)v * mag) >> 36);
-}
-
 // Two point rows of 4 floats, the first at an even slot.
 __device__ __forceinline__ void load_pair(const float4* p, float (&v)[8]) {
     asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
