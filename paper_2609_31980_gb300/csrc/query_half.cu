@@ -145,29 +145,6 @@ __device__ __forceinline__ int chunk_event(const EventHdr* qev, int E, int c) {
     return lo;
 }
 
-__device__ __forceinline__ void cswap(uint32_t& a, uint32_t& b) {
-    const uint32_t lo = min(a, b), hi = max(a, b);
-    a = lo;
-    b = hi;
-}
-
-// Batcher's odd-even merge sort of P keys in registers.
-template <int P>
-__device__ __forceinline__ void sort_regs(uint32_t (&k)[P]) {
-#pragma unroll
-    for (int p = 1; p < P; p <<= 1) {
-#pragma unroll
-        for (int q = p; q >= 1; q >>= 1) {
-#pragma unroll
-            for (int i = 0; i < P; ++i) {
-                const int j = q % p;   // the step's first key
-                if (i >= j && (i - j) % (2 * q) < q && i + q < P && i / (2 * p) == (i + q) / (2 * p))
-                    cswap(k[i], k[i + q]);
-            }
-        }
-    }
-}
-
 // Sort every query's list (n entries of query lane % 16 on its two lanes, at
 // most 2 P; warp-wide call) in place by (d2, original index); the places from
 // n to 2 P get the padding.
@@ -185,28 +162,8 @@ __device__ __forceinline__ void sort_rows(const WarpSmem& w, int n) {
         const uint32_t v = __float_as_uint(ld[e]);
         k[i] = e < n ? (v & ~31u) | (uint32_t)e : 0x80000000u | (uint32_t)(e * 33);
     }
-    sort_regs<P>(k);
-    // the pair's halves: the lower lane keeps the P smallest, the upper the
-    // rest (each a bitonic sequence), then one merge in registers
-    {
-        uint32_t o[P];
-#pragma unroll
-        for (int i = 0; i < P; ++i) o[i] = __shfl_xor_sync(kFull, k[P - 1 - i], 16);
-#pragma unroll
-        for (int i = 0; i < P; ++i) k[i] = hh ? max(k[i], o[i]) : min(k[i], o[i]);
-    }
-#pragma unroll
-    for (int j = P / 2; j > 0; j >>= 1)
-#pragma unroll
-        for (int i = 0; i < P; ++i)
-            if ((i & j) == 0) cswap(k[i], k[i | j]);
-    // neighbouring keys equal but for the place: the order needs the whole key
-    uint32_t near = 32u;
-#pragma unroll
-    for (int i = 0; i + 1 < P; ++i) near = min(near, k[i] ^ k[i + 1]);
-    const uint32_t edge = hh ? k[0] : k[P - 1];
-    near = min(near, edge ^ __shfl_xor_sync(kFull, edge, 16));
-    const unsigned tied = __ballot_sync(kFull, near < 32u);
+    const bool near = sort_pair<P>(k);
+    const unsigned tied = __ballot_sync(kFull, near);
     // entries to their places
     {
         float v[P];

@@ -34,14 +34,17 @@
 //
 // Kernel organisation (one persistent CTA per SM, 8 warps, 512 TMEM columns):
 //   * a producer warp issues cp.async.bulk copies of the A tile (128 query
-//     rows) and, per chunk of up to 128 candidates, of the B tile plus the
-//     float32 coordinates of the same candidates (for the recheck) into a
-//     3-deep ring, and the MMAs (K/16 instructions per chunk) into one of two
-//     TMEM accumulators (2 x 128 columns; two CTAs per SM share the 512);
-//   * four epilogue warps: warp w reads TMEM lanes 32w.. with tcgen05.ld
-//     32x32b.x32, tests 32 pairs per thread with a 3-input max tree, and where
-//     a value reaches t(x) compacts the warp's survivors so that all 32 lanes
-//     recheck them exactly from shared memory;
+//     rows) and, per chunk of up to 128 candidates, of the B tile into a ring
+//     (up to eight deep), and the MMAs (K/16 instructions per chunk) into one
+//     of two TMEM accumulators (2 x 128 columns; two CTAs per SM share the 512);
+//   * eight epilogue warps: warp w reads TMEM lanes 32 (w % 4).. and one half
+//     of the columns with tcgen05.ld 32x32b.x32, tests 32 pairs per thread with
+//     a 3-input max tree, looks closer only at the octets of columns in which
+//     some lane's maximum reaches t(x), and appends the survivors to a buffer;
+//     whenever 32 have come together, over groups and chunks, the warp's lanes
+//     recheck one each exactly, the candidate's float32 row from L2.  (A group
+//     of 32 x 32 pairs holds 1.7 survivors at 500k x 12: rechecking each
+//     group's own from staged coordinates left 30 lanes idle.)
 //   * per-query survivor lists in shared memory are sorted by (d2, index)
 //     with a register network and written as coalesced rows.  Lists longer
 //     than the capacity go to the exact selection kernel (query.cu).
@@ -53,6 +56,7 @@
 #include <cmath>
 
 #include "frnn_host.h"
+#include "warp_sort.cuh"
 
 namespace frnn {
 
@@ -61,7 +65,7 @@ constexpr int kTcN = 128;        // candidates per chunk = MMA N (multiple of 32
 constexpr int kTcAcc = 2;        // TMEM accumulators in flight (kTcAcc * kTcN = kTcCols)
 constexpr int kTcEpi = 256;      // epilogue threads: warp w < 8 owns TMEM lanes 32 (w % 4)..
                                  // and column half w / 4 of every chunk
-constexpr int kTcThreads = kTcEpi + 32;   // + one producer warp (bulk copies, MMA issue)
+constexpr int kTcThreads = kTcEpi + 64;   // + a loading warp (tasks, bulk copies) + an MMA warp
 constexpr int kTcLStr = kTcM + 1;         // list table: one column per query row
 constexpr int kTcMaxChunks = 128;         // chunk table entries kept in shared memory
 constexpr int kTcMaxRows = 256;           // neighbour rows per task (3^5 on a six-axis grid of half cells)
@@ -74,25 +78,27 @@ __host__ __device__ constexpr int tc_k_for(int D) { return ((3 * D + 2) + 15) / 
 
 // shared memory outside the operand ring
 __host__ __device__ constexpr size_t tc_smem_fixed(int K, int DP);
-// operand ring depth: as deep as fits two CTAs per SM (<= 110 KB each), 2..8
+// operand ring depth: as deep as fits two CTAs per SM (<= 107 KB each beside
+// the static part), 2..8
 __host__ __device__ constexpr int tc_ring_for(int D);
 
-constexpr int kTcSurvCap = 32 * 32;   // survivor (row, column) pairs of one warp and 32 columns
+constexpr int kTcSurvCap = 96;   // survivors a warp holds (it rechecks as soon as 32 have come together)
 
 __host__ __device__ constexpr size_t tc_smem_fixed(int K, int DP) {
     return (size_t)kTcM * K * 2                                // A tile
            + (size_t)kTcList * kTcLStr * 8                     // per-query lists
            + (size_t)kTcM * DP * 4                             // query coordinates
-           + (size_t)(kTcEpi / 32) * kTcSurvCap * 2;           // per-warp survivor buffers
+           + (size_t)(kTcEpi / 32) * kTcSurvCap * 5;           // per-warp survivor buffers
 }
 __host__ __device__ constexpr size_t tc_slot_bytes(int K, int DP) {
-    return (size_t)kTcN * K * 2 + (size_t)kTcN * DP * 4;       // B tile + float32 candidates
+    (void)DP;
+    return (size_t)kTcN * K * 2;       // B tile
 }
 __host__ __device__ constexpr int tc_ring_for(int D) {
     int r = 8;
     while (r > 2 && tc_smem_fixed(tc_k_for(D), padded_dim(D)) +
                             (size_t)r * tc_slot_bytes(tc_k_for(D), padded_dim(D)) >
-                        110 * 1024)
+                        107 * 1024)
         --r;
     return r;
 }
@@ -238,22 +244,6 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-        "%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-          "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
-          "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
-          "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-}
-
 // tcgen05.ld of 32 columns without the wait (several loads share one wait)
 __device__ __forceinline__ void tmem_ld32_nowait(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
@@ -310,39 +300,91 @@ struct TcArgs {
     int32_t* degree;
 };
 
+// Sort 16 lists held as columns (entry e of list r at Ld[e * kTcLStr + r]) by
+// (d2, original index), in place: lanes q and q + 16 share list r0 + q of n <=
+// 2 P entries (n the same on both).  Keys as in the half-cell scan: the
+// distance's bits with the low five cleared, then the entry's place; lists in
+// which two truncated distances agree are ordered by counting.
+template <int P>
+__device__ __forceinline__ void sort_columns(float* Ld, int32_t* Li, int r0, int n) {
+    const int lane = threadIdx.x & 31, hh = lane >> 4;
+    float* ld = Ld + r0 + (lane & 15);
+    int32_t* li = Li + r0 + (lane & 15);
+    uint32_t k[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+        const int e = hh * P + i;
+        // empty places: above every distance, 32 apart
+        k[i] = e < n ? (__float_as_uint(ld[e * kTcLStr]) & ~31u) | (uint32_t)e : 0x80000000u | (uint32_t)(e * 33);
+    }
+    const unsigned tied = __ballot_sync(kFull, sort_pair<P>(k));
+    {
+        float v[P];
+#pragma unroll
+        for (int i = 0; i < P; ++i) v[i] = hh * P + i < n ? ld[(k[i] & 31) * kTcLStr] : 0.f;
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < P; ++i)
+            if (hh * P + i < n) ld[(hh * P + i) * kTcLStr] = v[i];
+    }
+    {
+        int32_t v[P];
+#pragma unroll
+        for (int i = 0; i < P; ++i) v[i] = hh * P + i < n ? li[(k[i] & 31) * kTcLStr] : 0;
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < P; ++i)
+            if (hh * P + i < n) li[(hh * P + i) * kTcLStr] = v[i];
+    }
+    __syncwarp();
+    unsigned rows = (tied | (tied >> 16)) & 0xffffu;
+    while (rows) {
+        const int r = __ffs(rows) - 1;
+        rows &= rows - 1u;
+        const int nr = __shfl_sync(kFull, n, r);
+        const float d = lane < nr ? Ld[lane * kTcLStr + r0 + r] : 0.f;
+        const int32_t x = lane < nr ? Li[lane * kTcLStr + r0 + r] : 0;
+        int rank = 0;
+        for (int j = 0; j < nr; ++j) {
+            const float dj = __shfl_sync(kFull, d, j);
+            const int32_t xj = __shfl_sync(kFull, x, j);
+            rank += (dj < d || (dj == d && xj < x)) ? 1 : 0;
+        }
+        __syncwarp();
+        if (lane < nr) {
+            Ld[rank * kTcLStr + r0 + r] = d;
+            Li[rank * kTcLStr + r0 + r] = x;
+        }
+    }
+    __syncwarp();
+}
+
 // Chunk geometry of a task: neighbour row L covers slot range [rs, re); its
 // operand rows start at b8 = rs rounded down to 8 and end at e8 = re rounded
-// up to 8; chunks of up to 256 rows (the MMA N, rounded up to 16).
+// up to 8; chunks of up to kTcN rows (the MMA N, rounded up to 32).
 struct ChunkTab {
     int rs[kTcMaxRows], re[kTcMaxRows], pref[kTcMaxRows + 1];
-    int nrows, nch;
+    int nrows;
     int4 chunk[kTcMaxChunks];   // (start, n, lo, hi) of the first chunks
 };
 
-__device__ __forceinline__ void chunk_info_slow(const ChunkTab& t, int c, int& start, int& n,
-                                                int& lo, int& hi) {
+__device__ __forceinline__ int4 chunk_info(const ChunkTab& t, int c) {
+    if (c < kTcMaxChunks) return t.chunk[c];
     int L = 0;
     while (L + 1 < t.nrows && t.pref[L + 1] <= c) ++L;
-    start = (t.rs[L] & ~7) + (c - t.pref[L]) * kTcN;
+    const int start = (t.rs[L] & ~7) + (c - t.pref[L]) * kTcN;
     const int e8 = (t.re[L] + 7) & ~7;
-    n = min(kTcN, e8 - start);
-    n = (n + 31) & ~31;   // whole 32-column TMEM loads; extra rows are masked by [lo, hi)
-    lo = t.rs[L];
-    hi = t.re[L];
+    // whole 32-column TMEM loads; extra rows are masked by [lo, hi)
+    return make_int4(start, (min(kTcN, e8 - start) + 31) & ~31, t.rs[L], t.re[L]);
 }
 
-__device__ __forceinline__ void chunk_info(const ChunkTab& t, int c, int& start, int& n, int& lo,
-                                           int& hi) {
-    if (c < kTcMaxChunks) {
-        const int4 v = t.chunk[c];
-        start = v.x;
-        n = v.y;
-        lo = v.z;
-        hi = v.w;
-    } else {
-        chunk_info_slow(t, c, start, n, lo, hi);
-    }
-}
+// A task the loading warp has prepared.
+struct TcTask {
+    Task t;
+    int nch;        // chunks (0: nothing to compare, or an invalid event)
+    int done;       // no more tasks
+    float theta;    // the event's pre-filter radius, rounded up
+};
 
 template <int D>
 __global__ void __launch_bounds__(kTcThreads, 2) k_tc_query(TcArgs a) {
@@ -353,26 +395,25 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_query(TcArgs a) {
     extern __shared__ __align__(1024) unsigned char smem[];
     uint16_t* As = reinterpret_cast<uint16_t*>(smem);
     uint16_t* Bs = As + kTcM * K;
-    float* Fs = reinterpret_cast<float*>(Bs + kTcRing * kTcN * K);
-    float* Ld = Fs + kTcRing * kTcN * DP;
+    float* Ld = reinterpret_cast<float*>(Bs + kTcRing * kTcN * K);
     int32_t* Li = reinterpret_cast<int32_t*>(Ld + kTcList * kTcLStr);
     float* Qs = reinterpret_cast<float*>(Li + kTcList * kTcLStr);      // [128][DP]
-    uint16_t* Sv = reinterpret_cast<uint16_t*>(Qs + kTcM * DP);        // [4][kTcSurvCap]
+    uint32_t* Sv = reinterpret_cast<uint32_t*>(Qs + kTcM * DP);        // [warps][kTcSurvCap] slots, then rows
 
-    // bar_b: chunk operands landed; bar_mma: accumulator ready; bar_acc:
-    // epilogue done with an accumulator; bar_slot: epilogue done with a ring slot
+    // bar_b: chunk operands landed; bar_mma: accumulator ready and s_chunk
+    // written; bar_acc: epilogue has read an accumulator (and its s_chunk);
+    // bar_slot: MMAs done with a ring slot
     __shared__ __align__(8) uint64_t bar_a, bar_b[kTcRing], bar_mma[kTcAcc], bar_acc[kTcAcc],
         bar_slot[kTcRing];
     __shared__ uint32_t s_taddr;
-    __shared__ Task s_task;
-    __shared__ int s_done, s_abort;
-    __shared__ ChunkTab s_ct;
+    __shared__ TcTask s_task[2];
+    __shared__ int s_abort;
+    __shared__ ChunkTab s_ct;            // the loading warp's own
+    __shared__ int4 s_load[kTcRing];     // (start, n, lo, hi) of the chunk in each ring slot
+    __shared__ int4 s_chunk[kTcAcc];     // and in each accumulator
     __shared__ int s_cnt[kTcM];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const bool producer = warp == kTcEpi / 32;
-    const int half = (warp >> 2) & 1;          // column half of the chunk (epilogue warps)
-    const int row = 32 * (warp & 3) + lane;    // TMEM lane / query row
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -384,11 +425,11 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_query(TcArgs a) {
         mbar_init(&bar_a, 1);
         for (int i = 0; i < kTcRing; ++i) {
             mbar_init(&bar_b[i], 1);
-            mbar_init(&bar_slot[i], kTcEpi);   // every epilogue thread, every chunk
+            mbar_init(&bar_slot[i], 1);
         }
         for (int i = 0; i < kTcAcc; ++i) {
-            mbar_init(&bar_mma[i], 1);
-            mbar_init(&bar_acc[i], kTcEpi);
+            mbar_init(&bar_mma[i], 2);        // the MMAs' commit and the producer
+            mbar_init(&bar_acc[i], kTcEpi);   // every epilogue thread, every chunk
         }
         s_abort = 0;
         fence_mbar_init();
@@ -398,354 +439,470 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_query(TcArgs a) {
     tc_fence_after();
     const uint32_t taddr = s_taddr;
 
-    const uint32_t sA = smem_u32(As);
-    const uint32_t sB = smem_u32(Bs);
-    const uint32_t lbo = 128, sbo = (uint32_t)K * 16;
-    const float r2 = a.r2;
-    const int Kout = a.K;
-    const int ntasks = *a.ntasks;
-
-    uint32_t task_no = 0;
-    uint32_t g0 = 0;          // global chunk counter at the start of the task
-    unsigned long long n_surv = 0, n_acc = 0;
-
     auto abort_now = [&]() {
         atomicOr(a.status, kStatusTimeout);
         atomicExch(&s_abort, 1);
     };
     auto aborted = [&]() -> int { return *reinterpret_cast<volatile int*>(&s_abort); };
 
-    for (;;) {
-        __syncthreads();
-        if (tid == kTcEpi) {
-            const int t = atomicAdd(a.task_counter, 1);
-            s_done = (t >= ntasks) || aborted();
-            if (t < ntasks) s_task = a.tasks[t];
-        }
-        __syncthreads();
-        if (s_done) break;
-        const Task tk = s_task;
-        const EventHdr& h = a.ev[tk.ev];
-        if (a.path_filter >= 0 && h.path != a.path_filter) continue;   // another launch's event
-        int32_t* counts = a.counts ? a.counts : h.counts;
-        int32_t* oidx = a.counts ? a.idx : h.idx;
-        float* od2 = a.counts ? a.dist2 : h.dist2;
-        const int w0 = tk.qslot & ~7;
-        const int qs = w0 + row;
-        const bool active = !producer && qs >= tk.qslot && qs < tk.qslot + tk.nq;
-        const int qorig = active ? a.qperm[qs] : 0;
-        if (!h.valid) {
-            // grid built from non-finite input: empty rows (frnn_sync reports it)
-            if (active) {
-                for (int e = 0; e < Kout && !a.csr; ++e) {
-                    oidx[(int64_t)qorig * Kout + e] = -1;
-                    od2[(int64_t)qorig * Kout + e] = INFINITY;
-                }
-                counts[qorig] = 0;
-                if (a.degree) a.degree[qorig] = 0;
+    uint32_t g0 = 0;          // global chunk counter at the start of the task
+
+    if (warp == kTcEpi / 32) {
+        // ------------------------------------------------------ loading warp
+        const int ntasks = *a.ntasks;
+        int theta_ev = -1;
+        float theta = 0.f;
+        uint32_t a_loads = 0, g_loads = 0;   // query tiles and chunks sent for so far
+        // Take the next task and list its chunks, while the other warps still
+        // work on the task before.
+        auto prepare = [&](TcTask& out) -> int {
+            int t;
+            Task tk;
+            for (;;) {
+                t = 0;
+                if (lane == 0) t = aborted() ? ntasks : atomicAdd(a.task_counter, 1);
+                t = __shfl_sync(0xffffffffu, t, 0);
+                if (t >= ntasks) break;
+                tk = a.tasks[t];
+                if (a.path_filter < 0 || a.ev[tk.ev].path == a.path_filter) break;   // (else another launch's event)
             }
-            continue;
-        }
-        if (producer) {
-            // neighbour rows and chunk table
-            const int dims0 = h.dims[0], m = h.m;
-            const int xa = stored_cell(h, a.qcell[tk.qslot]) % dims0;
-            const int xb = stored_cell(h, a.qcell[tk.qslot + tk.nq - 1]) % dims0;
-            // (2m+1)^(naxes-1) <= kTcMaxRows rows (the grid parameters ensure
-            // it), 32 per round with a running chunk count
-            const int nrows = neighbour_rows(h);
+            if (t >= ntasks) {
+                if (lane == 0) out.done = 1;
+                return -1;
+            }
+            const EventHdr& h = a.ev[tk.ev];
             int carry = 0;
-            for (int rr = 0; rr * 32 < nrows; ++rr) {
-                const int l = rr * 32 + lane;
-                int rs = 0, re = 0;
-                int64_t rowbase;
-                if (l < nrows && neighbour_row(h, tk.row, l, rowbase)) {
-                    rs = a.cstart[rowbase + max(xa - m, 0)];
-                    re = a.cstart[rowbase + min(xb + m, dims0 - 1) + 1];
-                }
-                const int b8 = rs & ~7;
-                const int e8 = (re + 7) & ~7;
-                const int nch = re > rs ? (e8 - b8 + kTcN - 1) / kTcN : 0;
-                int pre = nch;
+            if (h.valid) {
+                const int dims0 = h.dims[0], m = h.m;
+                const int xa = stored_cell(h, a.qcell[tk.qslot]) % dims0;
+                const int xb = stored_cell(h, a.qcell[tk.qslot + tk.nq - 1]) % dims0;
+                // (2m+1)^(naxes-1) <= kTcMaxRows rows (the grid parameters ensure
+                // it), 32 per round with a running chunk count
+                const int nrows = neighbour_rows(h);
+                for (int rr = 0; rr * 32 < nrows; ++rr) {
+                    const int l = rr * 32 + lane;
+                    int rs = 0, re = 0;
+                    int64_t rowbase;
+                    if (l < nrows && neighbour_row(h, tk.row, l, rowbase)) {
+                        rs = a.cstart[rowbase + max(xa - m, 0)];
+                        re = a.cstart[rowbase + min(xb + m, dims0 - 1) + 1];
+                    }
+                    const int b8 = rs & ~7;
+                    const int e8 = (re + 7) & ~7;
+                    const int nch = re > rs ? (e8 - b8 + kTcN - 1) / kTcN : 0;
+                    int pre = nch;
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int v = __shfl_up_sync(0xffffffffu, pre, o);
-                    if (lane >= o) pre += v;
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int v = __shfl_up_sync(0xffffffffu, pre, o);
+                        if (lane >= o) pre += v;
+                    }
+                    if (l < kTcMaxRows) {
+                        s_ct.rs[l] = rs;
+                        s_ct.re[l] = re;
+                        s_ct.pref[l] = carry + pre - nch;
+                    }
+                    // this lane's row: its chunks' (start, n, lo, hi)
+                    for (int j = 0; j < nch; ++j) {
+                        const int c = carry + pre - nch + j;
+                        if (c >= kTcMaxChunks) break;
+                        const int start = b8 + j * kTcN;
+                        s_ct.chunk[c] = make_int4(start, (min(kTcN, e8 - start) + 31) & ~31, rs, re);
+                    }
+                    carry += __shfl_sync(0xffffffffu, pre, 31);
                 }
-                if (l < kTcMaxRows) {
-                    s_ct.rs[l] = rs;
-                    s_ct.re[l] = re;
-                    s_ct.pref[l] = carry + pre - nch;
+                if (lane == 0) s_ct.nrows = nrows;
+                if (tk.ev != theta_ev) {
+                    const double nu2 = fmax((double)ordered_to_float(a.nu_q[tk.ev]),
+                                            (double)ordered_to_float(a.nu_r[tk.ev]));
+                    const double nu = sqrt(fmax(nu2, 0.0));
+                    const double R = sqrt((double)a.r2 * (1.0 + 0x1p-18));
+                    theta = __double2float_ru((R + 0x1p-14 * nu) * (R + 0x1p-14 * nu) + 0x1p-12 * nu2);
+                    theta_ev = tk.ev;
                 }
-                // this lane's row: its chunks' (start, n, lo, hi)
-                for (int j = 0; j < nch; ++j) {
-                    const int c = carry + pre - nch + j;
-                    if (c >= kTcMaxChunks) break;
-                    const int start = b8 + j * kTcN;
-                    int n = min(kTcN, e8 - start);
-                    n = (n + 31) & ~31;
-                    s_ct.chunk[c] = make_int4(start, n, rs, re);
-                }
-                carry += __shfl_sync(0xffffffffu, pre, 31);
             }
             if (lane == 0) {
-                s_ct.nch = carry;
-                s_ct.nrows = nrows;
+                out.t = tk;
+                out.nch = carry;
+                out.done = 0;
+                out.theta = theta;
             }
-        } else if (half == 0) {
-            // this thread's query: float32 coordinates (shared: the recheck
-            // reads them from any lane)
-#pragma unroll
-            for (int k = 0; k < D; ++k)
-                Qs[row * DP + k] = active ? a.qpts[pt_index(qs, k, DP)] : 0.f;
-            s_cnt[row] = 0;
-        }
-        __syncthreads();
-        const int nch = s_ct.nch;
-
-        if (producer) {
-            // ---------------------------------------------------- producer
-            if (lane == 0 && nch > 0) {
-                // ring slot g % R is free once the epilogue of chunk g - R is done
-                auto slot_free_now = [&](uint32_t g) -> bool {
-                    if (g < (uint32_t)kTcRing) return true;
-                    uint32_t ok2;
-                    asm volatile(
-                        "{\n\t.reg .pred p;\n\t"
-                        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                        "selp.u32 %0, 1, 0, p;\n\t}"
-                        : "=r"(ok2)
-                        : "r"(smem_u32(&bar_slot[g % kTcRing])),
-                          "r"(((g - kTcRing) / kTcRing) & 1u)
-                        : "memory");
-                    return ok2 != 0;
-                };
-                auto issue_load = [&](int c, uint32_t g) {
-                    int start, n, lo, hi;
-                    chunk_info(s_ct, c, start, n, lo, hi);
-                    const int slot = g % kTcRing;
-                    const uint32_t bB = (uint32_t)n * K * 2;
-                    const uint32_t bF = (uint32_t)n * DP * 4;
-                    mbar_arrive_expect_tx(&bar_b[slot], bB + bF);
-                    bulk_g2s(Bs + (size_t)slot * kTcN * K, a.tcB + cm_off(start, 0, K), bB,
-                             &bar_b[slot]);
-                    bulk_g2s(Fs + (size_t)slot * kTcN * DP, a.rpts + (int64_t)start * DP, bF,
-                             &bar_b[slot]);
-                };
-                const uint32_t bA = (uint32_t)kTcM * K * 2;
-                mbar_arrive_expect_tx(&bar_a, bA);
-                bulk_g2s(As, a.tcA + cm_off(w0, 0, K), bA, &bar_a);
-                int next_load = 0, issued_mma = 0;
-                bool ok = true;
-                // loads run ahead as far as ring slots are free
-                while (next_load < nch && next_load < kTcRing && slot_free_now(g0 + next_load)) {
-                    issue_load(next_load, g0 + next_load);
-                    ++next_load;
-                }
-                ok = mbar_wait_bounded(&bar_a, task_no & 1u);
-                for (int c = 0; ok && c < nch; ++c) {
-                    const uint32_t g = g0 + c;
-                    const int slot = g % kTcRing;
-                    while (ok && next_load <= c) {   // this chunk's operands must be on their way
-                        const uint32_t gl = g0 + next_load;
-                        if (gl >= (uint32_t)kTcRing)
-                            ok = mbar_wait_bounded(&bar_slot[gl % kTcRing],
-                                                   ((gl - kTcRing) / kTcRing) & 1u);
-                        if (ok) {
-                            issue_load(next_load, gl);
-                            ++next_load;
-                        }
-                    }
-                    // operands landed and the accumulator's previous epilogue done
-                    if (ok) ok = mbar_wait_bounded(&bar_b[slot], (g / kTcRing) & 1u);
-                    if (ok && g >= (uint32_t)kTcAcc)
-                        ok = mbar_wait_bounded(&bar_acc[g % kTcAcc], ((g - kTcAcc) / kTcAcc) & 1u);
-                    if (!ok) break;
-                    tc_fence_after();
-                    int start, n, lo, hi;
-                    chunk_info(s_ct, c, start, n, lo, hi);
-                    const uint32_t idesc = mma_idesc(n);
-                    const uint32_t bbase = sB + (uint32_t)(slot * kTcN * K * 2);
-#pragma unroll
-                    for (int ks = 0; ks < KS; ++ks) {
-                        mma_bf16(taddr + (g % kTcAcc) * kTcN, smem_desc(sA + ks * 256, lbo, sbo),
-                                 smem_desc(bbase + ks * 256, lbo, sbo), idesc, ks > 0 ? 1u : 0u);
-                    }
-                    mma_commit(&bar_mma[g % kTcAcc]);
-                    issued_mma = c + 1;
-                    while (next_load < nch && next_load < c + 1 + kTcRing &&
-                           slot_free_now(g0 + next_load)) {
-                        issue_load(next_load, g0 + next_load);
-                        ++next_load;
-                    }
-                }
-                if (!ok) {
+            __syncwarp();
+            return carry;
+        };
+        // chunk c of the listed task into ring slot g % R, which is free once
+        // the MMAs of chunk g - R are done
+        auto load = [&](int c, uint32_t g) -> bool {
+            const int slot = g % kTcRing;
+            const int4 ci = chunk_info(s_ct, c);
+            if (g >= (uint32_t)kTcRing &&
+                !mbar_wait_bounded(&bar_slot[slot], ((g - kTcRing) / kTcRing) & 1u))
+                return false;
+            s_load[slot] = ci;
+            const uint32_t bB = (uint32_t)ci.y * K * 2;
+            mbar_arrive_expect_tx(&bar_b[slot], bB);
+            bulk_g2s(Bs + (size_t)slot * kTcN * K, a.tcB + cm_off(ci.x, 0, K), bB, &bar_b[slot]);
+            g_loads = g + 1;
+            return true;
+        };
+        // its query tile and its first chunks; the MMAs of the task before are
+        // done (they read the tile this overwrites)
+        auto start_loads = [&](const TcTask& tt, int nch) -> int {
+            if (lane != 0 || nch <= 0) return 0;
+            const uint32_t bA = (uint32_t)kTcM * K * 2;
+            mbar_arrive_expect_tx(&bar_a, bA);
+            bulk_g2s(As, a.tcA + cm_off(tt.t.qslot & ~7, 0, K), bA, &bar_a);
+            ++a_loads;
+            int c = 0;
+            for (; c < nch && c < kTcRing; ++c) {
+                if (!load(c, g0 + c)) {
                     abort_now();
-                    // wait (bounded) for the copies and MMAs in flight
-                    for (int c = issued_mma; c < next_load; ++c)
-                        mbar_wait_bounded(&bar_b[(g0 + c) % kTcRing], ((g0 + c) / kTcRing) & 1u);
-                    if (issued_mma > 0)
-                        mbar_wait_bounded(&bar_mma[(g0 + issued_mma - 1) % kTcAcc],
-                                          ((g0 + issued_mma - 1) / kTcAcc) & 1u);
+                    break;
+                }
+            }
+            return c;
+        };
+
+        int nch = prepare(s_task[0]);
+        int loaded = start_loads(s_task[0], nch);
+        for (uint32_t par = 0;; par ^= 1u) {
+            __syncthreads();   // this task is ready; the epilogue has finished the one before
+            if (nch < 0) break;
+            if (lane == 0) {
+                for (; loaded < nch && !aborted(); ++loaded) {
+                    if (!load(loaded, g0 + loaded)) {
+                        abort_now();
+                        break;
+                    }
                 }
             }
             __syncwarp();
-        } else {
-            // ---------------------------------------------------- epilogue
-            float tx = INFINITY;
-            if (active) {
-                const double nu2 = fmax((double)ordered_to_float(a.nu_q[tk.ev]),
-                                        (double)ordered_to_float(a.nu_r[tk.ev]));
-                const double nu = sqrt(fmax(nu2, 0.0));
-                const double R = sqrt((double)r2 * (1.0 + 0x1p-18));
-                const double th = (R + 0x1p-14 * nu) * (R + 0x1p-14 * nu) + 0x1p-12 * nu2;
-                tx = __double2float_rd(((double)a.qn[qs] - th) * 0.5);
+            const uint32_t g_end = g0 + (uint32_t)nch;
+            const int nch_next = prepare(s_task[par ^ 1u]);
+            // the query tile is free when the task's last MMAs are done
+            if (lane == 0 && nch > 0 && !aborted() &&
+                !mbar_wait_bounded(&bar_slot[(g_end - 1) % kTcRing], ((g_end - 1) / kTcRing) & 1u))
+                abort_now();
+            __syncwarp();
+            g0 = g_end;
+            nch = nch_next;
+            loaded = aborted() ? 0 : start_loads(s_task[par ^ 1u], nch);
+        }
+        // after a timeout: copies that no MMA waited for (chunk g's is the last
+        // phase of its slot's barrier)
+        if (lane == 0 && aborted()) {
+            if (a_loads > 0) mbar_wait_bounded(&bar_a, (a_loads - 1) & 1u);
+            for (uint32_t g = g_loads - min(g_loads, (uint32_t)kTcRing); g < g_loads; ++g)
+                mbar_wait_bounded(&bar_b[g % kTcRing], (g / kTcRing) & 1u);
+        }
+        __syncwarp();
+    } else if (warp == kTcEpi / 32 + 1) {
+        // ---------------------------------------------------------- MMA warp
+        const uint32_t lbo = 128, sbo = (uint32_t)K * 16;
+        const uint64_t descA = smem_desc(smem_u32(As), lbo, sbo);
+        const uint64_t descB = smem_desc(smem_u32(Bs), lbo, sbo);
+        uint32_t a_tiles = 0;     // query tiles waited for so far
+        for (uint32_t par = 0;; par ^= 1u) {
+            __syncthreads();
+            if (s_task[par].done) break;
+            const int nch = s_task[par].nch;
+            if (lane == 0 && nch > 0) {
+                bool ok = !aborted() && mbar_wait_bounded(&bar_a, a_tiles & 1u);
+                int issued = 0;
+                for (int c = 0; ok && c < nch; ++c) {
+                    const uint32_t g = g0 + c;
+                    const int slot = g % kTcRing;
+                    const uint32_t acc = g % kTcAcc;
+                    // operands landed and the accumulator's previous chunk read
+                    ok = !aborted() && mbar_wait_bounded(&bar_b[slot], (g / kTcRing) & 1u);
+                    const int4 ci = s_load[slot];
+                    const uint32_t idesc = mma_idesc(ci.y);
+                    const uint64_t db = descB + (uint32_t)slot * (kTcN * K * 2 / 16);
+                    if (ok && g >= (uint32_t)kTcAcc)
+                        ok = mbar_wait_bounded(&bar_acc[acc], ((g - kTcAcc) / kTcAcc) & 1u);
+                    if (!ok) break;
+                    tc_fence_after();
+#pragma unroll
+                    for (int ks = 0; ks < KS; ++ks)
+                        mma_bf16(taddr + acc * kTcN, descA + ks * 16, db + ks * 16, idesc,
+                                 ks > 0 ? 1u : 0u);
+                    mma_commit(&bar_mma[acc]);
+                    mma_commit(&bar_slot[slot]);
+                    s_chunk[acc] = ci;
+                    mbar_arrive(&bar_mma[acc]);
+                    issued = c + 1;
+                }
+                if (!ok) {
+                    abort_now();
+                    if (issued > 0) {   // the MMAs in flight
+                        const uint32_t g = g0 + issued - 1;
+                        mbar_wait_bounded(&bar_slot[g % kTcRing], (g / kTcRing) & 1u);
+                    }
+                }
+                ++a_tiles;
             }
+            __syncwarp();
+            g0 += nch;
+        }
+    } else {
+        // ---------------------------------------------------------- epilogue
+        const int half = warp >> 2;                // column half of the chunk
+        const int row = 32 * (warp & 3) + lane;    // TMEM lane / query row
+        const float r2 = a.r2;
+        const int Kout = a.K;
+        uint32_t* sv_slot = Sv + warp * kTcSurvCap;
+        uint8_t* sv_row = reinterpret_cast<uint8_t*>(Sv + (kTcEpi / 32) * kTcSurvCap) + warp * kTcSurvCap;
+        unsigned long long n_surv = 0, n_acc = 0;
+
+        for (uint32_t par = 0;; par ^= 1u) {
+            __syncthreads();   // the task is ready
+            const TcTask& ct = s_task[par];
+            if (ct.done) break;
+            const Task tk = ct.t;
+            const int nch = ct.nch;
+            const EventHdr& h = a.ev[tk.ev];
+            int32_t* counts = a.counts ? a.counts : h.counts;
+            int32_t* oidx = a.counts ? a.idx : h.idx;
+            float* od2 = a.counts ? a.dist2 : h.dist2;
+            const int qs = (tk.qslot & ~7) + row;
+            const bool active = qs >= tk.qslot && qs < tk.qslot + tk.nq;
+            const int qorig = active ? a.qperm[qs] : 0;
+            if (!h.valid) {
+                // grid built from non-finite input: empty rows (frnn_sync reports it)
+                if (active) {
+                    for (int e = 0; e < Kout && !a.csr; ++e) {
+                        oidx[(int64_t)qorig * Kout + e] = -1;
+                        od2[(int64_t)qorig * Kout + e] = INFINITY;
+                    }
+                    counts[qorig] = 0;
+                    if (a.degree) a.degree[qorig] = 0;
+                }
+                continue;
+            }
+            // this thread's query: float32 coordinates (shared: the recheck
+            // reads them from any lane)
+            if (half == 0) {
+                const float4* q4 = reinterpret_cast<const float4*>(a.qpts + (int64_t)(active ? qs : 0) * DP);
+#pragma unroll
+                for (int k4 = 0; k4 < DP / 4; ++k4) reinterpret_cast<float4*>(Qs + row * DP)[k4] = __ldg(q4 + k4);
+                s_cnt[row] = 0;
+            }
+            const float tx = active ? __fmul_rd(0.5f, __fsub_rd(a.qn[qs], ct.theta)) : INFINITY;
+            asm volatile("bar.sync 1, %0;" ::"n"(kTcEpi) : "memory");
+
             const int self_slot = a.self ? qs : -1;
-            uint16_t* sv = Sv + warp * kTcSurvCap;
+            int fill = 0;   // survivors waiting for the recheck
+            // recheck m entries from place p on, one per lane: the exact contract
+            // on the float32 rows (the candidate's from L2)
+            auto recheck = [&](int p, int m) {
+                __syncwarp();
+                if (lane < m) {
+                    const int r = sv_row[p + lane], cs = (int)sv_slot[p + lane];
+                    const float4* f4 = reinterpret_cast<const float4*>(a.rpts + (int64_t)cs * DP);
+                    const float* qv = Qs + r * DP;
+                    float f[DP];
+#pragma unroll
+                    for (int k4 = 0; k4 < DP / 4; ++k4) {
+                        const float4 x = __ldg(f4 + k4);
+                        f[4 * k4] = x.x;
+                        f[4 * k4 + 1] = x.y;
+                        f[4 * k4 + 2] = x.z;
+                        f[4 * k4 + 3] = x.w;
+                    }
+                    const int32_t orig = __ldg(a.rperm + cs);
+                    float sd = 0.f;
+#pragma unroll
+                    for (int k = 0; k < D; ++k) {
+                        const float d = __fsub_rn(qv[k], f[k]);
+                        sd = __fadd_rn(sd, __fmul_rn(d, d));
+                    }
+                    if (sd <= r2) {
+                        ++n_acc;
+                        const int pos = atomicAdd(&s_cnt[r], 1);
+                        if (pos < kTcList) {
+                            Ld[pos * kTcLStr + r] = sd;
+                            Li[pos * kTcLStr + r] = orig;
+                        }
+                    }
+                }
+                __syncwarp();
+            };
+            // survivors of one group of 32 columns starting at slot c0: each
+            // lane appends its own, behind those of the lanes before it
+            auto collect = [&](uint32_t mask, int c0) {
+                while (__any_sync(kFull, mask != 0)) {
+                    const int mine = __popc(mask);
+                    int pos = mine;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int v = __shfl_up_sync(kFull, pos, o);
+                        if (lane >= o) pos += v;
+                    }
+                    const int total = __shfl_sync(kFull, pos, 31);
+                    pos += fill - mine;
+                    // (what finds no place stays in the mask for the next round)
+                    while (mask && pos < kTcSurvCap) {
+                        const int j = __ffs(mask) - 1;
+                        mask &= mask - 1u;
+                        sv_slot[pos] = (uint32_t)(c0 + j);
+                        sv_row[pos] = (uint8_t)row;
+                        ++pos;
+                    }
+                    const int got = min(total, kTcSurvCap - fill);
+                    fill += got;
+                    n_surv += (lane == 0) ? got : 0;
+                    while (fill >= 32) {
+                        fill -= 32;
+                        recheck(fill, 32);
+                    }
+                }
+            };
             for (int c = 0; c < nch; ++c) {
                 const uint32_t g = g0 + c;
-                // accumulator ready and the chunk's staged coordinates visible
                 if (!aborted()) {
-                    if (!mbar_wait_bounded(&bar_mma[g % kTcAcc], (g / kTcAcc) & 1u) ||
-                        !mbar_wait_bounded(&bar_b[g % kTcRing], (g / kTcRing) & 1u))
-                        abort_now();
+                    if (!mbar_wait_bounded(&bar_mma[g % kTcAcc], (g / kTcAcc) & 1u)) abort_now();
                 }
                 __syncwarp();
                 tc_fence_after();
+                uint32_t masks[2] = {0u, 0u};
+                int c0h = 0;
                 if (!__shfl_sync(0xffffffffu, aborted(), 0)) {
-                    int start, n, lo, hi;
-                    chunk_info(s_ct, c, start, n, lo, hi);
-                    const float* F = Fs + (size_t)(g % kTcRing) * kTcN * DP;
+                    const int4 ci = s_chunk[g % kTcAcc];   // (start, n, lo, hi)
                     const uint32_t tbase =
                         taddr + ((uint32_t)(32 * (warp & 3)) << 16) + (g % kTcAcc) * kTcN;
-                    const int cend = min(n, kTcN / 2 * (half + 1));
-#pragma unroll 1
-                    for (int col0 = kTcN / 2 * half; col0 < cend; col0 += 32) {   // n: multiple of 32
-                        float v[32];
-                        __syncwarp();
-                        tmem_ld32(tbase + col0, v);
-                        float mx = fmax3(v[0], v[1], v[2]);
+                    c0h = ci.x + kTcN / 2 * half;
 #pragma unroll
-                        for (int j = 3; j < 31; j += 2) mx = fmax3(mx, v[j], v[j + 1]);
-                        mx = fmaxf(mx, v[31]);
-                        if (!__any_sync(0xffffffffu, mx >= tx)) continue;
-                        // columns of this group inside the chunk's own row range
-                        const int c0 = start + col0;
-                        const int jlo = max(lo - c0, 0), jhi = min(hi - c0, 32);
-                        uint32_t valid =
-                            jhi > jlo ? (((jhi - jlo) == 32 ? 0xffffffffu
-                                                            : ((1u << (jhi - jlo)) - 1u))
-                                         << jlo)
-                                      : 0u;
-                        if (self_slot >= c0 && self_slot < c0 + 32)
-                            valid &= ~(1u << (self_slot - c0));
-                        uint32_t mask = 0;
-                        if (mx >= tx) {
+                    for (int gr = 0; gr < 2; ++gr) {
+                        const int col0 = kTcN / 2 * half + 32 * gr;
+                        if (col0 < ci.y) {   // n: a multiple of 32
+                            uint32_t rv[32];
+                            __syncwarp();
+                            tmem_ld32_nowait(tbase + col0, rv);
+                            tmem_wait_ld();
+                            // maxima of the four octets of columns, then of all 32
+                            float oct[4];
 #pragma unroll
-                            for (int j = 0; j < 32; ++j)
-                                if (v[j] >= tx) mask |= 1u << j;
-                            mask &= valid;
-                        }
-                        // compact the warp's (row, column) survivors, then
-                        // recheck them with all 32 lanes
-                        const int nb = __popc(mask);
-                        int off = nb;
+                            for (int o = 0; o < 4; ++o) {
+                                const auto v = [&](int j) { return __uint_as_float(rv[8 * o + j]); };
+                                oct[o] = fmax3(fmax3(v(0), v(1), v(2)), fmax3(v(3), v(4), v(5)),
+                                               fmaxf(v(6), v(7)));
+                            }
+                            const float mx = fmaxf(fmax3(oct[0], oct[1], oct[2]), oct[3]);
+                            if (__any_sync(0xffffffffu, mx >= tx)) {
+                                // columns of this group inside the chunk's own row range
+                                const int c0 = ci.x + col0;
+                                const int jlo = max(ci.z - c0, 0), jhi = min(ci.w - c0, 32);
+                                uint32_t valid =
+                                    jhi > jlo ? (((jhi - jlo) == 32 ? 0xffffffffu
+                                                                    : ((1u << (jhi - jlo)) - 1u))
+                                                 << jlo)
+                                              : 0u;
+                                if ((unsigned)(self_slot - c0) < 32u) valid &= ~(1u << (self_slot - c0));
+                                uint32_t mask = 0;
 #pragma unroll
-                        for (int o = 1; o < 32; o <<= 1) {
-                            const int t2 = __shfl_up_sync(0xffffffffu, off, o);
-                            if (lane >= o) off += t2;
-                        }
-                        const int total = __shfl_sync(0xffffffffu, off, 31);
-                        off -= nb;
-                        while (mask) {
-                            const int j = __ffs(mask) - 1;
-                            mask &= mask - 1;
-                            sv[off++] = (uint16_t)((lane << 5) | j);
-                        }
-                        __syncwarp();
-                        n_surv += (lane == 0) ? total : 0;
-                        for (int b = 0; b < total; b += 32) {
-                            if (b + lane < total) {
-                                const int pr = sv[b + lane];
-                                const int r = 32 * (warp & 3) + (pr >> 5);
-                                const int cs = c0 + (pr & 31);
-                                // exact contract from the staged float32 coordinates
-                                const float* f = F + (size_t)(cs - start) * DP;
-                                const float* qv = Qs + r * DP;
-                                float sd = 0.f;
+                                for (int o = 0; o < 4; ++o) {
+                                    // (most octets hold no survivor of any lane)
+                                    if (__any_sync(0xffffffffu, oct[o] >= tx)) {
 #pragma unroll
-                                for (int k = 0; k < D; ++k) {
-                                    const float d = __fsub_rn(qv[k], f[k]);
-                                    sd = __fadd_rn(sd, __fmul_rn(d, d));
-                                }
-                                if (sd <= r2) {
-                                    ++n_acc;
-                                    const int pos = atomicAdd(&s_cnt[r], 1);
-                                    if (pos < kTcList) {   // original index looked up here
-                                        Ld[pos * kTcLStr + r] = sd;
-                                        Li[pos * kTcLStr + r] = a.rperm[cs];
+                                        for (int j = 0; j < 8; ++j)
+                                            if (__uint_as_float(rv[8 * o + j]) >= tx) mask |= 1u << (8 * o + j);
                                     }
                                 }
+                                masks[gr] = mask & valid;
                             }
                         }
-                        __syncwarp();
                     }
                 }
+                // the accumulator goes back before the survivors are looked at:
+                // they lie close together (16 of 100 groups hold them, 16 each),
+                // and a warp that has some no longer holds up the others
                 tc_fence_before();
                 mbar_arrive(&bar_acc[g % kTcAcc]);
-                mbar_arrive(&bar_slot[g % kTcRing]);
+                collect(masks[0], c0h);
+                collect(masks[1], c0h + 32);
             }
-        }
-        __syncthreads();
-        if (aborted()) break;
-        g0 += nch;
-        if (nch > 0) ++task_no;
-        if (producer) continue;
+            recheck(0, fill);
+            g0 += nch;
+            asm volatile("bar.sync 1, %0;" ::"n"(kTcEpi) : "memory");   // lists complete
 
-        // every query sorts its own list by (d2, original index), all threads
-        // in parallel (register bitonic network, see sort_list)
-        const int cnt = s_cnt[row];
-        const bool spill = active && cnt > kTcList;
-        if (half == 0) {
-            sort_list(Ld + row, Li + row, kTcLStr, (active && !spill) ? cnt : 0, nullptr);
-            if (active && !spill) counts[qorig] = min(cnt, Kout);
-            if (active && spill && a.csr) counts[qorig] = kCsrSpill;   // counted by the selection kernel
-            if (active && !spill && a.degree) a.degree[qorig] = cnt;
-        }
-        if (spill && half == 0) {
-            // longer than the list: the exact selection kernel finishes this row
-            const int pos = atomicAdd(a.ovf_count, 1);
-            if (pos < a.ovf_cap) {
-                a.ovf[pos].qslot = qs;
-                a.ovf[pos].ev = tk.ev;
-            } else {
-                atomicOr(a.status, kStatusCapacity);
+            const int cnt = s_cnt[row];
+            const bool spill = active && cnt > kTcList;
+            if (half == 0) {
+                if (active && !spill) counts[qorig] = min(cnt, Kout);
+                if (active && spill && a.csr) counts[qorig] = kCsrSpill;   // counted by the selection kernel
+                if (active && !spill && a.degree) a.degree[qorig] = cnt;
+                if (spill) {
+                    // longer than the list: the exact selection kernel finishes this row
+                    const int pos = atomicAdd(a.ovf_count, 1);
+                    if (pos < a.ovf_cap) {
+                        a.ovf[pos].qslot = qs;
+                        a.ovf[pos].ev = tk.ev;
+                    } else {
+                        atomicOr(a.status, kStatusCapacity);
+                    }
+                }
             }
-        }
-        // rows sorted by the half-0 threads; then coalesced row writes, each
-        // epilogue warp 16 of the 128 rows
-        asm volatile("bar.sync 1, %0;" ::"n"(kTcEpi) : "memory");
-        const unsigned skip = __ballot_sync(0xffffffffu, !active || spill);   // rows 32(w%4)..
-        for (int qq = 0; qq < 16; ++qq) {
-            const int ql = 16 * half + qq;                 // lane of this row in the warp
-            if (skip & (1u << ql)) continue;
-            const int r = 32 * (warp & 3) + ql;
-            const int c = min(__shfl_sync(0xffffffffu, cnt, ql), Kout);
-            const int qo = __shfl_sync(0xffffffffu, qorig, ql);
+            // each epilogue warp sorts 16 of the 128 rows and writes them
+            {
+                const int n = __shfl_sync(kFull, active && !spill ? cnt : 0, 16 * half + (lane & 15));
+                const unsigned most = __reduce_max_sync(kFull, (unsigned)n);
+                const int r0 = 32 * (warp & 3) + 16 * half;
+                if (most > 16) {
+                    sort_columns<16>(Ld, Li, r0, n);
+                } else if (most > 1) {
+                    sort_columns<8>(Ld, Li, r0, n);
+                }
+            }
+            const unsigned skip = __ballot_sync(0xffffffffu, !active || spill);   // rows 32(w%4)..
             const int rstride = a.csr ? kCsrStageW : Kout;   // compact: staging row, no padding
-            int32_t* irow = oidx + (int64_t)qo * rstride;
-            float* drow = od2 + (int64_t)qo * rstride;
-            for (int e = lane; e < (a.csr ? c : Kout); e += 32) {
-                const bool real = e < c;
-                irow[e] = real ? Li[e * kTcLStr + r] : -1;
-                drow[e] = real ? Ld[e * kTcLStr + r] : INFINITY;
+            // rows of whole, aligned 16-byte pieces (a compact row's last one
+            // may run past its entries, not past its staging row)
+            const bool vec = (rstride & 3) == 0 &&
+                             ((reinterpret_cast<uintptr_t>(oidx) | reinterpret_cast<uintptr_t>(od2)) & 15) == 0;
+            for (int qq = 0; qq < 16; ++qq) {
+                const int ql = 16 * half + qq;                 // lane of this row in the warp
+                if (skip & (1u << ql)) continue;
+                const int r = 32 * (warp & 3) + ql;
+                const int c = min(__shfl_sync(0xffffffffu, cnt, ql), Kout);
+                const int qo = __shfl_sync(0xffffffffu, qorig, ql);
+                const int w = a.csr ? c : Kout;
+                int32_t* irow = oidx + (int64_t)qo * rstride;
+                float* drow = od2 + (int64_t)qo * rstride;
+                if (vec) {
+                    for (int e = 4 * lane; e < w; e += 128) {
+                        int4 iv = make_int4(-1, -1, -1, -1);
+                        float4 dv = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+                        if (e < c) {
+                            iv.x = Li[e * kTcLStr + r];
+                            dv.x = Ld[e * kTcLStr + r];
+                        }
+                        if (e + 1 < c) {
+                            iv.y = Li[(e + 1) * kTcLStr + r];
+                            dv.y = Ld[(e + 1) * kTcLStr + r];
+                        }
+                        if (e + 2 < c) {
+                            iv.z = Li[(e + 2) * kTcLStr + r];
+                            dv.z = Ld[(e + 2) * kTcLStr + r];
+                        }
+                        if (e + 3 < c) {
+                            iv.w = Li[(e + 3) * kTcLStr + r];
+                            dv.w = Ld[(e + 3) * kTcLStr + r];
+                        }
+                        *reinterpret_cast<int4*>(irow + e) = iv;
+                        *reinterpret_cast<float4*>(drow + e) = dv;
+                    }
+                } else {
+                    for (int e = lane; e < w; e += 32) {
+                        const bool real = e < c;
+                        irow[e] = real ? Li[e * kTcLStr + r] : -1;
+                        drow[e] = real ? Ld[e * kTcLStr + r] : INFINITY;
+                    }
+                }
             }
         }
-    }
-    if (a.stat_survivors && !producer) {
-        atomicAdd(a.stat_survivors, n_surv);
-        atomicAdd(a.stat_accepted, n_acc);
+        if (a.stat_survivors) {
+            atomicAdd(a.stat_survivors, n_surv);
+            atomicAdd(a.stat_accepted, n_acc);
+        }
     }
     tc_fence_before();
     __syncthreads();
