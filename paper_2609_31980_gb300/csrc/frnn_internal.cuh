@@ -241,7 +241,6 @@ struct QueryArgs {
     const int64_t* row_off;      // CSR row offsets (ovf_mode 2)
     int64_t row_cap;             // entries idx / dist2 hold (ovf_mode 2): rows past it are skipped
     uint64_t* scratch;           // half-cell scan: kScratchKeys keys per warp (NULL: none)
-    uint64_t f2_one, f2_neg_one, f2_neg_zero;   // 1, -1 and -0 twice (query_half.cu, fma2)
     int32_t list_cap;            // entries it keeps per query: the list's, and kMoreCap with the scratch
     // compact output of the half-cell scan: pool entries behind the staging
     // rows (idx / dist2 from entry pool0 on), and the counter of those taken

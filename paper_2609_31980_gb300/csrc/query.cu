@@ -810,9 +810,6 @@ static QueryArgs query_args(const QueryLaunch& q) {
     a.degree = q.degree;
     a.row_off = q.row_off;
     a.row_cap = q.row_cap;
-    a.f2_one = 0x3f8000003f800000ull;
-    a.f2_neg_one = 0xbf800000bf800000ull;
-    a.f2_neg_zero = 0x8000000080000000ull;
     a.scratch = q.scratch;
     a.list_cap = 32 + (q.scratch ? kMoreCap : 0);
     a.pool0 = q.pool0;

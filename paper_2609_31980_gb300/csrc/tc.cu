@@ -32,24 +32,41 @@
 // path's output must equal the oracle's bit for bit), and the tightest slack
 // is what the false-candidate rate measures.
 //
-// Kernel organisation (one persistent CTA per SM, 8 warps, 512 TMEM columns):
-//   * a producer warp issues cp.async.bulk copies of the A tile (128 query
-//     rows) and, per chunk of up to 128 candidates, of the B tile into a ring
-//     (up to eight deep), and the MMAs (K/16 instructions per chunk) into one
-//     of two TMEM accumulators (2 x 128 columns; two CTAs per SM share the 512);
-//   * eight epilogue warps: warp w reads TMEM lanes 32 (w % 4).. and one half
-//     of the columns with tcgen05.ld 32x32b.x32, tests 32 pairs per thread with
-//     a 3-input max tree, looks closer only at the octets of columns in which
-//     some lane's maximum reaches t(x), and appends the survivors to a buffer;
-//     whenever 32 have come together, over groups and chunks, the warp's lanes
-//     recheck one each exactly, the candidate's float32 row from L2.  (A group
-//     of 32 x 32 pairs holds 1.7 survivors at 500k x 12: rechecking each
-//     group's own from staged coordinates left 30 lanes idle.)
-//   * per-query survivor lists in shared memory are sorted by (d2, index)
-//     with a register network and written as coalesced rows.  Lists longer
-//     than the capacity go to the exact selection kernel (query.cu).
+// Kernel organisation (persistent, two CTAs per SM of 10 warps and 256 TMEM
+// columns each; a task is 128 query slots of one row of cells):
+//   * a loading warp takes the next task, lists its chunks (up to 128
+//     candidates each) and sends for the query tile and for the chunks'
+//     operands with cp.async.bulk, into a ring up to eight deep, while the
+//     other warps still work on the task before;
+//   * an MMA warp issues K/16 instructions per chunk into one of two TMEM
+//     accumulators of 128 columns;
+//   * eight epilogue warps: warp w reads TMEM lanes 32 (w % 4).. of accumulator
+//     w / 4, so every other chunk, with tcgen05.ld 32x32b.x32; it tests 32
+//     pairs per thread with a 3-input max tree, looks closer only at the octets
+//     of columns in which some lane's maximum reaches t(x), gives the
+//     accumulator back and only then collects the survivors (a prefix sum over
+//     the lanes) in a buffer; whenever 32 have come together, over groups and
+//     chunks, its lanes recheck one each exactly, the candidate's float32 row
+//     from L2;
+//   * per-query survivor lists in shared memory are sorted by (d2, index) by
+//     pairs of lanes (warp_sort.cuh), 16 rows a warp, and written as coalesced
+//     rows.  Lists longer than the capacity go to select.cu.
 // Every mbarrier wait is bounded; on a timeout the CTA records the status,
 // stops, waits (bounded) for its copies and MMAs in flight and frees TMEM.
+//
+// What bounds it: latency.  500k x 12 on three axes (4,077 tasks of 31 chunks,
+// 1.9 G pairs, 6.3 M survivors in 16 % of the groups): 770 us, issue 42 % of
+// the slots with 19 warps an SM, tensor pipe 13 %; the lists and the operand
+// ring fill shared memory at two CTAs.  The steps, build and query, K = 128:
+// 1184 us with one warp for copies and MMAs, accumulators held during the
+// rechecks and candidate coordinates staged (D = 16: 1985, one CTA per SM) ->
+// 1105 (survivors rechecked 32 at a time from L2 rows, which 30 lanes idled
+// through before; D = 16: 1061) -> 1037 (accumulators given back early, next
+// task prepared during the last) -> 959 (loads and MMAs in two warps, 16-byte
+// row stores) -> 863 (32-bit sorting keys in all warps, prefix-sum appends) ->
+// 865 (a warp takes whole chunks instead of half of each: 50k x 12 210 -> 202;
+// D = 8, 500k 876 -> 863).  Slower: sixteen epilogue warps of 56 registers
+// (1542), both halves' TMEM loads in flight at once (1338, spills).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -64,14 +81,13 @@ constexpr int kTcM = 128;        // queries per task = MMA M = TMEM lanes
 constexpr int kTcN = 128;        // candidates per chunk = MMA N (multiple of 32)
 constexpr int kTcAcc = 2;        // TMEM accumulators in flight (kTcAcc * kTcN = kTcCols)
 constexpr int kTcEpi = 256;      // epilogue threads: warp w < 8 owns TMEM lanes 32 (w % 4)..
-                                 // and column half w / 4 of every chunk
+                                 // and accumulator w / 4
 constexpr int kTcThreads = kTcEpi + 64;   // + a loading warp (tasks, bulk copies) + an MMA warp
 constexpr int kTcLStr = kTcM + 1;         // list table: one column per query row
 constexpr int kTcMaxChunks = 128;         // chunk table entries kept in shared memory
 constexpr int kTcMaxRows = 256;           // neighbour rows per task (3^5 on a six-axis grid of half cells)
 constexpr int kTcCols = 256;     // TMEM columns per CTA: two accumulators (2 CTAs / SM)
-// (the producer warp is warp 4; epilogue warps 0..3 own the TMEM lane quarters)
-constexpr int kTcList = 30;      // per-query survivor list capacity (2 CTAs / SM up to D = 12)
+constexpr int kTcList = 30;      // per-query survivor list capacity (2 CTAs / SM)
 static_assert(kTcList <= kCsrStageW, "a staged compact row holds a whole list");
 
 __host__ __device__ constexpr int tc_k_for(int D) { return ((3 * D + 2) + 15) / 16 * 16; }
@@ -428,8 +444,8 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_query(TcArgs a) {
             mbar_init(&bar_slot[i], 1);
         }
         for (int i = 0; i < kTcAcc; ++i) {
-            mbar_init(&bar_mma[i], 2);        // the MMAs' commit and the producer
-            mbar_init(&bar_acc[i], kTcEpi);   // every epilogue thread, every chunk
+            mbar_init(&bar_mma[i], 2);        // the MMAs' commit and the MMA warp
+            mbar_init(&bar_acc[i], kTcEpi / kTcAcc);   // its epilogue threads, every chunk
         }
         s_abort = 0;
         fence_mbar_init();
@@ -645,7 +661,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_query(TcArgs a) {
         }
     } else {
         // ---------------------------------------------------------- epilogue
-        const int half = warp >> 2;                // column half of the chunk
+        const int half = warp >> 2;                // accumulator: every other chunk
         const int row = 32 * (warp & 3) + lane;    // TMEM lane / query row
         const float r2 = a.r2;
         const int Kout = a.K;
@@ -726,11 +742,11 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_query(TcArgs a) {
                 }
                 __syncwarp();
             };
-            // survivors of one group of 32 columns starting at slot c0: each
+            // survivors of 64 columns starting at slot c0: each
             // lane appends its own, behind those of the lanes before it
-            auto collect = [&](uint32_t mask, int c0) {
+            auto collect = [&](uint64_t mask, int c0) {
                 while (__any_sync(kFull, mask != 0)) {
-                    const int mine = __popc(mask);
+                    const int mine = __popcll(mask);
                     int pos = mine;
 #pragma unroll
                     for (int o = 1; o < 32; o <<= 1) {
@@ -741,7 +757,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_query(TcArgs a) {
                     pos += fill - mine;
                     // (what finds no place stays in the mask for the next round)
                     while (mask && pos < kTcSurvCap) {
-                        const int j = __ffs(mask) - 1;
+                        const int j = __ffsll((long long)mask) - 1;
                         mask &= mask - 1u;
                         sv_slot[pos] = (uint32_t)(c0 + j);
                         sv_row[pos] = (uint8_t)row;
@@ -756,27 +772,27 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_query(TcArgs a) {
                     }
                 }
             };
-            for (int c = 0; c < nch; ++c) {
+            // this warp's chunks: those of its accumulator
+            for (int c = (int)((g0 ^ (uint32_t)half) & 1u); c < nch; c += kTcAcc) {
                 const uint32_t g = g0 + c;
                 if (!aborted()) {
-                    if (!mbar_wait_bounded(&bar_mma[g % kTcAcc], (g / kTcAcc) & 1u)) abort_now();
+                    if (!mbar_wait_bounded(&bar_mma[half], (g / kTcAcc) & 1u)) abort_now();
                 }
                 __syncwarp();
                 tc_fence_after();
-                uint32_t masks[2] = {0u, 0u};
-                int c0h = 0;
+                uint64_t masks[2] = {0, 0};
+                int start = 0;
                 if (!__shfl_sync(0xffffffffu, aborted(), 0)) {
-                    const int4 ci = s_chunk[g % kTcAcc];   // (start, n, lo, hi)
+                    const int4 ci = s_chunk[half];   // (start, n, lo, hi)
                     const uint32_t tbase =
-                        taddr + ((uint32_t)(32 * (warp & 3)) << 16) + (g % kTcAcc) * kTcN;
-                    c0h = ci.x + kTcN / 2 * half;
-#pragma unroll
-                    for (int gr = 0; gr < 2; ++gr) {
-                        const int col0 = kTcN / 2 * half + 32 * gr;
-                        if (col0 < ci.y) {   // n: a multiple of 32
+                        taddr + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)half * kTcN;
+                    start = ci.x;
+#pragma unroll 4
+                    for (int gr = 0; gr < kTcN / 32; ++gr) {
+                        if (32 * gr < ci.y) {   // n: a multiple of 32
                             uint32_t rv[32];
                             __syncwarp();
-                            tmem_ld32_nowait(tbase + col0, rv);
+                            tmem_ld32_nowait(tbase + 32 * gr, rv);
                             tmem_wait_ld();
                             // maxima of the four octets of columns, then of all 32
                             float oct[4];
@@ -789,7 +805,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_query(TcArgs a) {
                             const float mx = fmaxf(fmax3(oct[0], oct[1], oct[2]), oct[3]);
                             if (__any_sync(0xffffffffu, mx >= tx)) {
                                 // columns of this group inside the chunk's own row range
-                                const int c0 = ci.x + col0;
+                                const int c0 = start + 32 * gr;
                                 const int jlo = max(ci.z - c0, 0), jhi = min(ci.w - c0, 32);
                                 uint32_t valid =
                                     jhi > jlo ? (((jhi - jlo) == 32 ? 0xffffffffu
@@ -807,7 +823,10 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_query(TcArgs a) {
                                             if (__uint_as_float(rv[8 * o + j]) >= tx) mask |= 1u << (8 * o + j);
                                     }
                                 }
-                                masks[gr] = mask & valid;
+                                {
+                                    const uint64_t mv = (uint64_t)(mask & valid) << (32 * (gr & 1));
+                                    if (gr < 2) masks[0] |= mv; else masks[1] |= mv;
+                                }
                             }
                         }
                     }
@@ -816,9 +835,9 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_query(TcArgs a) {
                 // they lie close together (16 of 100 groups hold them, 16 each),
                 // and a warp that has some no longer holds up the others
                 tc_fence_before();
-                mbar_arrive(&bar_acc[g % kTcAcc]);
-                collect(masks[0], c0h);
-                collect(masks[1], c0h + 32);
+                mbar_arrive(&bar_acc[half]);
+#pragma unroll 1
+                for (int hf = 0; hf < 2; ++hf) collect(hf ? masks[1] : masks[0], start + 64 * hf);
             }
             recheck(0, fill);
             g0 += nch;
