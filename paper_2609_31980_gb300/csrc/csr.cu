@@ -24,6 +24,8 @@ namespace {
 constexpr int kCsrThreads = 1024;
 constexpr int kCsrItems = 8;
 constexpr int kCsrChunk = kCsrThreads * kCsrItems;
+constexpr int kGatherRows = 8;   // rows a warp copies at once (k_csr_gather)
+static_assert(32 % kGatherRows == 0, "ranges of rows start at multiples of 32");
 
 __device__ __forceinline__ int64_t row_count(const int32_t* cnt, int64_t i, int64_t M) {
     return i < M ? (int64_t)(cnt[i] & kCsrCountMask) : 0;
@@ -137,32 +139,62 @@ __global__ void __launch_bounds__(256) k_csr_gather(const int32_t* cnt, const in
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     // rows [row0, row1) (row0 a multiple of 32)
-    for (int64_t w = (row0 >> 5) + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-         w * 32 < row1; w += nw) {
-        const int64_t i = w * 32 + lane;
-        const int32_t c = i < row1 ? cnt[i] : 0;
+    for (int64_t w = row0 / kGatherRows + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+         w * kGatherRows < row1; w += nw) {
+        const int64_t i = w * kGatherRows + lane;
+        const bool real = lane < kGatherRows && i < row1;
+        const int32_t c = real ? cnt[i] : 0;
         // spilled rows: written by the selection kernel
         const int own = (c & kCsrSpill) ? 0 : (c & kCsrCountMask);
         const int64_t src = (c & kCsrPool) ? *reinterpret_cast<const int64_t*>(sidx + i * kCsrStageW)
                                            : i * kCsrStageW;
-        const int64_t dst = i < row1 ? offsets[i] : 0;
-        const int rows = (int)min((int64_t)32, row1 - w * 32);
-#pragma unroll 4
-        for (int r = 0; r < rows; ++r) {
+        const int64_t dst = real ? offsets[i] : 0;
+        // cap: entries the output holds (a caller that gathers before it knows
+        // the edge count passes its capacity; the call then fails when the
+        // count exceeds it, and nothing past it is written)
+        int32_t x[kGatherRows];
+        float y[kGatherRows];
+#pragma unroll
+        for (int r = 0; r < kGatherRows; ++r) {
+            const int n = __shfl_sync(0xffffffffu, own, r);
+            const int64_t s = __shfl_sync(0xffffffffu, src, r);
+            x[r] = 0;
+            y[r] = 0.f;
+            if (lane < n) {
+                x[r] = __ldg(sidx + s + lane);
+                y[r] = __ldg(sd2 + s + lane);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < kGatherRows; ++r) {
+            const int n = __shfl_sync(0xffffffffu, own, r);
+            const int64_t d = __shfl_sync(0xffffffffu, dst, r);
+            if (lane < n && d + lane < cap) {
+                idx[d + lane] = x[r];
+                dist2[d + lane] = y[r];
+            }
+        }
+        if (!__any_sync(0xffffffffu, own > 32)) continue;
+        for (int r = 0; r < kGatherRows; ++r) {   // rows in the pool
             const int n = __shfl_sync(0xffffffffu, own, r);
             const int64_t s = __shfl_sync(0xffffffffu, src, r);
             const int64_t d = __shfl_sync(0xffffffffu, dst, r);
-            // cap: entries the output holds (a caller that gathers before
-            // it knows the edge count passes its capacity; the call then
-            // fails when the count exceeds it, and nothing past it is written)
-            if (lane < n && d + lane < cap) {
-                idx[d + lane] = __ldg(sidx + s + lane);
-                dist2[d + lane] = __ldg(sd2 + s + lane);
-            }
-            for (int e = 32 + lane; e < n; e += 32) {
-                if (d + e < cap) {
-                    idx[d + e] = __ldg(sidx + s + e);
-                    dist2[d + e] = __ldg(sd2 + s + e);
+            for (int e = 32 + lane; e < n; e += 96) {
+#pragma unroll
+                for (int u = 0; u < 3; ++u) {
+                    x[u] = 0;
+                    y[u] = 0.f;
+                    if (e + 32 * u < n) {
+                        x[u] = __ldg(sidx + s + e + 32 * u);
+                        y[u] = __ldg(sd2 + s + e + 32 * u);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 3; ++u) {
+                    if (e + 32 * u < n && d + e + 32 * u < cap) {
+                        idx[d + e + 32 * u] = x[u];
+                        dist2[d + e + 32 * u] = y[u];
+                    }
                 }
             }
         }
@@ -188,7 +220,7 @@ void enqueue_csr_gather(const int32_t* cnt, const int64_t* offsets, const int32_
                         cudaStream_t st, int64_t cap, int64_t row0, int64_t row1) {
     if (row1 < 0) row1 = M;
     if (row1 <= row0) return;
-    const int64_t warps = ceil_div(row1 - row0, 32);
+    const int64_t warps = ceil_div(row1 - row0, kGatherRows);
     const int64_t blocks = std::min<int64_t>(ceil_div(warps, 8), (int64_t)num_sms * 8);
     launch_pdl(k_csr_gather, dim3((unsigned)std::max<int64_t>(blocks, 1)), dim3(256), 0, st, cnt,
                offsets, sidx, sd2, M, idx, dist2, cap, row0, row1);
