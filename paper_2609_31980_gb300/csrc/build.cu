@@ -239,136 +239,155 @@ __device__ void event_params(EventHdr* hdr, int e, int D, int32_t* bbox, float r
                              int axes_mode, int naxes_req);
 
 // Per-event bounding boxes, and the zeroing of the cell counts.  One CTA takes
-// `sub` build blocks (256 points each, staged through shared memory with
-// 16-byte loads), keeps its points' extremes in registers and merges them once
-// per event into one of kBBoxCopies copies of the event's box (copy = block mod
-// kBBoxCopies), so that no address takes more than a few atomics.  The event's
-// last block to finish (a counter beside copy 0, taken after a memory fence)
-// combines the copies and derives the grid parameters; the zeroing of the other
-// blocks runs beside that chain.  `sub` build blocks a CTA: as many as make one
-// wave of kBoxWave CTAs, at most eight (each costs a round trip: 300k x 8 build
-// + query with 2, 4 and 8: 141, 148, 155 us; 1 M x 3 216, 214, 213).  One build
-// block a CTA, reduced by shuffles, and the zeroing in a launch of its own
-// measured 14 + 5 us at 300k x 8.
+// `sub` build blocks (256 points each); the ones that belong to one event are
+// one run of floats, read as 16-byte pieces, four in flight a thread.  The
+// threads that read (box_threads(D) of 256) stride by a multiple of D, so a
+// thread meets the same four coordinates every time and keeps their extremes
+// in registers; once per event the CTA's extremes are merged into one of
+// kBBoxCopies copies of the event's box (copy = block mod kBBoxCopies), so that
+// no address takes more than a few atomics.  The event's last block to finish
+// (a counter beside copy 0, taken after a memory fence) combines the copies and
+// derives the grid parameters; the zeroing of the other blocks runs beside that
+// chain.  `sub` build blocks a CTA: as many as make one wave of kBoxWave CTAs,
+// at most eight (a wave of 608, 304 or 1216 CTAs, build + query at 300k x 8:
+// 138.7, 140.8, 142.1 us).  What bounds it is the chain from the first load to
+// the derived parameters and, from a million points on, memory.  With the rows
+// staged in shared memory, build block by build block: 300k x 8 141.4 -> 138.7
+// us, 1 M x 3 215.3 -> 206.8, 500k x 12 335 -> 328, 16 events x 8 1551 -> 1513.
 constexpr int kBoxWave = 608;
 constexpr int kBoxMost = 8;
+
+// Threads of 256 that read a run of rows of D floats in 16-byte pieces: as many
+// as make 4 x threads a multiple of D.
+__host__ __device__ constexpr int box_threads(int D) {
+    const int period = D % 4 == 0 ? D / 4 : (D % 2 == 0 ? D / 2 : D);
+    return kBuildPtsPerBlock - kBuildPtsPerBlock % period;
+}
+
 __global__ void __launch_bounds__(kBuildPtsPerBlock, 4) k_bbox(EventHdr* hdr, int32_t* blk_start, int64_t* cell_off,
                                                             int E, int nblk, int sub, int D, int32_t* bbox,
                                                             int32_t* status, float r, int m, int axes_mode, int naxes_req,
                                                             int32_t* counts, int64_t L, int32_t* scalars,
                                                             OneEventTables t1) {
     pdl_trigger();
-    extern __shared__ float sm[];
-    __shared__ int32_t red_mn[kMaxD][kBuildPtsPerBlock / 32];
-    __shared__ int32_t red_mx[kMaxD][kBuildPtsPerBlock / 32];
+    __shared__ int32_t red_mn[4 * kBuildPtsPerBlock], red_mx[4 * kBuildPtsPerBlock];
     __shared__ int red_bad, s_last;
-    const bool pad = (D & 3) == 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int T = box_threads(D);
     // a one-event build reads its input (which no kernel of the chain writes)
     // before it waits for the previous work; else the tables come first
     if (!t1.set) pdl_wait();
-    int32_t mn[kMaxD], mx[kMaxD];   // ordered ints
-    bool bad = false;
-    auto clear = [&]() {
-#pragma unroll
-        for (int k = 0; k < kMaxD; ++k) {
-            mn[k] = INT_MAX;
-            mx[k] = INT_MIN;
-        }
-        bad = false;
-    };
-    // merge what the registers hold of event e (nb of its build blocks)
-    auto flush = [&](int e, int nb) {
-        if (threadIdx.x == 0) red_bad = 0;
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < kMaxD; ++k) {
-            if (k < D) {
-                const int32_t a = __reduce_min_sync(0xffffffffu, mn[k]);
-                const int32_t b = __reduce_max_sync(0xffffffffu, mx[k]);
-                if (lane == 0) {
-                    red_mn[k][warp] = a;
-                    red_mx[k][warp] = b;
-                }
-            }
-        }
-        if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&red_bad, 1);
-        __syncthreads();
-        int32_t* bb = bbox + ((int64_t)e * kBBoxCopies + (blockIdx.x % kBBoxCopies)) * kBBoxStride;
-        if (threadIdx.x < (unsigned)D) {
-            const int k = threadIdx.x;
-            int32_t a = INT_MAX, b = INT_MIN;
-            for (int w = 0; w < kBuildPtsPerBlock / 32; ++w) {
-                a = min(a, red_mn[k][w]);
-                b = max(b, red_mx[k][w]);
-            }
-            atomicMin(bb + k, a);
-            atomicMax(bb + 16 + k, b);
-        }
-        if (threadIdx.x == 0 && red_bad) {
-            atomicOr(bb + 32, 1);
-            atomicOr(status, kStatusNonFinite);
-        }
-        __threadfence();   // this block's box updates before its count
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const int total = t1.set ? t1.nblk : blk_start[e + 1] - blk_start[e];
-            int32_t* done = bbox + (int64_t)e * kBBoxCopies * kBBoxStride + kBBoxDone;
-            s_last = atomicAdd(done, nb) == total - nb;
-        }
-        __syncthreads();
-        if (!s_last) return;
-        __threadfence();   // every other block's updates before the reads
-        if (t1.set) {
-            copy_header(hdr, t1.hdr);
-            if (threadIdx.x == 0) {
-                blk_start[0] = 0;
-                blk_start[1] = t1.nblk;
-                cell_off[0] = 0;
-                cell_off[1] = t1.cell_end;
-            }
-            __syncthreads();
-        }
-        event_params(hdr, e, D, bbox, r, m, axes_mode, naxes_req);
-        __syncthreads();
-    };
-    clear();
-    int e_cur = -1, e_blocks = 0;
+    bool waited = !t1.set, zeroed = false;
     const int b1 = min((int)(blockIdx.x + 1) * sub, nblk);
-    bool waited = !t1.set;
-    for (int b = blockIdx.x * sub; b < b1; ++b) {
+    int b = blockIdx.x * sub;
+    while (b < b1) {
         const int e = t1.set ? 0 : find_event(blk_start, E, b);
-        if (e != e_cur && e_cur >= 0) {   // (several events only: the wait is done)
-            flush(e_cur, e_blocks);
-            clear();
-            e_blocks = 0;
-        }
-        e_cur = e;
-        ++e_blocks;
+        const int b_end = t1.set || e == E - 1 ? b1 : min(b1, blk_start[e + 1]);
         const float* refs = t1.set ? t1.hdr.refs : hdr[e].refs;
         const int64_t n = t1.set ? t1.hdr.n : hdr[e].n;
         const int64_t p0 = (int64_t)(t1.set ? b : b - blk_start[e]) * kBuildPtsPerBlock;
-        const int np = (int)max((int64_t)0, min((int64_t)kBuildPtsPerBlock, n - p0));
-        __syncthreads();   // the previous block's rows have been read
-        if (np > 0) stage_floats(sm, refs + p0 * D, np * D, pad);
-        __syncthreads();
-        if ((int)threadIdx.x < np) {
-            const StagedRow p{sm, (int)threadIdx.x * D, pad};
+        const int np = (int)max((int64_t)0, min((int64_t)(b_end - b) * kBuildPtsPerBlock, n - p0));
+        // thread t < T: elements head + 4 (t + i T) + c of the run; the head
+        // and tail short of 16 bytes (at most three each) go to threads 0.. and
+        // 32.. one by one
+        const float* src = refs + p0 * D;
+        const int nf = np * D;
+        const int head = min(nf, (int)((16u - (uint32_t)(reinterpret_cast<uintptr_t>(src) & 15u)) & 15u) >> 2);
+        const int n4 = (nf - head) >> 2;
+        int32_t mn[4], mx[4];   // ordered ints
 #pragma unroll
-            for (int k = 0; k < kMaxD; ++k) {
-                if (k < D) {
-                    const float v = p[k];
-                    bad |= !isfinite(v);
-                    const int32_t x = float_to_ordered(v);
-                    mn[k] = min(mn[k], x);
-                    mx[k] = max(mx[k], x);
+        for (int c = 0; c < 4; ++c) {
+            mn[c] = INT_MAX;
+            mx[c] = INT_MIN;
+        }
+        bool bad = false;
+        if ((int)threadIdx.x < T) {
+            const float4* s4 = reinterpret_cast<const float4*>(src + head);
+            constexpr int kAhead = 4;   // loads in flight per thread
+            for (int i0 = threadIdx.x; i0 < n4; i0 += kAhead * T) {
+                float4 v[kAhead];
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u)   // (past the end: the run's piece at i0 again)
+                    v[u] = __ldg(s4 + (i0 + u * T < n4 ? i0 + u * T : i0));
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    const float f[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        bad |= !isfinite(f[c]);
+                        const int32_t x = float_to_ordered(f[c]);
+                        mn[c] = min(mn[c], x);
+                        mx[c] = max(mx[c], x);
+                    }
                 }
             }
         }
+        int odd_at = -1;
+        if ((int)threadIdx.x < head) odd_at = threadIdx.x;
+        if (threadIdx.x >= 32 && (int)threadIdx.x - 32 < nf - head - 4 * n4) odd_at = head + 4 * n4 + (int)threadIdx.x - 32;
+        const float odd = odd_at >= 0 ? __ldg(src + odd_at) : 0.f;
+        bad |= !isfinite(odd);
+        if (!waited) pdl_wait();
+        waited = true;
+        if (!zeroed) zero_share(counts, L / 4, scalars);
+        zeroed = true;
+        // merge
+        if (threadIdx.x == 0) red_bad = 0;
+        *reinterpret_cast<int4*>(red_mn + 4 * threadIdx.x) = make_int4(mn[0], mn[1], mn[2], mn[3]);
+        *reinterpret_cast<int4*>(red_mx + 4 * threadIdx.x) = make_int4(mx[0], mx[1], mx[2], mx[3]);
+        __syncthreads();
+        int32_t* bb = bbox + ((int64_t)e * kBBoxCopies + (blockIdx.x % kBBoxCopies)) * kBBoxStride;
+        for (int k = warp; k < D; k += kBuildPtsPerBlock / 32) {
+            // entry q of the tables is an element of coordinate (head + q) % D
+            int32_t lo = INT_MAX, hi = INT_MIN;
+            for (int q = (k + 4 * D - head) % D + lane * D; q < 4 * T; q += 32 * D) {
+                lo = min(lo, red_mn[q]);
+                hi = max(hi, red_mx[q]);
+            }
+            lo = __reduce_min_sync(0xffffffffu, lo);
+            hi = __reduce_max_sync(0xffffffffu, hi);
+            if (lane == 0) {
+                atomicMin(bb + k, lo);
+                atomicMax(bb + 16 + k, hi);
+            }
+        }
+        if (odd_at >= 0) {
+            atomicMin(bb + odd_at % D, float_to_ordered(odd));
+            atomicMax(bb + 16 + odd_at % D, float_to_ordered(odd));
+        }
+        if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&red_bad, 1);
+        __threadfence();   // this block's box updates before its count
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            if (red_bad) {
+                atomicOr(bb + 32, 1);
+                atomicOr(status, kStatusNonFinite);
+                __threadfence();
+            }
+            const int total = t1.set ? t1.nblk : blk_start[e + 1] - blk_start[e];
+            int32_t* done = bbox + (int64_t)e * kBBoxCopies * kBBoxStride + kBBoxDone;
+            s_last = atomicAdd(done, b_end - b) == total - (b_end - b);
+        }
+        __syncthreads();
+        if (s_last) {
+            __threadfence();   // every other block's updates before the reads
+            if (t1.set) {
+                copy_header(hdr, t1.hdr);
+                if (threadIdx.x == 0) {
+                    blk_start[0] = 0;
+                    blk_start[1] = t1.nblk;
+                    cell_off[0] = 0;
+                    cell_off[1] = t1.cell_end;
+                }
+                __syncthreads();
+            }
+            event_params(hdr, e, D, bbox, r, m, axes_mode, naxes_req);
+        }
+        __syncthreads();   // (the tables and s_last are written again)
+        b = b_end;
     }
     if (!waited) pdl_wait();
-    zero_share(counts, L / 4, scalars);
-    if (e_cur >= 0) flush(e_cur, e_blocks);
+    if (!zeroed) zero_share(counts, L / 4, scalars);
 }
 
 // The start of a build with foreign parameters (a cross-set query's points,
@@ -1648,7 +1667,7 @@ frnn_status enqueue_build(GridBufs& g, const float* const* refs, const BuildOpts
     } else {
         if (!capturing) grid_clean(g, st);
         const int sub = box_sub(g.nblk);
-        launch_pdl(k_bbox, dim3((unsigned)ceil_div(g.nblk, sub)), dim3(kBuildPtsPerBlock), smem_pts, st, g.hdr,
+        launch_pdl(k_bbox, dim3((unsigned)ceil_div(g.nblk, sub)), dim3(kBuildPtsPerBlock), 0, st, g.hdr,
                    g.blk_start, g.cell_off, E, (int)g.nblk, sub, D, g.bbox, d_status, o.r, o.m, o.axes_mode, o.naxes,
                    g.cstart, g.L, g.scalars, t1);
     }
@@ -1673,7 +1692,7 @@ frnn_status enqueue_build_resident(GridBufs& g, const BuildOpts& o, int32_t* d_s
     // (the array's contents are anybody's: its boxes are emptied first)
     launch_pdl(k_box_reset, dim3(blocks_for((int64_t)E * kBBoxCopies * kBBoxStride, 256)), dim3(256), 0, st, g.bbox, E);
     const int sub = box_sub(g.nblk);
-    launch_pdl(k_bbox, dim3((unsigned)ceil_div(g.nblk, sub)), dim3(kBuildPtsPerBlock), smem_pts, st, g.hdr,
+    launch_pdl(k_bbox, dim3((unsigned)ceil_div(g.nblk, sub)), dim3(kBuildPtsPerBlock), 0, st, g.hdr,
                g.blk_start, g.cell_off, E, (int)g.nblk, sub, D, g.bbox, d_status, o.r, o.m, o.axes_mode, o.naxes, g.cstart,
                g.L, g.scalars, OneEventTables{});
     enqueue_sort(g, smem_pts, 0, d_status, st, EarlyPts{});

@@ -124,12 +124,12 @@ __global__ void __launch_bounds__(kCsrThreads) k_csr_down(const int32_t* cnt, in
         offsets[M] = tot + (parts ? parts[blockIdx.x] : 0);
 }
 
-// One warp per 32 consecutive rows, one row a step, its entries on the lanes:
-// a row's entries lie side by side in the staging area (or the pool) and in
-// the output.  Steps are independent and four are in flight, which is what
-// bounds this kernel; finding each lane's row in the 32 rows' flat range of
-// entries first (a five-step search before every load) measured 33 us a
-// quarter of the 300k x 8 event's rows, this 8.
+// One warp per kGatherRows consecutive rows: a row's entries lie side by side
+// in the staging area (or the pool) and in the output.  Latency bounds it, so a
+// warp loads the first 32 entries of all its rows before it stores any, and
+// rows are spread over four times the warps that 32 rows each would give: a
+// quarter of the 300k x 8 event's rows 9.4 us (32 rows a warp, four
+// steps of one row in flight: 23), rows of 84 at 271k x 12 46 us (66).
 __global__ void __launch_bounds__(256) k_csr_gather(const int32_t* cnt, const int64_t* offsets,
                                                     const int32_t* sidx, const float* sd2,
                                                     int64_t M, int32_t* idx, float* dist2,
