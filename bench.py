@@ -2,9 +2,9 @@
 shaped workload: N=300,000 points, D=8, 8,000 clusters x 30 (sigma 0.02) + 60,000
 uniform background in [-1,1]^8, r=0.1, K=64.
 
-One step = the whole hot path on one event: frnn_build_grid (cell ids, counting
-sort, prefix scan, scatter, tasks) + frnn_query (TMA-staged candidate scan,
-exact FP32 screen, warp top-K).  The metric is queries/s (value) and
+One step = the whole hot path on one event: frnn_build_grid (bounding box and grid
+parameters, cell ids, prefix scan, scatter) + frnn_query (half-cell scan of the
+neighbour rows, exact FP32 distances, sorted rows).  The metric is queries/s (value) and
 neighbour-pairs/s; the dominant kernel's achieved algorithmic bandwidth is
 reported against the measured HBM peak.
 
@@ -122,9 +122,10 @@ def profile_summary(path: str, wl: str):
     summary or the kernel's sources changed since the capture."""
     import hashlib
     key = (path, wl)
-    known = {("grid", "event300k"): ("grid_query_event300k_x8.md", ["query.cu", "frnn_internal.cuh"]),
-             ("rows", "event500k"): ("row_query_event500k_x12.md", ["query_rows.cu", "frnn_internal.cuh"]),
-             ("tc", "event500k"): ("tc_query_event500k_x12.md", ["tc.cu", "frnn_internal.cuh"])}
+    half = ["query_half.cu", "warp_sort.cuh", "frnn_internal.cuh"]
+    known = {("grid", "event300k"): ("half_query_event300k_x8.md", half),
+             ("grid", "event500k"): ("half_query_event500k_x12.md", half),
+             ("tc", "event500k"): ("tc_query_event500k_x12.md", ["tc.cu", "warp_sort.cuh", "frnn_internal.cuh"])}
     if key not in known:
         return None
     name, srcs = known[key]
@@ -210,11 +211,29 @@ def algorithmic_query_bytes(N: int, D: int, K: int) -> int:
     return N * DP * 4 * 2 + N * 4 + N * 4 + N * K * 8
 
 
-def _cell_cap(N: int, naxes: int) -> int:
+def scan_kernel(N: int, D: int, path: str, naxes_requested: int) -> str:
+    """The kernel a one-event self-query runs (mirrors the library's choice):
+    automatic grids take the half-cell scan from five dimensions on and one
+    query per lane below; requested axes the row tasks up to four and the chunk
+    scan at five (so does an automatic grid of nine or more dimensions up to
+    16,384 points, which asks for four)."""
+    if path == "tc":
+        return "k_tc_query"
+    if naxes_requested == 0 and D >= 9 and N <= 16384:
+        naxes_requested = 4
+    if naxes_requested == 0:
+        return "k_half_query" if D >= 5 else "k_low_query"
+    return "k_row_query" if naxes_requested <= 4 else "k_grid_query"
+
+
+def _cell_cap(N: int, D: int, naxes: int) -> int:
     """Cells the library allows an N-point grid requested with naxes axes
-    (mirrors cell_cap_for in build.cu: 18 N for five, 2 N for four)."""
-    c = 18 * N if naxes >= 5 else (2 * N if naxes == 4 else N // 2 + 1)
-    return min(max(16384, c), (1 << 27) if naxes >= 5 else (1 << 24))
+    (mirrors cell_cap_for in build.cu; 0: the automatic choice)."""
+    if naxes == 0 and D >= 5:
+        return min(max(16384, 12 * N), 1 << 26)
+    axes = naxes or D
+    c = 18 * N if axes >= 5 else (4 * N if naxes == 0 else (2 * N if axes == 4 else N // 2 + 1))
+    return min(max(16384, c), (1 << 27) if axes >= 5 else (1 << 24))
 
 
 def _scan_launches(L: int) -> int:
@@ -226,22 +245,20 @@ def _scan_launches(L: int) -> int:
 
 
 def launches_per_step(N: int, D: int, path: str = "grid", naxes_requested: int = 0) -> int:
-    """Kernels one build + query launches (mirrors the library's host code):
-    requested axes 0 (automatic, up to D = 8) or 5 take the chunk scan,
-    1..4 the row-task scan, whose query call first makes the pair copy and
-    the task list."""
-    if naxes_requested == 0 and path != "tc":
-        naxes_requested = 0 if D <= 8 else 4
-    cap_axes = naxes_requested or min(D, 5)
-    L = _cell_cap(N, cap_axes) + 1
-    build = 4 + _scan_launches(L)          # init bbox cellid scan(s) scatter
-    if path == "tc":
-        # operand preparation + 128-query tasks (rowtasks scan emit), tc query, selection pass
+    """Kernels one build + query of one event launches (mirrors the library's
+    host code)."""
+    kernel = scan_kernel(N, D, path, naxes_requested)
+    if naxes_requested == 0 and D >= 9 and N <= 16384:
+        naxes_requested = 4
+    L = _cell_cap(N, D, naxes_requested) + 1
+    if N <= 32768 and L <= 16 * 32768:
+        build = 1                              # one cluster
+    else:
+        build = 5 + (L > 4096 * 4096)          # bbox cellid reduce (parts) down scatter
+    if kernel in ("k_tc_query", "k_row_query"):
+        # operands or pair copy + tasks (rowtasks scan emit), query, selection pass
         return build + 1 + (1 + _scan_launches(L) + 1) + 2
-    if 1 <= naxes_requested <= 4:
-        # pair copy + 16-query tasks (rowtasks scan emit), row-task query, selection pass
-        return build + 1 + (1 + _scan_launches(L) + 1) + 2
-    return build + 2                       # chunk query + selection pass
+    return build + 2                           # query + selection pass
 
 
 def max_over_ranks(x: float, device) -> float:
@@ -334,7 +351,7 @@ def time_config(frnn, pts_np, r, K, path, dev, steps=20, warmup=3, opts=None, tc
 def run_design_points(args, dev):
     """Other configurations of the same path, each timed on its own:
     the 300k x 8 event on grids over three coordinates (cell multiple 1 and 2;
-    the library's default grids five up to D = 8), the uniform 4096 x 3 set, and the
+    the library's default grids up to six), the uniform 4096 x 3 set, and the
     500k x 12 event on the grid scan against the tensor-core pre-filter
     (false-candidate rate of the pre-filter; tensor-pipe activity from the
     committed ncu summary of that kernel)."""
@@ -431,7 +448,7 @@ def run_ours(args):
     torch.cuda.synchronize()
     wall = time.perf_counter() - wall0
     clocks = sampler.stop()
-    kern_is_tc = path == "tc"   # auto: a grid scan (five gridded axes up to D = 8, four above)
+    kern_is_tc = path == "tc"   # auto: a grid scan
     step_ms = [e[0].elapsed_time(e[2]) for e in evs]
     # attribution pass: the same K steps with events at the build/query
     # boundary and around the main query kernel (CUDA events on the launching
@@ -494,8 +511,10 @@ def run_ours(args):
     q_med = statistics.median(query_ms)
     k_mean = sum(kern_ms) / len(kern_ms)
     achieved = qbytes / (k_mean / 1e3) / 1e9
-    prof = profile_summary("tc" if kern_is_tc else ("rows" if gparams["kernel"] == "rows" else "grid"),
-                           args.workload)
+    kernel = scan_kernel(N, D, "tc" if kern_is_tc else "grid", ctx.get_option(frnn.FRNN_OPT_GRID_NAXES))
+    prof = None
+    if kernel in ("k_tc_query", "k_half_query"):
+        prof = profile_summary("tc" if kern_is_tc else "grid", args.workload)
     sm_count = int(getattr(torch.cuda.get_device_properties(dev), "multi_processor_count", 0))
     res = {
         "metric": METRIC,
@@ -523,8 +542,7 @@ def run_ours(args):
         "build_ms_median": statistics.median(build_ms),
         "query_ms_median": q_med,
         "roofline": {"bound": "hbm",
-                     "kernel": "k_tc_query" if kern_is_tc else
-                               ("k_row_query" if gparams["kernel"] == "rows" else "k_grid_query"),
+                     "kernel": kernel,
                      "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                      "kernel_ms_mean": k_mean,
                      "kernel_timing": "CUDA events around each launch of the kernel, on its stream, "
