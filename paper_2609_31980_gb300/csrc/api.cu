@@ -34,7 +34,7 @@ struct frnn_ctx {
     std::string err;
     // options (cell_mult 0 / exit_dims 0: tuned value, else the library default)
     int cell_mult = 0;
-    int grid_naxes = 0;       // gridded axes: 0 tuned / default, else 1..4
+    int grid_naxes = 0;       // gridded axes: 0 tuned / default, else 1..5
     int axes_mode = 0;
     int exit_dims = 0;
     int staging = 0;          // FRNN_OPT_STAGING (0: tuned, else 1)
@@ -198,6 +198,7 @@ static CellKind cell_kind(const frnn_ctx* ctx, int64_t N, int D) {
 // the selection kernel, as when the allocation fails).
 static void ensure_scratch(frnn_ctx* c, int K) {
     if (K <= kLongK || c->scratch_tried || c->budget != 0 || c->small_cells) return;
+    if (stream_capturing(c->stream)) return;   // (an allocation would end the caller's capture)
     c->scratch_tried = true;
     void* p = nullptr;
     if (cudaMalloc(&p, half_scratch_keys(c->num_sms) * sizeof(uint64_t)) != cudaSuccess) {

@@ -1589,13 +1589,13 @@ static int box_sub(int64_t nblk) {
     return (int)std::min<int64_t>(std::max<int64_t>(ceil_div(nblk, kBoxWave), 1), kBoxMost);
 }
 
-// Empty the boxes of buffers that no build has used yet (not inside a capture:
-// a replay would find them empty already).
+// Empty the boxes of buffers that no build has used yet.  Recorded into a
+// caller's capture it has not run yet, so the next build does it again.
 void grid_clean(GridBufs& g, cudaStream_t st) {
     if (g.clean_E >= g.E) return;
     launch_pdl(k_box_reset, dim3(blocks_for((int64_t)g.cap_E * kBBoxCopies * kBBoxStride, 256)), dim3(256), 0, st,
                g.bbox, (int)g.cap_E);
-    g.clean_E = g.cap_E;
+    if (!stream_capturing(st)) g.clean_E = g.cap_E;
 }
 
 frnn_status enqueue_build(GridBufs& g, const float* const* refs, const BuildOpts& o,

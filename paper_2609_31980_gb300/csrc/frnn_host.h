@@ -10,6 +10,16 @@
 
 namespace frnn {
 
+// Whether work on the stream is being captured (by the caller, say).
+inline bool stream_capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &c) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return c != cudaStreamCaptureStatusNone;
+}
+
 // Device buffers of one (possibly multi-event) cell-sorted point set: the
 // reference grid of frnn_build_grid / frnn_query_batched, or the binned query
 // set of a cross-set frnn_query.  One cudaMalloc block, carved into arrays.

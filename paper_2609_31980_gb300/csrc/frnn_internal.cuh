@@ -345,72 +345,4 @@ inline int32_t host_float_to_ordered(float f) {
 
 __host__ __device__ constexpr int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
-// ------------------------------------------------------------ per-thread sort
-// A thread's neighbour list lives in shared memory as a column of a
-// transposed table: entry e at d2[e * stride], idx[e * stride].  With perm,
-// idx holds the reference's sorted slot and sorting maps it to the original
-// index (the tie-break key); without, idx already holds the original index.
-// The sort builds 64-bit keys (d2 bits << 32 | index) (d2 >= +0, so the
-// unsigned order of the keys is the (d2, index) order) and runs a fixed
-// bitonic network in registers: no data-dependent branches, so the lanes of
-// a warp stay converged.
-template <int S>
-__device__ __forceinline__ void sort_list_net(float* d2, int32_t* idx, int stride, int cnt,
-                                              const int32_t* perm) {
-    uint64_t k[S];
-#pragma unroll
-    for (int e = 0; e < S; ++e) {
-        k[e] = ~0ull;
-        if (e < cnt) {
-            const int32_t slot = idx[e * stride];
-            k[e] = ((uint64_t)__float_as_uint(d2[e * stride]) << 32) |
-                   (uint32_t)(perm ? perm[slot] : slot);
-        }
-    }
-#pragma unroll
-    for (int kk = 2; kk <= S; kk <<= 1) {
-#pragma unroll
-        for (int j = kk >> 1; j > 0; j >>= 1) {
-#pragma unroll
-            for (int i = 0; i < S; ++i) {
-                const int l = i ^ j;
-                if (l > i) {
-                    const bool up = (i & kk) == 0;
-                    const uint64_t x = k[i], y = k[l];
-                    const bool sw = up ? (x > y) : (x < y);
-                    k[i] = sw ? y : x;
-                    k[l] = sw ? x : y;
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int e = 0; e < S; ++e) {
-        if (e < cnt) {
-            d2[e * stride] = __uint_as_float((uint32_t)(k[e] >> 32));
-            idx[e * stride] = (int32_t)(uint32_t)k[e];
-        }
-    }
-}
-
-// Sort one thread's list of cnt <= 32 entries (warp-uniform network size).
-__device__ __forceinline__ void sort_list(float* d2, int32_t* idx, int stride, int cnt,
-                                          const int32_t* perm) {
-    const unsigned full = __activemask();
-    int mx = cnt;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(full, mx, o));
-    if (mx <= 1) {
-        if (cnt == 1 && perm) idx[0] = perm[idx[0]];
-    } else if (mx <= 4) {
-        sort_list_net<4>(d2, idx, stride, cnt, perm);
-    } else if (mx <= 8) {
-        sort_list_net<8>(d2, idx, stride, cnt, perm);
-    } else if (mx <= 16) {
-        sort_list_net<16>(d2, idx, stride, cnt, perm);
-    } else {
-        sort_list_net<32>(d2, idx, stride, cnt, perm);
-    }
-}
-
 }  // namespace frnn

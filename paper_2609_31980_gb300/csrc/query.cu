@@ -1,6 +1,10 @@
-// query.cu — grid-path fixed-radius query: per-warp scan of the neighbouring
-// cells with candidate tiles staged in shared memory by bulk copies, the exact
-// float32 distance contract, and warp-level top-K.
+// query.cu — the launch of every grid scan, and the chunk scan: per-warp scan of
+// the neighbouring cells with candidate tiles staged in shared memory by bulk
+// copies (or loaded directly), the exact float32 distance contract, and
+// warp-level top-K.  Grids of five requested axes use it, and automatic grids of
+// five or more dimensions with a cell multiple above 1; the other automatic
+// grids have query_half.cu and query_low.cu, up to four requested axes
+// query_rows.cu.
 //
 // Method (Eq. 1, Sec. 1): for each query, every reference in the cells within
 // +-m cells along each gridded axis is a candidate (complete by the grid's
@@ -32,7 +36,7 @@
 //     order, never contracted), so lanes stay busy however few queries share
 //     a cell.  Accepted pairs (d2, slot) are appended to the query's list in
 //     shared memory (at most kListCap; a longer list sends the row to the
-//     exact selection kernel);
+//     exact selection kernel, select.cu);
 //   * for each query the warp loads the list (entry e on lane e), resolves the
 //     original indices (the deferred lookup, Table 3), sorts the keys (d2 bits
 //     << 32 | original index) with a bitonic network across the lanes, only as

@@ -2,8 +2,9 @@
 // tasks of 16 cell-sorted queries in one row of cells, the union of their
 // neighbour rows streamed through shared memory by bulk copies and screened
 // against all 16 queries at once, an exact float32 recheck and warp-level
-// top-K.  (Grids of five axes, whose cells hold few points, use the chunk
-// kernel of query.cu; the library picks by the requested axis count.)
+// top-K.  (Grids of five requested axes, whose cells hold few points, use
+// the chunk kernel of query.cu; automatic grids query_half.cu and query_low.cu;
+// the library picks by the requested axis count.)
 //
 // Method (Eq. 1, Sec. 1): for each query, every reference in the cells within
 // +-m cells along each gridded axis is a candidate (complete by the grid's
