@@ -333,8 +333,9 @@ typedef enum frnn_option {
     FRNN_OPT_USE_GRAPH = 4,   /* 1 (default): batched calls replay a CUDA graph */
     FRNN_OPT_AUTOTUNE = 5,    /* 1 (default): FRNN_PATH_AUTO consults the tuner;
                                  setting 0 also clears the tuned cache */
-    FRNN_OPT_AUTO_TC = 6,     /* 1 (default): FRNN_PATH_AUTO takes the tensor-core
-                                 path for D >= 8 */
+    FRNN_OPT_AUTO_TC = 6,     /* 1 (default): FRNN_PATH_AUTO may take the tensor-core
+                                 path (tuned, or large sets of D >= 11 on grids
+                                 requested with up to three axes) */
     FRNN_OPT_TC_SURVIVORS = 7,/* read: candidates that passed the tensor-core
                                  pre-filter since the last reset (synchronises);
                                  set (any value): reset both counters */

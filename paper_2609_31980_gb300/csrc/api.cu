@@ -40,7 +40,7 @@ struct frnn_ctx {
     int staging = 0;          // FRNN_OPT_STAGING (0: tuned, else 1)
     int use_graph = 1;
     int autotune = 1;
-    int auto_tc = 1;          // FRNN_PATH_AUTO uses the tensor-core path for D >= 8
+    int auto_tc = 1;          // FRNN_PATH_AUTO may use the tensor-core path (default_tc)
     // workspaces
     GridBufs qset;            // cross-set query binning
     GridBufs batch;           // batched multi-event grid
@@ -227,9 +227,9 @@ static frnn_status alloc_accounted(frnn_ctx* c, GridBufs& g, int E, const int64_
 }
 
 // Path choice: FRNN_PATH_TC forces the tensor-core pre-filter (D >= 8),
-// FRNN_PATH_GRID the scalar grid scan; FRNN_PATH_AUTO takes the tensor-core
-// path for D >= 8 unless the context's option says otherwise.
-static bool default_tc(const frnn_ctx* ctx, int D, int naxes);
+// FRNN_PATH_GRID the scalar grid scan; FRNN_PATH_AUTO takes the tuned choice,
+// else the tensor-core path where default_tc says so.
+static bool default_tc(const frnn_ctx* ctx, int64_t N, int D, int naxes);
 static const frnn_ctx::Tuned* find_tuned(const frnn_ctx* ctx, int64_t N, int D, int K);
 // naxes: gridded axes of the grid being queried (-1: what a build would use now)
 static bool use_tc_path(const frnn_ctx* ctx, int D, unsigned flags, int64_t N = -1, int K = -1,
@@ -241,7 +241,7 @@ static bool use_tc_path(const frnn_ctx* ctx, int D, unsigned flags, int64_t N = 
         const frnn_ctx::Tuned* t = find_tuned(ctx, N, D, K);
         if (t) return t->path == 1;
     }
-    return default_tc(ctx, D, naxes >= 0 ? naxes : build_naxes(ctx, std::max<int64_t>(N, 0), D));
+    return default_tc(ctx, N, D, naxes >= 0 ? naxes : build_naxes(ctx, std::max<int64_t>(N, 0), D));
 }
 
 // Build (or reuse) the tensor-core operands of a point set; accounted in the
@@ -343,12 +343,15 @@ static int build_naxes(const frnn_ctx* ctx, int64_t N, int D) {
     const frnn_ctx::Tuned* t = find_tuned(ctx, N, D, -1);
     return std::min(t ? t->naxes : default_naxes(ctx, N, D), D);
 }
-// default path when nothing is tuned: the tensor-core pre-filter beats the
-// grid scan over three gridded axes from about D = 10 on (0.90 vs 1.26 ms at
-// 500k x 12), but not the scan over four (0.70 ms): its 128-query tasks are
-// poorly filled by the shorter rows of a four-axis grid
-static bool default_tc(const frnn_ctx* ctx, int D, int naxes) {
-    return ctx->auto_tc && D >= 10 && naxes >= 1 && naxes <= 3;
+// default path when nothing is tuned: on grids requested with up to three axes
+// the tensor-core pre-filter, whose 128-query tasks want long rows of cells,
+// beats the row tasks in large sets of many dimensions only (build + query,
+// event sets, three axes, tensor core / row tasks, us): D = 10 500k 862 / 640,
+// 1 M 1696 / 1599; D = 12 500k 856 / 774, 700k 1195 / 1242, 1 M 1750 / 2131; D = 13
+// 300k 548 / 466, 500k 854 / 901; D = 16 50k 199 / 99, 300k 524 / 453, 500k 809 / 879,
+// 1 M 1665 / 2549
+static bool default_tc(const frnn_ctx* ctx, int64_t N, int D, int naxes) {
+    return ctx->auto_tc && D >= 11 && naxes >= 1 && naxes <= 3 && N >= (D >= 13 ? 450000 : 650000);
 }
 
 extern "C" {
