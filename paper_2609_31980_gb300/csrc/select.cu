@@ -138,6 +138,10 @@ __global__ void __launch_bounds__(kWarps * 32, BIG ? 1 : (D <= 8 ? 8 : (D <= 12 
         }
         const Overflow o = a.ovf[at_entry];
         const int ev = BIG ? ~o.ev : o.ev;
+        if constexpr (BIG) {
+            __syncwarp();   // every lane has read the entry
+            if (lane == 0) a.ovf[at_entry].ev = ev;   // no mark outlives the query
+        }
         const EventHdr& h = a.ev[ev];
         const int qs = o.qslot;
         const int qo = a.qperm[qs];

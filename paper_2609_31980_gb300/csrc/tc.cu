@@ -1141,6 +1141,12 @@ frnn_status enqueue_tc_query(const QueryLaunch& q, cudaStream_t st, std::string&
     o.ovf = qs.ovf;
     o.ovf_count = qs.scalars + kScOvfCount;
     o.ovf_cap = a.ovf_cap;
+    // the selection clears the list, as after a grid scan (a compact count
+    // pass leaves it to the fill, or to the next query of this point set)
+    o.ovf_done = qs.scalars + kScOvfDone;
+    o.task_counter = qs.scalars + kScTcCounter;
+    o.reset_ovf = q.ovf_mode == 1 ? 0 : 1;
+    qs.ovf_stale = q.ovf_mode == 1;
     o.path_filter = -1;   // the list only holds rows this launch queued
     o.csr = q.csr;
     o.ovf_mode = q.ovf_mode;
