@@ -76,7 +76,13 @@ struct OneEventTables {
 // A one-event build's input, passed by value to the kernels that stage it:
 // they stage their block's points before waiting for the previous kernel of
 // the chain (no kernel of the chain writes the caller's points, and the
-// header that would locate them is written by k_bbox in this case).
+// header that would locate them is written by k_bbox in this case).  The work
+// that wrote the points is complete by then, although it may itself have let
+// its successors start early: the chain's first kernel waits for it and only
+// then triggers, so nothing later in the chain starts before.  (Triggering
+// first and waiting in k_cellid instead: 0.5 to 1 us slower a chain.  Reading
+// the points before any wait, which is wrong after such work, was 0.5 to 1 us
+// faster a build: 300k x 8 138.7 against 139.7 us, 4096 x 3 20.4 against 21.)
 struct EarlyPts {
     const float* refs;
     int64_t n;
@@ -269,15 +275,15 @@ __global__ void __launch_bounds__(kBuildPtsPerBlock, 4) k_bbox(EventHdr* hdr, in
                                                             int32_t* status, float r, int m, int axes_mode, int naxes_req,
                                                             int32_t* counts, int64_t L, int32_t* scalars,
                                                             OneEventTables t1) {
+    // the first kernel of a chain: the caller's work on the stream may have let
+    // it start early, and wrote the points (see EarlyPts)
+    pdl_wait();
     pdl_trigger();
     __shared__ int32_t red_mn[4 * kBuildPtsPerBlock], red_mx[4 * kBuildPtsPerBlock];
     __shared__ int red_bad, s_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int T = box_threads(D);
-    // a one-event build reads its input (which no kernel of the chain writes)
-    // before it waits for the previous work; else the tables come first
-    if (!t1.set) pdl_wait();
-    bool waited = !t1.set, zeroed = false;
+    bool zeroed = false;
     const int b1 = min((int)(blockIdx.x + 1) * sub, nblk);
     int b = blockIdx.x * sub;
     while (b < b1) {
@@ -327,8 +333,6 @@ __global__ void __launch_bounds__(kBuildPtsPerBlock, 4) k_bbox(EventHdr* hdr, in
         if (threadIdx.x >= 32 && (int)threadIdx.x - 32 < nf - head - 4 * n4) odd_at = head + 4 * n4 + (int)threadIdx.x - 32;
         const float odd = odd_at >= 0 ? __ldg(src + odd_at) : 0.f;
         bad |= !isfinite(odd);
-        if (!waited) pdl_wait();
-        waited = true;
         if (!zeroed) zero_share(counts, L / 4, scalars);
         zeroed = true;
         // merge
@@ -386,7 +390,6 @@ __global__ void __launch_bounds__(kBuildPtsPerBlock, 4) k_bbox(EventHdr* hdr, in
         __syncthreads();   // (the tables and s_last are written again)
         b = b_end;
     }
-    if (!waited) pdl_wait();
     if (!zeroed) zero_share(counts, L / 4, scalars);
 }
 
@@ -394,8 +397,8 @@ __global__ void __launch_bounds__(kBuildPtsPerBlock, 4) k_bbox(EventHdr* hdr, in
 // binned by the reference grid's header src): tables, parameters, zeroed counts.
 __global__ void k_begin_foreign(OneEventTables t1, const EventHdr* src, EventHdr* hdr, int32_t* blk_start,
                                 int64_t* cell_off, int32_t* counts, int32_t* scalars) {
+    pdl_wait();      // (first of its chain: see EarlyPts)
     pdl_trigger();
-    pdl_wait();
     if (blockIdx.x == 0) {
         copy_header(hdr, t1.hdr);
         __syncthreads();
@@ -1171,8 +1174,8 @@ __global__ void __launch_bounds__(kCellThreads) k_cells_down(const EventHdr* hdr
 // the chain catches up.  Build + query, chain / cluster: 4096 x 3 30.8 / 21.1
 // us, 5,000 x 8 40.5 / 24.4, 20,000 x 8 45.8 / 38.4, 32,000 x 8 52.2 / 49.9
 // (eight CTAs without staged rows lost from 13,000 points on).
-//   1 bounding box of the CTA's points (input only, so before the wait for the
-//     previous kernel), zeroing of the cell counts; boxes to every CTA
+//   1 bounding box of the CTA's points, zeroing of the cell counts; boxes to
+//     every CTA
 //   2 grid parameters (one warp of every CTA, redundantly); cell ids, ranks
 //   3 per-warp sums of the counts; CTA sums to every CTA
 //   4 exclusive scan of the counts in place
@@ -1203,6 +1206,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     __shared__ int32_t s_mn[kMaxD], s_mx[kMaxD], s_bad;
     __shared__ int32_t s_box[kSmallCtas][2 * kMaxD + 1], s_all[2 * kMaxD];
     __shared__ int32_t s_wt[kWarps], s_tot[kSmallCtas];
+    pdl_wait();      // (first of its chain: the points may have just been written)
     pdl_trigger();
     cluster.barrier_arrive();   // (every CTA must run before its shared memory is written)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1245,7 +1249,6 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
             }
         }
     }
-    pdl_wait();   // the previous work on the stream may still read what is written from here on
     {
         // all of the cell array, or what the foreign parameters use of it
         const int L = src ? (t1.hdr.rowsort ? src->ncells / src->dims[0] : src->ncells) + 1 : t1.hdr.cell_cap + 1;
