@@ -1192,6 +1192,9 @@ constexpr int64_t kSmallCells = 16 * kSmallMax;   // cell-array entries
 __host__ __device__ constexpr size_t small_stage_floats(int64_t per, int D) {
     return (size_t)per * D + (size_t)per * D / 32 + 1;
 }
+// The most any set needs: the shared-memory limit set before every launch (it
+// is the function's, shared by every thread's calls, so no call may lower it).
+constexpr size_t kSmallSmemMost = sizeof(float) * small_stage_floats(kSmallPer * kSmallThreads, kMaxD);
 
 __global__ void __launch_bounds__(kSmallThreads, 1)
     k_build_small(OneEventTables t1, const EventHdr* src, int per, int D, int DP, float r, int m, int axes_mode,
@@ -1644,7 +1647,7 @@ frnn_status enqueue_build(GridBufs& g, const float* const* refs, const BuildOpts
         const size_t smem = sizeof(float) * small_stage_floats(per, D);
         cudaError_t ce = cudaFuncSetAttribute(k_build_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (ce == cudaSuccess)
-            ce = cudaFuncSetAttribute(k_build_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            ce = cudaFuncSetAttribute(k_build_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmemMost);
         if (ce == cudaSuccess)
             ce = launch_pdl_cluster(k_build_small, dim3(kSmallCtas), dim3(kSmallThreads), smem, st, kSmallCtas, t1,
                                     params_from ? (const EventHdr*)params_from->hdr : nullptr, per, D, g.DP, o.r, o.m,

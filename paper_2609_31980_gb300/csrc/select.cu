@@ -36,6 +36,7 @@ namespace sel {
 constexpr int kWarps = 4;
 constexpr int kSelKeys = 256;                 // buffer of the first pass (keys a warp)
 constexpr int kSelMaxCut = kSelKeys - 64;     // largest K whose cut leaves two rounds of room
+constexpr int kSelMostKeys = 2 * kMaxK;       // the second pass' buffer at the largest K
 
 // Sort the first 32 P keys of buf (entries past n hold any value).
 template <int P>
@@ -323,7 +324,10 @@ template <int D, bool BIG>
 cudaError_t launch(const QueryArgs& a, int cap, int num_sms, cudaStream_t st) {
     auto kern = &k_select<D, BIG>;
     const size_t smem = kWarps * warp_bytes(cap);
-    cudaError_t ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the limit is the function's, shared by every thread's calls: always the
+    // most any K needs, so that no call lowers it under another's launch)
+    constexpr size_t most = kWarps * warp_bytes(BIG ? kSelMostKeys : kSelKeys);
+    cudaError_t ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     if (ce != cudaSuccess) return ce;
     int per_sm = 0;
     ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarps * 32, smem);
