@@ -1653,13 +1653,14 @@ frnn_status enqueue_build(GridBufs& g, const float* const* refs, const BuildOpts
                                     params_from ? (const EventHdr*)params_from->hdr : nullptr, per, D, g.DP, o.r, o.m,
                                     o.axes_mode, o.naxes, g.hdr, g.blk_start, g.cell_off, g.cstart, g.scalars, g.pts,
                                     g.perm, g.cell, d_status);
-        g.tc_ready = false;
-        g.rows_ready = false;
-        if (ce != cudaSuccess) {
-            err = std::string("grid build launch failed: ") + cudaGetErrorString(ce);
-            return FRNN_ERR_CUDA;
+        if (ce == cudaSuccess) {
+            g.tc_ready = false;
+            g.rows_ready = false;
+            return FRNN_OK;
         }
-        return FRNN_OK;
+        // a cluster of this size is not portable: where it cannot be placed
+        // the launch is refused, and the separate kernels build the set
+        cudaGetLastError();
     }
     const size_t smem_pts = sizeof(float) * staged_floats(D);
     const EarlyPts ep{t1.hdr.refs, t1.hdr.n, t1.set};

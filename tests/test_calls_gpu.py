@@ -1,0 +1,76 @@
+"""What the library asks of the CUDA runtime, seen through a copy of it whose
+runtime calls are listed (cuda_calls.cpp): run in child processes that load
+that copy in place of the library."""
+import os
+import subprocess
+import sys
+import textwrap
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+WRAPPED = ("cudaMalloc", "cudaMemsetAsync", "cudaMemcpyAsync", "cudaLaunchKernelExC")
+
+PRELUDE = """
+import ctypes, sys
+import numpy as np
+import torch
+real = ctypes.CDLL
+ctypes.CDLL = lambda p, *a, **k: real(sys.argv[1] if str(p).endswith("libfrnn.so") else p, *a, **k)
+from oracle import oracle
+from paper_2609_31980_gb300 import frnn, synth
+lib = frnn._lib
+lib.calls_bytes.restype = ctypes.c_size_t
+def calls():
+    return [(lib.calls_kind(i), lib.calls_bytes(i)) for i in range(lib.calls_count())]
+def same(got, p, r, K):
+    rows = np.arange(0, len(p), 1 + len(p) // 500)
+    want = oracle.self_query(p, r, K, rows=rows)
+    for a, b in zip((x.cpu().numpy()[rows] for x in got), want):
+        assert np.array_equal(a.view(np.uint32), b.view(np.uint32))
+"""
+
+
+@pytest.fixture(scope="module")
+def listed_lib(tmp_path_factory):
+    from paper_2609_31980_gb300 import build
+    d = tmp_path_factory.mktemp("calls")
+    obj, so = str(d / "cuda_calls.o"), str(d / "listed.so")
+    subprocess.run([build._nvcc(), "-O2", "-std=c++17", "-Xcompiler", "-fPIC", "-c",
+                    os.path.join(HERE, "cuda_calls.cpp"), "-o", obj], check=True)
+    objs = [os.path.join(build.BUILD_DIR, os.path.basename(s)[:-3] + ".o") for s in build.sources()]
+    wraps = [f for w in WRAPPED for f in ("-Xlinker", f"--wrap={w}")]
+    subprocess.run([build._nvcc(), *build.ARCH, "-shared", "-o", so, *objs, obj, *wraps, "-lpthread"], check=True)
+    return so
+
+
+def _child(so, code):
+    r = subprocess.run([sys.executable, "-c", PRELUDE + textwrap.dedent(code), so], cwd=ROOT, timeout=300,
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-4000:]
+
+
+def test_small_sets_build_without_large_clusters(listed_lib):
+    """A device that cannot place a cluster of sixteen CTAs refuses the
+    one-launch build: the separate kernels build the set, no error stays."""
+    _child(listed_lib, """
+        lib.calls_refuse_clusters(1)
+        with frnn.Context() as ctx:
+            for n, D, r, K in ((1, 3, 0.1, 8), (3000, 3, 0.08, 32), (20_000, 8, 0.1, 64), (9_001, 12, 0.12, 64)):
+                p = synth.clustered(n // 50, 40, n - n // 50 * 40, D, 0.01, seed=70)
+                t = torch.from_numpy(p).cuda()
+                lib.calls_reset()
+                g = ctx.build_grid(t, r)
+                same(ctx.query(g, t, r, K), p, r, K)
+                same(ctx.query(g, t, r, K, path="grid"), p, r, K)
+                q = torch.from_numpy(p[:max(1, n // 3)].copy()).cuda()
+                c, i, d = (x.cpu().numpy() for x in ctx.query(g, q, r, K, self_query=False))
+                rows = np.arange(0, len(q), 1 + len(q) // 500)
+                want = oracle.frnn(p[rows], p, r, K)
+                assert np.array_equal(c[rows], want[0]) and np.array_equal(i[rows], want[1])
+                assert np.array_equal(d[rows].view(np.uint32), want[2].view(np.uint32))
+                ctx.sync()
+                assert sum(k == 4 for k, _ in calls()) == 2, calls()
+        """)
