@@ -61,7 +61,12 @@ typedef enum frnn_status {
 #define FRNN_PATH_AUTO 0x0u   /* library (autotuner) chooses the path */
 #define FRNN_PATH_GRID 0x2u   /* uniform-grid scan with the exact screen */
 #define FRNN_PATH_TC 0x4u     /* tensor-core BF16 pre-filter + exact recheck
-                                 (D >= 8 only) */
+                                 (D >= 8 only).  On a default grid (see
+                                 FRNN_OPT_GRID_NAXES) of half cells its first
+                                 query after a build makes a second grid of the
+                                 points, over three axes, kept with the
+                                 pre-filter's operands (4 D + 26 bytes a point
+                                 more, D rounded up to a multiple of 4) */
 
 typedef struct frnn_ctx frnn_ctx;
 typedef struct frnn_grid frnn_grid;

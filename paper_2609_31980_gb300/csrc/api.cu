@@ -19,7 +19,15 @@ struct frnn_grid {
     int D = 0;
     float r = 0.f;
     int naxes = 0;   // gridded axes requested at the build
+    int axes_mode = 0;   // and which ones (FRNN_OPT_GRID_AXES)
     bool half = false;   // half cells (half_cells at the build)
+    // the same points on a grid for tensor-core tiles (tc_set), made with the
+    // first tensor-core query after a build
+    GridBufs tiles;
+    bool tiles_ready = false;
+    size_t device_bytes() const {
+        return g.bytes + g.tc_bytes + g.rows_bytes + tiles.bytes + tiles.tc_bytes;
+    }
 };
 
 struct frnn_ctx {
@@ -244,13 +252,15 @@ static bool use_tc_path(const frnn_ctx* ctx, int D, unsigned flags, int64_t N = 
     return default_tc(ctx, N, D, naxes >= 0 ? naxes : build_naxes(ctx, std::max<int64_t>(N, 0), D));
 }
 
+static frnn_status alloc_batch(frnn_ctx* ctx, int E, const int64_t* n, int D, int K, unsigned flags);
+
 // Build (or reuse) the tensor-core operands of a point set; accounted in the
 // context's memory budget.
 namespace frnn {
 frnn_status ctx_reserve_batch(frnn_ctx* ctx, int E, int64_t n, int D, int K, unsigned flags) {
     if (E < 1 || n < 1) return FRNN_OK;
     std::vector<int64_t> ns(E, n);
-    frnn_status s = alloc_accounted(ctx, ctx->batch, E, ns.data(), D, nullptr);
+    frnn_status s = alloc_batch(ctx, E, ns.data(), D, K, flags);
     if (s != FRNN_OK || !use_tc_path(ctx, D, flags, n, K)) return s;
     std::string err;
     s = tc_reserve(ctx->batch, err);
@@ -354,6 +364,72 @@ static bool default_tc(const frnn_ctx* ctx, int64_t N, int D, int naxes) {
     return ctx->auto_tc && D >= 11 && naxes >= 1 && naxes <= 3 && N >= (D >= 13 ? 450000 : 650000);
 }
 
+// Tensor-core tiles of automatic grids.  A tile is 128 queries of one row of
+// cells against the neighbour rows' points, in chunks of up to 128: half cells
+// over six axes would give it 243 neighbour rows of a handful of points each
+// and few queries to a row (500k x 12 47 ms, 1 M x 8 107 ms).  Such point sets
+// get a grid of their own for the tiles, three axes of cells of r / 2 (as on
+// request), made from the cell-sorted rows with the first tensor-core query
+// after a build and kept with its operands.
+constexpr int kTcAxes = 3;
+static int tc_mult(const frnn_ctx* ctx) { return ctx->cell_mult > 0 ? ctx->cell_mult : 2; }
+
+// The point set a tensor-core query of the grid takes.  Where that grid cannot
+// be had (the context's budget, memory, an allocation inside a caller's
+// capture) the tiles walk the half cells: slower, the same rows.
+static GridBufs& tc_set(frnn_ctx* ctx, frnn_grid* grid) {
+    GridBufs& v = grid->tiles;
+    if (!grid->half || grid->N == 0) return grid->g;
+    if (grid->tiles_ready) return v;
+    const int64_t cap = cell_cap_for(grid->N, kTcAxes);
+    const bool held = v.base && v.tc_base && v.cap_n >= grid->g.n_total && v.cap_L >= cell_entries(cap);
+    if (!held && (stream_capturing(ctx->stream) ||
+                  !budget_allows(ctx, v.bytes, predict_grid_bytes(1, &grid->N, grid->D, &cap))))
+        return grid->g;
+    const size_t before = v.bytes + v.tc_bytes;
+    std::string err;
+    frnn_status s = grid_alloc(v, 1, &grid->N, grid->D, err, &cap);
+    if (!v.base) v.bytes = 0;
+    if (s == FRNN_OK) s = tc_reserve(v, err);
+    ctx->held = ctx->held - std::min(ctx->held, before) + v.bytes + v.tc_bytes;
+    if (s != FRNN_OK) return grid->g;
+    // the points in their original order, in the room the operands take later
+    float* pts = reinterpret_cast<float*>(v.tcA);
+    BuildOpts o;
+    o.r = grid->r;
+    o.m = tc_mult(ctx);
+    o.naxes = kTcAxes;
+    o.axes_mode = grid->axes_mode;
+    const float* ev_refs[1] = {pts};
+    // (a non-finite coordinate has been reported by the grid's own build)
+    if (enqueue_unsort(grid->g, pts, ctx->stream) != cudaSuccess ||
+        enqueue_build(v, ev_refs, o, nullptr, ctx->d_status + 1, ctx->stream, false, err) != FRNN_OK)
+        return grid->g;
+    grid->tiles_ready = true;
+    return v;
+}
+
+// Gridded axes and cell multiple of one event of a batch.
+struct EventGrid {
+    int naxes, m;
+    int64_t cap;   // cells allowed
+};
+static EventGrid event_grid(const frnn_ctx* ctx, int64_t n, int D, int K, unsigned flags) {
+    EventGrid g{build_naxes(ctx, n, D), build_mult(ctx, n, D), 0};
+    if (half_cells(D, g.naxes, g.m) && use_tc_path(ctx, D, flags, n, K)) {   // (see tc_set)
+        g = {kTcAxes, tc_mult(ctx), 0};
+        g.cap = cell_cap_for(n, g.naxes);
+    } else {
+        g.cap = cell_cap_for(n, cap_axes(g.naxes, D), cell_kind(ctx, n, D));
+    }
+    return g;
+}
+static frnn_status alloc_batch(frnn_ctx* ctx, int E, const int64_t* n, int D, int K, unsigned flags) {
+    std::vector<int64_t> caps(E);
+    for (int e = 0; e < E; ++e) caps[e] = event_grid(ctx, n[e], D, K, flags).cap;
+    return alloc_accounted(ctx, ctx->batch, E, n, D, caps.data());
+}
+
 extern "C" {
 
 const char* frnn_version(void) { return "0.1.0"; }
@@ -439,13 +515,13 @@ frnn_status frnn_grid_destroy(frnn_grid* grid) {
     if (grid->ctx) {
         cudaStreamSynchronize(grid->ctx->stream);
         grid->ctx->csr_pending = false;
-        grid->ctx->held -= std::min(grid->ctx->held,
-                                    grid->g.bytes + grid->g.tc_bytes + grid->g.rows_bytes);
+        grid->ctx->held -= std::min(grid->ctx->held, grid->device_bytes());
         grid->ctx->grids.erase(grid);
     } else {
         cudaDeviceSynchronize();   // context gone: its stream may still hold work on the buffers
     }
     grid_free(grid->g);
+    grid_free(grid->tiles);
     delete grid;
     return FRNN_OK;
 }
@@ -483,6 +559,7 @@ frnn_status frnn_destroy(frnn_ctx* ctx) {
         ctx->grids.erase(g);
         g->ctx = nullptr;
         grid_free(g->g);
+        grid_free(g->tiles);
         delete g;
     }
     // grids the caller still holds stay valid for frnn_grid_destroy only
@@ -537,6 +614,8 @@ frnn_status frnn_build_grid(frnn_ctx* ctx, const float* refs, int64_t N, int D, 
     o.naxes = build_naxes(ctx, N, D);
     o.axes_mode = ctx->axes_mode;
     g->naxes = o.naxes;
+    g->axes_mode = o.axes_mode;
+    g->tiles_ready = false;
     g->half = half_cells(D, o.naxes, o.m);
     g->g.h_hdr[0].half = g->half ? 1 : 0;
     std::string err;
@@ -584,8 +663,11 @@ static frnn_status query_impl(frnn_ctx* ctx, const frnn_grid* grid, const float*
     if ((flags & FRNN_PATH_TC) && grid->D < 8)
         return fail(ctx, FRNN_ERR_UNSUPPORTED, "the tensor-core path needs D >= 8");
     if (M == 0) return FRNN_OK;
+    const bool tc = use_tc_path(ctx, grid->D, flags, grid->N, K, grid->naxes);
+    frnn_grid* mgrid = const_cast<frnn_grid*>(grid);   // tensor-core operands are a lazy cache
+    GridBufs& rg = tc ? tc_set(ctx, mgrid) : mgrid->g;
     QueryLaunch q{};
-    q.rset = &grid->g;
+    q.rset = &rg;
     q.r2 = r * r;
     q.K = K;
     q.self = self ? 1 : 0;
@@ -628,23 +710,21 @@ static frnn_status query_impl(frnn_ctx* ctx, const frnn_grid* grid, const float*
         }
     }
     std::string err;
-    GridBufs& rg = const_cast<frnn_grid*>(grid)->g;   // tensor-core operands are a lazy cache
     if (self) {
         q.qset = &rg;
     } else {
-        const int64_t cap = grid->g.h_hdr[0].cell_cap;
+        const int64_t cap = rg.h_hdr[0].cell_cap;
         s = alloc_accounted(ctx, ctx->qset, 1, &M, grid->D, &cap);
         if (s != FRNN_OK) return s;
         // the half-cell scan needs its queries by rows of cells only
-        ctx->qset.h_hdr[0].rowsort =
-            grid->half && !use_tc_path(ctx, grid->D, flags, grid->N, K, grid->naxes) ? 1 : 0;
+        ctx->qset.h_hdr[0].rowsort = grid->half && !tc ? 1 : 0;
         BuildOpts o;
         const float* ev_q[1] = {queries};
-        s = enqueue_build(ctx->qset, ev_q, o, &grid->g, ctx->d_status, ctx->stream, false, err);
+        s = enqueue_build(ctx->qset, ev_q, o, &rg, ctx->d_status, ctx->stream, false, err);
         if (s != FRNN_OK) return fail(ctx, s, err);
         q.qset = &ctx->qset;
     }
-    if (use_tc_path(ctx, grid->D, flags, grid->N, K, grid->naxes)) {
+    if (tc) {
         s = prepare_tc(ctx, rg, rg);
         if (s == FRNN_OK && !self) s = prepare_tc(ctx, ctx->qset, rg);
         if (s != FRNN_OK) return s;
@@ -847,8 +927,9 @@ static frnn_status enqueue_batched(frnn_ctx* ctx, const frnn_event* ev, int n_ev
         h.idx = ev[e].idx;
         h.dist2 = ev[e].dist2;
         // per event: autotuned cell multiple, axes and path for its size class
-        h.m = build_mult(ctx, ev[e].n, D);
-        h.naxes = build_naxes(ctx, ev[e].n, D);
+        const EventGrid eg = event_grid(ctx, ev[e].n, D, K, flags);
+        h.m = eg.m;
+        h.naxes = eg.naxes;
         h.path = batch_path(ctx, ev[e].n, D, K, flags);
         h.half = h.path == 3 ? 1 : 0;
         if (ev[e].n > 0) any_path[h.path] = true;
@@ -983,7 +1064,7 @@ frnn_status frnn_query_batched(frnn_ctx* ctx, const frnn_event* ev, int n_events
     ev = ordered.data();
     std::vector<int64_t> n(n_events);
     for (int e = 0; e < n_events; ++e) n[e] = ev[e].n;
-    frnn_status s = alloc_accounted(ctx, ctx->batch, n_events, n.data(), D, nullptr);
+    frnn_status s = alloc_batch(ctx, n_events, n.data(), D, K, flags);
     if (s != FRNN_OK) return s;
     bool batch_tc = false, batch_rows = false;
     for (int e = 0; e < n_events; ++e) {

@@ -1713,4 +1713,18 @@ frnn_status enqueue_build_resident(GridBufs& g, const BuildOpts& o, int32_t* d_s
     return FRNN_OK;
 }
 
+// One thread per slot; an odd set's padding slot has no point.
+__global__ void k_unsort(const float* pts, const int32_t* perm, int64_t n, int D, int DP, float* out) {
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= n) return;
+    float* dst = out + (int64_t)perm[s] * D;
+    for (int k = 0; k < D; ++k) dst[k] = pts[pt_index(s, k, DP)];
+}
+
+cudaError_t enqueue_unsort(const GridBufs& g, float* out, cudaStream_t st) {
+    const int64_t n = g.h_hdr[0].n;
+    if (n > 0) k_unsort<<<blocks_for(n, 256), 256, 0, st>>>(g.pts, g.perm, n, g.D, g.DP, out);
+    return cudaGetLastError();
+}
+
 }  // namespace frnn

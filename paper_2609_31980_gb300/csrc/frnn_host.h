@@ -154,6 +154,9 @@ void enqueue_tasks(GridBufs& g, int W, int A, Task* out, int64_t out_cap, int32_
 frnn_status enqueue_build_resident(GridBufs& g, const BuildOpts& o, int32_t* d_status,
                                    cudaStream_t st, std::string& err);
 
+// The points of a one-event set in their original order: [n, D] floats at out.
+cudaError_t enqueue_unsort(const GridBufs& g, float* out, cudaStream_t st);
+
 // Exclusive scan of n int32 values in place; the total goes to *total.
 void enqueue_scan(int32_t* data, int64_t n, int32_t* parts, int32_t* total, cudaStream_t st);
 int64_t scan_parts_needed(int64_t n);
