@@ -201,6 +201,13 @@ static CellKind cell_kind(const frnn_ctx* ctx, int64_t N, int D) {
     return D <= 4 && naxes == 0 && ctx->budget == 0 && !ctx->small_cells ? CellKind::kLow : CellKind::kPlain;
 }
 
+// Cells a set may have.  A context with a memory budget gives up a few, to make
+// room for the larger headers and the rounding of the cell arrays: a request
+// that fitted its budget without them still does.
+static int64_t cells_for(const frnn_ctx* ctx, int64_t n, int naxes, CellKind kind) {
+    return cell_cap_for(n, naxes, kind) - (ctx->budget != 0 ? 32 : 0);
+}
+
 // The half-cell scan's scratch array, made with the first call that keeps long
 // rows (about 52 MB; none under a memory budget, whose contexts send them to
 // the selection kernel, as when the allocation fails).
@@ -221,7 +228,7 @@ static frnn_status alloc_accounted(frnn_ctx* c, GridBufs& g, int E, const int64_
     std::vector<int64_t> caps(E);
     for (int e = 0; e < E; ++e)
         caps[e] = caps_in ? caps_in[e]
-                          : cell_cap_for(n[e], cap_axes(build_naxes(c, n[e], D), D), cell_kind(c, n[e], D));
+                          : cells_for(c, n[e], cap_axes(build_naxes(c, n[e], D), D), cell_kind(c, n[e], D));
     const size_t old_bytes = g.bytes;
     const size_t need = predict_grid_bytes(E, n, D, caps.data());
     const bool reuse = g.base && need <= g.bytes;
@@ -381,7 +388,7 @@ static GridBufs& tc_set(frnn_ctx* ctx, frnn_grid* grid) {
     GridBufs& v = grid->tiles;
     if (!grid->half || grid->N == 0) return grid->g;
     if (grid->tiles_ready) return v;
-    const int64_t cap = cell_cap_for(grid->N, kTcAxes);
+    const int64_t cap = cells_for(ctx, grid->N, kTcAxes, CellKind::kPlain);
     const bool held = v.base && v.tc_base && v.cap_n >= grid->g.n_total && v.cap_L >= cell_entries(cap);
     if (!held && (stream_capturing(ctx->stream) ||
                   !budget_allows(ctx, v.bytes, predict_grid_bytes(1, &grid->N, grid->D, &cap))))
@@ -418,9 +425,9 @@ static EventGrid event_grid(const frnn_ctx* ctx, int64_t n, int D, int K, unsign
     EventGrid g{build_naxes(ctx, n, D), build_mult(ctx, n, D), 0};
     if (half_cells(D, g.naxes, g.m) && use_tc_path(ctx, D, flags, n, K)) {   // (see tc_set)
         g = {kTcAxes, tc_mult(ctx), 0};
-        g.cap = cell_cap_for(n, g.naxes);
+        g.cap = cells_for(ctx, n, g.naxes, CellKind::kPlain);
     } else {
-        g.cap = cell_cap_for(n, cap_axes(g.naxes, D), cell_kind(ctx, n, D));
+        g.cap = cells_for(ctx, n, cap_axes(g.naxes, D), cell_kind(ctx, n, D));
     }
     return g;
 }

@@ -412,7 +412,8 @@ __global__ void k_begin_foreign(OneEventTables t1, const EventHdr* src, EventHdr
     }
     // (t1.hdr.rowsort: used_entries of the finished header)
     const int used = (t1.hdr.rowsort ? src->ncells / src->dims[0] : src->ncells) + 1;
-    zero_share(counts, (used + kCellChunk - 1) / kCellChunk * (kCellChunk / 4), scalars);
+    const int64_t scanned = (int64_t)(used + kCellChunk - 1) / kCellChunk * kCellChunk;
+    zero_share(counts, min(scanned, cell_entries(t1.hdr.cell_cap)) / 4, scalars);
 }
 
 // Grid parameters of one event (one CTA: its warps combine the box copies,
@@ -1023,8 +1024,8 @@ void enqueue_scan(int32_t* data, int64_t n, int32_t* parts, int32_t* total, cuda
 // ------------------------------------------------------------------ cell scan
 // Exclusive scan of the cell counts, every event's on its own: an event's first
 // slot is known, so events share nothing, and only the entries a grid uses are
-// scanned.  Blocks of kCellChunk entries (an event's region starts on one), 16
-// entries a thread in four 16-byte loads; the down pass sums the totals of its
+// scanned.  Blocks of kCellChunk entries (an event's last one ends with its
+// region), 16 entries a thread in four 16-byte loads; the down pass sums the totals of its
 // event's blocks before it (beyond kCellSumParts of them a pass of one block per
 // event scans the totals first).  300k x 8 (3.5 M cells), reduce + down: 5.0 +
 // 9.6 us with 2,048-entry blocks and 4-byte accesses through shared memory.
@@ -1033,19 +1034,25 @@ constexpr int kCellThreads = 256;
 constexpr int kCellSumParts = 4096;
 static_assert(kCellChunk == 16 * kCellThreads, "four quads a thread");
 
-// Event of a block, its first block, whether the block holds used entries.
+// Event of a block, its first block, whether the block holds used entries, its
+// own entries (from `at` on, in `quads` 16-byte pieces).
 struct CellBlock {
-    int e, first;
+    int e, first, quads;
+    int64_t at;
     bool used;
     __device__ CellBlock(const EventHdr* hdr, int E) {
         int lo = 0, hi = E - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (hdr[mid].cell_off <= (int64_t)blockIdx.x * kCellChunk) lo = mid; else hi = mid - 1;
+            if (hdr[mid].cblk0 <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
         }
         e = lo;
-        first = (int)(hdr[lo].cell_off / kCellChunk);
-        used = ((int)blockIdx.x - first) * kCellChunk < used_entries(hdr[lo]);
+        const EventHdr& h = hdr[lo];
+        first = h.cblk0;
+        const int off = ((int)blockIdx.x - first) * kCellChunk;
+        at = h.cell_off + off;
+        quads = (int)min((int64_t)kCellChunk, cell_entries(h.cell_cap) - off) / 4;
+        used = off < used_entries(h);
     }
 };
 
@@ -1056,10 +1063,11 @@ __global__ void __launch_bounds__(kCellThreads) k_cells_reduce(const EventHdr* h
     __shared__ int32_t red[kCellThreads / 32];
     const CellBlock cb(hdr, E);
     if (!cb.used) return;
-    const int4* c4 = reinterpret_cast<const int4*>(counts + (int64_t)blockIdx.x * kCellChunk) + threadIdx.x;
+    const int4* c4 = reinterpret_cast<const int4*>(counts + cb.at) + threadIdx.x;
     int4 v[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = c4[j * kCellThreads];
+    for (int j = 0; j < 4; ++j)
+        v[j] = (int)threadIdx.x + j * kCellThreads < cb.quads ? c4[j * kCellThreads] : make_int4(0, 0, 0, 0);
     int s = 0;
 #pragma unroll
     for (int j = 0; j < 4; ++j) s += v[j].x + v[j].y + v[j].z + v[j].w;
@@ -1081,7 +1089,7 @@ __global__ void __launch_bounds__(1024) k_cells_parts(const EventHdr* hdr, int32
     const EventHdr& h = hdr[blockIdx.x];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nb = (used_entries(h) + kCellChunk - 1) / kCellChunk;
-    int32_t* p = parts + h.cell_off / kCellChunk;
+    int32_t* p = parts + h.cblk0;
     int carry = 0;
     for (int b0 = 0; b0 < nb; b0 += 1024) {
         const int i = b0 + threadIdx.x;
@@ -1115,10 +1123,11 @@ __global__ void __launch_bounds__(kCellThreads) k_cells_down(const EventHdr* hdr
     const CellBlock cb(hdr, E);
     if (!cb.used) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int4* c4 = reinterpret_cast<int4*>(counts + (int64_t)blockIdx.x * kCellChunk) + threadIdx.x;
+    int4* c4 = reinterpret_cast<int4*>(counts + cb.at) + threadIdx.x;
     int4 v[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = c4[j * kCellThreads];
+    for (int j = 0; j < 4; ++j)
+        v[j] = (int)threadIdx.x + j * kCellThreads < cb.quads ? c4[j * kCellThreads] : make_int4(0, 0, 0, 0);
     int before = 0;   // the event's entries before this block
     if (scanned) {
         if (threadIdx.x == 0) before = parts[blockIdx.x];
@@ -1157,7 +1166,8 @@ __global__ void __launch_bounds__(kCellThreads) k_cells_down(const EventHdr* hdr
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const int x = tot[j * kW + warp] + excl[j];
-        c4[j * kCellThreads] = make_int4(x, x + v[j].x, x + v[j].x + v[j].y, x + v[j].x + v[j].y + v[j].z);
+        if ((int)threadIdx.x + j * kCellThreads < cb.quads)
+            c4[j * kCellThreads] = make_int4(x, x + v[j].x, x + v[j].x + v[j].y, x + v[j].x + v[j].y + v[j].z);
     }
 }
 
@@ -1443,7 +1453,7 @@ void grid_free(GridBufs& g) {
 frnn_status grid_alloc(GridBufs& g, int E, const int64_t* n, int D, std::string& err,
                        const int64_t* caps, int naxes) {
     const int DP = padded_dim(D);
-    int64_t n_total = 0, L = 0, nblk = 0, nchunks = 0;
+    int64_t n_total = 0, L = 0, nblk = 0, nchunks = 0, ncblk = 0, cells = 0;
     g.h_hdr.assign(E, EventHdr{});
     g.h_blk_start.assign(E + 1, 0);
     g.h_cell_off.assign(E + 1, 0);
@@ -1458,13 +1468,16 @@ frnn_status grid_alloc(GridBufs& g, int E, const int64_t* n, int D, std::string&
         nchunks += ceil_div(n[e], kChunkQ);
         g.h_blk_start[e] = (int32_t)nblk;
         g.h_cell_off[e] = L;
+        h.cblk0 = (int32_t)ncblk;
+        ncblk += cell_blocks(cap);
+        cells += cap + 1;
         n_total += (n[e] + 1) & ~(int64_t)1;   // pair-aligned event regions
         L += cell_entries(cap);
         nblk += std::max<int64_t>(1, ceil_div(n[e], kBuildPtsPerBlock));
     }
     g.h_blk_start[E] = (int32_t)nblk;
     g.h_cell_off[E] = L;
-    if (n_total >= INT32_MAX || L >= ((int64_t)1 << 30) ||
+    if (n_total >= INT32_MAX || cells >= ((int64_t)1 << 30) ||
         nblk >= INT32_MAX || nchunks >= INT32_MAX) {
         err = "problem too large for one call (points, cells or tasks exceed the limits)";
         return FRNN_ERR_INVALID_ARG;
@@ -1474,8 +1487,9 @@ frnn_status grid_alloc(GridBufs& g, int E, const int64_t* n, int D, std::string&
     g.DP = DP;
     g.n_total = n_total;
     g.L = L;
+    g.ncblk = ncblk;
     g.nblk = nblk;
-    g.nparts = std::max(scan_parts_needed(L), L / kCellChunk);
+    g.nparts = std::max(scan_parts_needed(L), L / kCellChunk + E);   // (>= ncblk, and grows with L and E)
     g.nchunks = nchunks;
     // the buffers are reused only if every region is large enough, the
     // point rows included (a set of a higher dimension needs wider rows)
@@ -1574,13 +1588,11 @@ static inline unsigned blocks_for(int64_t n, int t) {
 static void enqueue_sort(GridBufs& g, size_t smem_pts, int check_finite, int32_t* d_status,
                          cudaStream_t st, EarlyPts ep) {
     const int E = g.E, D = g.D;
-    // (without host headers, the one event's entries are all of them)
-    auto cap_of = [&](int e) -> int64_t { return g.h_hdr.empty() ? g.L - 1 : g.h_hdr[e].cell_cap; };
     launch_pdl(k_cellid, dim3((unsigned)g.nblk), dim3(kBuildPtsPerBlock), smem_pts, st,
                g.hdr, g.blk_start, E, D, g.cstart, g.cid, g.rnk, check_finite, d_status, ep);
-    const int64_t nb = g.L / kCellChunk;
-    int64_t most = 0;   // blocks of the largest event
-    for (int e = 0; e < E; ++e) most = std::max(most, cell_entries(cap_of(e)) / kCellChunk);
+    const int64_t nb = g.ncblk;
+    int64_t most = g.h_hdr.empty() ? nb : 0;   // blocks of the largest event (without host headers: the only one)
+    for (const EventHdr& h : g.h_hdr) most = std::max(most, cell_blocks(h.cell_cap));
     launch_pdl(k_cells_reduce, dim3((unsigned)nb), dim3(kCellThreads), 0, st, g.hdr, E, g.cstart, g.parts);
     if (most > kCellSumParts)
         launch_pdl(k_cells_parts, dim3((unsigned)E), dim3(1024), 0, st, g.hdr, g.parts);

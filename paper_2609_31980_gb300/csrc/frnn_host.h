@@ -27,7 +27,8 @@ struct GridBufs {
     int E = 0;              // events
     int D = 0, DP = 0;      // dimensions, padded row length (floats)
     int64_t n_total = 0;    // points over all events
-    int64_t L = 0;          // cell-array entries: sum over events of (cell_cap + 1)
+    int64_t L = 0;          // cell-array entries: sum over events of cell_entries(cell_cap)
+    int64_t ncblk = 0;      // blocks of their scan
     int64_t nblk = 0;       // blocks of the per-point build kernels
     int64_t nparts = 0;     // scan partial sums needed
     int64_t nchunks = 0;    // query chunks (kChunkQ slots) over all events

@@ -95,6 +95,7 @@ struct EventHdr {
     int32_t path;          // batched queries: 0 = chunk scan, 1 = tensor-core pre-filter,
                            // 2 = row tasks, 3 = half-cell scan
     int32_t qchunk0;       // first query chunk (kChunkQ slots) of this event in its point set
+    int32_t cblk0;         // first block of this event in the scan of the cell counts
     float ctr[16];         // per-dimension centre of the bounding box (tensor-core operands)
     // query outputs for batched self-queries (row = original point index)
     int32_t* counts;
@@ -112,10 +113,12 @@ struct Task {
 };
 
 // Cell-array entries of an event allowed `cap` cells: one more than the cells
-// (the end of the last one), in whole blocks of the prefix scan.
+// (the end of the last one), in whole 16-byte pieces.
+__host__ __device__ constexpr int64_t cell_entries(int64_t cap) { return (cap + 4) & ~(int64_t)3; }
+// Entries a block of their prefix scan takes, and an event's blocks.
 constexpr int kCellChunk = 4096;
-__host__ __device__ constexpr int64_t cell_entries(int64_t cap) {
-    return (cap + kCellChunk) / kCellChunk * kCellChunk;
+__host__ __device__ constexpr int64_t cell_blocks(int64_t cap) {
+    return (cell_entries(cap) + kCellChunk - 1) / kCellChunk;
 }
 
 // A slot's stored cell id (its `cell` entry without the half bits).

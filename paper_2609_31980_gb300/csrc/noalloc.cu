@@ -86,6 +86,7 @@ static int32_t* carve(GridBufs& g, char* b, int64_t n, int D) {
     g.DP = padded_dim(D);
     g.n_total = (n + 1) & ~(int64_t)1;
     g.L = cell_entries(cap);
+    g.ncblk = cell_blocks(cap);
     g.nblk = std::max<int64_t>(1, ceil_div(n, kBuildPtsPerBlock));
     g.nparts = scan_parts_needed(g.L);
     g.nchunks = ceil_div(n, kChunkQ);   // the header's first chunk is 0
