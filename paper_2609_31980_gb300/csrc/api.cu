@@ -772,12 +772,14 @@ static frnn_status csr_reserve(frnn_ctx* ctx, int64_t M, int K) {
     const size_t rows = (size_t)std::max<int64_t>(M, 1);
     const size_t b_cnt = al(rows * 4);
     const size_t b_parts = al((size_t)csr_parts_needed(M) * 8);
-    // behind the staging rows, without a memory budget: a pool of as many
-    // entries for rows longer than a staging row (none if it cannot be had)
+    // calls whose scan keeps rows longer than a staging row (never under a
+    // memory budget): behind the staging rows a pool of as many entries for
+    // them (none if it cannot be had), and the counter of those taken
+    ensure_scratch(ctx, K);
+    const bool long_rows = K > kLongK && ctx->scratch != nullptr;
     const auto stage_bytes = [&](bool pool) { return al(rows * kCsrStageW * 4 * (pool ? 2 : 1)); };
     const auto total = [&](bool pool) { return b_cnt + 2 * stage_bytes(pool) + b_parts + 256; };
-    ensure_scratch(ctx, K);
-    bool pool = K > kLongK && ctx->scratch != nullptr;
+    bool pool = long_rows;
     if (pool && total(true) > ctx->csr_bytes) {
         cudaStreamSynchronize(ctx->stream);
         void* p = nullptr;
@@ -815,10 +817,12 @@ static frnn_status csr_reserve(frnn_ctx* ctx, int64_t M, int K) {
     ctx->csr_idx = reinterpret_cast<int32_t*>(b + b_cnt);
     ctx->csr_d2 = reinterpret_cast<float*>(b + b_cnt + b_stage);
     ctx->csr_parts = reinterpret_cast<int64_t*>(b + b_cnt + 2 * b_stage);
-    ctx->csr_pool_count = reinterpret_cast<unsigned long long*>(b + b_cnt + 2 * b_stage + b_parts);
+    ctx->csr_pool_count =
+        long_rows ? reinterpret_cast<unsigned long long*>(b + b_cnt + 2 * b_stage + b_parts) : nullptr;
     ctx->csr_pool0 = (int64_t)rows * kCsrStageW;
     ctx->csr_pool_cap = pool ? ctx->csr_pool0 : 0;
-    cudaMemsetAsync(ctx->csr_pool_count, 0, sizeof(unsigned long long), ctx->stream);
+    // (only then: the clear comes between the build and the query)
+    if (long_rows) cudaMemsetAsync(ctx->csr_pool_count, 0, sizeof(unsigned long long), ctx->stream);
     return FRNN_OK;
 }
 

@@ -74,3 +74,24 @@ def test_small_sets_build_without_large_clusters(listed_lib):
                 ctx.sync()
                 assert sum(k == 4 for k, _ in calls()) == 2, calls()
         """)
+
+
+def test_compact_queries_clear_the_pool_only_when_they_use_it(listed_lib):
+    """Rows past the staging width go to a pool in calls that keep more than
+    128 neighbours: only those clear its counter."""
+    _child(listed_lib, """
+        p = synth.clustered(500, 40, 20_000, 8, 0.01, seed=71)
+        t = torch.from_numpy(p).cuda()
+        with frnn.Context() as ctx:
+            g = ctx.build_grid(t, 0.1)
+            for K in (1000, 64, 128, 129, 64):
+                ctx.query_csr(g, t, 0.1, K)
+                ctx.sync()
+                lib.calls_reset()
+                g = ctx.build_grid(t, 0.1, grid=g)
+                ctx.query_csr(g, t, 0.1, K)
+                ctx.self_query_host_csr(p, 0.1, K)
+                ctx.self_query_host_csr(p, 0.1, K)
+                clears = [n for k, n in calls() if k == 2 and n == 8]
+                assert len(clears) == (3 if K > 128 else 0), (K, calls())
+        """)
