@@ -778,7 +778,7 @@ static frnn_status csr_reserve(frnn_ctx* ctx, int64_t M, int K) {
     ensure_scratch(ctx, K);
     const bool long_rows = K > kLongK && ctx->scratch != nullptr;
     const auto stage_bytes = [&](bool pool) { return al(rows * kCsrStageW * 4 * (pool ? 2 : 1)); };
-    const auto total = [&](bool pool) { return b_cnt + 2 * stage_bytes(pool) + b_parts + 256; };
+    const auto total = [&](bool pool) { return b_cnt + 2 * stage_bytes(pool) + b_parts + (long_rows ? 256 : 0); };
     bool pool = long_rows;
     if (pool && total(true) > ctx->csr_bytes) {
         cudaStreamSynchronize(ctx->stream);

@@ -95,3 +95,22 @@ def test_compact_queries_clear_the_pool_only_when_they_use_it(listed_lib):
                 clears = [n for k, n in calls() if k == 2 and n == 8]
                 assert len(clears) == (3 if K > 128 else 0), (K, calls())
         """)
+
+
+def test_compact_budget_holds_the_staging_rows_alone(listed_lib):
+    """Under a memory budget there is no pool: the staging of a compact query
+    is its counts, its rows of 32 and the scan totals, and no byte more."""
+    _child(listed_lib, """
+        n, D = 20_000, 8
+        p = synth.clustered(500, 40, 0, D, 0.01, seed=72)
+        t = torch.from_numpy(p).cuda()
+        al = lambda x: (x + 255) // 256 * 256
+        stage = al(4 * n) + 2 * al(128 * n) + al(8 * (-(-n // 8192)))
+        for K in (64, 200):
+            with frnn.Context(budget_bytes=64 << 20) as ctx:
+                lib.calls_reset()
+                g = ctx.build_grid(t, 0.1)
+                ctx.query_csr(g, t, 0.1, K)
+                ctx.sync()
+                assert (1, stage) in calls(), (K, stage, calls())
+        """)
