@@ -260,6 +260,7 @@ static bool use_tc_path(const frnn_ctx* ctx, int D, unsigned flags, int64_t N = 
 }
 
 static frnn_status alloc_batch(frnn_ctx* ctx, int E, const int64_t* n, int D, int K, unsigned flags);
+static int batch_path(const frnn_ctx* ctx, int64_t n, int D, int K, unsigned flags);
 
 // Build (or reuse) the tensor-core operands of a point set; accounted in the
 // context's memory budget.
@@ -268,6 +269,7 @@ frnn_status ctx_reserve_batch(frnn_ctx* ctx, int E, int64_t n, int D, int K, uns
     if (E < 1 || n < 1) return FRNN_OK;
     std::vector<int64_t> ns(E, n);
     frnn_status s = alloc_batch(ctx, E, ns.data(), D, K, flags);
+    if (s == FRNN_OK && batch_path(ctx, n, D, K, flags) == 3) ensure_scratch(ctx, K);
     if (s != FRNN_OK || !use_tc_path(ctx, D, flags, n, K)) return s;
     std::string err;
     s = tc_reserve(ctx->batch, err);
@@ -414,6 +416,16 @@ static GridBufs& tc_set(frnn_ctx* ctx, frnn_grid* grid) {
         return grid->g;
     grid->tiles_ready = true;
     return v;
+}
+
+// Path of one event of a batch: 0 grid scan by chunks, 3 half-cell scan, 2
+// grid scan by row tasks, 1 tensor core (autotuned per size class, else the
+// defaults).
+static int batch_path(const frnn_ctx* ctx, int64_t n, int D, int K, unsigned flags) {
+    if (use_tc_path(ctx, D, flags, n, K)) return 1;
+    const int naxes = build_naxes(ctx, n, D);
+    if (half_cells(D, naxes, build_mult(ctx, n, D))) return 3;
+    return grid_kernel(naxes) == 1 ? 2 : 0;
 }
 
 // Gridded axes and cell multiple of one event of a batch.
@@ -910,16 +922,6 @@ static bool same_events(const frnn_ctx* c, const frnn_event* ev, int n) {
             return false;
     }
     return true;
-}
-
-// Path of one event of a batch: 0 grid scan by chunks, 3 half-cell scan, 2
-// grid scan by row tasks, 1 tensor core (autotuned per size class, else the
-// defaults).
-static int batch_path(const frnn_ctx* ctx, int64_t n, int D, int K, unsigned flags) {
-    if (use_tc_path(ctx, D, flags, n, K)) return 1;
-    const int naxes = build_naxes(ctx, n, D);
-    if (half_cells(D, naxes, build_mult(ctx, n, D))) return 3;
-    return grid_kernel(naxes) == 1 ? 2 : 0;
 }
 
 // ev: ordered by path (chunks, half cells, row tasks, tensor core), so that

@@ -114,3 +114,19 @@ def test_compact_budget_holds_the_staging_rows_alone(listed_lib):
                 ctx.sync()
                 assert (1, stage) in calls(), (K, stage, calls())
         """)
+
+
+def test_serving_allocates_before_the_first_request(listed_lib):
+    """Every slot's workspace, the scan's scratch of calls that keep more than
+    128 neighbours included, is made before the loop copies its first input."""
+    _child(listed_lib, """
+        ev = [synth.clustered(100, 40, 1000, 8, 0.01, seed=73 + i) for i in range(6)]
+        with frnn.Context() as ctx:
+            lib.calls_reset()
+            outs, lat, st = ctx.serve(ev, [0.0] * len(ev), 0.1, 200, slots=2, max_batch=2)
+            kinds = [k for k, n in calls()]
+            copy = next(i for i, (k, n) in enumerate(calls()) if k == 3 and n == ev[0].nbytes)
+            assert 1 in kinds[:copy] and 1 not in kinds[copy:], calls()
+            for p, o in zip(ev, outs):
+                same([torch.from_numpy(x) for x in o], p, 0.1, 200)
+        """)
