@@ -339,10 +339,10 @@ def time_config(frnn, pts_np, r, K, path, dev, steps=20, warmup=3, opts=None, tc
         res["prefilter_survivors"] = surv
         res["exact_accepted"] = acc
         res["false_candidate_rate"] = (surv - acc) / surv if surv else None
-    gp = grid.params()
-    res["gridded_axes"] = gp["naxes"]
-    res["cell_mult"] = gp["cell_mult"]
-    res["grid_kernel"] = gp["kernel"]
+    sc = grid.scan()
+    res["gridded_axes"] = sc["naxes"]
+    res["cell_mult"] = grid.params()["cell_mult"]
+    res["grid_kernel"] = sc["scan"]
     ctx.close()
     del out, pts, flush
     return res
@@ -414,7 +414,7 @@ def run_ours(args):
     grid = ctx.build_grid(pts, r)
     ctx.query(grid, pts, r, K, True, path, (counts, idx, d2))
     ctx.sync()
-    gparams = grid.params()
+    gscan, cell_mult = grid.scan(), grid.params()["cell_mult"]
 
     def step(ev=None, split=False):
         # split: an event at the build/query boundary as well (the attribution
@@ -531,9 +531,9 @@ def run_ours(args):
         "data": "synthetic (seeded clusters + background shaped like a tracking event)",
         "config": {"workload": w.name, "N": N, "D": D, "r": r, "K": K, "path": path,
                    "grid_naxes_option": ctx.get_option(frnn.FRNN_OPT_GRID_NAXES),
-                   "gridded_axes": gparams["naxes"], "cell_mult": gparams["cell_mult"],
-                   "grid_dims": gparams["dims"], "grid_cells": gparams["cells"],
-                   "grid_kernel": gparams["kernel"],
+                   "gridded_axes": gscan["naxes"], "cell_mult": cell_mult,
+                   "grid_dims": gscan["dims"], "grid_cells": gscan["cells"],
+                   "grid_kernel": gscan["scan"],
                    "staging": ctx.get_option(frnn.FRNN_OPT_STAGING),
                    "self_query": True, "l2": "flushed between timed steps (256 MB write)",
                    "parallelism": f"replicas x{ws}" if ws > 1 else "single GPU"},

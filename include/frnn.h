@@ -132,15 +132,36 @@ typedef struct frnn_grid_info {
     int dims[5];        /* cells per gridded axis */
     float cell_edge;    /* 1 / inv_h, the cell edge (about r / m) */
     int64_t cells;      /* product of dims */
-    int kernel;         /* grid scan used for this grid: 0 chunks of 16 queries
-                           (candidates on lanes), 1 row tasks of 16 queries
-                           (grids requested with up to four axes).  axes, dims
-                           and cells leave out the coordinate that a default
-                           grid may divide its cells along besides these */
+    int kernel;         /* 1: grids requested with up to four axes, scanned by
+                           row tasks of 16 queries; 0: all others (frnn_grid_scan
+                           says how) */
     int valid;          /* 0 if a coordinate was non-finite */
 } frnn_grid_info;
 
 frnn_status frnn_grid_params(const frnn_grid* grid, frnn_grid_info* info);
+
+/* How a built grid is stored and scanned.  frnn_grid_params describes a grid
+ * of half cells by its cells of edge r over (at most) its first five axes; this
+ * is the grid itself: the sixth axis if there is one, and the cells stored.
+ * Synchronises the grid's context stream.  Errors: as frnn_grid_params. */
+typedef struct frnn_grid_scan_info {
+    int scan;           /* 0 chunks of 16 queries, candidates on lanes
+                             (query.cu: five requested axes; default grids of
+                             D >= 5 with a cell multiple above 1)
+                           1 row tasks of 16 queries (query_rows.cu: up to four
+                             requested axes)
+                           2 half cells: chunks of 16 queries, candidates on
+                             lanes, cells stored two by two along every axis but
+                             the first (query_half.cu: default grids of D >= 5)
+                           3 one query a lane (query_low.cu: D <= 4, default
+                             grids) */
+    int naxes;          /* gridded coordinates (1..6) */
+    int axes[6];        /* gridded coordinate indices (the first naxes) */
+    int dims[6];        /* stored cells per gridded axis */
+    int64_t cells;      /* product of dims */
+} frnn_grid_scan_info;
+
+frnn_status frnn_grid_scan(const frnn_grid* grid, frnn_grid_scan_info* info);
 
 /* Free a grid (after its pending work completes).  NULL is accepted.  A grid
  * is the device-resident cell structure of Sec. 2's uniform-grid method; it

@@ -529,6 +529,28 @@ frnn_status frnn_grid_params(const frnn_grid* grid, frnn_grid_info* info) {
     return FRNN_OK;
 }
 
+frnn_status frnn_grid_scan(const frnn_grid* grid, frnn_grid_scan_info* info) {
+    if (!grid || !info || !grid->ctx) return FRNN_ERR_INVALID_ARG;
+    frnn_ctx* ctx = grid->ctx;
+    *info = frnn_grid_scan_info{};
+    // as the query takes it (query_impl, enqueue_grid_query)
+    const int kernel = grid->half ? 2 : grid_kernel(grid->naxes);
+    info->scan = kernel == 0 && grid->D <= 4 ? 3 : kernel;
+    if (grid->g.E < 1 || !grid->g.hdr) return FRNN_OK;
+    cudaError_t e = cudaStreamSynchronize(ctx->stream);
+    EventHdr h{};
+    if (e == cudaSuccess) e = cudaMemcpy(&h, grid->g.hdr, sizeof(h), cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "reading the grid header");
+    info->naxes = h.naxes;
+    info->cells = 1;
+    for (int a = 0; a < kHdrAxes; ++a) {
+        info->axes[a] = a < h.naxes ? h.axes[a] : 0;
+        info->dims[a] = h.dims[a];
+        info->cells *= h.dims[a];
+    }
+    return FRNN_OK;
+}
+
 frnn_status frnn_grid_destroy(frnn_grid* grid) {
     if (!grid) return FRNN_OK;
     if (grid->ctx) {

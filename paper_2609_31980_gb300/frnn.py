@@ -54,7 +54,8 @@ EXPORTED = ["frnn_version", "frnn_create", "frnn_destroy", "frnn_build_grid",
             "frnn_sync", "frnn_last_error", "frnn_set_option", "frnn_get_option",
             "frnn_autotune", "frnn_serve_run", "frnn_self_query_noalloc",
             "frnn_kernel_times", "frnn_query_csr_count", "frnn_query_csr_fill",
-            "frnn_self_query_host_csr", "frnn_check_wait_timeout", "frnn_grid_params"]
+            "frnn_self_query_host_csr", "frnn_check_wait_timeout", "frnn_grid_params",
+            "frnn_grid_scan"]
 
 
 class frnn_tune_result(ctypes.Structure):
@@ -66,6 +67,11 @@ class frnn_grid_info(ctypes.Structure):
     _fields_ = [("naxes", ctypes.c_int), ("cell_mult", ctypes.c_int), ("axes", ctypes.c_int * 5),
                 ("dims", ctypes.c_int * 5), ("cell_edge", ctypes.c_float), ("cells", ctypes.c_int64),
                 ("kernel", ctypes.c_int), ("valid", ctypes.c_int)]
+
+
+class frnn_grid_scan_info(ctypes.Structure):
+    _fields_ = [("scan", ctypes.c_int), ("naxes", ctypes.c_int), ("axes", ctypes.c_int * 6),
+                ("dims", ctypes.c_int * 6), ("cells", ctypes.c_int64)]
 
 
 class frnn_request(ctypes.Structure):
@@ -94,6 +100,7 @@ _sigs = {
     "frnn_build_grid": ([_vp, _vp, _i64, _int, _f32, ctypes.POINTER(_vp)], _int),
     "frnn_grid_destroy": ([_vp], _int),
     "frnn_grid_params": ([_vp, ctypes.c_void_p], _int),
+    "frnn_grid_scan": ([_vp, ctypes.c_void_p], _int),
     "frnn_query": ([_vp, _vp, _vp, _i64, _f32, _int, _u32, _vp, _vp, _vp], _int),
     "frnn_query_batched": ([_vp, ctypes.POINTER(frnn_event), _int, _int, _f32, _int, _u32], _int),
     "frnn_self_query_host": ([_vp, _vp, _i64, _int, _f32, _int, _u32, _vp, _vp, _vp], _int),
@@ -169,6 +176,14 @@ class Grid:
         return {"naxes": n, "cell_mult": info.cell_mult, "axes": list(info.axes)[:n],
                 "dims": list(info.dims)[:n], "cell_edge": info.cell_edge, "cells": info.cells,
                 "kernel": "rows" if info.kernel == 1 else "chunks", "valid": bool(info.valid)}
+
+    def scan(self) -> dict:
+        """frnn_grid_scan: how this grid is stored and scanned."""
+        info = frnn_grid_scan_info()
+        _check(self.ctx.handle, frnn_grid_scan(self.handle, ctypes.byref(info)))
+        n = info.naxes
+        return {"scan": ("chunks", "rows", "half cells", "query per lane")[info.scan], "naxes": n,
+                "axes": list(info.axes)[:n], "dims": list(info.dims)[:n], "cells": info.cells}
 
     def close(self):
         if self.handle:
