@@ -154,7 +154,10 @@ typedef struct frnn_grid_scan_info {
                              lanes, cells stored two by two along every axis but
                              the first (query_half.cu: default grids of D >= 5)
                            3 one query a lane (query_low.cu: D <= 4, default
-                             grids) */
+                             grids)
+                           4 as 2, but plain cells over four or five axes, where
+                             an axis holds so few cells that half cells would cover
+                             more of the points (query_half.cu) */
     int naxes;          /* gridded coordinates (1..6) */
     int axes[6];        /* gridded coordinate indices (the first naxes) */
     int dims[6];        /* stored cells per gridded axis */

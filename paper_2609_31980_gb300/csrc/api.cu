@@ -541,6 +541,7 @@ frnn_status frnn_grid_scan(const frnn_grid* grid, frnn_grid_scan_info* info) {
     EventHdr h{};
     if (e == cudaSuccess) e = cudaMemcpy(&h, grid->g.hdr, sizeof(h), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "reading the grid header");
+    if (grid->half && h.valid && !h.half) info->scan = 4;   // (the build's choice)
     info->naxes = h.naxes;
     info->cells = 1;
     for (int a = 0; a < kHdrAxes; ++a) {

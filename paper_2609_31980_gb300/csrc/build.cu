@@ -459,10 +459,11 @@ struct GridFit {
     bool at_start = false;   // the starting cell edge fitted (no enlargement)
 };
 
-// lo_j, hi_j: the extremes of coordinate j on lane j < D.  Called by all
-// lanes of warp 0.
+// lo_j, hi_j: the extremes of coordinate j on lane j < D.  once: no grid (an
+// infinite fraction) where the starting cell edge does not fit.  Called by all
+// lanes of a warp.
 __device__ void grid_fit(GridFit& f, float lo_j, float hi_j, int D, int k, int m, int axes_mode,
-                         float r, int64_t cap, bool valid, int max_rows, bool half) {
+                         float r, int64_t cap, bool valid, int max_rows, bool half, bool once = false) {
     constexpr unsigned kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int la = lane & 7;   // the lane's axis (every eighth lane alike, for the products below)
@@ -542,6 +543,7 @@ __device__ void grid_fit(GridFit& f, float lo_j, float hi_j, int D, int k, int m
             f.at_start = it == 0;
             break;
         }
+        if (once) return;   // (frac as it was: infinite)
         // too many cells: by the ratio the budget asks for (the dims' rounding
         // may need another step); a failed bound or axis limit: by a tenth
         float shrink = 0.9f;
@@ -584,10 +586,19 @@ __device__ __forceinline__ uint64_t division_multiplier(uint32_t d) {
 // coordinate j in shared memory, bad a non-finite input.  Warp w fits the
 // candidate of k_hi - w axes; the best one's warp writes the parameters.
 // H: the event's header (global or shared memory), everything else of it set.
+// Half cells reach four cells along an axis where plain ones reach three, which
+// is all of an axis of few cells: two more warps fit five and four axes of
+// plain cells, taken (H.half = 0) where the expected candidates of a query, at
+// kWideCost of a half cell's each (grids of few cells only: the starting edge
+// must fit the budget) and with kWideMore5 or kWideMore4 for the
+// look-ups (five axes: three times as many), are fewer.
 constexpr int kFitWarps = 3;
+constexpr int kWideWarps = 2;
+constexpr float kWideCost = 0.45f;
+constexpr float kWideMore5 = 350.f, kWideMore4 = 150.f;
 __device__ void derive_params(EventHdr& H, const int32_t* box, bool bad, int D, float r, int m, int axes_mode,
                               int naxes_req) {
-    __shared__ float s_frac[kFitWarps];
+    __shared__ float s_frac[kFitWarps + kWideWarps];
     __shared__ int s_start[kFitWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t n = H.n;
@@ -613,6 +624,10 @@ __device__ void derive_params(EventHdr& H, const int32_t* box, bool bad, int D, 
     f.frac = INFINITY;
     if (warp < kFitWarps && k_hi - warp >= k_lo)
         grid_fit(f, lo_j, hi_j, D, k_hi - warp, half ? 1 : m_req, axes_mode, r, cap, valid, max_rows, half);
+    if (warp >= kFitWarps && warp < kFitWarps + kWideWarps) {
+        if (half) grid_fit(f, lo_j, hi_j, D, kMaxAxes - (warp - kFitWarps), 1, axes_mode, r, cap, valid, kMaxNbrRows, false, true);
+        if (lane == 0) s_frac[warp] = f.frac;
+    }
     if (warp < kFitWarps && lane == 0) {
         s_frac[warp] = f.frac;
         s_start[warp] = f.at_start ? 1 : 0;
@@ -623,6 +638,14 @@ __device__ void derive_params(EventHdr& H, const int32_t* box, bool bad, int D, 
     int best = 0;
     for (int w = 1; w < kFitWarps && k_hi - w >= k_lo && !s_start[w - 1]; ++w)
         if (s_frac[w] < s_frac[best]) best = w;
+    float cost = (float)n * s_frac[best];
+    for (int w = 0; w < kWideWarps && half && valid; ++w) {
+        const float c = kWideCost * (float)n * s_frac[kFitWarps + w] + (w == 0 ? kWideMore5 : kWideMore4);
+        if (c < cost) {
+            cost = c;
+            best = kFitWarps + w;
+        }
+    }
     if (warp != best) return;
     const int na = f.naxes;
     if (lane < kHdrAxes) {
@@ -644,6 +667,7 @@ __device__ void derive_params(EventHdr& H, const int32_t* box, bool bad, int D, 
         H.ctr[lane] = c;
     }
     if (lane == 0) {
+        if (best >= kFitWarps) H.half = 0;
         H.naxes = na;
         H.m = f.m;
         H.valid = valid ? 1 : 0;

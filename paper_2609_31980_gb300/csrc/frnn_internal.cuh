@@ -221,7 +221,7 @@ struct QueryArgs {
     int32_t* idx;
     float* dist2;
     float r2;                    // fl(r * r)
-    float r2_screen;             // row-task kernel: r2 (1 + 2^-16) rounded up, the packed screen's bound
+    float r2_screen;             // r2 (1 + 2^-16) rounded up: the packed screens' bound (query_rows.cu)
     int32_t K;
     int32_t self;                // 1: query slot == reference slot is excluded
     int32_t D;

@@ -797,6 +797,7 @@ static QueryArgs query_args(const QueryLaunch& q) {
     a.idx = q.idx;
     a.dist2 = q.dist2;
     a.r2 = q.r2;
+    a.r2_screen = std::nextafter((float)((double)q.r2 * (1.0 + 0x1p-16)), INFINITY);
     a.K = q.K;
     a.self = q.self;
     a.D = rs.D;

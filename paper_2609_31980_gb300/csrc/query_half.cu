@@ -49,6 +49,17 @@
 //   * the sorted rows go back to shared memory and are written with 16-byte
 //     stores (row width a multiple of 4 and aligned outputs; else 4-byte).
 //
+// Grids of few cells (EventHdr::half 0; the build's rule is derive_params in
+// build.cu).  Half cells reach 4 cells along an axis, all of one that has no
+// more, where plain cells reach 3, and at radii of a fifth of the extent a query
+// has thousands of candidates.  Such events get plain cells over four axes (27
+// rows, one a lane) or five (walked in three rounds), and wide_stream screens
+// the candidates against four queries a step in packed arithmetic.  Uniform
+// points in the unit cube, build + query, row tasks or chunks of the axes that
+// were the default before / half cells / now: 60k x 8, r = 0.26 1.51 / 3.79 /
+// 0.82 ms; 60k x 12, r = 0.3 1.76 / 6.0 / 1.72; 200k x 16, r = 0.22 5.8 / 23.2 /
+// 3.0; 20k x 10, r = 0.18 0.110 / 0.143 / 0.079.
+//
 // What bounds it: instruction issue (70 % of the slots, 84 M warp instructions
 // at 300k x 8 where the chunk scan over five axes took 143 M) and the
 // load/store pipe (65 %).  Kernel alone, 300k x 8, K = 64: 193 us (chunk scan)
@@ -60,6 +71,7 @@
 // -> 350, 20k x 8 66 -> 45.
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 #include "frnn_host.h"
 #include "warp_sort.cuh"
@@ -264,22 +276,169 @@ __device__ __noinline__ void write_long_row(const float* ld, const int32_t* li, 
     }
 }
 
-// LONG: rows past the shared-memory lists are kept (scratch, pool) and written
-// here; else they go to select.cu.
+// Packed float32 pairs (query_rows.cu has the proof of the screen's bound).
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ uint64_t screen2(uint64_t s, uint64_t q, uint64_t c) {
+    uint64_t d, t;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(q), "l"(c));
+    asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(t) : "l"(d), "l"(s));
+    return t;
+}
+__device__ __forceinline__ float min2(uint64_t v) {
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    return fminf(a, b);
+}
+
+// The candidates of one batch of groups (U of them in nr ranges) on a grid of
+// plain cells: few, full cells, so whole chunks of queries against thousands of
+// candidates, of which few are neighbours.  A lane takes one candidate a round;
+// a step screens it against four queries, two to a packed instruction, and the
+// rest of the dimensions is left out when no lane's partial sum is within the
+// bound (sums of squares never decrease).  What passes is computed again by the
+// contract.  The queries lie pair-interleaved in w.Q.
 template <int D, bool LONG>
-__global__ void __launch_bounds__(kWarps * 32, Cfg<D>::MINB) k_half_query(QueryArgs a, int sub_shift) {
-    pdl_trigger();
-    pdl_wait();
+__device__ __forceinline__ void wide_stream(const WarpSmem& w, const QueryArgs& a, int nr, int U) {
     constexpr int DP = Cfg<D>::DP;
-    extern __shared__ __align__(128) unsigned char smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const WarpSmem w = carve<D>(smem + (size_t)warp * warp_bytes<D>());
+    // dimensions summed before each vote (the gridded ones come last)
+    constexpr int VOTE1 = D <= 5 ? D : (D == 9 || D == 10 ? 6 : 4), VOTE2 = D <= 10 ? D : 8;
+    const int lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1u;
     const unsigned le_mask = lt_mask | (1u << lane);
+    const float r2 = a.r2, rs2 = a.r2_screen;
+    int cur = -1;
+    auto load_cand = [&](int k0, int& qq, int32_t& orig, float (&cv)[DP]) {
+        const int ri = cur + 1 + lane;
+        const int d = ri < nr ? w.rpre[ri] - k0 : 32;
+        const unsigned starts = __reduce_or_sync(kFull, d < 32 ? 1u << d : 0u);
+        const int i = cur + __popc(starts & le_mask);
+        cur += __popc(starts);
+        qq = 0;
+        orig = -1;
+#pragma unroll
+        for (int k = 0; k < DP; ++k) cv[k] = 0.f;
+        const int u = k0 + lane;
+        if (u < U) {
+            const int slot = u + w.rdel[i];
+            qq = w.rq[i];
+            orig = __ldg(a.rperm + slot);
+            load_row<DP>(a.rpts + (int64_t)slot * DP, cv);
+        }
+    };
+    int qq;
+    int32_t orig;
+    float cv[DP];
+    load_cand(0, qq, orig, cv);
+#pragma unroll 1
+    for (int k0 = 0; k0 < U; k0 += 32) {
+        int qq_n;
+        int32_t orig_n;
+        float cvn[DP];
+        load_cand(k0 + 32, qq_n, orig_n, cvn);   // next round in flight
+        const int qa = qq & 255, qb = qq >> 8;
+        const int pa = qa >> 1, np = ((qb + 1) >> 1) - pa;   // pairs of queries (the first and last may be half)
+        const int mx = __reduce_max_sync(kFull, (unsigned)np);
+        const int qq_p = __shfl_up_sync(kFull, qq, 1);
+        const unsigned firsts = __ballot_sync(kFull, lane == 0 || qq != qq_p);
+        const unsigned g_lo = lt_mask & ~((1u << (31 - __clz(firsts & le_mask))) - 1u);
+        const unsigned later = firsts & ~le_mask;
+        const unsigned g_hi = ~le_mask & (later ? (later & (0u - later)) - 1u : kFull);
+        uint64_t cc[D];
+#pragma unroll
+        for (int k = 0; k < D; ++k) cc[k] = pack2(cv[k], cv[k]);
+#pragma unroll 1
+        for (int j = 0; j < mx; j += 2) {
+            const float* Q0 = w.Q + (j < np ? pa + j : 0) * 2 * DP;
+            const float* Q1 = w.Q + (j + 1 < np ? pa + j + 1 : 0) * 2 * DP;
+            uint64_t s0 = 0, s1 = 0;
+            auto dims = [&](auto from, auto to) {
+#pragma unroll
+                for (int k = decltype(from)::value; k < decltype(to)::value; k += 2) {
+                    const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(Q0 + 2 * k);
+                    const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(Q1 + 2 * k);
+                    s0 = screen2(s0, x.x, cc[k]);
+                    s1 = screen2(s1, y.x, cc[k]);
+                    if (k + 1 < D) {
+                        s0 = screen2(s0, x.y, cc[k + 1 < D ? k + 1 : k]);
+                        s1 = screen2(s1, y.y, cc[k + 1 < D ? k + 1 : k]);
+                    }
+                }
+            };
+            auto near = [&]() {
+                return __any_sync(kFull, (j < np && min2(s0) <= rs2) || (j + 1 < np && min2(s1) <= rs2));
+            };
+            dims(std::integral_constant<int, 0>{}, std::integral_constant<int, VOTE1>{});
+            if (!near()) continue;
+            if constexpr (VOTE1 < D) {
+                dims(std::integral_constant<int, VOTE1>{}, std::integral_constant<int, VOTE2>{});
+                if (VOTE2 < D && !near()) continue;
+                dims(std::integral_constant<int, VOTE2>{}, std::integral_constant<int, D>{});
+            }
+            // the step's queries 2 (pa + j) + b, b < 4: bit b if it passes
+            unsigned pass = 0;
+            {
+                float v[4];
+                asm("mov.b64 {%0, %1}, %2;" : "=f"(v[0]), "=f"(v[1]) : "l"(s0));
+                asm("mov.b64 {%0, %1}, %2;" : "=f"(v[2]), "=f"(v[3]) : "l"(s1));
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    const int q = 2 * (pa + j) + b;
+                    if (q >= qa && q < qb && v[b] <= rs2) pass |= 1u << b;
+                }
+            }
+            unsigned left = __reduce_or_sync(kFull, pass);
+            while (left) {
+                const int b = __ffs(left) - 1;
+                left &= left - 1u;
+                const bool on = (pass >> b) & 1u;
+                const int q = on ? 2 * (pa + j) + b : 0;
+                const int held = w.cnt[q];
+                const float* qp = w.Q + (q >> 1) * 2 * DP + (q & 1);
+                float s = 0.f;
+#pragma unroll
+                for (int k = 0; k < D; ++k) {
+                    const float d = __fsub_rn(qp[2 * k], cv[k]);
+                    s = __fadd_rn(s, __fmul_rn(d, d));
+                }
+                const bool acc = on && s <= r2 && !(a.self && orig == w.qor[q]);
+                const unsigned am = __ballot_sync(kFull, acc);
+                const int p = held + __popc(am & g_lo);
+                if (acc && p < kListCap) {
+                    w.Ld[q * kListStr + p] = s;
+                    w.Li[q * kListStr + p] = orig;
+                }
+                if (acc && (am & g_hi) == 0) w.cnt[q] = p + 1;
+                if (LONG && acc && p >= kListCap && p < a.list_cap)
+                    (a.scratch + (size_t)(blockIdx.x * kWarps + (threadIdx.x >> 5)) * kScratchKeys +
+                     q * kMoreCap)[p - kListCap] = make_key(s, orig);
+                __syncwarp();
+            }
+        }
+        qq = qq_n;
+        orig = orig_n;
+#pragma unroll
+        for (int k = 0; k < DP; ++k) cv[k] = cvn[k];
+    }
+}
+
+// LONG: rows past the shared-memory lists are kept (scratch, pool) and written
+// here; else they go to select.cu.
+// WIDE: a grid of plain cells (EventHdr::half 0).  Task t: the queries `part`
+// x `per` of chunk c, of event e.
+template <int D, bool LONG, bool WIDE>
+__device__ __forceinline__ void do_task(const QueryArgs& a, const WarpSmem& w, int e, int c, int part, int per) {
+    constexpr int DP = Cfg<D>::DP;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const unsigned le_mask = lt_mask | (1u << lane);
+    const EventHdr& hq = a.qev[e];
+    const EventHdr& h = a.ev[e];
     const float r2 = a.r2;
     const int K = a.K;
-    const int per = kQ >> sub_shift;
-    const int ntasks = a.nchunks << sub_shift;
     // row width of the output (compact staging rows have no padding) and, for
     // the 16-byte stores, its quarter
     const int width = a.csr ? kCsrStageW : K;
@@ -288,346 +447,425 @@ __global__ void __launch_bounds__(kWarps * 32, Cfg<D>::MINB) k_half_query(QueryA
     auto scratch = [&](int q) {
         return a.scratch + (size_t)(blockIdx.x * kWarps + (threadIdx.x >> 5)) * kScratchKeys + q * kMoreCap;
     };
-
-    for (;;) {
-        int t = 0;
-        if (lane == 0) t = atomicAdd(a.task_counter, 1);
-        t = __shfl_sync(kFull, t, 0);
-        if (t >= ntasks) break;
-        const int c = t >> sub_shift;
-        const int e = a.nev > 1 ? chunk_event(a.qev, a.nev, c) : 0;
-        const EventHdr& hq = a.qev[e];
-        const EventHdr& h = a.ev[e];
-        if (a.path_filter >= 0 && h.path != a.path_filter) continue;   // another launch's event
-        int32_t* counts = a.counts ? a.counts : h.counts;
-        int32_t* oidx = a.counts ? a.idx : h.idx;
-        float* od2 = a.counts ? a.dist2 : h.dist2;
-        const int64_t q_end = hq.pt_off + hq.n;
-        const int s0 = (int)(hq.pt_off + (int64_t)(c - hq.qchunk0) * kQ) + (t & ((1 << sub_shift) - 1)) * per;
-        const int nqc = (int)min((int64_t)per, q_end - (int64_t)s0);
-        if (nqc <= 0) continue;   // past the event's last query
-        const bool act = lane < nqc;
-        const int qorig0 = act ? a.qperm[s0 + lane] : 0;
-        if (!h.valid) {
-            // grid built from non-finite input: empty rows (frnn_sync reports it)
-            for (int ql = 0; ql < nqc && !a.csr; ++ql) {
-                const int qo = __shfl_sync(kFull, qorig0, ql);
-                for (int e2 = lane; e2 < K; e2 += 32) {
-                    oidx[(int64_t)qo * K + e2] = -1;
-                    od2[(int64_t)qo * K + e2] = INFINITY;
-                }
+    int32_t* counts = a.counts ? a.counts : h.counts;
+    int32_t* oidx = a.counts ? a.idx : h.idx;
+    float* od2 = a.counts ? a.dist2 : h.dist2;
+    const int64_t q_end = hq.pt_off + hq.n;
+    const int s0 = (int)(hq.pt_off + (int64_t)(c - hq.qchunk0) * kQ) + part * per;
+    const int nqc = (int)min((int64_t)per, q_end - (int64_t)s0);
+    if (nqc <= 0) return;   // past the event's last query
+    const bool act = lane < nqc;
+    const int qorig0 = act ? a.qperm[s0 + lane] : 0;
+    if (!h.valid) {
+        // grid built from non-finite input: empty rows (frnn_sync reports it)
+        for (int ql = 0; ql < nqc && !a.csr; ++ql) {
+            const int qo = __shfl_sync(kFull, qorig0, ql);
+            for (int e2 = lane; e2 < K; e2 += 32) {
+                oidx[(int64_t)qo * K + e2] = -1;
+                od2[(int64_t)qo * K + e2] = INFINITY;
             }
-            if (act) counts[qorig0] = 0;
-            if (act && a.degree) a.degree[qorig0] = 0;
-            continue;
         }
-        const int naxes = h.naxes, dims0 = h.dims[0];
-        const int32_t* cells = a.cstart + h.cell_off;
+        if (act) counts[qorig0] = 0;
+        if (act && a.degree) a.degree[qorig0] = 0;
+        return;
+    }
+    const int naxes = h.naxes, dims0 = h.dims[0];
+    const int32_t* cells = a.cstart + h.cell_off;
 
-        // the chunk's queries by (row of cells, half bits, cell on the row)
-        int x, row, src, pk;
-        {
-            const int key = act ? a.qcell[s0 + lane] : 0;
-            const int id = key >> kHalfBits;
-            row = div_mag(id, h.mag[0]);
-            x = id - row * dims0;
-            const int prev = __shfl_up_sync(kFull, row, 1);
-            const int rr = __popc(__ballot_sync(kFull, act && (lane == 0 || row != prev)) & le_mask);
-            uint32_t sk = act ? ((uint32_t)rr << 20) | ((uint32_t)(key & ((1 << kHalfBits) - 1)) << 15) |
-                                    ((uint32_t)x << 5) | (uint32_t)lane
-                              : 0xffffffffu;
+    // the chunk's queries by (row of cells, half bits, cell on the row)
+    int x, row, src, pk;
+    {
+        const int key = act ? a.qcell[s0 + lane] : 0;
+        const int id = WIDE ? key : key >> kHalfBits;
+        row = div_mag(id, h.mag[0]);
+        x = id - row * dims0;
+        const int prev = __shfl_up_sync(kFull, row, 1);
+        const int rr = __popc(__ballot_sync(kFull, act && (lane == 0 || row != prev)) & le_mask);
+        uint32_t sk = act ? ((uint32_t)rr << 20) | ((uint32_t)(WIDE ? 0 : key & ((1 << kHalfBits) - 1)) << 15) |
+                                ((uint32_t)x << 5) | (uint32_t)lane
+                          : 0xffffffffu;
 #pragma unroll
-            for (int k2 = 2; k2 <= kQ; k2 <<= 1) {
+        for (int k2 = 2; k2 <= kQ; k2 <<= 1) {
 #pragma unroll
-                for (int j = k2 >> 1; j > 0; j >>= 1) {
-                    const uint32_t o = __shfl_xor_sync(kFull, sk, j);
-                    const bool take_min = ((lane & j) == 0) == ((lane & k2) == 0 || k2 == kQ);
-                    sk = take_min ? min(sk, o) : max(sk, o);
-                }
+            for (int j = k2 >> 1; j > 0; j >>= 1) {
+                const uint32_t o = __shfl_xor_sync(kFull, sk, j);
+                const bool take_min = ((lane & j) == 0) == ((lane & k2) == 0 || k2 == kQ);
+                sk = take_min ? min(sk, o) : max(sk, o);
             }
-            src = (int)(sk & 31u);
-            pk = (int)(sk >> 5);
-            x = pk & 1023;
-            row = __shfl_sync(kFull, row, src);
         }
-        const int bits = (pk >> 10) & 31;
-        const int qs = s0 + src;
-        const int qorig = __shfl_sync(kFull, qorig0, src);
-        if (act) {
-            const float4* q4 = reinterpret_cast<const float4*>(a.qpts + (int64_t)qs * DP);
-            float4* dst = reinterpret_cast<float4*>(w.Q + lane * DP);
+        src = (int)(sk & 31u);
+        pk = (int)(sk >> 5);
+        x = pk & 1023;
+        row = __shfl_sync(kFull, row, src);
+    }
+    const int bits = (pk >> 10) & 31;
+    const int qs = s0 + src;
+    const int qorig = __shfl_sync(kFull, qorig0, src);
+    if (act) {
+        const float4* q4 = reinterpret_cast<const float4*>(a.qpts + (int64_t)qs * DP);
+        float4* dst = reinterpret_cast<float4*>(w.Q + lane * DP);
+        if constexpr (!WIDE) {
 #pragma unroll
             for (int k4 = 0; k4 < DP / 4; ++k4) dst[k4] = q4[k4];
-            w.qor[lane] = qorig;
-            w.cnt[lane] = 0;
         }
-        // per query: the moves (bits of a neighbour row's number) that would
-        // leave the grid; per lane: the row offset its own bits move by
-        int bad = 0, mv[kHdrAxes - 1];
-        {
-            int v = row, rs = 1;
+        w.qor[lane] = qorig;
+        w.cnt[lane] = 0;
+    }
+    if (WIDE && lane < kQ) {   // pair-interleaved; no query: never within the radius
+        const float* p = a.qpts + (int64_t)qs * DP;
+        float* dst = w.Q + (lane >> 1) * 2 * DP + (lane & 1);
+#pragma unroll 1
+        for (int k = 0; k < DP; ++k) dst[2 * k] = act ? p[k] : __int_as_float(0x7fc00000);
+    }
+    // per query: the moves (bits of a neighbour row's number; plain cells:
+    // two bits an axis, down and up) that would leave the grid; per lane:
+    // the moves its row makes, and the row offset its own bits move by
+    int bad = 0, moves = lane & 31, mv[kHdrAxes - 1], back = 0;
+    // plain cells: a lane has one of the 27 rows of four axes; a fifth axis is
+    // walked group by group, its rows last_rs apart
+    const int rounds = WIDE && naxes == 5 ? 3 : 1;
+    int last_rs = 0;
+    if constexpr (WIDE) {
+        int v = row, rs = 1, l = lane;
+        moves = 0;
 #pragma unroll
-            for (int ax = 1; ax < kHdrAxes; ++ax) {
-                mv[ax - 1] = 0;
-                if (ax < naxes) {
-                    const int da = h.dims[ax];
-                    const int qv = div_mag(v, h.mag[ax]);
-                    const int ca = v - qv * da;
-                    v = qv;
-                    if (((bits >> (ax - 1)) & 1) ? ca == da - 1 : ca == 0) bad |= 1 << (ax - 1);
-                    if ((lane >> (ax - 1)) & 1) mv[ax - 1] = rs;
-                    rs *= da;
-                }
+        for (int ax = 1; ax < kHdrAxes; ++ax) mv[ax - 1] = 0;
+#pragma unroll 1
+        for (int ax = 1; ax < naxes; ++ax) {
+            const int da = h.dims[ax];
+            const int qv = div_mag(v, h.mag[ax]);
+            const int ca = v - qv * da;
+            v = qv;
+            if (ca == 0) bad |= 1 << (2 * ax - 2);
+            if (ca == da - 1) bad |= 2 << (2 * ax - 2);
+            if (ax < 4) {
+                const int d = l % 3 - 1;
+                l /= 3;
+                if (d != 0) moves |= (d < 0 ? 1 : 2) << (2 * ax - 2);
+                back += d * rs;
+            } else {
+                last_rs = rs;
+            }
+            rs *= da;
+        }
+        if (l > 0) moves |= 1 << 8;   // (past the last neighbour row)
+        bad |= 1 << 8;
+    } else {
+        int v = row, rs = 1;
+#pragma unroll
+        for (int ax = 1; ax < kHdrAxes; ++ax) {
+            mv[ax - 1] = 0;
+            if (ax < naxes) {
+                const int da = h.dims[ax];
+                const int qv = div_mag(v, h.mag[ax]);
+                const int ca = v - qv * da;
+                v = qv;
+                if (((bits >> (ax - 1)) & 1) ? ca == da - 1 : ca == 0) bad |= 1 << (ax - 1);
+                if ((lane >> (ax - 1)) & 1) mv[ax - 1] = rs;
+                rs *= da;
             }
         }
-        const int back = -(mv[0] + mv[1] + mv[2] + mv[3] + mv[4]);
-        const bool lane_row = lane < (1 << (naxes - 1));
-        const int gp = bits | (bad << 5) | (x << 10);
-        // groups
-        const int ppk = __shfl_up_sync(kFull, pk, 1);
-        const bool head = act && (lane == 0 || (pk >> 10) != (ppk >> 10) || x > (ppk & 1023) + 1);
-        const unsigned gmask = __ballot_sync(kFull, head);
-        const int ng = __popc(gmask);
+    }
+    if constexpr (!WIDE) back = -(mv[0] + mv[1] + mv[2] + mv[3] + mv[4]);
+    const bool lane_row = WIDE || lane < (1 << (naxes - 1));
+    const int gp = bits | (bad << 5) | (x << 14);
+    // groups
+    const int ppk = __shfl_up_sync(kFull, pk, 1);
+    const bool head = act && (lane == 0 || (pk >> 10) != (ppk >> 10) || x > (ppk & 1023) + 1);
+    const unsigned gmask = __ballot_sync(kFull, head);
+    const int ng = __popc(gmask) * rounds;
 
-        // slot range of the neighbour row of group g (first query hl, past its
-        // last hn) on this lane
-        int nlo = 0, nhi = 0;
-        unsigned gleft = gmask;   // heads of the groups not fetched yet
-        int f_hl = 0, f_hn = 0;   // queries of the fetched group
-        auto fetch = [&]() {
+    // slot range of the neighbour row of group g (first query hl, past its
+    // last hn) on this lane
+    int nlo = 0, nhi = 0;
+    unsigned gleft = gmask;   // heads of the groups not fetched yet
+    int f_hl = 0, f_hn = 0;   // queries of the fetched group
+    int f_round = rounds - 1;
+    auto fetch = [&]() {
+        if (!WIDE || ++f_round == rounds) {
             f_hl = __ffs(gleft) - 1;
             gleft &= gleft - 1u;
             f_hn = gleft ? __ffs(gleft) - 1 : nqc;
-            const int g = __shfl_sync(kFull, gp, f_hl);
-            const int grow = __shfl_sync(kFull, row, f_hl);
-            const int xl = __shfl_sync(kFull, x, f_hn - 1);
-            const int x0 = max((g >> 10) - 1, 0), x1 = min(xl + 1, dims0 - 1) + 1;
-            nlo = 0;
-            nhi = 0;
-            if (lane_row && (lane & (g >> 5) & 31) == 0) {
-                int off = back;
+            f_round = 0;
+        }
+        const int g = __shfl_sync(kFull, gp, f_hl);
+        const int grow = __shfl_sync(kFull, row, f_hl);
+        const int xl = __shfl_sync(kFull, x, f_hn - 1);
+        const int x0 = max((g >> 14) - 1, 0), x1 = min(xl + 1, dims0 - 1) + 1;
+        nlo = 0;
+        nhi = 0;
+        int need = moves, off = back;
+        if (WIDE && rounds == 3) {
+            need |= f_round == 0 ? 1 << 6 : (f_round == 2 ? 2 << 6 : 0);
+            off += (f_round - 1) * last_rs;
+        }
+        if (lane_row && (need & (g >> 5) & 511) == 0) {
 #pragma unroll
-                for (int ax = 0; ax < kHdrAxes - 1; ++ax)
-                    if ((g >> ax) & 1) off += 2 * mv[ax];
-                const int base = (grow + off) * dims0;
-                nlo = __ldg(cells + base + x0);
-                nhi = __ldg(cells + base + x1);
+            for (int ax = 0; ax < kHdrAxes - 1; ++ax)
+                if ((g >> ax) & 1) off += 2 * mv[ax];
+            const int base = (grow + off) * dims0;
+            nlo = __ldg(cells + base + x0);
+            nhi = __ldg(cells + base + x1);
+        }
+    };
+    fetch();
+    __syncwarp();
+
+    int gdone = 0;   // groups taken into a batch
+    while (gdone < ng) {
+        int nr = 0;
+        for (;;) {
+            const int n = nhi - nlo;
+            const unsigned bal = __ballot_sync(kFull, n > 0);
+            if (nr + __popc(bal) > kRangeCap) break;   // this group opens the next batch
+            if (n > 0) {
+                const int pos = nr + __popc(bal & lt_mask);
+                w.rdel[pos] = nlo;
+                w.rpre[pos] = n;   // a count until the batch's scan
+                w.rq[pos] = (uint16_t)(f_hl | (f_hn << 8));
             }
-        };
-        fetch();
+            nr += __popc(bal);
+            if (++gdone == ng) break;
+            fetch();
+        }
+        // counts -> stream positions
+        __syncwarp();
+        int U = 0;
+        for (int b0 = 0; b0 < nr; b0 += 32) {
+            const int i = b0 + lane;
+            const int v = i < nr ? w.rpre[i] : 0;
+            int incl = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (i < nr) {
+                const int start = U + incl - v;
+                w.rpre[i] = start;
+                w.rdel[i] -= start;
+            }
+            U += __shfl_sync(kFull, incl, 31);
+        }
         __syncwarp();
 
-        int gdone = 0;   // groups taken into a batch
-        while (gdone < ng) {
-            int nr = 0;
-            for (;;) {
-                const int n = nhi - nlo;
-                const unsigned bal = __ballot_sync(kFull, n > 0);
-                if (nr + __popc(bal) > kRangeCap) break;   // this group opens the next batch
-                if (n > 0) {
-                    const int pos = nr + __popc(bal & lt_mask);
-                    w.rdel[pos] = nlo;
-                    w.rpre[pos] = n;   // a count until the batch's scan
-                    w.rq[pos] = (uint16_t)(f_hl | (f_hn << 8));
-                }
-                nr += __popc(bal);
-                if (++gdone == ng) break;
-                fetch();
-            }
-            // counts -> stream positions
+        if constexpr (WIDE) {
+            wide_stream<D, LONG>(w, a, nr, U);
             __syncwarp();
-            int U = 0;
-            for (int b0 = 0; b0 < nr; b0 += 32) {
-                const int i = b0 + lane;
-                const int v = i < nr ? w.rpre[i] : 0;
-                int incl = v;
+            continue;
+        }
+        int cur = -1;   // last range that starts before the next round
+        auto load_cand = [&](int k0, int& qq, int32_t& orig, float (&cv)[DP]) {
+            const int ri = cur + 1 + lane;
+            const int d = ri < nr ? w.rpre[ri] - k0 : 32;
+            const unsigned starts = __reduce_or_sync(kFull, d < 32 ? 1u << d : 0u);
+            const int i = cur + __popc(starts & le_mask);
+            cur += __popc(starts);
+            qq = 0;
+            orig = -1;
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(kFull, incl, o);
-                    if (lane >= o) incl += y;
-                }
-                if (i < nr) {
-                    const int start = U + incl - v;
-                    w.rpre[i] = start;
-                    w.rdel[i] -= start;
-                }
-                U += __shfl_sync(kFull, incl, 31);
+            for (int k = 0; k < DP; ++k) cv[k] = 0.f;
+            const int u = k0 + lane;
+            if (u < U) {
+                const int slot = u + w.rdel[i];
+                qq = w.rq[i];
+                orig = __ldg(a.rperm + slot);
+                load_row<DP>(a.rpts + (int64_t)slot * DP, cv);
             }
-            __syncwarp();
-
-            int cur = -1;   // last range that starts before the next round
-            auto load_cand = [&](int k0, int& qq, int32_t& orig, float (&cv)[DP]) {
-                const int ri = cur + 1 + lane;
-                const int d = ri < nr ? w.rpre[ri] - k0 : 32;
-                const unsigned starts = __reduce_or_sync(kFull, d < 32 ? 1u << d : 0u);
-                const int i = cur + __popc(starts & le_mask);
-                cur += __popc(starts);
-                qq = 0;
-                orig = -1;
-#pragma unroll
-                for (int k = 0; k < DP; ++k) cv[k] = 0.f;
-                const int u = k0 + lane;
-                if (u < U) {
-                    const int slot = u + w.rdel[i];
-                    qq = w.rq[i];
-                    orig = __ldg(a.rperm + slot);
-                    load_row<DP>(a.rpts + (int64_t)slot * DP, cv);
-                }
-            };
-            int qq;
-            int32_t orig;
-            float cv[DP];
-            load_cand(0, qq, orig, cv);
+        };
+        int qq;
+        int32_t orig;
+        float cv[DP];
+        load_cand(0, qq, orig, cv);
 #pragma unroll 1
-            for (int k0 = 0; k0 < U; k0 += 32) {
-                int qq_n;
-                int32_t orig_n;
-                float cvn[DP];
-                load_cand(k0 + 32, qq_n, orig_n, cvn);   // next round in flight
-                const int qa = qq & 255;
-                const int nq = (qq >> 8) - qa;
-                const int mx = __reduce_max_sync(kFull, (unsigned)nq);
-                // the lanes of this lane's group before and after it (a group's
-                // lanes are consecutive)
-                const int qq_p = __shfl_up_sync(kFull, qq, 1);
-                const unsigned firsts = __ballot_sync(kFull, lane == 0 || qq != qq_p);
-                const unsigned g_lo = lt_mask & ~((1u << (31 - __clz(firsts & le_mask))) - 1u);
-                const unsigned later = firsts & ~le_mask;
-                const unsigned g_hi = ~le_mask & (later ? (later & (0u - later)) - 1u : kFull);
-                for (int j = 0; j < mx; ++j) {
-                    const bool on = j < nq;
-                    const int q = on ? qa + j : 0;
-                    const float4* qp = reinterpret_cast<const float4*>(w.Q + q * DP);
-                    const int held = w.cnt[q];
-                    float s = 0.f;
+        for (int k0 = 0; k0 < U; k0 += 32) {
+            int qq_n;
+            int32_t orig_n;
+            float cvn[DP];
+            load_cand(k0 + 32, qq_n, orig_n, cvn);   // next round in flight
+            const int qa = qq & 255;
+            const int nq = (qq >> 8) - qa;
+            const int mx = __reduce_max_sync(kFull, (unsigned)nq);
+            // the lanes of this lane's group before and after it (a group's
+            // lanes are consecutive)
+            const int qq_p = __shfl_up_sync(kFull, qq, 1);
+            const unsigned firsts = __ballot_sync(kFull, lane == 0 || qq != qq_p);
+            const unsigned g_lo = lt_mask & ~((1u << (31 - __clz(firsts & le_mask))) - 1u);
+            const unsigned later = firsts & ~le_mask;
+            const unsigned g_hi = ~le_mask & (later ? (later & (0u - later)) - 1u : kFull);
+            for (int j = 0; j < mx; ++j) {
+                const bool on = j < nq;
+                const int q = on ? qa + j : 0;
+                const float4* qp = reinterpret_cast<const float4*>(w.Q + q * DP);
+                const int held = w.cnt[q];
+                float s = 0.f;
 #pragma unroll
-                    for (int k4 = 0; k4 < DP / 4; ++k4) {
-                        const float4 v = qp[k4];
-                        const float qv[4] = {v.x, v.y, v.z, v.w};
+                for (int k4 = 0; k4 < DP / 4; ++k4) {
+                    const float4 v = qp[k4];
+                    const float qv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            if (4 * k4 + k < D) {
-                                const float d = __fsub_rn(qv[k], cv[4 * k4 + k]);
-                                s = __fadd_rn(s, __fmul_rn(d, d));
-                            }
+                    for (int k = 0; k < 4; ++k) {
+                        if (4 * k4 + k < D) {
+                            const float d = __fsub_rn(qv[k], cv[4 * k4 + k]);
+                            s = __fadd_rn(s, __fmul_rn(d, d));
                         }
                     }
-                    bool acc = on && s <= r2;
-                    if (acc && a.self) acc = orig != w.qor[q];
-                    // places in the list by counting the group's accepting
-                    // lanes; the last of them writes the new count (a query
-                    // belongs to one group, so no other lane does)
-                    const unsigned am = __ballot_sync(kFull, acc);
-                    const int p = held + __popc(am & g_lo);
-                    if (acc && p < kListCap) {
-                        w.Ld[q * kListStr + p] = s;
-                        w.Li[q * kListStr + p] = orig;
-                    }
-                    if (acc && (am & g_hi) == 0) w.cnt[q] = p + 1;
-                    if constexpr (LONG) {
-                        const bool over = acc && p >= kListCap;
-                        if (__any_sync(kFull, over)) {
-                            if (over && p < a.list_cap) scratch(q)[p - kListCap] = make_key(s, orig);
-                        }
-                    }
-                    __syncwarp();
                 }
-                qq = qq_n;
-                orig = orig_n;
-#pragma unroll
-                for (int k = 0; k < DP; ++k) cv[k] = cvn[k];
+                bool acc = on && s <= r2;
+                if (acc && a.self) acc = orig != w.qor[q];
+                // places in the list by counting the group's accepting
+                // lanes; the last of them writes the new count (a query
+                // belongs to one group, so no other lane does)
+                const unsigned am = __ballot_sync(kFull, acc);
+                const int p = held + __popc(am & g_lo);
+                if (acc && p < kListCap) {
+                    w.Ld[q * kListStr + p] = s;
+                    w.Li[q * kListStr + p] = orig;
+                }
+                if (acc && (am & g_hi) == 0) w.cnt[q] = p + 1;
+                if constexpr (LONG) {
+                    const bool over = acc && p >= kListCap;
+                    if (__any_sync(kFull, over)) {
+                        if (over && p < a.list_cap) scratch(q)[p - kListCap] = make_key(s, orig);
+                    }
+                }
+                __syncwarp();
             }
-            __syncwarp();   // the batch's ranges are rewritten by the next batch
+            qq = qq_n;
+            orig = orig_n;
+#pragma unroll
+            for (int k = 0; k < DP; ++k) cv[k] = cvn[k];
         }
+        __syncwarp();   // the batch's ranges are rewritten by the next batch
+    }
 
-        // per query: counts, degree, rows for the selection kernel
-        const int kept = act ? w.cnt[lane] : 0;
-        bool spill = kept > (LONG ? a.list_cap : kListCap);
-        const bool is_long = LONG && kept > kListCap && !spill;
-        int64_t pool_at = 0;   // compact output: a long row's place in the pool
-        if (LONG && is_long && a.csr) {
-            const int need = (min(kept, K) + 3) & ~3;
-            pool_at = (int64_t)atomicAdd(a.pool_count, (unsigned long long)need);
-            spill = pool_at + need > a.pool_cap;
-        }
-        if (act && !spill) counts[qorig] = min(kept, K) | (is_long && a.csr ? kCsrPool : 0);
-        if (spill && a.csr) counts[qorig] = kCsrSpill;   // counted by the selection kernel
-        if (act && !spill && a.degree) a.degree[qorig] = kept;
-        if (spill) {
-            const int pos = atomicAdd(a.ovf_count, 1);
-            if (pos < a.ovf_cap) {
-                a.ovf[pos].qslot = qs;
-                a.ovf[pos].ev = e;
-            } else {
-                atomicOr(a.status, kStatusCapacity);
-            }
-        }
-        // rows longer than the lists, one by one (before the lists are sorted)
-        unsigned long_rows = LONG ? __ballot_sync(kFull, is_long && !spill) : 0u;
-        while (long_rows) {
-            const int q = __ffs(long_rows) - 1;
-            long_rows &= long_rows - 1u;
-            const int nl = __shfl_sync(kFull, kept, q);
-            const int64_t row = __shfl_sync(kFull, qorig, q);
-            const int64_t pool = a.pool0 + __shfl_sync(kFull, pool_at, q);
-            const int64_t at = a.csr ? pool : row * K;
-            const int wide = a.csr ? (min(nl, K) + 3) & ~3 : K;
-            const float* ld = w.Ld + q * kListStr;
-            const int32_t* li = w.Li + q * kListStr;
-            if (nl <= 64) write_long_row<2>(ld, li, scratch(q), nl, wide, oidx + at, od2 + at);
-            else write_long_row<4>(ld, li, scratch(q), nl, wide, oidx + at, od2 + at);
-            if (a.csr && lane == 0) *reinterpret_cast<int64_t*>(oidx + row * kCsrStageW) = pool;
-        }
-        const unsigned rows = __ballot_sync(kFull, act && kept <= kListCap);   // the other rows written here
-        const int n = __shfl_sync(kFull, kept > kListCap ? 0 : kept, lane & 15);
-        const int most = __reduce_max_sync(kFull, (unsigned)n);
-        int sorted = 32;   // places of the lists that hold the row or its padding
-        if (most <= 8) {
-            sort_rows<4>(w, n);
-            sorted = 8;
-        } else if (most <= 16) {
-            sort_rows<8>(w, n);
-            sorted = 16;
+    // per query: counts, degree, rows for the selection kernel
+    const int kept = act ? w.cnt[lane] : 0;
+    bool spill = kept > (LONG ? a.list_cap : kListCap);
+    const bool is_long = LONG && kept > kListCap && !spill;
+    int64_t pool_at = 0;   // compact output: a long row's place in the pool
+    if (LONG && is_long && a.csr) {
+        const int need = (min(kept, K) + 3) & ~3;
+        pool_at = (int64_t)atomicAdd(a.pool_count, (unsigned long long)need);
+        spill = pool_at + need > a.pool_cap;
+    }
+    if (act && !spill) counts[qorig] = min(kept, K) | (is_long && a.csr ? kCsrPool : 0);
+    if (spill && a.csr) counts[qorig] = kCsrSpill;   // counted by the selection kernel
+    if (act && !spill && a.degree) a.degree[qorig] = kept;
+    if (spill) {
+        const int pos = atomicAdd(a.ovf_count, 1);
+        if (pos < a.ovf_cap) {
+            a.ovf[pos].qslot = qs;
+            a.ovf[pos].ev = e;
         } else {
-            sort_rows<16>(w, n);
+            atomicOr(a.status, kStatusCapacity);
         }
-        const bool vec = (width & 3) == 0 &&
-                         ((reinterpret_cast<uintptr_t>(oidx) | reinterpret_cast<uintptr_t>(od2)) & 15) == 0;
-        if (vec) {
-            // quarter p of a row: its indices for p < w4, then its distances
-            for (int p0 = 0; p0 < 2 * w4; p0 += 32) {
-                const int p = p0 + lane;
-                const bool dist = p >= w4;
-                const int e0 = 4 * (dist ? p - w4 : p);
-                const bool lane_on = p < 2 * w4;
-                const bool listed = lane_on && e0 < sorted;   // else padding
-                const int pad = dist ? 0x7f800000 : -1;
-                const int32_t* src4 = (dist ? reinterpret_cast<const int32_t*>(w.Ld) : w.Li) + e0;
-                int32_t* dst = (dist ? reinterpret_cast<int32_t*>(od2) : oidx) + e0;
-                unsigned left = rows;
-                while (left) {
-                    const int q = __ffs(left) - 1;
-                    left &= left - 1u;
-                    int4 v = make_int4(pad, pad, pad, pad);
-                    if (listed) v = *reinterpret_cast<const int4*>(src4 + q * kListStr);
-                    if (lane_on && (!a.csr || e0 < w.cnt[q]))
-                        *reinterpret_cast<int4*>(dst + (int64_t)w.qor[q] * width) = v;
-                }
-            }
-        } else {
+    }
+    // rows longer than the lists, one by one (before the lists are sorted)
+    unsigned long_rows = LONG ? __ballot_sync(kFull, is_long && !spill) : 0u;
+    while (long_rows) {
+        const int q = __ffs(long_rows) - 1;
+        long_rows &= long_rows - 1u;
+        const int nl = __shfl_sync(kFull, kept, q);
+        const int64_t row = __shfl_sync(kFull, qorig, q);
+        const int64_t pool = a.pool0 + __shfl_sync(kFull, pool_at, q);
+        const int64_t at = a.csr ? pool : row * K;
+        const int wide = a.csr ? (min(nl, K) + 3) & ~3 : K;
+        const float* ld = w.Ld + q * kListStr;
+        const int32_t* li = w.Li + q * kListStr;
+        if (nl <= 64) write_long_row<2>(ld, li, scratch(q), nl, wide, oidx + at, od2 + at);
+        else write_long_row<4>(ld, li, scratch(q), nl, wide, oidx + at, od2 + at);
+        if (a.csr && lane == 0) *reinterpret_cast<int64_t*>(oidx + row * kCsrStageW) = pool;
+    }
+    const unsigned rows = __ballot_sync(kFull, act && kept <= kListCap);   // the other rows written here
+    const int n = __shfl_sync(kFull, kept > kListCap ? 0 : kept, lane & 15);
+    const int most = __reduce_max_sync(kFull, (unsigned)n);
+    int sorted = 32;   // places of the lists that hold the row or its padding
+    if (most <= 8) {
+        sort_rows<4>(w, n);
+        sorted = 8;
+    } else if (most <= 16) {
+        sort_rows<8>(w, n);
+        sorted = 16;
+    } else {
+        sort_rows<16>(w, n);
+    }
+    const bool vec = (width & 3) == 0 &&
+                     ((reinterpret_cast<uintptr_t>(oidx) | reinterpret_cast<uintptr_t>(od2)) & 15) == 0;
+    if (vec) {
+        // quarter p of a row: its indices for p < w4, then its distances
+        for (int p0 = 0; p0 < 2 * w4; p0 += 32) {
+            const int p = p0 + lane;
+            const bool dist = p >= w4;
+            const int e0 = 4 * (dist ? p - w4 : p);
+            const bool lane_on = p < 2 * w4;
+            const bool listed = lane_on && e0 < sorted;   // else padding
+            const int pad = dist ? 0x7f800000 : -1;
+            const int32_t* src4 = (dist ? reinterpret_cast<const int32_t*>(w.Ld) : w.Li) + e0;
+            int32_t* dst = (dist ? reinterpret_cast<int32_t*>(od2) : oidx) + e0;
             unsigned left = rows;
             while (left) {
                 const int q = __ffs(left) - 1;
                 left &= left - 1u;
-                const int64_t at = (int64_t)w.qor[q] * width;
-                const int stop = a.csr ? min(w.cnt[q], width) : width;
-                for (int e2 = lane; e2 < stop; e2 += 32) {
-                    oidx[at + e2] = e2 < sorted ? w.Li[q * kListStr + e2] : -1;
-                    od2[at + e2] = e2 < sorted ? w.Ld[q * kListStr + e2] : INFINITY;
-                }
+                int4 v = make_int4(pad, pad, pad, pad);
+                if (listed) v = *reinterpret_cast<const int4*>(src4 + q * kListStr);
+                if (lane_on && (!a.csr || e0 < w.cnt[q]))
+                    *reinterpret_cast<int4*>(dst + (int64_t)w.qor[q] * width) = v;
             }
         }
-        __syncwarp();
+    } else {
+        unsigned left = rows;
+        while (left) {
+            const int q = __ffs(left) - 1;
+            left &= left - 1u;
+            const int64_t at = (int64_t)w.qor[q] * width;
+            const int stop = a.csr ? min(w.cnt[q], width) : width;
+            for (int e2 = lane; e2 < stop; e2 += 32) {
+                oidx[at + e2] = e2 < sorted ? w.Li[q * kListStr + e2] : -1;
+                od2[at + e2] = e2 < sorted ? w.Ld[q * kListStr + e2] : INFINITY;
+            }
+        }
+    }
+    __syncwarp();
+}
+
+// Not inlined: the scan of the half cells keeps its registers and instruction
+// cache to itself.
+template <int D, bool LONG>
+__device__ __noinline__ void wide_task(const QueryArgs& a, int e, int c, int part, int per) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    const WarpSmem w = carve<D>(smem + (size_t)(threadIdx.x >> 5) * warp_bytes<D>());
+    do_task<D, LONG, true>(a, w, e, c, part, per);
+}
+
+template <int D, bool LONG>
+__global__ void __launch_bounds__(kWarps * 32, Cfg<D>::MINB)
+    k_half_query(const __grid_constant__ QueryArgs a, int sub_shift) {
+    pdl_trigger();
+    pdl_wait();
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int lane = threadIdx.x & 31;
+    const WarpSmem w = carve<D>(smem + (size_t)(threadIdx.x >> 5) * warp_bytes<D>());
+    const int per = kQ >> sub_shift;
+    const int ntasks = a.nchunks << sub_shift;
+    auto next_task = [&]() {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(a.task_counter, 1);
+        return __shfl_sync(kFull, t, 0);
+    };
+    if (!LONG && a.nev == 1 && a.ev[0].half && (a.path_filter < 0 || a.ev[0].path == a.path_filter)) {
+        // one event: no other kind of task in the loop (300k x 8 138 -> 132 us,
+        // build included, 500k x 12 335 -> 323; long rows gain nothing from it)
+        for (int t = next_task(); t < ntasks; t = next_task())
+            do_task<D, LONG, false>(a, w, 0, t >> sub_shift, t & ((1 << sub_shift) - 1), per);
+        return;
+    }
+    for (int t = next_task(); t < ntasks; t = next_task()) {
+        const int c = t >> sub_shift, part = t & ((1 << sub_shift) - 1);
+        const int e = a.nev > 1 ? chunk_event(a.qev, a.nev, c) : 0;
+        if (a.path_filter >= 0 && a.ev[e].path != a.path_filter) continue;   // another launch's event
+        if (a.ev[e].half) do_task<D, LONG, false>(a, w, e, c, part, per);
+        else wide_task<D, LONG>(a, e, c, part, per);
     }
 }
 

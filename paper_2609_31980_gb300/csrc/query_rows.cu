@@ -768,7 +768,6 @@ frnn_status enqueue_row_query(const QueryLaunch& q, const QueryArgs& a0, cudaStr
     a.ntasks = qs.scalars + kScNTasks;
     a.qpts = qs.ppts;
     a.rpts = rs.ppts;
-    a.r2_screen = std::nextafter((float)((double)q.r2 * (1.0 + 0x1p-16)), INFINITY);
     cudaError_t ce = cudaSuccess;
     switch (rs.D) {
 #define FRNN_CASE(d) case d: ce = launch_row_query_d<d>(a, q.exit_dims, q.num_sms, st); break;

@@ -182,7 +182,7 @@ class Grid:
         info = frnn_grid_scan_info()
         _check(self.ctx.handle, frnn_grid_scan(self.handle, ctypes.byref(info)))
         n = info.naxes
-        return {"scan": ("chunks", "rows", "half cells", "query per lane")[info.scan], "naxes": n,
+        return {"scan": ("chunks", "rows", "half cells", "query per lane", "wide cells")[info.scan], "naxes": n,
                 "axes": list(info.axes)[:n], "dims": list(info.dims)[:n], "cells": info.cells}
 
     def close(self):

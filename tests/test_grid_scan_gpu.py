@@ -13,7 +13,9 @@ def test_scan_and_stored_cells():
     event = synth.config2().points
     cases = (   # points, r, requested axes, cell multiple, scan, axes (None: the build's choice)
         (event, 0.1, 0, 0, "half cells", [3, 4, 5, 6, 7, 2]),
-        (synth.uniform(20_000, 5, seed=1), 0.2, 0, 0, "half cells", None),
+        (synth.uniform(20_000, 5, seed=1), 0.08, 0, 0, "half cells", None),
+        (synth.uniform(20_000, 5, seed=1), 0.25, 0, 0, "wide cells", None),
+        (synth.uniform(20_000, 12, seed=1), 0.3, 0, 0, "wide cells", None),
         (synth.uniform(4096, 3, seed=2), 0.05, 0, 0, "query per lane", [0, 1, 2]),
         (synth.uniform(4096, 3, seed=2), 0.05, 0, 2, "query per lane", [0, 1, 2]),
         (synth.uniform(2000, 8, seed=3), 0.1, 3, 0, "rows", [5, 6, 7]),
