@@ -113,28 +113,30 @@ __global__ void __launch_bounds__(kWarps * 32, BIG ? 1 : (D <= 8 ? 8 : (D <= 12 
     const bool count_only = a.ovf_mode == 1;
     const bool csr_rows = a.ovf_mode == 2;
     const unsigned lt_mask = (1u << lane) - 1u;
+    // a warp has every stride-th row of the list; the second pass looks for the
+    // marked ones 32 at a time (rows next to each other in the list, which come
+    // from the same dense place, go to different warps: uniform 3000 x 3, K =
+    // 300, degrees of 1,500, 0.35 ms, with 32 consecutive rows a warp 3.1)
     const int stride = gridDim.x * kWarps;
-    // the first pass takes the list's rows one by one; the second looks for the
-    // marked ones 32 entries at a time
-    int w = (blockIdx.x * kWarps + warp) * (BIG ? 32 : 1) - (BIG ? 0 : stride);
+    int64_t w = (int64_t)blockIdx.x * kWarps + warp - (BIG ? 0 : stride);
+    int64_t w_base = 0;
     unsigned marked = 0;
-    int w_base = 0;
     for (;;) {
         if constexpr (BIG) {
             while (!marked && w < nov) {
-                const int i = w + lane;
+                const int64_t i = w + (int64_t)lane * stride;
                 marked = __ballot_sync(kFull, i < nov && a.ovf[i].ev < 0);
                 w_base = w;
-                w += stride * 32;
+                w += (int64_t)stride * 32;
             }
             if (!marked) break;
         } else {
             w += stride;
             if (w >= nov) break;
         }
-        int at_entry = w;
+        int64_t at_entry = w;
         if constexpr (BIG) {
-            at_entry = w_base + __ffs(marked) - 1;
+            at_entry = w_base + (int64_t)(__ffs(marked) - 1) * stride;
             marked &= marked - 1u;
         }
         const Overflow o = a.ovf[at_entry];
