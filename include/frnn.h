@@ -379,8 +379,8 @@ typedef enum frnn_option {
                                  choice (the smallest expected neighbourhood
                                  under the cell budget among min(D, 5) axes,
                                  one fewer and, from D = 6, one more), from
-                                 D = 9 four for up to 16,384 points or under
-                                 a memory budget.
+                                 D = 9 four for up to 16,384 points, under a
+                                 memory budget or with a cell multiple above 1.
                                  Grids requested with 1..4 axes are scanned by
                                  16-query row tasks, five-axis and automatic
                                  ones by 16-query chunks.  The cell multiple

@@ -343,19 +343,22 @@ static int build_mult(const frnn_ctx* ctx, int64_t N, int D) {
 }
 // gridded axes when neither the option nor the tuner fixes them: 0, the
 // build's automatic choice (all of them for D < 5; from D = 5 half cells, six
-// to four axes).  From D = 9 three kinds of sets keep four axes and the
-// row-task scan: up to kRowsDefaultMax points, where that grid is the
-// documented default that frnn_grid_params reports (the half-cell scan is the
-// faster one there too: 13k x 12 points 41 against 61 us, build + query);
-// contexts with a memory budget, whose calls were sized for the four-axis
-// grid's smaller cell array; and batches whose cell arrays would not fit
-// their 2^30 entries.  Measured above that line (build + query, K = 64, row
+// to four axes, or plain cells where an axis holds few).  From D = 9 four kinds
+// of sets keep four axes and the row-task scan: up to kRowsDefaultMax points,
+// where that grid is the documented default that frnn_grid_params reports (the
+// half-cell scan is the faster one there too: 13k x 12 points 41 against 61 us,
+// build + query); contexts with a memory budget, whose calls were sized for the
+// four-axis grid's smaller cell array; batches whose cell arrays would not fit
+// their 2^30 entries; and requested cell multiples above 1, which half cells do
+// not have (60k x 12 uniform, r = 0.3: chunk scan of the automatic axes 2.45 ms,
+// row tasks 1.73).  Measured above the line of points (build + query, K = 64, row
 // tasks / half cells): 20k x 12 65 / 44 us, 100k x 12 128 / 77, 300k x 9
 // 313 / 167, 300k x 16 327 / 235.
 constexpr int64_t kRowsDefaultMax = 16384;
 constexpr int64_t kHalfBatchMax = (int64_t)1 << 26;   // points of a batch
 static int default_naxes(const frnn_ctx* ctx, int64_t N, int D) {
-    return D >= 9 && (N <= kRowsDefaultMax || ctx->budget != 0 || ctx->batch_points > kHalfBatchMax) ? 4 : 0;
+    return D >= 9 && (N <= kRowsDefaultMax || ctx->budget != 0 || ctx->batch_points > kHalfBatchMax ||
+                      ctx->cell_mult > 1) ? 4 : 0;
 }
 static int build_naxes(const frnn_ctx* ctx, int64_t N, int D) {
     if (ctx->grid_naxes > 0) return std::min(ctx->grid_naxes, D);
