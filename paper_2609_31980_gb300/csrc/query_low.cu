@@ -18,9 +18,9 @@
 //   * a persistent grid; a warp takes 32 query slots (two chunks) at a time
 //     from an atomic counter; every lane carries its own event's parameters, so
 //     a warp may straddle the events of a batch.  Sets too small to fill the
-//     chip give each query G = 2, 4 or 8 lanes, which share its neighbour rows
-//     (a query's search is a serial chain: 4096 x 4 points, G = 1 53 us, build
-//     included);
+//     chip give each query G = 4 or 8 lanes, which share its neighbour rows,
+//     every G-th to a lane (a query's search is a serial chain: 4096 x 4 points,
+//     G = 1 53 us, build included);
 //   * each lane looks up kRows neighbour rows at a time, all loads in flight,
 //     and keeps the non-empty ranges in its column of a shared-memory table;
 //     it then walks them back to back, two candidates a step, moving to its
@@ -240,10 +240,15 @@ __global__ void __launch_bounds__(kWarps * 32, kMinBlocks) k_low_query(QueryArgs
                 }
             }
             const int self_slot = a.self ? qs : -1;
-            // the neighbour rows' offsets, counted like digits
-            int d0 = naxes > 1 ? -m : 0, d1 = naxes > 2 ? -m : 0, d2 = naxes > 3 ? -m : 0;
+            // the neighbour rows' offsets, counted like digits of base 2m + 1;
+            // of a query's G lanes each takes every G-th row
+            const int side = 2 * m + 1, first = G > 1 ? lane % G : 0;
+            const int step0 = G % side, step1 = G / side;   // (below side: G <= 8)
+            int d0 = (naxes > 1 ? -m : 0) + first % side;
+            int d1 = (naxes > 2 ? -m : 0) + first / side % side;
+            int d2 = (naxes > 3 ? -m : 0) + first / side / side;
             const int row0 = row * dims0;
-            for (int l0 = 0; l0 < nrows; l0 += kRows) {
+            for (int l0 = first; l0 < nrows; l0 += kRows * G) {
                 int k = 0;
                 {
                     int lo[kRows], hi[kRows];
@@ -251,7 +256,7 @@ __global__ void __launch_bounds__(kWarps * 32, kMinBlocks) k_low_query(QueryArgs
                     for (int j = 0; j < kRows; ++j) {
                         lo[j] = 0;
                         hi[j] = 0;
-                        const bool ok = l0 + j < nrows && (G == 1 || (l0 + j) % G == lane % G) && (unsigned)(cc[0] + d0) < (unsigned)dm[0] &&
+                        const bool ok = l0 + j * G < nrows && (unsigned)(cc[0] + d0) < (unsigned)dm[0] &&
                                         (unsigned)(cc[1] + d1) < (unsigned)dm[1] &&
                                         (unsigned)(cc[2] + d2) < (unsigned)dm[2];
                         if (ok) {
@@ -259,10 +264,23 @@ __global__ void __launch_bounds__(kWarps * 32, kMinBlocks) k_low_query(QueryArgs
                             lo[j] = __ldg(cells + at + x0);
                             hi[j] = __ldg(cells + at + x1);
                         }
-                        if (++d0 > m) {
-                            d0 = -m;
-                            if (++d1 > m) {
-                                d1 = -m;
+                        if constexpr (G == 1) {
+                            if (++d0 > m) {
+                                d0 = -m;
+                                if (++d1 > m) {
+                                    d1 = -m;
+                                    ++d2;
+                                }
+                            }
+                        } else {
+                            d0 += step0;
+                            d1 += step1;
+                            if (d0 > m) {
+                                d0 -= side;
+                                ++d1;
+                            }
+                            if (d1 > m) {
+                                d1 -= side;
                                 ++d2;
                             }
                         }
@@ -478,14 +496,17 @@ cudaError_t launch_g(const QueryArgs& a, int num_sms, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// lanes per query: one, more while that leaves resident warps without a task
+// lanes per query: one, more while that leaves resident warps without a task.
+// Never two: half the rows a lane, but places in the lists from a counter
+// (build + query, cells of r / r/2, us: 30,000 x 4 G = 1 50 / 77, G = 2 58 / 112,
+// G = 4 46 / 89; 50,000 x 4 62 / 102, 68 / 140, 58 / 128; 20,000 x 4 -, 51 / 100,
+// 38 / 78; 30,000 x 3 38 / 42, 38 / 50, 41 / 41).
 template <int D>
 cudaError_t launch(const QueryArgs& a, int num_sms, cudaStream_t st) {
     // (half the resident warps: 20,000 x 2 points 33.5 us with G = 4, 35 with 8)
     const int64_t warps = (int64_t)num_sms * kMinBlocks * kWarps / 2;
     const int64_t tasks = ceil_div(a.nchunks, 2);   // with one lane a query
-    if (tasks >= warps) return launch_g<D, 1>(a, num_sms, st);
-    if (2 * tasks >= warps) return launch_g<D, 2>(a, num_sms, st);
+    if (2 * tasks >= warps) return launch_g<D, 1>(a, num_sms, st);
     if (4 * tasks >= warps) return launch_g<D, 4>(a, num_sms, st);
     return launch_g<D, 8>(a, num_sms, st);
 }
