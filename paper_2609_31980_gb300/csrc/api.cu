@@ -103,6 +103,7 @@ struct frnn_ctx {
     bool csr_pending = false;
     QueryLaunch csr_q{};
     int64_t csr_M = 0, csr_E = 0;
+    int64_t csr_listed = 0;   // rows the fill's selection writes
     const int64_t* csr_off = nullptr;
     // kernel timing (FRNN_OPT_KERNEL_TIMING): event pairs, reused across reads
     int ktime = 0;
@@ -805,7 +806,7 @@ frnn_status frnn_query(frnn_ctx* ctx, const frnn_grid* grid, const float* querie
     return query_impl(ctx, grid, queries, M, r, K, flags, counts, idx, dist2, nullptr, nullptr);
 }
 
-static frnn_status csr_reserve(frnn_ctx* ctx, int64_t M, int K) {
+static frnn_status csr_reserve(frnn_ctx* ctx, int64_t M, int K, bool half_scan) {
     auto al = [](size_t x) { return (x + 255) / 256 * 256; };
     const size_t rows = (size_t)std::max<int64_t>(M, 1);
     const size_t b_cnt = al(rows * 4);
@@ -813,8 +814,8 @@ static frnn_status csr_reserve(frnn_ctx* ctx, int64_t M, int K) {
     // calls whose scan keeps rows longer than a staging row (never under a
     // memory budget): behind the staging rows a pool of as many entries for
     // them (none if it cannot be had), and the counter of those taken
-    ensure_scratch(ctx, K);
-    const bool long_rows = K > kLongK && ctx->scratch != nullptr;
+    if (half_scan) ensure_scratch(ctx, K);
+    const bool long_rows = half_scan && K > kLongK && ctx->scratch != nullptr;
     const auto stage_bytes = [&](bool pool) { return al(rows * kCsrStageW * 4 * (pool ? 2 : 1)); };
     const auto total = [&](bool pool) { return b_cnt + 2 * stage_bytes(pool) + b_parts + (long_rows ? 256 : 0); };
     bool pool = long_rows;
@@ -865,8 +866,9 @@ static frnn_status csr_reserve(frnn_ctx* ctx, int64_t M, int K) {
 }
 
 // The count pass of the compact output, enqueued: the search with staged
-// rows, the offset scan, and the copy of the edge count into page-locked
-// *h_edges (valid once the stream reaches it).  q: the search's launch.
+// rows, the offset scan, and the copy of the edge count and of the number of
+// rows left to the selection kernel into page-locked (*h_edges)[0..1] (valid
+// once the stream reaches them).  q: the search's launch.
 static frnn_status csr_count_enqueue(frnn_ctx* ctx, const frnn_grid* grid, const float* queries,
                                      int64_t M, float r, int K, unsigned flags, int64_t* offsets,
                                      int32_t* degree, int64_t** h_edges, QueryLaunch* q) {
@@ -874,7 +876,7 @@ static frnn_status csr_count_enqueue(frnn_ctx* ctx, const frnn_grid* grid, const
     int32_t dummy = 0;   // check_query_args wants row outputs: the staging is ours
     frnn_status s = check_query_args(ctx, M, r, K, flags, &dummy, &dummy, reinterpret_cast<float*>(&dummy));
     if (s != FRNN_OK) return s;
-    s = csr_reserve(ctx, M, K);
+    s = csr_reserve(ctx, M, K, grid->half && !use_tc_path(ctx, grid->D, flags, grid->N, K, grid->naxes));
     if (s != FRNN_OK) return s;
     *q = QueryLaunch{};
     if (M > 0) {
@@ -883,9 +885,11 @@ static frnn_status csr_count_enqueue(frnn_ctx* ctx, const frnn_grid* grid, const
                        ctx->csr_d2, &cp, q);
         if (s != FRNN_OK) return s;
     }
-    enqueue_csr_offsets(ctx->csr_cnt, M, ctx->csr_parts, offsets, ctx->stream);
+    int64_t* totals = reinterpret_cast<int64_t*>(ctx->d_status + 4);   // (the status block has room)
+    enqueue_csr_offsets(ctx->csr_cnt, M, ctx->csr_parts, offsets,
+                        q->qset ? q->qset->scalars + kScOvfCount : nullptr, totals, ctx->stream);
     *h_edges = reinterpret_cast<int64_t*>(ctx->h_status + 2);
-    cudaError_t e = cudaMemcpyAsync(*h_edges, offsets + M, sizeof(int64_t), cudaMemcpyDeviceToHost,
+    cudaError_t e = cudaMemcpyAsync(*h_edges, totals, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost,
                                     ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "reading the edge count");
     return FRNN_OK;
@@ -904,10 +908,11 @@ frnn_status frnn_query_csr_count(frnn_ctx* ctx, const frnn_grid* grid, const flo
     if (s != FRNN_OK) return s;
     s = frnn_sync(ctx);
     if (s != FRNN_OK) return s;
-    *n_edges = *h_edges;
+    *n_edges = h_edges[0];
     ctx->csr_q = q;
     ctx->csr_M = M;
-    ctx->csr_E = *h_edges;
+    ctx->csr_E = h_edges[0];
+    ctx->csr_listed = h_edges[1];
     ctx->csr_off = offsets;
     ctx->csr_pending = true;
     return FRNN_OK;
@@ -930,9 +935,13 @@ frnn_status frnn_query_csr_fill(frnn_ctx* ctx, int32_t* idx, float* dist2) {
     q.idx = idx;
     q.dist2 = dist2;
     q.degree = nullptr;
-    std::string err;
-    frnn_status s = enqueue_overflow_only(q, ctx->stream, err);
-    if (s != FRNN_OK) return fail(ctx, s, err);
+    if (ctx->csr_listed > 0) {
+        std::string err;
+        frnn_status s = enqueue_overflow_only(q, ctx->stream, err);
+        if (s != FRNN_OK) return fail(ctx, s, err);
+    } else {
+        q.qset->ovf_stale = false;   // (the list is empty)
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "compact-output gather launch");
     return FRNN_OK;
@@ -1294,7 +1303,7 @@ frnn_status frnn_self_query_host_csr(frnn_ctx* ctx, const float* refs_host, int6
     cut[0] = 0;
     cut[kParts] = N;
     for (int p = 1; p < kParts; ++p) cut[p] = std::min<int64_t>(N, (N * p / kParts + 31) / 32 * 32);
-    int64_t* h_cut = h_edges + 1;
+    int64_t* h_cut = h_edges + 2;
     for (int p = 1; p < kParts && e == cudaSuccess; ++p)
         e = cudaMemcpyAsync(h_cut + (p - 1), d_off + cut[p], sizeof(int64_t), cudaMemcpyDeviceToHost,
                             ctx->stream);

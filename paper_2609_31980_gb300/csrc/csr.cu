@@ -8,10 +8,15 @@
 //
 // Here the search runs once.  Its kernels write every row (sorted, at most 32
 // entries) into a staging area of the context, 32 entries per original query
-// index, and its count into cnt[i]; rows longer than the in-kernel list are
-// marked (kCsrSpill) and counted exactly by the selection kernel.  Then:
+// index, and its count into cnt[i].  The half-cell scan keeps rows of up to 128
+// entries in calls with K > 128: those past 32 lie in a pool behind the staging
+// rows (kCsrPool; the first pool entry's index in the staging row).  Rows longer
+// than the scan keeps are marked (kCsrSpill) and counted exactly by the
+// selection kernel.  Then:
 //   * k_csr_reduce / k_csr_scan_parts / k_csr_down: exclusive int64 prefix
-//     scan of the counts -> offsets[0..M] (offsets[M] = number of edges);
+//     scan of the counts -> offsets[0..M] (offsets[M] = number of edges); the
+//     number of marked rows goes to the host with it, so that a fill pass
+//     without any launches no selection;
 //   * k_csr_gather: after the caller has allocated offsets[M] entries, copies
 //     each unmarked row from the staging area to [offsets[i], offsets[i+1]);
 //     the marked rows are written there by the selection kernel.
@@ -99,9 +104,11 @@ __global__ void __launch_bounds__(kCsrThreads) k_csr_scan_parts(int64_t* parts, 
 }
 
 // offsets of one chunk: the chunk's exclusive scan plus its part's prefix;
-// the last chunk also writes offsets[M]
+// the last chunk also writes offsets[M], and for the host that number and the
+// rows left to the selection kernel (listed: NULL: none)
 __global__ void __launch_bounds__(kCsrThreads) k_csr_down(const int32_t* cnt, int64_t M,
-                                                          const int64_t* parts, int64_t* offsets) {
+                                                          const int64_t* parts, int64_t* offsets,
+                                                          const int32_t* listed, int64_t* totals) {
     pdl_trigger();
     pdl_wait();
     __shared__ int64_t warp_tot[kCsrThreads / 32];
@@ -120,8 +127,12 @@ __global__ void __launch_bounds__(kCsrThreads) k_csr_down(const int32_t* cnt, in
         if (base + k < M) offsets[base + k] = ex;
         ex += v[k];
     }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0)
-        offsets[M] = tot + (parts ? parts[blockIdx.x] : 0);
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+        const int64_t edges = tot + (parts ? parts[blockIdx.x] : 0);
+        offsets[M] = edges;
+        totals[0] = edges;
+        totals[1] = listed ? *listed : 0;
+    }
 }
 
 // One warp per kGatherRows consecutive rows: a row's entries lie side by side
@@ -204,13 +215,14 @@ __global__ void __launch_bounds__(256) k_csr_gather(const int32_t* cnt, const in
 }  // namespace
 
 void enqueue_csr_offsets(const int32_t* cnt, int64_t M, int64_t* parts, int64_t* offsets,
-                         cudaStream_t st) {
+                         const int32_t* listed, int64_t* totals, cudaStream_t st) {
     const int64_t nb = std::max<int64_t>(1, ceil_div(M, kCsrChunk));
     if (nb > 1) {
         launch_pdl(k_csr_reduce, dim3((unsigned)nb), dim3(kCsrThreads), 0, st, cnt, M, parts);
         launch_pdl(k_csr_scan_parts, dim3(1), dim3(kCsrThreads), 0, st, parts, nb);
     }
-    launch_pdl(k_csr_down, dim3((unsigned)nb), dim3(kCsrThreads), 0, st, cnt, M, nb > 1 ? parts : nullptr, offsets);
+    launch_pdl(k_csr_down, dim3((unsigned)nb), dim3(kCsrThreads), 0, st, cnt, M, nb > 1 ? parts : nullptr, offsets,
+               listed, totals);
 }
 
 int64_t csr_parts_needed(int64_t M) { return std::max<int64_t>(1, ceil_div(M, kCsrChunk)); }

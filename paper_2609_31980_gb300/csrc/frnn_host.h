@@ -215,10 +215,11 @@ cudaError_t enqueue_low_query(const QueryArgs& a, int num_sms, cudaStream_t st);
 // (compact output, second pass: q.ovf_mode 2, q.row_off).
 frnn_status enqueue_overflow_only(const QueryLaunch& q, cudaStream_t st, std::string& err);
 // Compact output (csr.cu): offsets[0..M] from the marked counts; the gather
-// of the staged rows.  parts: csr_parts_needed(M) int64 scratch.
+// of the staged rows.  parts: csr_parts_needed(M) int64 scratch.  totals[0..1]
+// (device): the edges, and *listed, the rows in the query's selection list.
 int64_t csr_parts_needed(int64_t M);
 void enqueue_csr_offsets(const int32_t* cnt, int64_t M, int64_t* parts, int64_t* offsets,
-                         cudaStream_t st);
+                         const int32_t* listed, int64_t* totals, cudaStream_t st);
 // cap: entries idx / dist2 hold; entries at or past it are not written.
 // [row0, row1): the rows gathered (row0 a multiple of 32; row1 < 0: to M).
 void enqueue_csr_gather(const int32_t* cnt, const int64_t* offsets, const int32_t* sidx,

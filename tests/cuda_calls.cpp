@@ -9,7 +9,7 @@
 namespace {
 constexpr int kMax = 4096;
 struct Call {
-    int kind;   // 1 cudaMalloc, 2 cudaMemsetAsync, 3 cudaMemcpyAsync, 4 refused launch
+    int kind;   // 1 cudaMalloc, 2 cudaMemsetAsync, 3 cudaMemcpyAsync, 4 refused launch, 5 launch
     size_t bytes;
 };
 Call g_calls[kMax];
@@ -47,6 +47,7 @@ cudaError_t __wrap_cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* 
             return cudaErrorInvalidClusterSize;
         }
     }
+    note(5, 0);
     return __real_cudaLaunchKernelExC(c, f, a);
 }
 

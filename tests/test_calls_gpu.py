@@ -130,3 +130,41 @@ def test_serving_allocates_before_the_first_request(listed_lib):
             for p, o in zip(ev, outs):
                 same([torch.from_numpy(x) for x in o], p, 0.1, 200)
         """)
+
+
+def test_compact_queries_without_long_rows_launch_no_second_selection(listed_lib):
+    """Search, its selection, offsets, gather: nothing more when the count pass
+    left no row to the selection, whatever K; the rows when it did."""
+    _child(listed_lib, """
+        for D, n in ((3, 3000), (8, 3000), (12, 3000), (8, 20_000)):
+            p = synth.clustered(n // 50, 10, n - n // 50 * 10, D, 0.01, seed=75)
+            long = p.copy()
+            long[:700] = long[0] + np.random.default_rng(1).uniform(-1e-3, 1e-3, (700, D)).astype(np.float32)
+            with frnn.Context() as ctx:
+                for K in (64, 200):
+                    for pts, r in ((p, 0.02), (long, 0.02), (p, 0.02)):
+                        t = torch.from_numpy(pts).cuda()
+                        g = ctx.build_grid(t, r)
+                        ctx.query(g, t, r, K)      # (per-build preparation)
+                        ctx.query_csr(g, t, r, K)
+                        ctx.sync()
+                        lib.calls_reset()
+                        off, i, d, _ = ctx.query_csr(g, t, r, K)
+                        launches = sum(k == 5 for k, _ in calls())
+                        memsets = sum(k == 2 for k, _ in calls())
+                        ctx.sync()
+                        c = np.diff(off.cpu().numpy())
+                        rows = np.arange(0, n, 7)
+                        want = oracle.self_query(pts, r, K, rows=rows)
+                        assert np.array_equal(c[rows], want[0])
+                        off, i, d = off.cpu().numpy(), i.cpu().numpy(), d.cpu().numpy()
+                        for k, row in enumerate(rows):
+                            assert np.array_equal(i[off[row]:off[row + 1]], want[1][k, :want[0][k]])
+                        half = g.scan()["scan"] in ("half cells", "wide cells")
+                        assert memsets == (1 if half and K > 128 else 0), (D, n, K, calls())
+                        parts = 2 if n > 8192 else 0
+                        if pts is p:
+                            assert launches == 4 + parts, (D, n, K, launches)
+                        else:
+                            assert launches > 4 + parts, (D, n, K, launches)
+        """)
