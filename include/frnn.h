@@ -114,7 +114,8 @@ frnn_status frnn_destroy(frnn_ctx* ctx);
  * (r/m)(1+2^-10), m = the cell-multiple option, enlarged when needed so that
  * the cell count stays bounded.  The default grid of five or more dimensions
  * stores cells two by two along every axis but the first and may divide them
- * along one more coordinate.  The choice never changes results (the cell
+ * along one more coordinate, or has plain cells over four or five where an axis
+ * holds few (frnn_grid_scan).  The choice never changes results (the cell
  * assignment is proven conservative).  A non-finite coordinate makes frnn_sync return
  * FRNN_ERR_NONFINITE and later queries on the grid return no neighbours.
  */
@@ -146,8 +147,7 @@ frnn_status frnn_grid_params(const frnn_grid* grid, frnn_grid_info* info);
  * Synchronises the grid's context stream.  Errors: as frnn_grid_params. */
 typedef struct frnn_grid_scan_info {
     int scan;           /* 0 chunks of 16 queries, candidates on lanes
-                             (query.cu: five requested axes; default grids of
-                             D >= 5 with a cell multiple above 1)
+                             (query.cu: five requested axes)
                            1 row tasks of 16 queries (query_rows.cu: up to four
                              requested axes)
                            2 half cells: chunks of 16 queries, candidates on
@@ -316,14 +316,13 @@ const char* frnn_last_error(const frnn_ctx* ctx);
 /*
  * Autotuner.  Times the candidate configurations on the given point set (a
  * representative event, device memory, self-query): the automatic axis
- * choice with cell multiple m = 1 (scanned by chunks of 16 queries,
- * candidates on lanes; up to D = 4 with either candidate staging), four
+ * choice with cell multiple m = 1 (scanned as frnn_grid_scan says), four
  * coordinates with
  * m = 1 and three with m = 2 (scanned by 16-query row tasks, at the default
  * and a later warp vote); fewer axes when D is smaller; for D <= 4 the
  * automatic choice with m = 2 as well, and for D <= 3 with m = 3 (where
- * the chunk scan's 128-row neighbour table holds the (2m + 1)^(axes - 1)
- * rows); on each grid, the tensor-core pre-filter (D >= 8).
+ * the (2m + 1)^(axes - 1) neighbour rows are at most 128); on each grid,
+ * the tensor-core pre-filter (D >= 8).
  * Each candidate runs whole steps, build then query (first run untimed,
  * best of three timed with CUDA events on the context's stream, the L2
  * cache flushed before each run), and the fastest is cached for the event
@@ -342,7 +341,7 @@ typedef struct frnn_tune_result {
     int exit_dims;   /* warp vote point of the row-task scan (0 = default) */
     float ms;        /* build + query time of the winner, milliseconds */
     int grid_axes;   /* gridded coordinates requested (0: the automatic choice; 3 or 4) */
-    int staging;     /* grid scan candidate staging (FRNN_OPT_STAGING values 1, 2) */
+    int staging;     /* grid scan candidate staging (1: the candidates have one) */
 } frnn_tune_result;
 
 frnn_status frnn_autotune(frnn_ctx* ctx, const float* refs, int64_t N, int D, float r, int K,
@@ -379,21 +378,22 @@ typedef enum frnn_option {
                                  choice (the smallest expected neighbourhood
                                  under the cell budget among min(D, 5) axes,
                                  one fewer and, from D = 6, one more), from
-                                 D = 9 four for up to 16,384 points, under a
-                                 memory budget or with a cell multiple above 1.
-                                 Grids requested with 1..4 axes are scanned by
-                                 16-query row tasks, five-axis and automatic
-                                 ones by 16-query chunks.  The cell multiple
+                                 D = 9 four for up to 16,384 points or under
+                                 a memory budget.  Grids requested with 1..4
+                                 axes are scanned by 16-query row tasks, five
+                                 requested axes by 16-query chunks, automatic
+                                 ones as frnn_grid_scan says.  The cell multiple
                                  is lowered until the neighbour rows,
                                  (2m+1)^(axes-1), are at most 32 (row tasks)
-                                 or 128 (chunks). */
+                                 or 128 (chunks, D <= 4); it is 1 on automatic
+                                 grids of D >= 5. */
     FRNN_OPT_STAGING = 11     /* candidate staging of the grid scan: 1 each lane
                                  loads its candidate's row from global memory
                                  (L2), the next round in flight; 2 bulk copies
                                  (cp.async.bulk) of tiles into a shared-memory
-                                 ring; 0 (default): autotuned, else 1.  The
-                                 default grids of five or more dimensions and
-                                 row tasks have one staging each */
+                                 ring; 0 (default): autotuned, else 1.  For
+                                 the chunk scan (five requested axes); the
+                                 other scans have one staging each */
 } frnn_option;
 
 frnn_status frnn_set_option(frnn_ctx* ctx, frnn_option opt, int64_t value);
@@ -413,7 +413,9 @@ frnn_status frnn_get_option(const frnn_ctx* ctx, frnn_option opt, int64_t* value
  *   n_edges  host out: offsets[M], the entries the caller must allocate.
  * Synchronises the context's stream (the count has to reach the host).  The
  * context holds 8 * 32 + 4 bytes of staging per query, reused
- * across calls (charged to the memory budget).  Errors: those of frnn_query
+ * across calls (charged to the memory budget); without a budget, for K > 128 on
+ * default grids of D >= 5, 16 * 32 + 4 and, as every query there with such a K,
+ * a scratch array of about 52 MB for rows of 33 to 128 entries.  Errors: those of frnn_query
  * (INVALID_ARG, UNSUPPORTED, BUDGET, OUT_OF_MEMORY, NONFINITE, CAPACITY,
  * TIMEOUT, CUDA); NULL offsets or n_edges: INVALID_ARG. */
 frnn_status frnn_query_csr_count(frnn_ctx* ctx, const frnn_grid* grid, const float* queries,

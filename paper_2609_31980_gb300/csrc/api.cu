@@ -198,7 +198,7 @@ static int cap_axes(int naxes, int D) { return naxes > 0 ? naxes : std::min(D, k
 // by it.
 static CellKind cell_kind(const frnn_ctx* ctx, int64_t N, int D) {
     const int naxes = build_naxes(ctx, N, D);
-    if (half_cells(D, naxes, build_mult(ctx, N, D))) return CellKind::kHalf;
+    if (half_cells(D, naxes)) return CellKind::kHalf;
     return D <= 4 && naxes == 0 && ctx->budget == 0 && !ctx->small_cells ? CellKind::kLow : CellKind::kPlain;
 }
 
@@ -290,11 +290,11 @@ static frnn_status prepare_tc(frnn_ctx* ctx, GridBufs& g, const GridBufs& center
     return FRNN_OK;
 }
 
-// The grid scan for a grid requested with naxes gridded axes (0: the
-// build's automatic choice, five or four): the row-task kernel for grids
-// requested with up to four axes (cells holding many points, long candidate
-// streams shared by 16 queries), the chunk kernel otherwise (few points per
-// cell, candidates on lanes).
+// The grid scan for a grid requested with naxes gridded axes: 1, the row-task
+// kernel, for grids requested with up to four axes (cells holding many points,
+// long candidate streams shared by 16 queries); 0 otherwise: the chunk kernel
+// for five requested axes, and for the automatic choice (naxes 0) the half-cell
+// scan from D = 5 (half_cells), one query a lane up to D = 4.
 static int grid_kernel(int naxes) { return (naxes >= 1 && naxes <= 4) ? 1 : 0; }
 
 // Pair copy and tasks of a point set for the row-task kernel; accounted in
@@ -344,22 +344,19 @@ static int build_mult(const frnn_ctx* ctx, int64_t N, int D) {
 }
 // gridded axes when neither the option nor the tuner fixes them: 0, the
 // build's automatic choice (all of them for D < 5; from D = 5 half cells, six
-// to four axes, or plain cells where an axis holds few).  From D = 9 four kinds
+// to four axes, or plain cells where an axis holds few).  From D = 9 three kinds
 // of sets keep four axes and the row-task scan: up to kRowsDefaultMax points,
 // where that grid is the documented default that frnn_grid_params reports (the
 // half-cell scan is the faster one there too: 13k x 12 points 41 against 61 us,
 // build + query); contexts with a memory budget, whose calls were sized for the
-// four-axis grid's smaller cell array; batches whose cell arrays would not fit
-// their 2^30 entries; and requested cell multiples above 1, which half cells do
-// not have (60k x 12 uniform, r = 0.3: chunk scan of the automatic axes 2.45 ms,
-// row tasks 1.73).  Measured above the line of points (build + query, K = 64, row
+// four-axis grid's smaller cell array; and batches whose cell arrays would not
+// fit their 2^30 entries.  Measured above the line of points (build + query, K = 64, row
 // tasks / half cells): 20k x 12 65 / 44 us, 100k x 12 128 / 77, 300k x 9
 // 313 / 167, 300k x 16 327 / 235.
 constexpr int64_t kRowsDefaultMax = 16384;
 constexpr int64_t kHalfBatchMax = (int64_t)1 << 26;   // points of a batch
 static int default_naxes(const frnn_ctx* ctx, int64_t N, int D) {
-    return D >= 9 && (N <= kRowsDefaultMax || ctx->budget != 0 || ctx->batch_points > kHalfBatchMax ||
-                      ctx->cell_mult > 1) ? 4 : 0;
+    return D >= 9 && (N <= kRowsDefaultMax || ctx->budget != 0 || ctx->batch_points > kHalfBatchMax) ? 4 : 0;
 }
 static int build_naxes(const frnn_ctx* ctx, int64_t N, int D) {
     if (ctx->grid_naxes > 0) return std::min(ctx->grid_naxes, D);
@@ -384,15 +381,19 @@ static bool default_tc(const frnn_ctx* ctx, int64_t N, int D, int naxes) {
 // get a grid of their own for the tiles, three axes of cells of r / 2 (as on
 // request), made from the cell-sorted rows with the first tensor-core query
 // after a build and kept with its operands.
+// Up to kTilesMin points and queries (and where that grid cannot be had) the
+// tiles walk the half cells (D = 8 event sets, build + query, walk / own grid:
+// 2,000 142 / 158 us, 4,000 147 / 166, 6,000 178 / 172, 12,000 237 / 182).
 constexpr int kTcAxes = 3;
+constexpr int64_t kTilesMin = 5000;
 static int tc_mult(const frnn_ctx* ctx) { return ctx->cell_mult > 0 ? ctx->cell_mult : 2; }
 
-// The point set a tensor-core query of the grid takes.  Where that grid cannot
-// be had (the context's budget, memory, an allocation inside a caller's
+// The point set a tensor-core query of M points takes.  Where the tiles' grid
+// cannot be had (the context's budget, memory, an allocation inside a caller's
 // capture) the tiles walk the half cells: slower, the same rows.
-static GridBufs& tc_set(frnn_ctx* ctx, frnn_grid* grid) {
+static GridBufs& tc_set(frnn_ctx* ctx, frnn_grid* grid, int64_t M) {
     GridBufs& v = grid->tiles;
-    if (!grid->half || grid->N == 0) return grid->g;
+    if (!grid->half || grid->N == 0 || std::max(grid->N, M) < kTilesMin) return grid->g;
     if (grid->tiles_ready) return v;
     const int64_t cap = cells_for(ctx, grid->N, kTcAxes, CellKind::kPlain);
     const bool held = v.base && v.tc_base && v.cap_n >= grid->g.n_total && v.cap_L >= cell_entries(cap);
@@ -428,7 +429,7 @@ static GridBufs& tc_set(frnn_ctx* ctx, frnn_grid* grid) {
 static int batch_path(const frnn_ctx* ctx, int64_t n, int D, int K, unsigned flags) {
     if (use_tc_path(ctx, D, flags, n, K)) return 1;
     const int naxes = build_naxes(ctx, n, D);
-    if (half_cells(D, naxes, build_mult(ctx, n, D))) return 3;
+    if (half_cells(D, naxes)) return 3;
     return grid_kernel(naxes) == 1 ? 2 : 0;
 }
 
@@ -439,7 +440,7 @@ struct EventGrid {
 };
 static EventGrid event_grid(const frnn_ctx* ctx, int64_t n, int D, int K, unsigned flags) {
     EventGrid g{build_naxes(ctx, n, D), build_mult(ctx, n, D), 0};
-    if (half_cells(D, g.naxes, g.m) && use_tc_path(ctx, D, flags, n, K)) {   // (see tc_set)
+    if (half_cells(D, g.naxes) && use_tc_path(ctx, D, flags, n, K)) {   // (see tc_set)
         g = {kTcAxes, tc_mult(ctx), 0};
         g.cap = cells_for(ctx, n, g.naxes, CellKind::kPlain);
     } else {
@@ -662,7 +663,7 @@ frnn_status frnn_build_grid(frnn_ctx* ctx, const float* refs, int64_t N, int D, 
     g->naxes = o.naxes;
     g->axes_mode = o.axes_mode;
     g->tiles_ready = false;
-    g->half = half_cells(D, o.naxes, o.m);
+    g->half = half_cells(D, o.naxes);
     g->g.h_hdr[0].half = g->half ? 1 : 0;
     std::string err;
     const float* ev_refs[1] = {refs};
@@ -711,7 +712,7 @@ static frnn_status query_impl(frnn_ctx* ctx, const frnn_grid* grid, const float*
     if (M == 0) return FRNN_OK;
     const bool tc = use_tc_path(ctx, grid->D, flags, grid->N, K, grid->naxes);
     frnn_grid* mgrid = const_cast<frnn_grid*>(grid);   // tensor-core operands are a lazy cache
-    GridBufs& rg = tc ? tc_set(ctx, mgrid) : mgrid->g;
+    GridBufs& rg = tc ? tc_set(ctx, mgrid, M) : mgrid->g;
     QueryLaunch q{};
     q.rset = &rg;
     q.r2 = r * r;
@@ -1507,13 +1508,12 @@ frnn_status frnn_autotune(frnn_ctx* ctx, const float* refs, int64_t N, int D, fl
         ms = bestms;
         return frnn_sync(ctx);
     };
-    // grid configurations: the automatic axis choice (five axes, or four
-    // when the cell budget makes five-axis cells too coarse; chunk kernel),
-    // four axes with cells of r and three with cells of r/2 (row-task
-    // kernel); fewer for smaller D.  Cells of r/2 and r/3 on the automatic
-    // choice too, where its (2m + 1)^(axes - 1) neighbour rows stay within
-    // the chunk kernel's table (m = 2 up to D = 4, m = 3 up to D = 3):
-    // beyond that the grid lowers m and the configuration repeats another
+    // grid configurations: the automatic axis choice (half-cell scan, or one
+    // query a lane up to D = 4), four axes with cells of r and three with cells
+    // of r/2 (row-task kernel); fewer for smaller D.  Cells of r/2 and r/3 on
+    // the automatic choice too, where its (2m + 1)^(axes - 1) neighbour rows
+    // are at most kMaxNbrRows (m = 2 up to D = 4, m = 3 up to D = 3): beyond
+    // that the grid lowers m and the configuration repeats another
     struct GridCfg { int naxes, m; };
     std::vector<GridCfg> gcfg;
     auto add_cfg = [&](int na, int m) {
@@ -1534,16 +1534,13 @@ frnn_status frnn_autotune(frnn_ctx* ctx, const float* refs, int64_t N, int D, fl
         const int m = gcfg[gi].m;
         ctx->cell_mult = m;
         ctx->grid_naxes = gcfg[gi].naxes;
-        // the chunk kernel with either staging; the row-task kernel with its
-        // default vote point and a later one
+        // the automatic grids' scans have one form; the row-task kernel with
+        // its default vote point and a later one
         struct Cand { unsigned path; int staging, exit_dims; };
         std::vector<Cand> cands;
         if (!(flags & FRNN_PATH_TC)) {
             if (grid_kernel(gcfg[gi].naxes) == 0) {
                 cands.push_back({FRNN_PATH_GRID, 1, 0});
-                // the chunk scan's other staging (half cells and grids of up to
-                // four dimensions have scans of their own)
-                if (D > 4 && !half_cells(D, gcfg[gi].naxes, m)) cands.push_back({FRNN_PATH_GRID, 2, 0});
             } else {
                 cands.push_back({FRNN_PATH_GRID, 1, 0});
                 if (D >= 5) cands.push_back({FRNN_PATH_GRID, 1, 3});

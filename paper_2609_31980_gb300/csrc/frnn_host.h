@@ -121,9 +121,13 @@ void grid_free(GridBufs& g);
 void grid_clean(GridBufs& g, cudaStream_t st);
 
 // Whether a grid requested with naxes gridded axes (0: the automatic choice)
-// and cell multiple m stores half cells (EventHdr::half) for the half-cell
-// scan (query_half.cu): the automatic grids of five or more dimensions.
-inline bool half_cells(int D, int naxes, int m) { return naxes == 0 && m == 1 && D > 4; }
+// is made for the half-cell scan (query_half.cu, EventHdr::half): the automatic
+// grids of five or more dimensions.  Their cell multiple is 1, whatever was
+// requested: the neighbour rows of a larger one over five axes were too many for
+// the chunk scan too, which lowered it (60k x 12, requested 2, chunk scan / row
+// tasks / half cells: event, r = 0.12 83 / 97 / 57 us, uniform, r = 0.3 2.45 /
+// 1.74 / 1.72 ms).
+inline bool half_cells(int D, int naxes) { return naxes == 0 && D > 4; }
 
 struct BuildOpts {
     float r = 0.f;          // grid radius

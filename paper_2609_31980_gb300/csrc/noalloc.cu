@@ -151,7 +151,7 @@ frnn_status frnn_self_query_noalloc(const float* pts, int64_t N, int D, float r,
     GridBufs g;
     int32_t* status = carve(g, base, N, D);
     k_noalloc_tables<<<1, 32, 0, st>>>(g.hdr, g.blk_start, g.cell_off, pts, N,
-                                      (int32_t)na_cap(N), (int32_t)g.nblk, half_cells(D, 0, 1), status);
+                                      (int32_t)na_cap(N), (int32_t)g.nblk, half_cells(D, 0), status);
     BuildOpts o;
     o.r = r;
     o.m = 1;
@@ -165,7 +165,7 @@ frnn_status frnn_self_query_noalloc(const float* pts, int64_t N, int D, float r,
     q.K = K;
     q.self = 1;
     q.exit_dims = 0;
-    q.kernel = half_cells(D, 0, 1) ? 2 : 0;
+    q.kernel = half_cells(D, 0) ? 2 : 0;
     q.counts = counts;
     q.idx = idx;
     q.dist2 = dist2;

@@ -1,10 +1,8 @@
 // query.cu — the launch of every grid scan, and the chunk scan: per-warp scan of
 // the neighbouring cells with candidate tiles staged in shared memory by bulk
 // copies (or loaded directly), the exact float32 distance contract, and
-// warp-level top-K.  Grids of five requested axes use it, and automatic grids of
-// five or more dimensions with a cell multiple above 1; the other automatic
-// grids have query_half.cu and query_low.cu, up to four requested axes
-// query_rows.cu.
+// warp-level top-K.  Grids of five requested axes use it; automatic grids have
+// query_half.cu and query_low.cu, up to four requested axes query_rows.cu.
 //
 // Method (Eq. 1, Sec. 1): for each query, every reference in the cells within
 // +-m cells along each gridded axis is a candidate (complete by the grid's

@@ -20,7 +20,7 @@ def test_scan_and_stored_cells():
         (synth.uniform(4096, 3, seed=2), 0.05, 0, 2, "query per lane", [0, 1, 2]),
         (synth.uniform(2000, 8, seed=3), 0.1, 3, 0, "rows", [5, 6, 7]),
         (synth.uniform(2000, 8, seed=3), 0.1, 5, 0, "chunks", [3, 4, 5, 6, 7]),
-        (synth.uniform(2000, 8, seed=3), 0.3, 0, 2, "chunks", None),
+        (synth.uniform(2000, 8, seed=3), 0.05, 0, 2, "half cells", None),
         (synth.clustered(400, 25, 3000, 12, 0.025, seed=4), 0.12, 0, 0, "rows", [8, 9, 10, 11]))
     with frnn.Context() as ctx:
         for pts, r, naxes, mult, scan, axes in cases:
