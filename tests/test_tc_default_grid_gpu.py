@@ -22,7 +22,7 @@ def _pts(n, D, seed):
     return synth.clustered(n // 50, 40, n - n // 50 * 40, D, 0.01, seed=seed)
 
 
-@pytest.mark.parametrize("n,D,r,K", [(1, 8, 0.1, 8), (2001, 8, 0.1, 64), (16_385, 9, 0.1, 64),
+@pytest.mark.parametrize("n,D,r,K", [(1, 8, 0.1, 8), (2001, 8, 0.1, 64), (4999, 8, 0.1, 64), (5000, 8, 0.1, 64), (16_385, 9, 0.1, 64),
                                      (20_000, 12, 0.12, 200), (33_001, 16, 0.12, 64), (40_000, 13, 0.12, 20)])
 @pytest.mark.parametrize("axes", [0, 1])
 def test_rows_on_the_automatic_grid(n, D, r, K, axes):
