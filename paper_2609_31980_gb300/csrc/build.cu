@@ -3,7 +3,7 @@
 //
 // The uniform grid / cell list is the method of the original FRNN the paper
 // starts from (Sec. 2: uniform-grid kernel, spacing chosen so that r is an
-// integer multiple of it).  Here at most 5 coordinates are gridded; the cell
+// integer multiple of it).  Here at most six coordinates are gridded; the cell
 // assignment is "roundoff-safe" (Table 1): it provably never separates two
 // points the float32 contract accepts by more than m cells per axis (proof at
 // event_params below).

@@ -73,7 +73,8 @@ struct EventHdr {
     int32_t naxes;         // gridded axes (1..6); preset by the host: requested count (0: default)
     int32_t m;             // cell multiple: neighbours are within +-m cells per gridded axis
     int32_t valid;         // 0 if a coordinate was non-finite
-    // 1: a grid of half cells (preset by the host).  Cell coordinates are those
+    // 1: a grid of half cells (preset by the host; the build sets 0 where it takes
+    // plain cells instead, derive_params).  Cell coordinates are those
     // of a grid with m = 1, but along every axis except axes[0] two neighbouring
     // cells share one stored cell: stored coordinate = cell coordinate >> 1,
     // and the low bits say which half.  The cells within +-1 of cell c are then

@@ -2,7 +2,7 @@
 // tiles, followed by the exact float32 recheck of every survivor.
 //
 // The squared distance is written as n(x) + n(y) - 2 x.y, the dot products of
-// a 128-query tile with a chunk of up to 256 candidates computed by one
+// a 128-query tile with a chunk of up to 128 candidates computed by one
 // tcgen05.mma (kind::f16, BF16 operands, FP32 accumulator in tensor memory).
 // The filter only has to be conservative: every pair the float32 contract
 // accepts must pass it; each survivor is then recomputed with the exact
