@@ -60,15 +60,15 @@
 // 0.82 ms; 60k x 12, r = 0.3 1.76 / 6.0 / 1.72; 200k x 16, r = 0.22 5.8 / 23.2 /
 // 3.0; 20k x 10, r = 0.18 0.110 / 0.143 / 0.079.
 //
-// What bounds it: instruction issue (70 % of the slots, 84 M warp instructions
+// What bounds it: instruction issue (71 % of the slots, 80 M warp instructions
 // at 300k x 8 where the chunk scan over five axes took 143 M) and the
-// load/store pipe (65 %).  Kernel alone, 300k x 8, K = 64: 193 us (chunk scan)
+// load/store pipe (70 %).  Kernel alone, 300k x 8, K = 64: 193 us (chunk scan)
 // -> 129 (8 CTAs per SM, 64 registers, 100 B of spills, one shared-memory
 // atomic per accepted pair) -> 111 (7 CTAs, 72 registers) -> 105 (places in the
 // lists by ballots instead of atomics, whose same-address conflicts were a
-// fifth of the load/store pipe, and 32-byte row loads).  Build + query: 300k x
-// 8 242 -> 151 us, 300k x 5 1334 -> 199, 500k x 12 (four-axis row tasks) 523
-// -> 350, 20k x 8 66 -> 45.
+// fifth of the load/store pipe, and 32-byte row loads) -> 99 (a single event's
+// tasks in a loop of their own).  Build + query, chunk scan or four-axis row
+// tasks / now: 300k x 8 242 / 133 us, 500k x 12 523 / 323, 20k x 8 66 / 38.
 #include <algorithm>
 #include <climits>
 #include <type_traits>
