@@ -1009,8 +1009,11 @@ frnn_status tc_reserve(GridBufs& g, std::string& err) {
     g.tc_cap_tasks = tcap;
     g.tc_cap_E = g.E;
     g.tc_K = K;
-    // rows past the last slot stay zero (chunks may read them)
+    // rows past the last slot stay zero (chunks may read them).  Waited for: the
+    // call returns before the device has run it, and a context's stream that
+    // does not synchronise with the default one would write the operands first
     ce = cudaMemset(base, 0, 2 * bA + bn);
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(nullptr);
     if (ce != cudaSuccess) {
         cudaGetLastError();
         err = "zeroing tensor-core operands failed";
