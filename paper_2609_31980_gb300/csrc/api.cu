@@ -1628,8 +1628,9 @@ frnn_status frnn_set_option(frnn_ctx* ctx, frnn_option opt, int64_t value) {
             return FRNN_OK;
         case FRNN_OPT_TC_SURVIVORS:
         case FRNN_OPT_TC_ACCEPTED:
+            // in order with the context's queries, whatever the default stream does
+            cudaMemsetAsync(ctx->d_tcstat, 0, 2 * sizeof(unsigned long long), ctx->stream);
             cudaStreamSynchronize(ctx->stream);
-            cudaMemset(ctx->d_tcstat, 0, 2 * sizeof(unsigned long long));
             return FRNN_OK;
         case FRNN_OPT_KERNEL_TIMING:
             cudaStreamSynchronize(ctx->stream);
